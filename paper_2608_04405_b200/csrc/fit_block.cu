@@ -1,0 +1,990 @@
+// Algorithm 1 (fit) in blocks of 32 bits: four kernels per block instead of one pass over the keys per bit.
+//
+// Algorithm 1 decides bit i of every key by t = R_i d_i (R_i = K - sum_{j<i} u_j v_j, d_i the caller's direction) and forms
+// v_i = u_i^T R_i / n.  With the plain rule (no power iterations) all directions are known from the start, so what a bit
+// needs from its predecessors is not the residual rows but only the scalars c_{j,i} = v_j . d_i:
+//     t_i = (K D^T)_i - sum_{j<i} u_j c_{j,i}.
+// Per block of 32 bits:
+//   * project: T = K D_blk^T - U_prev C_prev for the block's 32 columns, one key per row; both terms are contractions and
+//     run on the tensor cores (directions and scalars as three bf16 terms each: 24 mantissa bits, products exact).
+//   * sweep: the 32 sequential bits on T alone.  A key costs 4 bytes of new data per bit (its entry of the next column)
+//     where the row pass costs 272.  Pass j decides bit j from column j and already sums u_i T[:, j+1] for all i <= j;
+//     those sums and the agreement counts u_j . u_i give c_{i,j+1} by forward substitution in fp64, because
+//     n c_{i,l} = u_i^T T_l - sum_{m<i} (u_i . u_m) c_{m,l}.  One thread block cluster per unit: the exchange per bit is a
+//     few hundred bytes through distributed shared memory and one cluster barrier.
+//   * gather: W = U_blk^T K and the agreement counts of the block's bits with all bits so far (tensor cores again, the key
+//     tile read channel-major).
+//   * rows: v_i = (W_i - sum_{j<i} (u_i . u_j) v_j) / n in fp64, then the next block's scalars C = V D_next^T in fp64.
+// The keys are read twice per 32 bits instead of 32 times.  fp32 caches take CUDA-core versions of project and gather.
+#include <mutex>
+#include "umma.cuh"
+#include "fit_block.h"
+
+namespace {
+using namespace umma;
+
+constexpr int kTileKeys = 128;
+constexpr int kGroupThreads = 128;
+constexpr int kTileBytes = kTileKeys * 256;
+constexpr int kBits = 32;                                  // bits of a block = one code word
+
+__device__ __forceinline__ void group_sync(int g) { asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "r"(kGroupThreads) : "memory"); }
+
+// 32 consecutive accumulator columns of this thread's TMEM lane (no wait: several can be in flight)
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+               "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
+                 "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
+                 "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
+                 "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+               : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// signs of bits s, s + 1 of x as a pair of bf16 (1 -> +1, 0 -> -1)
+__device__ __forceinline__ uint32_t sign_pair(uint32_t x, int s) {
+  const uint32_t nx = ~x;
+  const uint32_t lo = s <= 15 ? nx << (15 - s) : nx >> (s - 15);
+  const uint32_t hi = nx << (30 - s);
+  return 0x3F803F80u | (lo & 0x8000u) | (hi & 0x80000000u);
+}
+
+__device__ __forceinline__ void split3(float v, __nv_bfloat16 (&t)[3]) {   // v = t0 + t1 + t2 (24 mantissa bits)
+  t[0] = __float2bfloat16_rn(v);
+  const float r1 = v - __bfloat162float(t[0]);
+  t[1] = __float2bfloat16_rn(r1);
+  t[2] = __float2bfloat16_rn(r1 - __bfloat162float(t[1]));
+}
+
+// 32 x 32 bit transpose across the lanes of a warp: lane i returns bit i of every lane
+__device__ __forceinline__ uint32_t warp_transpose(uint32_t x, int lane) {
+  uint32_t m = 0x0000FFFFu;
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) {
+    const uint32_t y = __shfl_xor_sync(0xffffffffu, x, o);
+    x = (lane & o) ? ((x & ~m) | ((y >> o) & m)) : ((x & m) | ((y & m) << o));
+    m ^= m << (o >> 1);
+  }
+  return x;
+}
+
+// rows of a unit that block `blk` of `blocks` takes: equal shares of whole tiles
+__host__ __device__ inline int block_rows(int n, int blocks) { return ((n + blocks - 1) / blocks + kTileKeys - 1) / kTileKeys * kTileKeys; }
+
+// --------------------------------------------------------------------------- project (tensor cores, bf16 caches)
+// T[l][key] for the 32 columns of block `blk`.  Per tile of 128 keys: eight MMAs K_tile x D (N = 96: three bf16 terms of
+// the 32 directions), then two MMAs per earlier code word, U x (-C), into the same accumulator.  GROUPS warpgroups with
+// their own tile, sign operand and accumulator; a tile's buffer is refilled as soon as its K MMAs are done, so the next
+// load runs under the sign part and the 32 column stores.
+constexpr int kSignCols = 96;                              // signs expanded at a time (three words)
+constexpr int kProjN = 3 * kBits;
+
+template <int GROUPS>
+__global__ void __launch_bounds__(kGroupThreads * GROUPS, 1)
+fit_project_tc_kernel(const __nv_bfloat16* __restrict__ k_cache, const uint32_t* __restrict__ hfit, const float* __restrict__ v_star,
+                      const float* __restrict__ cross, float* __restrict__ T, const int32_t* __restrict__ unit_lens,
+                      int32_t* __restrict__ err, int n_max, int row_stride, int b, int blk, int t_stride) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  constexpr int kThreads = kGroupThreads * GROUPS;
+  constexpr int U_BYTES = kTileKeys * kSignCols * 2;
+  constexpr unsigned U_LBO = (kTileKeys / 8) * 128, C_LBO = (kProjN / 8) * 128;
+  const int tid = threadIdx.x, warp = tid >> 5;
+  const int grp = tid / kGroupThreads, gtid = tid % kGroupThreads;
+  unsigned char* a_t = smem + (size_t)grp * kTileBytes;
+  unsigned char* b_s = smem + (size_t)GROUPS * kTileBytes;             // directions, three terms: [96 x 128], 128-byte swizzle
+  unsigned char* u_s = b_s + kProjN * 256 + (size_t)grp * U_BYTES;     // this warpgroup's signs: [128 x 96], no swizzle
+  unsigned char* c_s = b_s + kProjN * 256 + (size_t)GROUPS * U_BYTES;  // -C, three terms: [96 x 32 blk], no swizzle
+  __shared__ unsigned long long bar_s[GROUPS];
+  __shared__ uint32_t tmem_base_s;
+  __shared__ int timed_out_g[GROUPS];
+  const int unit = blockIdx.y;
+  const int n = min(unit_lens[unit], n_max);
+  const int rows = block_rows(n, gridDim.x);
+  const int row0 = blockIdx.x * rows;
+  if (row0 >= n) return;                                               // uniform over the block, nothing set up yet
+  const int row_end = min(n, row0 + rows);
+  const int ntile = (row_end - row0 + kTileKeys - 1) / kTileKeys;
+  const int words = b / 32;
+
+  if (tid == 0) {
+    for (int g = 0; g < GROUPS; ++g) { mbar_init(&bar_s[g], 1); timed_out_g[g] = 0; }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"(512) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  const unsigned char* kbase = reinterpret_cast<const unsigned char*>(k_cache) + (size_t)unit * n_max * (size_t)row_stride * 2;
+  auto load_tile = [&](int tile) {                                     // rows past the end are zero-filled
+    const int r0 = row0 + tile * kTileKeys;
+    for (int c = gtid; c < kTileKeys * 16; c += kGroupThreads) {
+      const int r = c >> 4, ch = c & 15;
+      unsigned char* d = a_t + sw128_offset(kTileKeys, r, ch);
+      if (r0 + r < row_end) cp_async16(d, kbase + (size_t)(r0 + r) * row_stride * 2 + ch * 16);
+      else *reinterpret_cast<uint4*>(d) = make_uint4(0u, 0u, 0u, 0u);
+    }
+    cp_async_commit();
+  };
+  if (grp < ntile) load_tile(grp);
+  for (int c = tid; c < kBits * BPC_D; c += kThreads) {
+    const int l = c >> 7, ch = c & 127;
+    __nv_bfloat16 t3[3];
+    split3(v_star[((size_t)unit * b + kBits * blk + l) * BPC_D + ch], t3);
+#pragma unroll
+    for (int p = 0; p < 3; ++p)
+      *reinterpret_cast<__nv_bfloat16*>(b_s + sw128_offset(kProjN, p * kBits + l, ch >> 3) + (size_t)(ch & 7) * 2) = t3[p];
+  }
+  for (int c = tid; c < kBits * blk * kBits; c += kThreads) {
+    const int j = c >> 5, l = c & 31;                                  // earlier bit, column
+    __nv_bfloat16 t3[3];
+    split3(-cross[((size_t)unit * b + j) * kBits + l], t3);
+#pragma unroll
+    for (int p = 0; p < 3; ++p) *reinterpret_cast<__nv_bfloat16*>(c_s + nosw_offset(kProjN, p * kBits + l, j)) = t3[p];
+  }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem_all = tmem_base_s;
+  const uint32_t tm_d = tmem_all + (uint32_t)(grp * kProjN);
+  const uint32_t lane_off = (uint32_t)(32 * (warp & 3)) << 16;
+  unsigned long long* bar = &bar_s[grp];
+  const uint32_t idesc = umma_idesc_bf16(kTileKeys, kProjN);
+
+  unsigned ph = 0;
+  for (int tl = grp; tl < ntile; tl += GROUPS) {
+    const int row = row0 + tl * kTileKeys + gtid;
+    const bool live = row < row_end;
+    const uint32_t* hrow = hfit + ((size_t)unit * n_max + (live ? row : row0)) * words;
+    uint32_t first[kSignCols / 32];                                    // (requested before the wait for the tile)
+#pragma unroll
+    for (int w = 0; w < kSignCols / 32; ++w) first[w] = w < blk ? hrow[w] : 0u;
+    cp_async_wait_all();
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    group_sync(grp);                                                   // the tile has landed for all 128 threads
+    if (timed_out_g[grp]) break;                                       // (set before a barrier, so all 128 threads agree)
+    if (gtid == 0) {
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+      for (int ks = 0; ks < 8; ++ks) {
+        const size_t aoff = (size_t)(ks >> 2) * (kTileKeys * 128) + (size_t)(ks & 3) * 32;
+        const size_t boff = (size_t)(ks >> 2) * (kProjN * 128) + (size_t)(ks & 3) * 32;
+        umma_bf16(tm_d, umma_desc_sw128(a_t + aoff), umma_desc_sw128(b_s + boff), idesc, ks > 0 ? 1u : 0u);
+      }
+      umma_commit(bar);
+    }
+    bool refilled = false;
+    for (int w0 = 0; w0 < blk; w0 += kSignCols / 32) {                 // (one round for up to 128-bit codes)
+      const int wn = min(blk - w0, kSignCols / 32);
+      if (w0 > 0) {                                                    // the previous round's MMAs have read the operand
+        if (!mbar_wait(bar, ph)) timed_out_g[grp] = 1;
+        ph ^= 1u;
+      }
+#pragma unroll
+      for (int w = 0; w < kSignCols / 32; ++w) {
+        if (w >= wn) break;
+        const uint32_t x = w0 == 0 ? first[w] : hrow[w0 + w];
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          *reinterpret_cast<uint4*>(u_s + (size_t)(4 * w + c) * U_LBO + (size_t)(gtid >> 3) * 128 + (size_t)(gtid & 7) * 16) =
+              make_uint4(sign_pair(x, 8 * c), sign_pair(x, 8 * c + 2), sign_pair(x, 8 * c + 4), sign_pair(x, 8 * c + 6));
+      }
+      if (w0 == 0) {                                                   // the K MMAs are done: refill the tile under the rest
+        if (!mbar_wait(bar, ph)) timed_out_g[grp] = 1;
+        ph ^= 1u;
+        if (tl + GROUPS < ntile) load_tile(tl + GROUPS);
+        refilled = true;
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      group_sync(grp);
+      if (gtid == 0) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        for (int ks = 0; ks < 2 * wn; ++ks)
+          umma_bf16(tm_d, umma_desc_nosw(u_s + (size_t)ks * 2 * U_LBO, U_LBO, 128),
+                    umma_desc_nosw(c_s + (size_t)(4 * w0 + 2 * ks) * C_LBO, C_LBO, 128), idesc, 1u);
+        umma_commit(bar);
+      }
+    }
+    if (!mbar_wait(bar, ph)) timed_out_g[grp] = 1;
+    ph ^= 1u;
+    if (!refilled && tl + GROUPS < ntile) load_tile(tl + GROUPS);
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    uint32_t r0[32], r1[32], r2[32];
+    tmem_ld32(tm_d + lane_off, r0);
+    tmem_ld32(tm_d + lane_off + 32, r1);
+    tmem_ld32(tm_d + lane_off + 64, r2);
+    tmem_wait_ld();
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    float* dst = T + (size_t)unit * kBits * t_stride + row;            // (rows of the last tile past the end: zeros)
+#pragma unroll
+    for (int l = 0; l < kBits; ++l) {
+      const float v = (__uint_as_float(r0[l]) + __uint_as_float(r1[l])) + __uint_as_float(r2[l]);
+      dst[(size_t)l * t_stride] = live ? v : 0.f;
+    }
+  }
+  if (timed_out_g[grp] && gtid == 0) atomicOr(err, BPC_DEVERR_TIMEOUT);
+  cp_async_wait_all();
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_all), "r"(512) : "memory");
+}
+
+// --------------------------------------------------------------------------- project (CUDA cores, fp32 caches)
+// One thread per key: dot products in fp32 over 16 channels (or 32 earlier bits) at a time, added in fp64.
+__global__ void __launch_bounds__(kTileKeys)
+fit_project_f32_kernel(const float* __restrict__ k_cache, const uint32_t* __restrict__ hfit, const float* __restrict__ v_star,
+                       const float* __restrict__ cross, float* __restrict__ T, const int32_t* __restrict__ unit_lens,
+                       int n_max, int row_stride, int b, int blk, int t_stride) {
+  const int unit = blockIdx.y, tid = threadIdx.x;
+  const int n = min(unit_lens[unit], n_max);
+  const int row = blockIdx.x * kTileKeys + tid;
+  if (blockIdx.x * kTileKeys >= n) return;
+  const bool live = row < n;
+  __shared__ __align__(16) float d_s[BPC_D][kBits];                    // directions, channel-major; then the scalars of 32 bits
+  double acc[kBits];
+#pragma unroll
+  for (int l = 0; l < kBits; ++l) acc[l] = 0.0;
+  for (int c = tid; c < kBits * BPC_D; c += kTileKeys) d_s[c & 127][c >> 7] = v_star[((size_t)unit * b + kBits * blk + (c >> 7)) * BPC_D + (c & 127)];
+  __syncthreads();
+  const float4* kr = reinterpret_cast<const float4*>(k_cache + ((size_t)unit * n_max + (live ? row : 0)) * row_stride);
+  for (int c0 = 0; c0 < BPC_D; c0 += 16) {
+    float x[16], p[kBits];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) { const float4 q = kr[c0 / 4 + v]; x[4 * v] = q.x; x[4 * v + 1] = q.y; x[4 * v + 2] = q.z; x[4 * v + 3] = q.w; }
+#pragma unroll
+    for (int l = 0; l < kBits; ++l) p[l] = 0.f;
+#pragma unroll
+    for (int c = 0; c < 16; ++c)
+#pragma unroll
+      for (int l = 0; l < kBits; ++l) p[l] = fmaf(x[c], d_s[c0 + c][l], p[l]);
+#pragma unroll
+    for (int l = 0; l < kBits; ++l) acc[l] += (double)p[l];
+  }
+  for (int w = 0; w < blk; ++w) {
+    __syncthreads();
+    for (int c = tid; c < kBits * kBits; c += kTileKeys) d_s[c >> 5][c & 31] = cross[((size_t)unit * b + 32 * w + (c >> 5)) * kBits + (c & 31)];
+    __syncthreads();
+    const uint32_t x = hfit[((size_t)unit * n_max + (live ? row : 0)) * (b / 32) + w];
+    float p[kBits];
+#pragma unroll
+    for (int l = 0; l < kBits; ++l) p[l] = 0.f;
+    for (int j = 0; j < 32; ++j) {
+      const float u = ((x >> j) & 1u) ? 1.f : -1.f;
+#pragma unroll
+      for (int l = 0; l < kBits; ++l) p[l] = fmaf(u, d_s[j][l], p[l]);
+    }
+#pragma unroll
+    for (int l = 0; l < kBits; ++l) acc[l] -= (double)p[l];
+  }
+  float* dst = T + (size_t)unit * kBits * t_stride + row;
+#pragma unroll
+  for (int l = 0; l < kBits; ++l) dst[(size_t)l * t_stride] = live ? (float)acc[l] : 0.f;
+}
+
+// --------------------------------------------------------------------------- gather (tensor cores, bf16 caches)
+// W[i][c] = sum over keys of u_i K[c] for the block's 32 bits, and the inner products u_i . u_j with all bits j so far.
+// Per tile of 128 keys the signs of all bits so far are laid out bit-major, U [bits x 128 keys] (each warp transposes its
+// 32 keys' code words across lanes, one lane then writes one bit's 32 keys); then eight MMAs K_tile^T (channel-major view of
+// the tile, M = 128 channels) x U_blk (N = 32) and eight (sixteen for 256-bit codes) U x U_blk.  Channel sums move to fp64
+// registers every kFlushTiles tiles (1024 rows); the inner products are integers below 2^24 and stay exact in fp32.
+constexpr int kGatherGroups = 2;
+constexpr int kFlushTiles = 8;
+
+template <int HALVES, int NBUF>                            // HALVES = 128-bit halves of a code, NBUF = key-tile buffers per warpgroup
+__global__ void __launch_bounds__(kGroupThreads * kGatherGroups, 1)
+fit_gather_tc_kernel(const __nv_bfloat16* __restrict__ k_cache, const uint32_t* __restrict__ hfit, double* __restrict__ wpart,
+                     int32_t* __restrict__ apart, const int32_t* __restrict__ unit_lens, int32_t* __restrict__ err, int n_max,
+                     int row_stride, int b, int blk) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  constexpr int kThreads = kGroupThreads * kGatherGroups;
+  constexpr int R = 128 * HALVES;                          // operand rows (bits)
+  constexpr int U_BYTES = R * kTileKeys * 2;
+  constexpr unsigned LBO = (R / 8) * 128;                  // bytes between core matrices along K (keys)
+  constexpr int kCols = 32 * (1 + HALVES);                 // accumulator columns of a warpgroup
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int grp = tid / kGroupThreads, gtid = tid % kGroupThreads;
+  unsigned char* a_g = smem + (size_t)grp * NBUF * kTileBytes;
+  unsigned char* u_s = smem + (size_t)kGatherGroups * NBUF * kTileBytes + (size_t)grp * U_BYTES;
+  __shared__ unsigned long long bar_s[kGatherGroups];
+  __shared__ uint32_t tmem_base_s;
+  __shared__ int timed_out_g[kGatherGroups];
+  const int unit = blockIdx.y, words = b / 32;
+  const int n = min(unit_lens[unit], n_max);
+  const int rows = block_rows(n, gridDim.x);
+  const int row0 = blockIdx.x * rows;
+  if (row0 >= n) return;                                   // (the reduction skips blocks without rows)
+  const int row_end = min(n, row0 + rows);
+  const int ntile = (row_end - row0 + kTileKeys - 1) / kTileKeys;
+  if (tid == 0) {
+    for (int g = 0; g < kGatherGroups; ++g) { mbar_init(&bar_s[g], 1); timed_out_g[g] = 0; }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"(256) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  const unsigned char* kbase = reinterpret_cast<const unsigned char*>(k_cache) + (size_t)unit * n_max * (size_t)row_stride * 2;
+  auto load_tile = [&](int tile, int buf) {                // rows past the end are zero-filled
+    const int r0 = row0 + tile * kTileKeys;
+    unsigned char* a = a_g + (size_t)buf * kTileBytes;
+    for (int c = gtid; c < kTileKeys * 16; c += kGroupThreads) {
+      const int r = c >> 4, ch = c & 15;
+      unsigned char* d = a + sw128_offset(kTileKeys, r, ch);
+      if (r0 + r < row_end) cp_async16(d, kbase + (size_t)(r0 + r) * row_stride * 2 + ch * 16);
+      else *reinterpret_cast<uint4*>(d) = make_uint4(0u, 0u, 0u, 0u);
+    }
+    cp_async_commit();
+  };
+  uint32_t nxt[4 * HALVES];                                // code words of this thread's key of the next tile
+  auto load_words = [&](int tile) {
+    const int r = row0 + tile * kTileKeys + gtid;
+    const uint32_t* h = hfit + ((size_t)unit * n_max + r) * words;
+#pragma unroll
+    for (int w = 0; w < 4 * HALVES; ++w) nxt[w] = (w <= blk && r < row_end) ? h[w] : 0u;
+  };
+  if (grp < ntile) { load_tile(grp, 0); load_words(grp); }
+  for (int i = tid; i < kGatherGroups * U_BYTES / 16; i += kThreads)   // rows of bits to come stay zero
+    reinterpret_cast<uint4*>(smem + (size_t)kGatherGroups * NBUF * kTileBytes)[i] = make_uint4(0u, 0u, 0u, 0u);
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem_all = tmem_base_s;
+  const uint32_t tm_w = tmem_all + (uint32_t)(grp * kCols), tm_a = tm_w + 32;
+  const uint32_t lane_off = (uint32_t)(32 * (warp & 3)) << 16;
+  unsigned long long* bar = &bar_s[grp];
+  const uint32_t idesc = umma_idesc_bf16(128, kBits);
+  double acc[kBits];                                       // channel gtid
+#pragma unroll
+  for (int i = 0; i < kBits; ++i) acc[i] = 0.0;
+  unsigned ph = 0;
+  bool pend = false;
+  int since_flush = 0, idx = 0;
+  for (int tl = grp; tl < ntile; tl += kGatherGroups, ++idx) {
+    const int buf = NBUF == 2 ? (idx & 1) : 0;
+    const unsigned char* a = a_g + (size_t)buf * kTileBytes;
+    uint32_t mine[4 * HALVES];
+#pragma unroll
+    for (int w = 0; w < 4 * HALVES; ++w) mine[w] = nxt[w];
+    if (tl + kGatherGroups < ntile) load_words(tl + kGatherGroups);
+    if (pend) {                                            // the previous tile's MMAs: their operands are free afterwards
+      if (!mbar_wait(bar, ph)) timed_out_g[grp] = 1;
+      ph ^= 1u;
+      pend = false;
+      if (NBUF == 1) load_tile(tl, 0);
+    }
+    if (NBUF == 2 && tl + kGatherGroups < ntile) load_tile(tl + kGatherGroups, buf ^ 1);
+    // this warp's 32 keys, one bit per lane; keys past the end become 0 instead of +-1
+    const int r_w = row0 + tl * kTileKeys + 32 * (warp & 3);
+    const int live = min(max(row_end - r_w, 0), 32);
+#pragma unroll
+    for (int w = 0; w < 4 * HALVES; ++w) {
+      if (w > blk) break;
+      const uint32_t m = warp_transpose(mine[w], lane);
+      unsigned char* dst = u_s + (size_t)(4 * (warp & 3)) * LBO + (size_t)(32 * w + lane) * 16;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        uint32_t h[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) h[e] = sign_pair(m, 8 * c + 2 * e);
+        if (live < 32) {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int k0 = 8 * c + 2 * e;
+            h[e] &= (k0 < live ? 0xFFFFu : 0u) | (k0 + 1 < live ? 0xFFFF0000u : 0u);
+          }
+        }
+        *reinterpret_cast<uint4*>(dst + (size_t)c * LBO) = make_uint4(h[0], h[1], h[2], h[3]);
+      }
+    }
+    if (NBUF == 2 && tl + kGatherGroups < ntile) asm volatile("cp.async.wait_group 1;" ::: "memory");
+    else cp_async_wait_all();
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");   // (a flush's accumulator reads are done)
+    group_sync(grp);
+    if (timed_out_g[grp]) break;
+    if (gtid == 0) {
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const unsigned char* ub = u_s + (size_t)(4 * blk) * 128;          // rows of this block's 32 bits
+#pragma unroll
+      for (int ks = 0; ks < 8; ++ks)
+        umma_bf16(tm_w, umma_desc_sw128_mn(a + (size_t)ks * 2048, 16384, 1024), umma_desc_nosw(ub + (size_t)ks * 2 * LBO, LBO, 128),
+                  idesc | kIdescAMnMajor, (since_flush > 0 || ks > 0) ? 1u : 0u);
+#pragma unroll
+      for (int hf = 0; hf < HALVES; ++hf) {
+        if (4 * hf > blk) break;
+#pragma unroll
+        for (int ks = 0; ks < 8; ++ks)
+          umma_bf16(tm_a + (uint32_t)(32 * hf), umma_desc_nosw(u_s + (size_t)hf * 2048 + (size_t)ks * 2 * LBO, LBO, 128),
+                    umma_desc_nosw(ub + (size_t)ks * 2 * LBO, LBO, 128), idesc, (idx > 0 || ks > 0) ? 1u : 0u);
+      }
+      umma_commit(bar);
+    }
+    pend = true;
+    ++since_flush;
+    if (since_flush == kFlushTiles || tl + kGatherGroups >= ntile) {
+      if (!mbar_wait(bar, ph)) timed_out_g[grp] = 1;
+      ph ^= 1u;
+      pend = false;
+      if (NBUF == 1 && tl + kGatherGroups < ntile) load_tile(tl + kGatherGroups, 0);
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      uint32_t r[32];
+      tmem_ld32(tm_w + lane_off, r);
+      tmem_wait_ld();
+#pragma unroll
+      for (int i = 0; i < kBits; ++i) acc[i] += (double)__uint_as_float(r[i]);
+      since_flush = 0;
+    }
+  }
+  if (timed_out_g[grp] && gtid == 0) atomicOr(err, BPC_DEVERR_TIMEOUT);
+  cp_async_wait_all();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  __syncthreads();                                         // the tile buffers are free in both warpgroups
+  double* red = reinterpret_cast<double*>(smem);           // [groups][32][128]
+#pragma unroll
+  for (int i = 0; i < kBits; ++i) red[((size_t)grp * kBits + i) * BPC_D + gtid] = acc[i];
+  int32_t* redc = reinterpret_cast<int32_t*>(smem + (size_t)kGatherGroups * kBits * BPC_D * 8);   // [groups][R][33]
+#pragma unroll
+  for (int hf = 0; hf < HALVES; ++hf) {
+    uint32_t r[32];
+    tmem_ld32(tm_a + (uint32_t)(32 * hf) + lane_off, r);
+    tmem_wait_ld();
+    const bool any = grp < ntile && 4 * hf <= blk;
+#pragma unroll
+    for (int i = 0; i < kBits; ++i) redc[((size_t)grp * R + 128 * hf + gtid) * 33 + i] = any ? (int)__uint_as_float(r[i]) : 0;
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  double* wo = wpart + ((size_t)unit * gridDim.x + blockIdx.x) * kBits * BPC_D;
+  for (int e = tid; e < kBits * BPC_D; e += kThreads) wo[e] = red[e] + red[kBits * BPC_D + e];
+  int32_t* ao = apart + ((size_t)unit * gridDim.x + blockIdx.x) * kBits * b;
+  const int nj = kBits * (blk + 1);
+  for (int e = tid; e < kBits * nj; e += kThreads) {
+    const int i = e / nj, j = e % nj;
+    ao[(size_t)i * b + j] = redc[(size_t)j * 33 + i] + redc[((size_t)R + j) * 33 + i];
+  }
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_all), "r"(256) : "memory");
+}
+
+// --------------------------------------------------------------------------- gather (CUDA cores, fp32 caches)
+// Thread (half, channel) adds +-K over at most 1024 rows in fp32; the inner products come from ballots: lane i holds bit i of
+// the block over a warp's 32 keys, every earlier bit's 32 keys are one broadcast word.
+__global__ void __launch_bounds__(256)
+fit_gather_f32_kernel(const float* __restrict__ k_cache, const uint32_t* __restrict__ hfit, double* __restrict__ wpart,
+                      int32_t* __restrict__ apart, const int32_t* __restrict__ unit_lens, int n_max, int row_stride, int b, int blk) {
+  const int unit = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, words = b / 32;
+  const int n = min(unit_lens[unit], n_max);
+  const int rows = block_rows(n, gridDim.x);
+  const int row0 = blockIdx.x * rows;
+  if (row0 >= n) return;
+  const int row_end = min(n, row0 + rows);
+  __shared__ int cnt_s[kBits][256 + 1];
+  for (int e = tid; e < kBits * 257; e += 256) (&cnt_s[0][0])[e] = 0;
+  const int half = tid >> 7, c = tid & 127;
+  double acc64[kBits];
+#pragma unroll
+  for (int i = 0; i < kBits; ++i) acc64[i] = 0.0;
+  const uint32_t* h = hfit + (size_t)unit * n_max * words;
+  for (int r0 = row0; r0 < row_end; r0 += 1024) {
+    float acc[kBits];
+#pragma unroll
+    for (int i = 0; i < kBits; ++i) acc[i] = 0.f;
+    for (int r = r0 + half; r < min(row_end, r0 + 1024); r += 2) {
+      const float x = k_cache[((size_t)unit * n_max + r) * row_stride + c];
+      const uint32_t w = h[(size_t)r * words + blk];
+#pragma unroll
+      for (int i = 0; i < kBits; ++i) acc[i] += ((w >> i) & 1u) ? x : -x;
+    }
+#pragma unroll
+    for (int i = 0; i < kBits; ++i) acc64[i] += (double)acc[i];
+  }
+  __syncthreads();
+  for (int r0 = row0 + 32 * warp; r0 < row_end; r0 += 256) {
+    const int r = r0 + lane;
+    const uint32_t live = __ballot_sync(0xffffffffu, r < row_end);
+    const uint32_t mine = warp_transpose(r < row_end ? h[(size_t)r * words + blk] : 0u, lane);   // bit `lane` of the block
+    for (int w = 0; w <= blk; ++w) {
+      const uint32_t other = warp_transpose(r < row_end ? h[(size_t)r * words + w] : 0u, lane);
+      for (int j = 0; j < 32; ++j) {
+        const uint32_t x = __shfl_sync(0xffffffffu, other, j);
+        const int d = __popc(live) - 2 * __popc((mine ^ x) & live);
+        atomicAdd(&cnt_s[lane][32 * w + j], d);
+      }
+    }
+  }
+  double* wo = wpart + ((size_t)unit * gridDim.x + blockIdx.x) * kBits * BPC_D;
+  if (half == 0)
+    for (int i = 0; i < kBits; ++i) wo[(size_t)i * BPC_D + c] = acc64[i];
+  __syncthreads();
+  if (half == 1)
+    for (int i = 0; i < kBits; ++i) wo[(size_t)i * BPC_D + c] += acc64[i];
+  int32_t* ao = apart + ((size_t)unit * gridDim.x + blockIdx.x) * kBits * b;
+  const int nj = kBits * (blk + 1);
+  for (int e = tid; e < kBits * nj; e += 256) ao[(size_t)(e / nj) * b + e % nj] = cnt_s[e / nj][e % nj];
+}
+
+// --------------------------------------------------------------------------- sweep
+// The 32 sequential bits of a block on the columns T.  Block r of the unit's cluster owns an equal share of the keys; a
+// thread takes four consecutive keys at a time.  Per key and bit: subtract sum_i u_i c_i (two table look-ups per eight
+// bits), decide, and add the next column's entry to the running sums of the bits that are set (the sum over set bits
+// gives u_i^T T = 2 sum - total).  Agreements with the earlier bits are counted bit-sliced, 32 bits per operation.
+// The loop body is compiled for 8, 16, 24 and 32 bits in play.
+constexpr int kSweepThreads = 512;
+constexpr int kSweepWarps = kSweepThreads / 32;
+constexpr int kSweepPlanes = 8;
+constexpr int kSweepFlush = 60;                            // rounds of four keys between flushes: 240 < 2^kSweepPlanes counts
+
+struct SweepSums {                                         // lane i: bit i
+  double s, tot;
+  int cnt;
+};
+
+// values v[0..N-1] of every lane summed over the warp: lane l returns the sum of v[l] (l & (N - 1) for N < 32)
+template <int N>
+__device__ __forceinline__ float warp_sum_scatter(float (&v)[N], int lane) {
+  static_assert(N == 8 || N == 16 || N == 32, "");
+#pragma unroll
+  for (int o = 16; o >= N; o >>= 1)
+#pragma unroll
+    for (int i = 0; i < N; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+#pragma unroll
+  for (int o = N / 2; o >= 1; o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < o; ++i) {
+      const float keep = up ? v[i + o] : v[i], give = up ? v[i] : v[i + o];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+  }
+  return v[0];
+}
+
+__device__ __forceinline__ void full_add(uint32_t a, uint32_t b, uint32_t c, uint32_t& s, uint32_t& cy) {
+  s = a ^ b ^ c;
+  cy = (a & b) | (c & (a | b));
+}
+
+// One pass over this block's keys: decides bit j; unless it is the block's last bit, also the sums for column j + 1.
+template <int JB, bool LAST>
+__device__ __forceinline__ void sweep_pass(const float* __restrict__ tc, const float* __restrict__ tn, uint32_t* __restrict__ ws,
+                                           const float* __restrict__ lut, int j, int nk, int nkeys, int warp, int lane, SweepSums& out) {
+  constexpr int NS = JB == 3 ? 32 : 8 * JB;                // running sums (a power of two for the warp reduction)
+  out.s = out.tot = 0.0;
+  out.cnt = 0;
+  const uint32_t bit = 1u << j;
+  for (int g0 = warp; g0 < nk / 128; g0 += kSweepWarps * kSweepFlush) {
+    float s[NS];
+    float tot = 0.f;
+    uint32_t pl[kSweepPlanes];
+#pragma unroll
+    for (int i = 0; i < NS; ++i) s[i] = 0.f;
+#pragma unroll
+    for (int k = 0; k < kSweepPlanes; ++k) pl[k] = 0u;
+    const int g1 = min(nk / 128, g0 + kSweepWarps * kSweepFlush);
+    float4 t4 = *reinterpret_cast<const float4*>(tc + g0 * 128 + 4 * lane), n4;
+    if (!LAST) n4 = *reinterpret_cast<const float4*>(tn + g0 * 128 + 4 * lane);
+    for (int g = g0; g < g1; g += kSweepWarps) {
+      const int key = g * 128 + 4 * lane;
+      const float t[4] = {t4.x, t4.y, t4.z, t4.w};
+      const float nx[4] = {n4.x, n4.y, n4.z, n4.w};
+      if (g + kSweepWarps < g1) {                          // (requested one round ahead)
+        t4 = *reinterpret_cast<const float4*>(tc + key + kSweepWarps * 128);
+        if (!LAST) n4 = *reinterpret_cast<const float4*>(tn + key + kSweepWarps * 128);
+      }
+      const uint4 w4 = *reinterpret_cast<const uint4*>(ws + key);
+      uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w}, x[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        float c0 = 0.f, c1 = 0.f;
+#pragma unroll
+        for (int nb = 0; nb < 2 * JB; nb += 2) {
+          c0 += lut[nb * 16 + ((w[e] >> (4 * nb)) & 15u)];
+          c1 += lut[nb * 16 + 16 + ((w[e] >> (4 * nb + 4)) & 15u)];
+        }
+        const bool pos = t[e] - (c0 + c1) >= 0.f;
+        x[e] = pos ? w[e] : ~w[e];
+        w[e] |= pos ? bit : 0u;
+        if (!LAST) {
+          tot += nx[e];
+#pragma unroll
+          for (int i = 0; i < 8 * JB; ++i)
+            if (w[e] & (1u << i)) s[i] += nx[e];
+        }
+      }
+      *reinterpret_cast<uint4*>(ws + key) = make_uint4(w[0], w[1], w[2], w[3]);
+      if (!LAST) {
+        if (key + 4 > nkeys) {                             // keys past the end agree with nothing
+#pragma unroll
+          for (int e = 0; e < 4; ++e) if (key + e >= nkeys) x[e] = 0u;
+        }
+        uint32_t s1, ca, cb, cc;
+        full_add(x[0], x[1], x[2], s1, ca);
+        full_add(pl[0], s1, x[3], pl[0], cb);
+        full_add(pl[1], ca, cb, pl[1], cc);
+#pragma unroll
+        for (int k = 2; k < kSweepPlanes; ++k) {
+          const uint32_t nc = pl[k] & cc;
+          pl[k] ^= cc;
+          cc = nc;
+        }
+      }
+    }
+    if (!LAST) {
+      out.s += (double)warp_sum_scatter<NS>(s, lane);
+#pragma unroll
+      for (int o = 16; o >= 1; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+      out.tot += (double)tot;
+      const int keys_per_lane = 4 * ((g1 - g0 + kSweepWarps - 1) / kSweepWarps);
+#pragma unroll
+      for (int k = 0; k < kSweepPlanes; ++k) {
+        if ((keys_per_lane >> k) == 0) break;              // higher planes are empty
+        out.cnt += __popc(warp_transpose(pl[k], lane)) << k;
+      }
+    }
+  }
+}
+
+template <bool SMEM_WORDS>
+__global__ void __launch_bounds__(kSweepThreads, 1)
+fit_sweep_kernel(const float* __restrict__ T, uint32_t* __restrict__ hfit, uint32_t* __restrict__ words_g,
+                 const int32_t* __restrict__ unit_lens, int n_max, int b, int blk, int t_stride, int cluster_size) {
+  extern __shared__ __align__(16) uint32_t words_s[];
+  __shared__ __align__(16) float lut[8 * 16];              // lut[nibble][pattern] = sum of +-c over the nibble's bits
+  __shared__ double red_s[kSweepWarps][32], red_t[kSweepWarps];
+  __shared__ int red_c[kSweepWarps][32];
+  __shared__ double slot_s[2][BPC_MAX_CLUSTER][32];        // the cluster's sums of bit i, by rank; two passes alternate
+  __shared__ int slot_c[2][BPC_MAX_CLUSTER][32];
+  __shared__ double agree[32][33];                         // u_i . u_m
+  __shared__ float c_s[32];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int rank = blockIdx.x % cluster_size, unit = blockIdx.x / cluster_size;
+  const int n = min(unit_lens[unit], n_max);
+  if (n <= 0) return;                                      // (the whole cluster)
+  const int share = block_rows(n, cluster_size);
+  const int row0 = rank * share;
+  const int nkeys = max(0, min(n - row0, share));          // keys of this block; nk = the same in whole groups of 128
+  const int nk = (nkeys + 127) / 128 * 128;
+  uint32_t* ws = SMEM_WORDS ? words_s : words_g + (size_t)unit * t_stride + row0;
+  for (int i = tid; i < nk / 4; i += kSweepThreads) reinterpret_cast<uint4*>(ws)[i] = make_uint4(0u, 0u, 0u, 0u);
+  if (tid < 128) lut[tid] = 0.f;
+  __syncthreads();
+  const float* Tu = T + (size_t)unit * kBits * t_stride + row0;
+  const double inv_n = 1.0 / (double)n;
+  for (int j = 0; j < kBits; ++j) {
+    const float* tc = Tu + (size_t)j * t_stride;
+    SweepSums sums;
+    if (j == kBits - 1) { sweep_pass<4, true>(tc, tc, ws, lut, j, nk, nkeys, warp, lane, sums); break; }
+    if (j < 8) sweep_pass<1, false>(tc, tc + t_stride, ws, lut, j, nk, nkeys, warp, lane, sums);
+    else if (j < 16) sweep_pass<2, false>(tc, tc + t_stride, ws, lut, j, nk, nkeys, warp, lane, sums);
+    else if (j < 24) sweep_pass<3, false>(tc, tc + t_stride, ws, lut, j, nk, nkeys, warp, lane, sums);
+    else sweep_pass<4, false>(tc, tc + t_stride, ws, lut, j, nk, nkeys, warp, lane, sums);
+    red_s[warp][lane] = sums.s;
+    red_c[warp][lane] = sums.cnt;
+    if (lane == 0) red_t[warp] = sums.tot;
+    __syncthreads();
+    const int buf = j & 1;
+    if (warp == 0) {
+      double s = 0.0, tot = 0.0;
+      int c = 0;
+#pragma unroll
+      for (int w = 0; w < kSweepWarps; ++w) { s += red_s[w][lane]; tot += red_t[w]; c += red_c[w][lane]; }
+      s = 2.0 * s - tot;                                   // u_lane^T T[:, j + 1] over this block's keys
+      const unsigned as = (unsigned)__cvta_generic_to_shared(&slot_s[buf][rank][lane]);
+      const unsigned ac = (unsigned)__cvta_generic_to_shared(&slot_c[buf][rank][lane]);
+      for (int r = 0; r < cluster_size; ++r) {
+        unsigned ps, pc;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ps) : "r"(as), "r"(r));
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(pc) : "r"(ac), "r"(r));
+        asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(ps), "d"(s) : "memory");
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(pc), "r"(c) : "memory");
+      }
+    }
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (warp == 0) {
+      double s = 0.0;
+      int c = 0;
+      for (int r = 0; r < cluster_size; ++r) { s += slot_s[buf][r][lane]; c += slot_c[buf][r][lane]; }
+      agree[j][lane] = (double)(2 * (long long)c - (long long)n);        // u_j . u_lane (lane < j)
+      __syncwarp();
+      // c_{i,j+1} = (u_i^T T - sum_{m<i} (u_i . u_m) c_{m,j+1}) / n
+      double mine = 0.0;
+      for (int m = 0; m <= j; ++m) {
+        const double cm = __shfl_sync(0xffffffffu, s, m) * inv_n;
+        if (lane == m) mine = cm;
+        if (lane > m) s -= agree[lane][m] * cm;
+      }
+      c_s[lane] = lane <= j ? (float)mine : 0.f;
+      __syncwarp();
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int e = lane + 32 * q;
+        float v = 0.f;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) { const float d = c_s[4 * (e >> 4) + i]; v += ((e >> i) & 1) ? d : -d; }
+        lut[e] = v;
+      }
+    }
+    __syncthreads();
+  }
+  __syncthreads();
+  uint32_t* h = hfit + ((size_t)unit * n_max + row0) * (b / 32) + blk;
+  for (int i = tid; i < nkeys; i += kSweepThreads) h[(size_t)i * (b / 32)] = ws[i];
+}
+
+// --------------------------------------------------------------------------- rows and scalars
+// v_i = (W_i - sum_{j<i} (u_i . u_j) v_j) / n for the block's 32 bits, one block per unit; four thread groups split the
+// partial sums and the earlier bits, one thread per channel runs the block's own triangle in registers.  Fixed order.
+__global__ void __launch_bounds__(BPC_D * 4)
+fit_rows_kernel(const double* __restrict__ wpart, const int32_t* __restrict__ apart, float* __restrict__ P,
+                const int32_t* __restrict__ unit_lens, int n_max, int b, int blk, int parts) {
+  extern __shared__ __align__(16) double rows_smem[];
+  double* corr = rows_smem;                                // [32][32 (blk + 1)] u_i . u_j
+  double* w_s = corr + kBits * kBits * (blk + 1);          // [32][128]
+  const int unit = blockIdx.x, tid = threadIdx.x, c = tid & 127, q = tid >> 7;
+  const int n = min(unit_lens[unit], n_max);
+  float* Pu = P + (size_t)unit * b * BPC_D;
+  if (n <= 0) {
+    for (int e = tid; e < kBits * BPC_D; e += 512) Pu[(size_t)kBits * blk * BPC_D + e] = 0.f;
+    return;
+  }
+  const int rows = block_rows(n, parts), used = (n + rows - 1) / rows;
+  const int nj = kBits * (blk + 1);
+  for (int e = tid; e < kBits * nj; e += 512) {
+    long long a = 0;
+    for (int p = 0; p < used; ++p) a += apart[(((size_t)unit * parts + p) * kBits + e / nj) * b + e % nj];
+    corr[e] = (double)a;
+  }
+  __syncthreads();
+  for (int i0 = 8 * q; i0 < 8 * q + 8; i0 += 4) {          // group q: rows 8q .. 8q + 7
+    double acc[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[i] = 0.0;
+    for (int p = 0; p < used; ++p)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[i] += wpart[(((size_t)unit * parts + p) * kBits + i0 + i) * BPC_D + c];
+    for (int j = 0; j < kBits * blk; ++j) {
+      const double v = (double)Pu[(size_t)j * BPC_D + c];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[i] -= corr[(i0 + i) * nj + j] * v;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w_s[(i0 + i) * BPC_D + c] = acc[i];
+  }
+  __syncthreads();
+  if (q == 0) {
+    double w[kBits];
+#pragma unroll
+    for (int i = 0; i < kBits; ++i) w[i] = w_s[i * BPC_D + c];
+    const double inv_n = 1.0 / (double)n;
+#pragma unroll
+    for (int i = 0; i < kBits; ++i) {
+      const float v = (float)(w[i] * inv_n);
+      Pu[(size_t)(kBits * blk + i) * BPC_D + c] = v;
+#pragma unroll
+      for (int i2 = i + 1; i2 < kBits; ++i2) w[i2] -= corr[i2 * nj + kBits * blk + i] * (double)v;
+    }
+  }
+}
+
+// cross[j][l] = v_j . d_l for 32 bits j so far and the 32 columns l of block `blk`; grid (blk, units), fp64 sums
+__global__ void __launch_bounds__(256)
+fit_cross_kernel(const float* __restrict__ P, const float* __restrict__ v_star, float* __restrict__ cross, int b, int blk) {
+  __shared__ float v_s[kBits][BPC_D + 1], d_s[kBits][BPC_D + 1];
+  const int unit = blockIdx.y, w = blockIdx.x, tid = threadIdx.x;
+  for (int e = tid; e < kBits * BPC_D; e += 256) {
+    v_s[e >> 7][e & 127] = P[((size_t)unit * b + kBits * w) * BPC_D + e];
+    d_s[e >> 7][e & 127] = v_star[((size_t)unit * b + kBits * blk) * BPC_D + e];
+  }
+  __syncthreads();
+  const int l = tid & 31;
+  for (int j = tid >> 5; j < kBits; j += 8) {
+    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+#pragma unroll 8
+    for (int c = 0; c < BPC_D; c += 4) {
+      a0 = fma((double)v_s[j][c], (double)d_s[l][c], a0);
+      a1 = fma((double)v_s[j][c + 1], (double)d_s[l][c + 1], a1);
+      a2 = fma((double)v_s[j][c + 2], (double)d_s[l][c + 2], a2);
+      a3 = fma((double)v_s[j][c + 3], (double)d_s[l][c + 3], a3);
+    }
+    cross[((size_t)unit * b + kBits * w + j) * kBits + l] = (float)((a0 + a1) + (a2 + a3));
+  }
+}
+
+// --------------------------------------------------------------------------- host side
+constexpr int kSms = 148;
+constexpr size_t kSweepMaxSmem = 196 * 1024;               // code words of a sweep block kept in shared memory
+
+inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
+inline int t_stride_of(const bpc_config* c) { return (c->n_max + kTileKeys - 1) / kTileKeys * kTileKeys; }
+
+// Blocks per unit of project and gather (one block per SM): the first count from one wave up whose last wave is at least
+// 90 % full (32 units: 9, 8 units: 18, 128 units: 8), not below 384 keys per block.
+int parts_of(const bpc_config* c) {
+  const int units = c->batch * c->n_kv_heads;
+  int p = kSms / units > 0 ? kSms / units : 1;
+  for (int tries = 0; tries < 16; ++tries) {
+    const int rem = (int)(((long long)units * p) % kSms);
+    if (rem == 0 || rem * 10 >= kSms * 9) break;
+    ++p;
+  }
+  const int most = (c->n_max + 383) / 384;
+  return p < most ? p : most;
+}
+
+struct Layout {
+  size_t t, words, wpart, apart, cross, total;
+  explicit Layout(const bpc_config* c) {
+    const size_t units = (size_t)c->batch * c->n_kv_heads, ts = t_stride_of(c), parts = parts_of(c);
+    t = 0;
+    words = align256(units * kBits * ts * 4);
+    wpart = words + align256(units * ts * 4);
+    apart = wpart + align256(units * parts * kBits * BPC_D * 8);
+    cross = apart + align256(units * parts * kBits * c->code_bits * 4);
+    total = cross + align256(units * c->code_bits * kBits * 4);
+  }
+};
+
+// Resident sweep clusters by size on a device (the kernel takes a whole SM per block, so this depends on nothing else);
+// asked for once per device.
+struct SweepLimits {
+  std::once_flag once;
+  int active[BPC_MAX_CLUSTER + 1];
+  cudaError_t status;
+};
+SweepLimits g_sweep_limits[64];
+
+cudaLaunchConfig_t sweep_config(cudaLaunchAttribute* attr, int units, int cs, size_t smem, cudaStream_t stream) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(units * cs));
+  cfg.blockDim = dim3(kSweepThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = (unsigned)cs;
+  attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+const SweepLimits* sweep_limits(int device) {
+  if (device < 0 || device >= 64) return nullptr;
+  SweepLimits* l = &g_sweep_limits[device];
+  std::call_once(l->once, [l]() {
+    cudaError_t e = cudaFuncSetAttribute(fit_sweep_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSweepMaxSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fit_sweep_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fit_sweep_kernel<false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    for (int cs = 1; cs <= BPC_MAX_CLUSTER && e == cudaSuccess; ++cs) {
+      cudaLaunchAttribute attr;
+      cudaLaunchConfig_t cfg = sweep_config(&attr, 1, cs, kSweepMaxSmem, nullptr);
+      if (cudaOccupancyMaxActiveClusters(&l->active[cs], fit_sweep_kernel<true>, &cfg) != cudaSuccess) {
+        (void)cudaGetLastError();
+        l->active[cs] = 0;
+      }
+    }
+    l->status = e;
+  });
+  return l;
+}
+
+// Cluster size of the sweep: the smallest estimate of waves x (rounds of 128 keys per warp + the exchange of a bit), in
+// units of one round.
+int sweep_cluster(const bpc_config* c, const SweepLimits* l) {
+  const int units = c->batch * c->n_kv_heads;
+  double best_cost = 0.0;
+  int best = 1;
+  for (int cs = 1; cs <= BPC_MAX_CLUSTER; ++cs) {
+    if (l->active[cs] < 1) continue;
+    const int nk = block_rows(c->n_max, cs);
+    const int rounds = (nk / 128 + kSweepWarps - 1) / kSweepWarps;
+    const int waves = (units + l->active[cs] - 1) / l->active[cs];
+    const double cost = waves * (rounds * ((size_t)nk * 4 > kSweepMaxSmem ? 1.5 : 1.0) + 4.0 + 0.1 * cs);
+    if (best_cost == 0.0 || cost < best_cost) { best_cost = cost; best = cs; }
+  }
+  return best;
+}
+
+template <int GROUPS>
+cudaError_t launch_project_tc(const bpc_ctx* ctx, const void* k_cache, const uint32_t* hfit, const float* v_star, const float* cross, float* T,
+                              int blk, int parts, int ts, cudaStream_t stream) {
+  const bpc_config& c = ctx->cfg;
+  const size_t smem = (size_t)GROUPS * (kTileBytes + kTileKeys * kSignCols * 2) + (size_t)kProjN * 256 + (size_t)blk * kProjN * 64 + 1024;
+  cudaError_t e = cudaFuncSetAttribute(fit_project_tc_kernel<GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  fit_project_tc_kernel<GROUPS><<<dim3(parts, ctx->units), kGroupThreads * GROUPS, smem, stream>>>(
+      (const __nv_bfloat16*)k_cache, hfit, v_star, cross, T, ctx->unit_lens, ctx->dev_err, c.n_max, ctx->row_stride, c.code_bits, blk, ts);
+  return cudaGetLastError();
+}
+
+template <int HALVES, int NBUF>
+cudaError_t launch_gather_tc(const bpc_ctx* ctx, const void* k_cache, const uint32_t* hfit, double* wpart, int32_t* apart, int blk, int parts,
+                             cudaStream_t stream) {
+  const bpc_config& c = ctx->cfg;
+  const size_t smem = (size_t)kGatherGroups * (NBUF * kTileBytes + 128 * HALVES * kTileKeys * 2) + 1024;
+  cudaError_t e = cudaFuncSetAttribute(fit_gather_tc_kernel<HALVES, NBUF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  fit_gather_tc_kernel<HALVES, NBUF><<<dim3(parts, ctx->units), kGroupThreads * kGatherGroups, smem, stream>>>(
+      (const __nv_bfloat16*)k_cache, hfit, wpart, apart, ctx->unit_lens, ctx->dev_err, c.n_max, ctx->row_stride, c.code_bits, blk);
+  return cudaGetLastError();
+}
+
+}  // namespace
+
+size_t bpc_fit_blocked_bytes(const bpc_config* c) { return Layout(c).total; }
+
+cudaError_t bpc_launch_fit_blocked(bpc_ctx* ctx, const void* k_cache, const float* v_star, uint32_t* hfit, unsigned char* ws,
+                                   cudaStream_t stream, int* launches) {
+  const bpc_config& c = ctx->cfg;
+  const Layout lay(&c);
+  float* T = (float*)(ws + lay.t);
+  uint32_t* words_g = (uint32_t*)(ws + lay.words);
+  double* wpart = (double*)(ws + lay.wpart);
+  int32_t* apart = (int32_t*)(ws + lay.apart);
+  float* cross = (float*)(ws + lay.cross);
+  const int ts = t_stride_of(&c), parts = parts_of(&c), b = c.code_bits;
+  const SweepLimits* lim = sweep_limits(ctx->device);
+  if (lim == nullptr || lim->status != cudaSuccess) return lim == nullptr ? cudaErrorInvalidDevice : lim->status;
+  const int cs = sweep_cluster(&c, lim);
+  const size_t words_bytes = (size_t)block_rows(c.n_max, cs) * 4;
+  const bool tc = c.kv_dtype == BPC_BF16;
+  const dim3 grid(parts, ctx->units);
+  cudaError_t e = cudaSuccess;
+  for (int blk = 0; blk < b / kBits && e == cudaSuccess; ++blk) {
+    if (blk > 0) fit_cross_kernel<<<dim3(blk, ctx->units), 256, 0, stream>>>(ctx->P, v_star, cross, b, blk);
+    if (tc) {
+      // three warpgroups while the scalars of the earlier bits leave room for them (up to five earlier words)
+      e = blk <= 5 ? launch_project_tc<3>(ctx, k_cache, hfit, v_star, cross, T, blk, parts, ts, stream)
+                   : launch_project_tc<2>(ctx, k_cache, hfit, v_star, cross, T, blk, parts, ts, stream);
+    } else {
+      fit_project_f32_kernel<<<dim3((c.n_max + kTileKeys - 1) / kTileKeys, ctx->units), kTileKeys, 0, stream>>>(
+          (const float*)k_cache, hfit, v_star, cross, T, ctx->unit_lens, c.n_max, ctx->row_stride, b, blk, ts);
+    }
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute attr;
+    if (words_bytes <= kSweepMaxSmem) {
+      cudaLaunchConfig_t cfg = sweep_config(&attr, ctx->units, cs, words_bytes, stream);
+      e = cudaLaunchKernelEx(&cfg, fit_sweep_kernel<true>, (const float*)T, hfit, words_g, (const int32_t*)ctx->unit_lens, (int)c.n_max, b, blk, ts, cs);
+    } else {
+      cudaLaunchConfig_t cfg = sweep_config(&attr, ctx->units, cs, 0, stream);
+      e = cudaLaunchKernelEx(&cfg, fit_sweep_kernel<false>, (const float*)T, hfit, words_g, (const int32_t*)ctx->unit_lens, (int)c.n_max, b, blk, ts, cs);
+    }
+    if (e != cudaSuccess) return e;
+    if (tc) {
+      e = b <= 128 ? launch_gather_tc<1, 2>(ctx, k_cache, hfit, wpart, apart, blk, parts, stream)
+                   : launch_gather_tc<2, 1>(ctx, k_cache, hfit, wpart, apart, blk, parts, stream);
+    } else {
+      fit_gather_f32_kernel<<<grid, 256, 0, stream>>>((const float*)k_cache, hfit, wpart, apart, ctx->unit_lens, c.n_max, ctx->row_stride, b, blk);
+    }
+    if (e != cudaSuccess) return e;
+    const size_t rows_smem = (size_t)(kBits * kBits * (blk + 1) + kBits * BPC_D) * 8;
+    e = cudaFuncSetAttribute(fit_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rows_smem);
+    if (e != cudaSuccess) return e;
+    fit_rows_kernel<<<ctx->units, BPC_D * 4, rows_smem, stream>>>(wpart, apart, ctx->P, ctx->unit_lens, c.n_max, b, blk, parts);
+    e = cudaGetLastError();
+    *launches += blk > 0 ? 5 : 4;
+  }
+  return e;
+}
