@@ -40,14 +40,27 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
                  "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
                : "r"(taddr));
 }
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+                 "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+               : "r"(taddr));
+}
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// signs of bits s, s + 1 of x as a pair of bf16 (1 -> +1, 0 -> -1)
-__device__ __forceinline__ uint32_t sign_pair(uint32_t x, int s) {
-  const uint32_t nx = ~x;
-  const uint32_t lo = s <= 15 ? nx << (15 - s) : nx >> (s - 15);
-  const uint32_t hi = nx << (30 - s);
-  return 0x3F803F80u | (lo & 0x8000u) | (hi & 0x80000000u);
+// Signs as bf16 (bit 1 -> +1, 0 -> -1): nibble q of x as four values, from a table of the 16 patterns in shared memory
+// (address 128-byte aligned; one look-up replaces eight logic operations).
+__device__ __forceinline__ uint2 signs4(unsigned table, uint32_t x, int q) {
+  const uint32_t i = q == 0 ? x << 3 : x >> (4 * q - 3);
+  uint2 v;
+  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"((i & 0x78u) | table));
+  return v;
+}
+__device__ __forceinline__ void fill_sign_table(uint2* table, int tid) {
+  if (tid < 16) {
+    const uint32_t p[4] = {(tid & 1) ? 0x3F80u : 0xBF80u, (tid & 2) ? 0x3F80u : 0xBF80u, (tid & 4) ? 0x3F80u : 0xBF80u, (tid & 8) ? 0x3F80u : 0xBF80u};
+    table[tid] = make_uint2(p[0] | (p[1] << 16), p[2] | (p[3] << 16));
+  }
 }
 
 __device__ __forceinline__ void split3(float v, __nv_bfloat16 (&t)[3]) {   // v = t0 + t1 + t2 (24 mantissa bits)
@@ -69,14 +82,28 @@ __device__ __forceinline__ uint32_t warp_transpose(uint32_t x, int lane) {
   return x;
 }
 
+__device__ __forceinline__ void warp_transpose4(uint32_t (&x)[4], int lane) {   // four at once: the shuffles overlap
+  uint32_t m = 0x0000FFFFu;
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) {
+    const bool up = lane & o;
+    uint32_t y[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) y[k] = __shfl_xor_sync(0xffffffffu, x[k], o);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) x[k] = up ? ((x[k] & ~m) | ((y[k] >> o) & m)) : ((x[k] & m) | ((y[k] << o) & ~m));
+    m ^= m << (o >> 1);
+  }
+}
+
 // rows of a unit that block `blk` of `blocks` takes: equal shares of whole tiles
 __host__ __device__ inline int block_rows(int n, int blocks) { return ((n + blocks - 1) / blocks + kTileKeys - 1) / kTileKeys * kTileKeys; }
 
 // --------------------------------------------------------------------------- project (tensor cores, bf16 caches)
 // T[l][key] for the 32 columns of block `blk`.  Per tile of 128 keys: eight MMAs K_tile x D (N = 96: three bf16 terms of
 // the 32 directions), then two MMAs per earlier code word, U x (-C), into the same accumulator.  GROUPS warpgroups with
-// their own tile, sign operand and accumulator; a tile's buffer is refilled as soon as its K MMAs are done, so the next
-// load runs under the sign part and the 32 column stores.
+// their own tile, sign operand and accumulator.  The signs are laid out while the tile is on its way; the tile's buffer is
+// refilled as soon as the MMAs are done, so the next load runs under the 32 column stores.
 constexpr int kSignCols = 96;                              // signs expanded at a time (three words)
 constexpr int kProjN = 3 * kBits;
 
@@ -96,9 +123,11 @@ fit_project_tc_kernel(const __nv_bfloat16* __restrict__ k_cache, const uint32_t*
   unsigned char* b_s = smem + (size_t)GROUPS * kTileBytes;             // directions, three terms: [96 x 128], 128-byte swizzle
   unsigned char* u_s = b_s + kProjN * 256 + (size_t)grp * U_BYTES;     // this warpgroup's signs: [128 x 96], no swizzle
   unsigned char* c_s = b_s + kProjN * 256 + (size_t)GROUPS * U_BYTES;  // -C, three terms: [96 x 32 blk], no swizzle
+  __shared__ __align__(128) uint2 sign_table[16];
   __shared__ unsigned long long bar_s[GROUPS];
   __shared__ uint32_t tmem_base_s;
   __shared__ int timed_out_g[GROUPS];
+  const unsigned st_a = smem_u32(sign_table);
   const int unit = blockIdx.y;
   const int n = min(unit_lens[unit], n_max);
   const int rows = block_rows(n, gridDim.x);
@@ -128,6 +157,7 @@ fit_project_tc_kernel(const __nv_bfloat16* __restrict__ k_cache, const uint32_t*
     cp_async_commit();
   };
   if (grp < ntile) load_tile(grp);
+  fill_sign_table(sign_table, tid);
   for (int c = tid; c < kBits * BPC_D; c += kThreads) {
     const int l = c >> 7, ch = c & 127;
     __nv_bfloat16 t3[3];
@@ -154,16 +184,38 @@ fit_project_tc_kernel(const __nv_bfloat16* __restrict__ k_cache, const uint32_t*
   const uint32_t idesc = umma_idesc_bf16(kTileKeys, kProjN);
 
   unsigned ph = 0;
+  uint32_t first[kSignCols / 32];                                      // the next tile's first code words of this thread's key
+  auto load_words = [&](int tile) {
+    const int r = row0 + tile * kTileKeys + gtid;
+    const uint32_t* h = hfit + ((size_t)unit * n_max + r) * words;
+#pragma unroll
+    for (int w = 0; w < kSignCols / 32; ++w) first[w] = (w < blk && r < row_end) ? h[w] : 0u;
+  };
+  auto put_signs = [&](int w, uint32_t x) {                            // word w of the operand's row `gtid`
+    unsigned char* d = u_s + (size_t)(4 * w) * U_LBO + (size_t)(gtid >> 3) * 128 + (size_t)(gtid & 7) * 16;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const uint2 lo = signs4(st_a, x, 2 * c), hi = signs4(st_a, x, 2 * c + 1);
+      *reinterpret_cast<uint4*>(d + (size_t)c * U_LBO) = make_uint4(lo.x, lo.y, hi.x, hi.y);
+    }
+  };
+  auto issue_signs = [&](int w0, int wn) {
+    for (int ks = 0; ks < 2 * wn; ++ks)
+      umma_bf16(tm_d, umma_desc_nosw(u_s + (size_t)ks * 2 * U_LBO, U_LBO, 128),
+                umma_desc_nosw(c_s + (size_t)(4 * w0 + 2 * ks) * C_LBO, C_LBO, 128), idesc, 1u);
+  };
+  if (grp < ntile) load_words(grp);
   for (int tl = grp; tl < ntile; tl += GROUPS) {
     const int row = row0 + tl * kTileKeys + gtid;
     const bool live = row < row_end;
-    const uint32_t* hrow = hfit + ((size_t)unit * n_max + (live ? row : row0)) * words;
-    uint32_t first[kSignCols / 32];                                    // (requested before the wait for the tile)
+    const int w1 = min(blk, kSignCols / 32);
 #pragma unroll
-    for (int w = 0; w < kSignCols / 32; ++w) first[w] = w < blk ? hrow[w] : 0u;
+    for (int w = 0; w < kSignCols / 32; ++w)                           // (while the tile is on its way)
+      if (w < w1) put_signs(w, first[w]);
+    if (tl + GROUPS < ntile) load_words(tl + GROUPS);
     cp_async_wait_all();
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    group_sync(grp);                                                   // the tile has landed for all 128 threads
+    group_sync(grp);                                                   // tile and signs are there
     if (timed_out_g[grp]) break;                                       // (set before a barrier, so all 128 threads agree)
     if (gtid == 0) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -173,43 +225,26 @@ fit_project_tc_kernel(const __nv_bfloat16* __restrict__ k_cache, const uint32_t*
         const size_t boff = (size_t)(ks >> 2) * (kProjN * 128) + (size_t)(ks & 3) * 32;
         umma_bf16(tm_d, umma_desc_sw128(a_t + aoff), umma_desc_sw128(b_s + boff), idesc, ks > 0 ? 1u : 0u);
       }
+      issue_signs(0, w1);
       umma_commit(bar);
     }
-    bool refilled = false;
-    for (int w0 = 0; w0 < blk; w0 += kSignCols / 32) {                 // (one round for up to 128-bit codes)
+    if (!mbar_wait(bar, ph)) timed_out_g[grp] = 1;
+    ph ^= 1u;
+    if (tl + GROUPS < ntile) load_tile(tl + GROUPS);
+    for (int w0 = kSignCols / 32; w0 < blk; w0 += kSignCols / 32) {    // 256-bit codes: the words beyond the third
       const int wn = min(blk - w0, kSignCols / 32);
-      if (w0 > 0) {                                                    // the previous round's MMAs have read the operand
-        if (!mbar_wait(bar, ph)) timed_out_g[grp] = 1;
-        ph ^= 1u;
-      }
-#pragma unroll
-      for (int w = 0; w < kSignCols / 32; ++w) {
-        if (w >= wn) break;
-        const uint32_t x = w0 == 0 ? first[w] : hrow[w0 + w];
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-          *reinterpret_cast<uint4*>(u_s + (size_t)(4 * w + c) * U_LBO + (size_t)(gtid >> 3) * 128 + (size_t)(gtid & 7) * 16) =
-              make_uint4(sign_pair(x, 8 * c), sign_pair(x, 8 * c + 2), sign_pair(x, 8 * c + 4), sign_pair(x, 8 * c + 6));
-      }
-      if (w0 == 0) {                                                   // the K MMAs are done: refill the tile under the rest
-        if (!mbar_wait(bar, ph)) timed_out_g[grp] = 1;
-        ph ^= 1u;
-        if (tl + GROUPS < ntile) load_tile(tl + GROUPS);
-        refilled = true;
-      }
+      const uint32_t* h = hfit + ((size_t)unit * n_max + (live ? row : row0)) * words + w0;
+      for (int w = 0; w < wn; ++w) put_signs(w, h[w]);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       group_sync(grp);
       if (gtid == 0) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        for (int ks = 0; ks < 2 * wn; ++ks)
-          umma_bf16(tm_d, umma_desc_nosw(u_s + (size_t)ks * 2 * U_LBO, U_LBO, 128),
-                    umma_desc_nosw(c_s + (size_t)(4 * w0 + 2 * ks) * C_LBO, C_LBO, 128), idesc, 1u);
+        issue_signs(w0, wn);
         umma_commit(bar);
       }
+      if (!mbar_wait(bar, ph)) timed_out_g[grp] = 1;
+      ph ^= 1u;
     }
-    if (!mbar_wait(bar, ph)) timed_out_g[grp] = 1;
-    ph ^= 1u;
-    if (!refilled && tl + GROUPS < ntile) load_tile(tl + GROUPS);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     uint32_t r0[32], r1[32], r2[32];
     tmem_ld32(tm_d + lane_off, r0);
@@ -221,7 +256,7 @@ fit_project_tc_kernel(const __nv_bfloat16* __restrict__ k_cache, const uint32_t*
 #pragma unroll
     for (int l = 0; l < kBits; ++l) {
       const float v = (__uint_as_float(r0[l]) + __uint_as_float(r1[l])) + __uint_as_float(r2[l]);
-      dst[(size_t)l * t_stride] = live ? v : 0.f;
+      dst[(size_t)l * t_stride] = live ? v + 0.f : 0.f;                // (never -0)
     }
   }
   if (timed_out_g[grp] && gtid == 0) atomicOr(err, BPC_DEVERR_TIMEOUT);
@@ -280,37 +315,41 @@ fit_project_f32_kernel(const float* __restrict__ k_cache, const uint32_t* __rest
   }
   float* dst = T + (size_t)unit * kBits * t_stride + row;
 #pragma unroll
-  for (int l = 0; l < kBits; ++l) dst[(size_t)l * t_stride] = live ? (float)acc[l] : 0.f;
+  for (int l = 0; l < kBits; ++l) dst[(size_t)l * t_stride] = live ? (float)acc[l] + 0.f : 0.f;   // (never -0)
 }
 
 // --------------------------------------------------------------------------- gather (tensor cores, bf16 caches)
 // W[i][c] = sum over keys of u_i K[c] for the block's 32 bits, and the inner products u_i . u_j with all bits j so far.
-// Per tile of 128 keys the signs of all bits so far are laid out bit-major, U [bits x 128 keys] (each warp transposes its
-// 32 keys' code words across lanes, one lane then writes one bit's 32 keys); then eight MMAs K_tile^T (channel-major view of
-// the tile, M = 128 channels) x U_blk (N = 32) and eight (sixteen for 256-bit codes) U x U_blk.  Channel sums move to fp64
+// Per tile of 128 keys the signs of all R = 32 (blk + 1) bits so far are laid out bit-major, U [R x 128 keys] (each warp
+// transposes its 32 keys' code words across lanes, one lane then writes one bit's 32 keys); then eight MMAs K_tile^T
+// (channel-major view of the tile, M = 128 channels) x U_blk (N = 32) and eight per 128 bits U x U_blk.  An A operand of 128
+// rows reaches past the R rows of U into whatever follows; those accumulator rows are not read.  Channel sums move to fp64
 // registers every kFlushTiles tiles (1024 rows); the inner products are integers below 2^24 and stay exact in fp32.
-constexpr int kGatherGroups = 2;
+// A tile occupies its buffer from the start of its load to the end of its MMAs and the load is most of that, so as many
+// warpgroups with one buffer each as shared memory holds beat fewer with two (two groups of two buffers: 261 to 372 us at
+// 32 x 128K keys).
 constexpr int kFlushTiles = 8;
 
-template <int HALVES, int NBUF>                            // HALVES = 128-bit halves of a code, NBUF = key-tile buffers per warpgroup
-__global__ void __launch_bounds__(kGroupThreads * kGatherGroups, 1)
+template <int GROUPS>
+__global__ void __launch_bounds__(kGroupThreads * GROUPS, 1)
 fit_gather_tc_kernel(const __nv_bfloat16* __restrict__ k_cache, const uint32_t* __restrict__ hfit, double* __restrict__ wpart,
                      int32_t* __restrict__ apart, const int32_t* __restrict__ unit_lens, int32_t* __restrict__ err, int n_max,
                      int row_stride, int b, int blk) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-  constexpr int kThreads = kGroupThreads * kGatherGroups;
-  constexpr int R = 128 * HALVES;                          // operand rows (bits)
-  constexpr int U_BYTES = R * kTileKeys * 2;
-  constexpr unsigned LBO = (R / 8) * 128;                  // bytes between core matrices along K (keys)
-  constexpr int kCols = 32 * (1 + HALVES);                 // accumulator columns of a warpgroup
+  constexpr int kThreads = kGroupThreads * GROUPS;
+  constexpr int kMaxWords = 8;
+  const int R = kBits * (blk + 1);                         // operand rows (bits)
+  const unsigned LBO = (unsigned)(R / 8) * 128;            // bytes between core matrices along K (keys)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int grp = tid / kGroupThreads, gtid = tid % kGroupThreads;
-  unsigned char* a_g = smem + (size_t)grp * NBUF * kTileBytes;
-  unsigned char* u_s = smem + (size_t)kGatherGroups * NBUF * kTileBytes + (size_t)grp * U_BYTES;
-  __shared__ unsigned long long bar_s[kGatherGroups];
+  unsigned char* a_t = smem + (size_t)grp * kTileBytes;
+  unsigned char* u_s = smem + (size_t)GROUPS * kTileBytes + (size_t)grp * R * kTileKeys * 2;
+  __shared__ __align__(128) uint2 sign_table[16];
+  __shared__ unsigned long long bar_s[GROUPS];
   __shared__ uint32_t tmem_base_s;
-  __shared__ int timed_out_g[kGatherGroups];
+  __shared__ int timed_out_g[GROUPS];
+  const unsigned st_a = smem_u32(sign_table);
   const int unit = blockIdx.y, words = b / 32;
   const int n = min(unit_lens[unit], n_max);
   const int rows = block_rows(n, gridDim.x);
@@ -319,40 +358,38 @@ fit_gather_tc_kernel(const __nv_bfloat16* __restrict__ k_cache, const uint32_t* 
   const int row_end = min(n, row0 + rows);
   const int ntile = (row_end - row0 + kTileKeys - 1) / kTileKeys;
   if (tid == 0) {
-    for (int g = 0; g < kGatherGroups; ++g) { mbar_init(&bar_s[g], 1); timed_out_g[g] = 0; }
+    for (int g = 0; g < GROUPS; ++g) { mbar_init(&bar_s[g], 1); timed_out_g[g] = 0; }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"(256) : "memory");
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"(512) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   const unsigned char* kbase = reinterpret_cast<const unsigned char*>(k_cache) + (size_t)unit * n_max * (size_t)row_stride * 2;
-  auto load_tile = [&](int tile, int buf) {                // rows past the end are zero-filled
+  auto load_tile = [&](int tile) {                         // rows past the end are zero-filled
     const int r0 = row0 + tile * kTileKeys;
-    unsigned char* a = a_g + (size_t)buf * kTileBytes;
     for (int c = gtid; c < kTileKeys * 16; c += kGroupThreads) {
       const int r = c >> 4, ch = c & 15;
-      unsigned char* d = a + sw128_offset(kTileKeys, r, ch);
+      unsigned char* d = a_t + sw128_offset(kTileKeys, r, ch);
       if (r0 + r < row_end) cp_async16(d, kbase + (size_t)(r0 + r) * row_stride * 2 + ch * 16);
       else *reinterpret_cast<uint4*>(d) = make_uint4(0u, 0u, 0u, 0u);
     }
     cp_async_commit();
   };
-  uint32_t nxt[4 * HALVES];                                // code words of this thread's key of the next tile
+  uint32_t nxt[kMaxWords];                                 // code words of this thread's key of the next tile
   auto load_words = [&](int tile) {
     const int r = row0 + tile * kTileKeys + gtid;
     const uint32_t* h = hfit + ((size_t)unit * n_max + r) * words;
 #pragma unroll
-    for (int w = 0; w < 4 * HALVES; ++w) nxt[w] = (w <= blk && r < row_end) ? h[w] : 0u;
+    for (int w = 0; w < kMaxWords; ++w) nxt[w] = (w <= blk && r < row_end) ? h[w] : 0u;
   };
-  if (grp < ntile) { load_tile(grp, 0); load_words(grp); }
-  for (int i = tid; i < kGatherGroups * U_BYTES / 16; i += kThreads)   // rows of bits to come stay zero
-    reinterpret_cast<uint4*>(smem + (size_t)kGatherGroups * NBUF * kTileBytes)[i] = make_uint4(0u, 0u, 0u, 0u);
+  if (grp < ntile) { load_tile(grp); load_words(grp); }
+  fill_sign_table(sign_table, tid);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_all = tmem_base_s;
-  const uint32_t tm_w = tmem_all + (uint32_t)(grp * kCols), tm_a = tm_w + 32;
+  const uint32_t tm_w = tmem_all + (uint32_t)(grp * 96), tm_a = tm_w + 32;   // channel sums; inner products, 128 bits per 32 columns
   const uint32_t lane_off = (uint32_t)(32 * (warp & 3)) << 16;
   unsigned long long* bar = &bar_s[grp];
   const uint32_t idesc = umma_idesc_bf16(128, kBits);
@@ -360,35 +397,20 @@ fit_gather_tc_kernel(const __nv_bfloat16* __restrict__ k_cache, const uint32_t* 
 #pragma unroll
   for (int i = 0; i < kBits; ++i) acc[i] = 0.0;
   unsigned ph = 0;
-  bool pend = false;
-  int since_flush = 0, idx = 0;
-  for (int tl = grp; tl < ntile; tl += kGatherGroups, ++idx) {
-    const int buf = NBUF == 2 ? (idx & 1) : 0;
-    const unsigned char* a = a_g + (size_t)buf * kTileBytes;
-    uint32_t mine[4 * HALVES];
+  int since_flush = 0;
+  bool first = true;
+  for (int tl = grp; tl < ntile; tl += GROUPS) {
+    // this warp's 32 keys, one bit per lane; keys past the end become 0 instead of +-1 (while the tile is on its way)
+    const int live = min(max(row_end - (row0 + tl * kTileKeys + 32 * (warp & 3)), 0), 32);
 #pragma unroll
-    for (int w = 0; w < 4 * HALVES; ++w) mine[w] = nxt[w];
-    if (tl + kGatherGroups < ntile) load_words(tl + kGatherGroups);
-    if (pend) {                                            // the previous tile's MMAs: their operands are free afterwards
-      if (!mbar_wait(bar, ph)) timed_out_g[grp] = 1;
-      ph ^= 1u;
-      pend = false;
-      if (NBUF == 1) load_tile(tl, 0);
-    }
-    if (NBUF == 2 && tl + kGatherGroups < ntile) load_tile(tl + kGatherGroups, buf ^ 1);
-    // this warp's 32 keys, one bit per lane; keys past the end become 0 instead of +-1
-    const int r_w = row0 + tl * kTileKeys + 32 * (warp & 3);
-    const int live = min(max(row_end - r_w, 0), 32);
-#pragma unroll
-    for (int w = 0; w < 4 * HALVES; ++w) {
+    for (int w = 0; w < kMaxWords; ++w) {
       if (w > blk) break;
-      const uint32_t m = warp_transpose(mine[w], lane);
+      const uint32_t m = warp_transpose(nxt[w], lane);
       unsigned char* dst = u_s + (size_t)(4 * (warp & 3)) * LBO + (size_t)(32 * w + lane) * 16;
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
-        uint32_t h[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) h[e] = sign_pair(m, 8 * c + 2 * e);
+        const uint2 lo = signs4(st_a, m, 2 * c), hi = signs4(st_a, m, 2 * c + 1);
+        uint32_t h[4] = {lo.x, lo.y, hi.x, hi.y};
         if (live < 32) {
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
@@ -399,73 +421,84 @@ fit_gather_tc_kernel(const __nv_bfloat16* __restrict__ k_cache, const uint32_t* 
         *reinterpret_cast<uint4*>(dst + (size_t)c * LBO) = make_uint4(h[0], h[1], h[2], h[3]);
       }
     }
-    if (NBUF == 2 && tl + kGatherGroups < ntile) asm volatile("cp.async.wait_group 1;" ::: "memory");
-    else cp_async_wait_all();
+    if (tl + GROUPS < ntile) load_words(tl + GROUPS);
+    cp_async_wait_all();
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");   // (a flush's accumulator reads are done)
     group_sync(grp);
-    if (timed_out_g[grp]) break;
+    if (timed_out_g[grp]) break;                           // (set before a barrier, so all 128 threads agree)
     if (gtid == 0) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const unsigned char* ub = u_s + (size_t)(4 * blk) * 128;          // rows of this block's 32 bits
 #pragma unroll
       for (int ks = 0; ks < 8; ++ks)
-        umma_bf16(tm_w, umma_desc_sw128_mn(a + (size_t)ks * 2048, 16384, 1024), umma_desc_nosw(ub + (size_t)ks * 2 * LBO, LBO, 128),
+        umma_bf16(tm_w, umma_desc_sw128_mn(a_t + (size_t)ks * 2048, 16384, 1024), umma_desc_nosw(ub + (size_t)ks * 2 * LBO, LBO, 128),
                   idesc | kIdescAMnMajor, (since_flush > 0 || ks > 0) ? 1u : 0u);
-#pragma unroll
-      for (int hf = 0; hf < HALVES; ++hf) {
-        if (4 * hf > blk) break;
+      for (int hf = 0; 4 * hf <= blk; ++hf) {
 #pragma unroll
         for (int ks = 0; ks < 8; ++ks)
           umma_bf16(tm_a + (uint32_t)(32 * hf), umma_desc_nosw(u_s + (size_t)hf * 2048 + (size_t)ks * 2 * LBO, LBO, 128),
-                    umma_desc_nosw(ub + (size_t)ks * 2 * LBO, LBO, 128), idesc, (idx > 0 || ks > 0) ? 1u : 0u);
+                    umma_desc_nosw(ub + (size_t)ks * 2 * LBO, LBO, 128), idesc, (!first || ks > 0) ? 1u : 0u);
       }
       umma_commit(bar);
     }
-    pend = true;
+    first = false;
+    if (!mbar_wait(bar, ph)) timed_out_g[grp] = 1;
+    ph ^= 1u;
+    if (tl + GROUPS < ntile) load_tile(tl + GROUPS);
     ++since_flush;
-    if (since_flush == kFlushTiles || tl + kGatherGroups >= ntile) {
-      if (!mbar_wait(bar, ph)) timed_out_g[grp] = 1;
-      ph ^= 1u;
-      pend = false;
-      if (NBUF == 1 && tl + kGatherGroups < ntile) load_tile(tl + kGatherGroups, 0);
+    if (since_flush == kFlushTiles || tl + GROUPS >= ntile) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      uint32_t r[32];
-      tmem_ld32(tm_w + lane_off, r);
-      tmem_wait_ld();
 #pragma unroll
-      for (int i = 0; i < kBits; ++i) acc[i] += (double)__uint_as_float(r[i]);
+      for (int h = 0; h < 2; ++h) {
+        uint32_t r[16];
+        tmem_ld16(tm_w + lane_off + 16 * h, r);
+        tmem_wait_ld();
+#pragma unroll
+        for (int i = 0; i < 16; ++i) acc[16 * h + i] += (double)__uint_as_float(r[i]);
+      }
       since_flush = 0;
     }
   }
   if (timed_out_g[grp] && gtid == 0) atomicOr(err, BPC_DEVERR_TIMEOUT);
   cp_async_wait_all();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  __syncthreads();                                         // the tile buffers are free in both warpgroups
+  __syncthreads();                                         // the tile buffers are free in all warpgroups
   double* red = reinterpret_cast<double*>(smem);           // [groups][32][128]
 #pragma unroll
   for (int i = 0; i < kBits; ++i) red[((size_t)grp * kBits + i) * BPC_D + gtid] = acc[i];
-  int32_t* redc = reinterpret_cast<int32_t*>(smem + (size_t)kGatherGroups * kBits * BPC_D * 8);   // [groups][R][33]
+  int32_t* redc = reinterpret_cast<int32_t*>(smem + (size_t)GROUPS * kBits * BPC_D * 8);   // [groups][R][33]
+  for (int hf = 0; 4 * hf <= blk; ++hf) {
+    const int j = 128 * hf + gtid;
 #pragma unroll
-  for (int hf = 0; hf < HALVES; ++hf) {
-    uint32_t r[32];
-    tmem_ld32(tm_a + (uint32_t)(32 * hf) + lane_off, r);
-    tmem_wait_ld();
-    const bool any = grp < ntile && 4 * hf <= blk;
+    for (int h = 0; h < 2; ++h) {
+      uint32_t r[16];
+      tmem_ld16(tm_a + (uint32_t)(32 * hf + 16 * h) + lane_off, r);
+      tmem_wait_ld();
+      if (j < R) {
 #pragma unroll
-    for (int i = 0; i < kBits; ++i) redc[((size_t)grp * R + 128 * hf + gtid) * 33 + i] = any ? (int)__uint_as_float(r[i]) : 0;
+        for (int i = 0; i < 16; ++i) redc[((size_t)grp * R + j) * 33 + 16 * h + i] = grp < ntile ? (int)__uint_as_float(r[i]) : 0;
+      }
+    }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   double* wo = wpart + ((size_t)unit * gridDim.x + blockIdx.x) * kBits * BPC_D;
-  for (int e = tid; e < kBits * BPC_D; e += kThreads) wo[e] = red[e] + red[kBits * BPC_D + e];
-  int32_t* ao = apart + ((size_t)unit * gridDim.x + blockIdx.x) * kBits * b;
-  const int nj = kBits * (blk + 1);
-  for (int e = tid; e < kBits * nj; e += kThreads) {
-    const int i = e / nj, j = e % nj;
-    ao[(size_t)i * b + j] = redc[(size_t)j * 33 + i] + redc[((size_t)R + j) * 33 + i];
+  for (int e = tid; e < kBits * BPC_D; e += kThreads) {
+    double v = 0.0;
+#pragma unroll
+    for (int g = 0; g < GROUPS; ++g) v += red[(size_t)g * kBits * BPC_D + e];
+    wo[e] = v;
   }
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_all), "r"(256) : "memory");
+  int32_t* ao = apart + ((size_t)unit * gridDim.x + blockIdx.x) * kBits * b;
+  for (int e = tid; e < kBits * R; e += kThreads) {
+    const int i = e / R, j = e % R;
+    int v = 0;
+#pragma unroll
+    for (int g = 0; g < GROUPS; ++g) v += redc[((size_t)g * R + j) * 33 + i];
+    ao[(size_t)i * b + j] = v;
+  }
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_all), "r"(512) : "memory");
 }
 
 // --------------------------------------------------------------------------- gather (CUDA cores, fp32 caches)
@@ -534,11 +567,38 @@ fit_gather_f32_kernel(const float* __restrict__ k_cache, const uint32_t* __restr
 constexpr int kSweepThreads = 512;
 constexpr int kSweepWarps = kSweepThreads / 32;
 constexpr int kSweepPlanes = 8;
+constexpr int kSweepSlots = 3;                             // rounds of the two columns in flight or in use, per thread 32 bytes each
+constexpr int kSweepSlotBytes = 2 * kSweepThreads * 16;
+constexpr int kSweepRing = kSweepSlots * kSweepSlotBytes;
 constexpr int kSweepFlush = 60;                            // rounds of four keys between flushes: 240 < 2^kSweepPlanes counts
 
 struct SweepSums {                                         // lane i: bit i
-  double s, tot;
-  int cnt;
+  double s;                                                // u_i^T T over this warp's keys
+  int cnt;                                                 // keys whose new bit agrees with bit i
+};
+
+// The columns on their way to a warp: round after round and pass after pass without a break, so that the first entries of
+// a pass arrive while the block still exchanges the previous one's sums.
+struct SweepStream {
+  const float* base;                                       // this lane's entry of column 0, round 0
+  const float* next;                                       // ... of the next request
+  int t_stride, rounds;                                    // rounds of this warp per pass
+  int bit, round;                                          // of the next request
+  unsigned char* ring;                                     // this thread's slots
+  int at;                                                  // offset of the slot to be read next
+  __device__ __forceinline__ void request(unsigned char* slot) {      // (always a group, so that the waits can count)
+    if (bit < kBits) {
+      cp_async16(slot, next);
+      if (bit + 1 < kBits) cp_async16(slot + kSweepThreads * 16, next + t_stride);
+      next += kSweepWarps * 128;
+      if (++round == rounds) {
+        round = 0;
+        ++bit;
+        next = base + (size_t)bit * t_stride;
+      }
+    }
+    cp_async_commit();
+  }
 };
 
 // values v[0..N-1] of every lane summed over the warp: lane l returns the sum of v[l] (l & (N - 1) for N < 32)
@@ -566,15 +626,45 @@ __device__ __forceinline__ void full_add(uint32_t a, uint32_t b, uint32_t c, uin
   cy = (a & b) | (c & (a | b));
 }
 
+// acc += v where w has bit I set (written out so that the tests of a word become predicates, not selects)
+template <int I>
+__device__ __forceinline__ void add_if(float& acc, float v, uint32_t w) {
+  asm("{\n\t.reg .pred p;\n\t.reg .b32 q;\n\tand.b32 q, %1, %2;\n\tsetp.ne.b32 p, q, 0;\n\t@p add.f32 %0, %0, %3;\n\t}\n"
+      : "+f"(acc) : "r"(w), "n"(1u << I), "f"(v));
+}
+template <int I, int N, int NS>
+__device__ __forceinline__ void add_bits(float (&acc)[NS], float v, uint32_t w) {
+  if constexpr (I < N) {
+    add_if<I>(acc[I], v, w);
+    add_bits<I + 1, N>(acc, v, w);
+  }
+}
+// entry (w >> 4 NB) & 15 of the look-up table's row NB; `base` is the table's shared-memory address, 512-byte aligned
+template <int NB>
+__device__ __forceinline__ float lut_at(unsigned base, uint32_t w) {
+  const uint32_t x = NB == 0 ? w << 2 : w >> (4 * NB - 2);
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1 + %2];" : "=f"(v) : "r"((x & 0x3Cu) | base), "n"(64 * NB));
+  return v;
+}
+template <int NB, int N>
+__device__ __forceinline__ float lut_sum(unsigned base, uint32_t w) {      // rows NB, NB + 2, ...
+  if constexpr (NB + 2 < N) return lut_at<NB>(base, w) + lut_sum<NB + 2, N>(base, w);
+  else return lut_at<NB>(base, w);
+}
+
 // One pass over this block's keys: decides bit j; unless it is the block's last bit, also the sums for column j + 1.
-template <int JB, bool LAST>
-__device__ __forceinline__ void sweep_pass(const float* __restrict__ tc, const float* __restrict__ tn, uint32_t* __restrict__ ws,
-                                           const float* __restrict__ lut, int j, int nk, int nkeys, int warp, int lane, SweepSums& out) {
-  constexpr int NS = JB == 3 ? 32 : 8 * JB;                // running sums (a power of two for the warp reduction)
-  out.s = out.tot = 0.0;
+// Q4 = groups of four bits in play (j / 4 + 1).  Keys past the end (up to 127, all in the last group of the unit's last
+// block, entries zero) take part like any others and are subtracted at the end: they all carry the same code word.
+template <int Q4, bool LAST>
+__device__ __forceinline__ void sweep_pass(SweepStream& in, uint32_t* __restrict__ ws, unsigned lut, int j, int nk, int nkeys, int warp,
+                                           int lane, SweepSums& out) {
+  constexpr int NS = Q4 <= 2 ? 8 : Q4 <= 4 ? 16 : 32;      // running sums (a power of two for the warp reduction)
+  out.s = 0.0;
   out.cnt = 0;
   const uint32_t bit = 1u << j;
-  for (int g0 = warp; g0 < nk / 128; g0 += kSweepWarps * kSweepFlush) {
+  const int ng = nk / 128;
+  for (int g0 = warp; g0 < ng; g0 += kSweepWarps * kSweepFlush) {
     float s[NS];
     float tot = 0.f;
     uint32_t pl[kSweepPlanes];
@@ -582,43 +672,35 @@ __device__ __forceinline__ void sweep_pass(const float* __restrict__ tc, const f
     for (int i = 0; i < NS; ++i) s[i] = 0.f;
 #pragma unroll
     for (int k = 0; k < kSweepPlanes; ++k) pl[k] = 0u;
-    const int g1 = min(nk / 128, g0 + kSweepWarps * kSweepFlush);
-    float4 t4 = *reinterpret_cast<const float4*>(tc + g0 * 128 + 4 * lane), n4;
-    if (!LAST) n4 = *reinterpret_cast<const float4*>(tn + g0 * 128 + 4 * lane);
+    const int g1 = min(ng, g0 + kSweepWarps * kSweepFlush);
+    uint32_t* pw = ws + g0 * 128 + 4 * lane;
     for (int g = g0; g < g1; g += kSweepWarps) {
-      const int key = g * 128 + 4 * lane;
+      int ahead = in.at + 2 * kSweepSlotBytes;
+      if (ahead >= kSweepRing) ahead -= kSweepRing;
+      in.request(in.ring + ahead);
+      asm volatile("cp.async.wait_group 2;" ::: "memory");
+      const float4 t4 = *reinterpret_cast<const float4*>(in.ring + in.at);
+      const float4 n4 = *reinterpret_cast<const float4*>(in.ring + in.at + kSweepThreads * 16);
+      in.at += kSweepSlotBytes;
+      if (in.at == kSweepRing) in.at = 0;
       const float t[4] = {t4.x, t4.y, t4.z, t4.w};
       const float nx[4] = {n4.x, n4.y, n4.z, n4.w};
-      if (g + kSweepWarps < g1) {                          // (requested one round ahead)
-        t4 = *reinterpret_cast<const float4*>(tc + key + kSweepWarps * 128);
-        if (!LAST) n4 = *reinterpret_cast<const float4*>(tn + key + kSweepWarps * 128);
-      }
-      const uint4 w4 = *reinterpret_cast<const uint4*>(ws + key);
+      const uint4 w4 = *reinterpret_cast<const uint4*>(pw);
       uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w}, x[4];
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        float c0 = 0.f, c1 = 0.f;
-#pragma unroll
-        for (int nb = 0; nb < 2 * JB; nb += 2) {
-          c0 += lut[nb * 16 + ((w[e] >> (4 * nb)) & 15u)];
-          c1 += lut[nb * 16 + 16 + ((w[e] >> (4 * nb + 4)) & 15u)];
-        }
-        const bool pos = t[e] - (c0 + c1) >= 0.f;
-        x[e] = pos ? w[e] : ~w[e];
-        w[e] |= pos ? bit : 0u;
+        const float c = Q4 == 1 ? lut_at<0>(lut, w[e]) : lut_sum<0, Q4>(lut, w[e]) + lut_sum<1, Q4>(lut, w[e]);
+        const uint32_t neg = (uint32_t)((int)__float_as_uint(t[e] - c) >> 31);   // (never -0: columns hold no -0)
+        x[e] = w[e] ^ neg;                                 // bit i: agrees with the new bit
+        w[e] |= bit & ~neg;
         if (!LAST) {
           tot += nx[e];
-#pragma unroll
-          for (int i = 0; i < 8 * JB; ++i)
-            if (w[e] & (1u << i)) s[i] += nx[e];
+          add_bits<0, 4 * Q4>(s, nx[e], w[e]);
         }
       }
-      *reinterpret_cast<uint4*>(ws + key) = make_uint4(w[0], w[1], w[2], w[3]);
+      *reinterpret_cast<uint4*>(pw) = make_uint4(w[0], w[1], w[2], w[3]);
+      pw += kSweepWarps * 128;
       if (!LAST) {
-        if (key + 4 > nkeys) {                             // keys past the end agree with nothing
-#pragma unroll
-          for (int e = 0; e < 4; ++e) if (key + e >= nkeys) x[e] = 0u;
-        }
         uint32_t s1, ca, cb, cc;
         full_add(x[0], x[1], x[2], s1, ca);
         full_add(pl[0], s1, x[3], pl[0], cb);
@@ -632,32 +714,70 @@ __device__ __forceinline__ void sweep_pass(const float* __restrict__ tc, const f
       }
     }
     if (!LAST) {
-      out.s += (double)warp_sum_scatter<NS>(s, lane);
 #pragma unroll
       for (int o = 16; o >= 1; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
-      out.tot += (double)tot;
+      out.s += 2.0 * (double)warp_sum_scatter<NS>(s, lane) - (double)tot;
       const int keys_per_lane = 4 * ((g1 - g0 + kSweepWarps - 1) / kSweepWarps);
 #pragma unroll
-      for (int k = 0; k < kSweepPlanes; ++k) {
-        if ((keys_per_lane >> k) == 0) break;              // higher planes are empty
-        out.cnt += __popc(warp_transpose(pl[k], lane)) << k;
+      for (int k0 = 0; k0 < kSweepPlanes; k0 += 4) {       // four independent transposes at a time
+        if ((keys_per_lane >> k0) == 0) break;             // higher planes are empty
+        uint32_t x[4] = {pl[k0], pl[k0 + 1], pl[k0 + 2], pl[k0 + 3]};
+        warp_transpose4(x, lane);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) out.cnt += __popc(x[k]) << (k0 + k);
+      }
+      if (g1 == ng && nkeys < nk && (ng - 1 - warp) % kSweepWarps == 0) {   // this warp took the group with keys past the end
+        __syncwarp();
+        const uint32_t wp = ws[nk - 1];
+        const uint32_t same = (wp & bit) ? wp : ~wp;
+        out.cnt -= (nk - nkeys) * (int)((same >> lane) & 1u);
       }
     }
   }
 }
 
+// arrival of this thread plus `bytes` still to come on the barrier's current phase
+__device__ __forceinline__ void mbar_expect(unsigned long long* bar, unsigned bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+}
+// bounded wait for a phase whose data other blocks of the cluster sent; false when the iteration budget runs out
+__device__ __forceinline__ bool mbar_wait_cluster(unsigned long long* bar, unsigned parity) {
+  for (int it = 0; it < 20000000; ++it) {
+    unsigned ok;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
+                 : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+    if (ok) return true;
+  }
+  return false;
+}
+// asynchronous store into rank r's copy of `dst`, counted on rank r's copy of `bar`
+__device__ __forceinline__ void send_b64(const void* dst, const void* bar, int r, unsigned long long v) {
+  asm volatile("{\n\t.reg .b32 d, b;\n\tmapa.shared::cluster.u32 d, %0, %2;\n\tmapa.shared::cluster.u32 b, %1, %2;\n\t"
+               "st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [d], %3, [b];\n\t}\n"
+               ::"r"(smem_u32(dst)), "r"(smem_u32(bar)), "r"(r), "l"(v) : "memory");
+}
+__device__ __forceinline__ void send_b32(const void* dst, const void* bar, int r, uint32_t v) {
+  asm volatile("{\n\t.reg .b32 d, b;\n\tmapa.shared::cluster.u32 d, %0, %2;\n\tmapa.shared::cluster.u32 b, %1, %2;\n\t"
+               "st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [d], %3, [b];\n\t}\n"
+               ::"r"(smem_u32(dst)), "r"(smem_u32(bar)), "r"(r), "r"(v) : "memory");
+}
+
 template <bool SMEM_WORDS>
 __global__ void __launch_bounds__(kSweepThreads, 1)
 fit_sweep_kernel(const float* __restrict__ T, uint32_t* __restrict__ hfit, uint32_t* __restrict__ words_g,
-                 const int32_t* __restrict__ unit_lens, int n_max, int b, int blk, int t_stride, int cluster_size) {
-  extern __shared__ __align__(16) uint32_t words_s[];
-  __shared__ __align__(16) float lut[8 * 16];              // lut[nibble][pattern] = sum of +-c over the nibble's bits
-  __shared__ double red_s[kSweepWarps][32], red_t[kSweepWarps];
+                 const int32_t* __restrict__ unit_lens, int32_t* __restrict__ err, int n_max, int b, int blk, int t_stride, int cluster_size) {
+  extern __shared__ __align__(16) unsigned char sweep_smem[];   // the copy ring, then (SMEM_WORDS) this block's code words
+  __shared__ __align__(512) float lut[8 * 16];             // lut[nibble][pattern] = sum of +-c over the nibble's bits
+  __shared__ double red_s[kSweepWarps][32];
   __shared__ int red_c[kSweepWarps][32];
   __shared__ double slot_s[2][BPC_MAX_CLUSTER][32];        // the cluster's sums of bit i, by rank; two passes alternate
   __shared__ int slot_c[2][BPC_MAX_CLUSTER][32];
-  __shared__ double agree[32][33];                         // u_i . u_m
-  __shared__ float c_s[32];
+  __shared__ unsigned long long bar_s[2];                  // the cluster's sums of this parity have arrived
+  __shared__ double sum_s[32];
+  __shared__ double inv_s[32][33];                         // c = inv_s * sums: the inverse of the triangle n I + (u_i . u_m), m < i
+  __shared__ double agree_s[32];                           // u_j . u_m of the newest bit
+  __shared__ __align__(16) float c_s[32];
+  __shared__ int timed_out;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int rank = blockIdx.x % cluster_size, unit = blockIdx.x / cluster_size;
   const int n = min(unit_lens[unit], n_max);
@@ -666,156 +786,219 @@ fit_sweep_kernel(const float* __restrict__ T, uint32_t* __restrict__ hfit, uint3
   const int row0 = rank * share;
   const int nkeys = max(0, min(n - row0, share));          // keys of this block; nk = the same in whole groups of 128
   const int nk = (nkeys + 127) / 128 * 128;
-  uint32_t* ws = SMEM_WORDS ? words_s : words_g + (size_t)unit * t_stride + row0;
+  uint32_t* ws = SMEM_WORDS ? reinterpret_cast<uint32_t*>(sweep_smem + kSweepRing) : words_g + (size_t)unit * t_stride + row0;
   for (int i = tid; i < nk / 4; i += kSweepThreads) reinterpret_cast<uint4*>(ws)[i] = make_uint4(0u, 0u, 0u, 0u);
   if (tid < 128) lut[tid] = 0.f;
-  __syncthreads();
+  if (tid < 32) c_s[tid] = 0.f;
+  for (int i = tid; i < 32 * 33; i += kSweepThreads) (&inv_s[0][0])[i] = 0.0;
+  if (tid == 0) {
+    timed_out = 0;
+    for (int q = 0; q < 2; ++q) {
+      mbar_init(&bar_s[q], 1);
+      mbar_expect(&bar_s[q], (unsigned)cluster_size * 32u * 12u);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");      // every rank's barriers are armed
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  double new_row = 0.0;
   const float* Tu = T + (size_t)unit * kBits * t_stride + row0;
   const double inv_n = 1.0 / (double)n;
+  const unsigned lut_a = smem_u32(lut);
+  auto prefetch = [&](int c) {                             // column c of this block's keys into L2, a part per warp
+    const int part = (nk / 4 + kSweepWarps - 1) / kSweepWarps, at = warp * part, cnt = min(part, nk / 4 - at);
+    if (c < kBits && lane == 0 && cnt > 0)
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(Tu + (size_t)c * t_stride + 4 * at), "r"(16 * cnt) : "memory");
+  };
+  SweepStream in;
+  in.base = in.next = Tu + warp * 128 + 4 * lane;
+  in.t_stride = t_stride;
+  in.rounds = (nk / 128 - warp + kSweepWarps - 1) / kSweepWarps;
+  in.bit = in.rounds > 0 ? 0 : kBits;                      // (a warp without keys requests nothing)
+  in.round = 0;
+  in.ring = sweep_smem + 16 * tid;
+  in.at = 0;
+  in.request(in.ring);
+  in.request(in.ring + kSweepSlotBytes);
   for (int j = 0; j < kBits; ++j) {
-    const float* tc = Tu + (size_t)j * t_stride;
     SweepSums sums;
-    if (j == kBits - 1) { sweep_pass<4, true>(tc, tc, ws, lut, j, nk, nkeys, warp, lane, sums); break; }
-    if (j < 8) sweep_pass<1, false>(tc, tc + t_stride, ws, lut, j, nk, nkeys, warp, lane, sums);
-    else if (j < 16) sweep_pass<2, false>(tc, tc + t_stride, ws, lut, j, nk, nkeys, warp, lane, sums);
-    else if (j < 24) sweep_pass<3, false>(tc, tc + t_stride, ws, lut, j, nk, nkeys, warp, lane, sums);
-    else sweep_pass<4, false>(tc, tc + t_stride, ws, lut, j, nk, nkeys, warp, lane, sums);
+    if (j == kBits - 1) { sweep_pass<8, true>(in, ws, lut_a, j, nk, nkeys, warp, lane, sums); break; }
+    prefetch(j + 2);
+    switch (j >> 2) {
+      case 0: sweep_pass<1, false>(in, ws, lut_a, j, nk, nkeys, warp, lane, sums); break;
+      case 1: sweep_pass<2, false>(in, ws, lut_a, j, nk, nkeys, warp, lane, sums); break;
+      case 2: sweep_pass<3, false>(in, ws, lut_a, j, nk, nkeys, warp, lane, sums); break;
+      case 3: sweep_pass<4, false>(in, ws, lut_a, j, nk, nkeys, warp, lane, sums); break;
+      case 4: sweep_pass<5, false>(in, ws, lut_a, j, nk, nkeys, warp, lane, sums); break;
+      case 5: sweep_pass<6, false>(in, ws, lut_a, j, nk, nkeys, warp, lane, sums); break;
+      case 6: sweep_pass<7, false>(in, ws, lut_a, j, nk, nkeys, warp, lane, sums); break;
+      default: sweep_pass<8, false>(in, ws, lut_a, j, nk, nkeys, warp, lane, sums); break;
+    }
     red_s[warp][lane] = sums.s;
     red_c[warp][lane] = sums.cnt;
-    if (lane == 0) red_t[warp] = sums.tot;
     __syncthreads();
     const int buf = j & 1;
-    if (warp == 0) {
-      double s = 0.0, tot = 0.0;
+    const unsigned phase = (unsigned)(j >> 1) & 1u;
+    // Exchange within the cluster: warps 0..3 send the block's sums, 4..7 its counts, each to every fourth rank; the sends
+    // complete on the receiver's barrier of this parity (a rank sends bit j + 2 only after it has everybody's bit j + 1).
+    if (warp < 4) {
+      double v[kSweepWarps];
+#pragma unroll
+      for (int w = 0; w < kSweepWarps; ++w) v[w] = red_s[w][lane];
+#pragma unroll
+      for (int o = kSweepWarps / 2; o >= 1; o >>= 1)
+#pragma unroll
+        for (int w = 0; w < o; ++w) v[w] += v[w + o];
+      for (int r = warp; r < cluster_size; r += 4)
+        send_b64(&slot_s[buf][rank][lane], &bar_s[buf], r, (unsigned long long)__double_as_longlong(v[0]));
+    } else if (warp < 8) {
       int c = 0;
 #pragma unroll
-      for (int w = 0; w < kSweepWarps; ++w) { s += red_s[w][lane]; tot += red_t[w]; c += red_c[w][lane]; }
-      s = 2.0 * s - tot;                                   // u_lane^T T[:, j + 1] over this block's keys
-      const unsigned as = (unsigned)__cvta_generic_to_shared(&slot_s[buf][rank][lane]);
-      const unsigned ac = (unsigned)__cvta_generic_to_shared(&slot_c[buf][rank][lane]);
-      for (int r = 0; r < cluster_size; ++r) {
-        unsigned ps, pc;
-        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ps) : "r"(as), "r"(r));
-        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(pc) : "r"(ac), "r"(r));
-        asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(ps), "d"(s) : "memory");
-        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(pc), "r"(c) : "memory");
-      }
+      for (int w = 0; w < kSweepWarps; ++w) c += red_c[w][lane];
+      for (int r = warp - 4; r < cluster_size; r += 4) send_b32(&slot_c[buf][rank][lane], &bar_s[buf], r, (uint32_t)c);
     }
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    if (warp == 0) {
-      double s = 0.0;
+    // n c_{i,j+1} = u_i^T T - sum_{m<i} (u_i . u_m) c_{m,j+1}: c_i for i < j are rows of the triangle's inverse times the
+    // sums, c_j follows from them (warp 0); the new bit's row of the inverse (warp 8) is needed one bit later.
+    if (warp == 0 || warp == 8) {
+      if (!timed_out && !mbar_wait_cluster(&bar_s[buf], phase)) timed_out = 1;
       int c = 0;
-      for (int r = 0; r < cluster_size; ++r) { s += slot_s[buf][r][lane]; c += slot_c[buf][r][lane]; }
-      agree[j][lane] = (double)(2 * (long long)c - (long long)n);        // u_j . u_lane (lane < j)
-      __syncwarp();
-      // c_{i,j+1} = (u_i^T T - sum_{m<i} (u_i . u_m) c_{m,j+1}) / n
-      double mine = 0.0;
-      for (int m = 0; m <= j; ++m) {
-        const double cm = __shfl_sync(0xffffffffu, s, m) * inv_n;
-        if (lane == m) mine = cm;
-        if (lane > m) s -= agree[lane][m] * cm;
-      }
-      c_s[lane] = lane <= j ? (float)mine : 0.f;
-      __syncwarp();
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int e = lane + 32 * q;
-        float v = 0.f;
+      for (int r = 0; r < BPC_MAX_CLUSTER; ++r) c += r < cluster_size ? slot_c[buf][r][lane] : 0;
+      const double agree = lane < j ? (double)(2 * c - n) : 0.0;         // u_j . u_lane
+      if (warp == 0) {
+        double v[BPC_MAX_CLUSTER];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) { const float d = c_s[4 * (e >> 4) + i]; v += ((e >> i) & 1) ? d : -d; }
-        lut[e] = v;
+        for (int r = 0; r < BPC_MAX_CLUSTER; ++r) v[r] = r < cluster_size ? slot_s[buf][r][lane] : 0.0;
+#pragma unroll
+        for (int o = BPC_MAX_CLUSTER / 2; o >= 1; o >>= 1)
+#pragma unroll
+          for (int r = 0; r < o; ++r) v[r] += v[r + o];
+        sum_s[lane] = v[0];
+        __syncwarp();
+        double a[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 2
+        for (int m = 0; m < j; m += 4)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) a[q] += inv_s[lane][m + q] * sum_s[m + q];   // (zero beyond the row's own bit)
+        double ci = (a[0] + a[1]) + (a[2] + a[3]);
+        double x = lane < j ? agree * ci : 0.0;
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if (lane == j) ci = (v[0] - x) * inv_n;
+        c_s[lane] = lane <= j ? (float)ci : 0.f;
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int e = lane + 32 * q;
+          const float4 d = *reinterpret_cast<const float4*>(&c_s[4 * (e >> 4)]);
+          lut[e] = (((e & 1) ? d.x : -d.x) + ((e & 2) ? d.y : -d.y)) + (((e & 4) ? d.z : -d.z) + ((e & 8) ? d.w : -d.w));
+        }
+      } else {
+        agree_s[lane] = agree;
+        __syncwarp();
+        double a[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 2
+        for (int k = 0; k < j; k += 4)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) a[q] += agree_s[k + q] * inv_s[k + q][lane];    // (rows from j on are zero)
+        new_row = lane == j ? inv_n : -((a[0] + a[1]) + (a[2] + a[3])) * inv_n;
       }
     }
     __syncthreads();
+    if (warp == 8) inv_s[j][lane] = new_row;               // (warp 0 has read the inverse; it reads it again two barriers on)
+    if (tid == 0) mbar_expect(&bar_s[buf], (unsigned)cluster_size * 32u * 12u);   // arms the barrier for bit j + 2
   }
+  cp_async_wait_all();
   __syncthreads();
   uint32_t* h = hfit + ((size_t)unit * n_max + row0) * (b / 32) + blk;
   for (int i = tid; i < nkeys; i += kSweepThreads) h[(size_t)i * (b / 32)] = ws[i];
+  if (timed_out && tid == 0) atomicOr(err, BPC_DEVERR_TIMEOUT);
 }
 
 // --------------------------------------------------------------------------- rows and scalars
-// v_i = (W_i - sum_{j<i} (u_i . u_j) v_j) / n for the block's 32 bits, one block per unit; four thread groups split the
-// partial sums and the earlier bits, one thread per channel runs the block's own triangle in registers.  Fixed order.
-__global__ void __launch_bounds__(BPC_D * 4)
-fit_rows_kernel(const double* __restrict__ wpart, const int32_t* __restrict__ apart, float* __restrict__ P,
-                const int32_t* __restrict__ unit_lens, int n_max, int b, int blk, int parts) {
-  extern __shared__ __align__(16) double rows_smem[];
-  double* corr = rows_smem;                                // [32][32 (blk + 1)] u_i . u_j
-  double* w_s = corr + kBits * kBits * (blk + 1);          // [32][128]
-  const int unit = blockIdx.x, tid = threadIdx.x, c = tid & 127, q = tid >> 7;
+// The blocks' partial sums of a unit, added in block order into the first block's place; grid (16 + 4 (blk + 1), units), one
+// sum per thread (the loads are independent: a latency or two in all).
+__global__ void __launch_bounds__(256)
+fit_sum_parts_kernel(double* __restrict__ wpart, int32_t* __restrict__ apart, const int32_t* __restrict__ unit_lens, int n_max, int b,
+                     int blk, int parts) {
+  const int unit = blockIdx.y;
   const int n = min(unit_lens[unit], n_max);
-  float* Pu = P + (size_t)unit * b * BPC_D;
-  if (n <= 0) {
-    for (int e = tid; e < kBits * BPC_D; e += 512) Pu[(size_t)kBits * blk * BPC_D + e] = 0.f;
-    return;
-  }
+  if (n <= 0) return;
   const int rows = block_rows(n, parts), used = (n + rows - 1) / rows;
-  const int nj = kBits * (blk + 1);
-  for (int e = tid; e < kBits * nj; e += 512) {
-    long long a = 0;
-    for (int p = 0; p < used; ++p) a += apart[(((size_t)unit * parts + p) * kBits + e / nj) * b + e % nj];
-    corr[e] = (double)a;
-  }
-  __syncthreads();
-  for (int i0 = 8 * q; i0 < 8 * q + 8; i0 += 4) {          // group q: rows 8q .. 8q + 7
-    double acc[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) acc[i] = 0.0;
-    for (int p = 0; p < used; ++p)
-#pragma unroll
-      for (int i = 0; i < 4; ++i) acc[i] += wpart[(((size_t)unit * parts + p) * kBits + i0 + i) * BPC_D + c];
-    for (int j = 0; j < kBits * blk; ++j) {
-      const double v = (double)Pu[(size_t)j * BPC_D + c];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) acc[i] -= corr[(i0 + i) * nj + j] * v;
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) w_s[(i0 + i) * BPC_D + c] = acc[i];
-  }
-  __syncthreads();
-  if (q == 0) {
-    double w[kBits];
-#pragma unroll
-    for (int i = 0; i < kBits; ++i) w[i] = w_s[i * BPC_D + c];
-    const double inv_n = 1.0 / (double)n;
-#pragma unroll
-    for (int i = 0; i < kBits; ++i) {
-      const float v = (float)(w[i] * inv_n);
-      Pu[(size_t)(kBits * blk + i) * BPC_D + c] = v;
-#pragma unroll
-      for (int i2 = i + 1; i2 < kBits; ++i2) w[i2] -= corr[i2 * nj + kBits * blk + i] * (double)v;
-    }
+  if (blockIdx.x < 16) {
+    double* w = wpart + (size_t)unit * parts * kBits * BPC_D + blockIdx.x * 256 + threadIdx.x;
+    double s = w[0];
+#pragma unroll 16
+    for (int p = 1; p < used; ++p) s += w[(size_t)p * kBits * BPC_D];
+    w[0] = s;
+  } else {
+    const int e = (blockIdx.x - 16) * 256 + threadIdx.x, nj = kBits * (blk + 1);
+    int32_t* a = apart + (size_t)unit * parts * kBits * b + (size_t)(e / nj) * b + e % nj;
+    int s = a[0];
+#pragma unroll 16
+    for (int p = 1; p < used; ++p) s += a[(size_t)p * kBits * b];
+    a[0] = s;
   }
 }
 
-// cross[j][l] = v_j . d_l for 32 bits j so far and the 32 columns l of block `blk`; grid (blk, units), fp64 sums
-__global__ void __launch_bounds__(256)
-fit_cross_kernel(const float* __restrict__ P, const float* __restrict__ v_star, float* __restrict__ cross, int b, int blk) {
-  __shared__ float v_s[kBits][BPC_D + 1], d_s[kBits][BPC_D + 1];
-  const int unit = blockIdx.y, w = blockIdx.x, tid = threadIdx.x;
-  for (int e = tid; e < kBits * BPC_D; e += 256) {
-    v_s[e >> 7][e & 127] = P[((size_t)unit * b + kBits * w) * BPC_D + e];
-    d_s[e >> 7][e & 127] = v_star[((size_t)unit * b + kBits * blk) * BPC_D + e];
+// v_i = (W_i - sum_{j<i} (u_i . u_j) v_j) / n for the block's 32 bits; grid (4, units), a block has 32 channels.  Thread
+// (row pair, channel) takes off the earlier blocks' rows, then one warp runs the block's own triangle in registers.
+__global__ void __launch_bounds__(512)
+fit_rows_kernel(const double* __restrict__ wpart, const int32_t* __restrict__ apart, float* __restrict__ P,
+                const int32_t* __restrict__ unit_lens, int n_max, int b, int blk, int parts) {
+  extern __shared__ __align__(16) double rows_smem[];
+  const int nj = kBits * (blk + 1), np = kBits * blk;
+  double* corr = rows_smem;                                // [32][nj] u_i . u_j
+  double* v_s = corr + kBits * nj;                         // [np][32] earlier rows, this block's channels
+  double* w_s = v_s + (size_t)np * 32;                     // [32][32]
+  const int unit = blockIdx.y, tid = threadIdx.x, lane = tid & 31, r = tid >> 5, c = 32 * blockIdx.x + lane;
+  const int n = min(unit_lens[unit], n_max);
+  float* Pu = P + (size_t)unit * b * BPC_D;
+  if (n <= 0) {
+    for (int i = r; i < kBits; i += 16) Pu[(size_t)(np + i) * BPC_D + c] = 0.f;
+    return;
   }
+  const double* w = wpart + (size_t)unit * parts * kBits * BPC_D;
+  const int32_t* a = apart + (size_t)unit * parts * kBits * b;
+  double acc[2][2] = {{w[(size_t)r * BPC_D + c], 0.0}, {w[(size_t)(r + 16) * BPC_D + c], 0.0}};
+  for (int e = tid; e < kBits * nj; e += 512) corr[e] = (double)a[(size_t)(e / nj) * b + e % nj];
+  for (int j = r; j < np; j += 16) v_s[j * 32 + lane] = (double)Pu[(size_t)j * BPC_D + c];
   __syncthreads();
-  const int l = tid & 31;
-  for (int j = tid >> 5; j < kBits; j += 8) {
-    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-#pragma unroll 8
-    for (int c = 0; c < BPC_D; c += 4) {
-      a0 = fma((double)v_s[j][c], (double)d_s[l][c], a0);
-      a1 = fma((double)v_s[j][c + 1], (double)d_s[l][c + 1], a1);
-      a2 = fma((double)v_s[j][c + 2], (double)d_s[l][c + 2], a2);
-      a3 = fma((double)v_s[j][c + 3], (double)d_s[l][c + 3], a3);
+#pragma unroll 4
+  for (int j = 0; j < np; j += 2) {
+#pragma unroll
+    for (int o = 0; o < 2; ++o) {
+      const double v = v_s[(j + o) * 32 + lane];
+      acc[0][o] -= corr[r * nj + j + o] * v;
+      acc[1][o] -= corr[(r + 16) * nj + j + o] * v;
     }
-    cross[((size_t)unit * b + kBits * w + j) * kBits + l] = (float)((a0 + a1) + (a2 + a3));
+  }
+  w_s[r * 32 + lane] = acc[0][0] + acc[0][1];
+  w_s[(r + 16) * 32 + lane] = acc[1][0] + acc[1][1];
+  __syncthreads();
+  if (r != 0) return;
+  double x[kBits];
+#pragma unroll
+  for (int i = 0; i < kBits; ++i) x[i] = w_s[i * 32 + lane];
+  const double inv_n = 1.0 / (double)n;
+#pragma unroll
+  for (int i = 0; i < kBits; ++i) {
+    const float v = (float)(x[i] * inv_n);
+    Pu[(size_t)(np + i) * BPC_D + c] = v;
+#pragma unroll
+    for (int k = i + 1; k < kBits; ++k) x[k] -= corr[k * nj + np + i] * (double)v;
   }
 }
 
 // --------------------------------------------------------------------------- host side
 constexpr int kSms = 148;
-constexpr size_t kSweepMaxSmem = 196 * 1024;               // code words of a sweep block kept in shared memory
+constexpr size_t kSweepMaxSmem = 196 * 1024;               // dynamic shared memory of a sweep block: copy ring and code words
+
+constexpr size_t kMaxSmem = 226 * 1024;                    // dynamic shared memory a block may ask for next to its static part
+// tiles, signs of 32 (blk + 1) bits, room for the last A operand (128 rows a half) to reach past its signs, and alignment
+inline size_t gather_smem(int groups, int blk) {
+  return (size_t)groups * (kTileBytes + (size_t)kBits * (blk + 1) * kTileKeys * 2) + (size_t)(2048 * (blk / 4 + 1) - 512 * (blk + 1)) + 1024;
+}
 
 inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 inline int t_stride_of(const bpc_config* c) { return (c->n_max + kTileKeys - 1) / kTileKeys * kTileKeys; }
@@ -875,6 +1058,7 @@ const SweepLimits* sweep_limits(int device) {
   SweepLimits* l = &g_sweep_limits[device];
   std::call_once(l->once, [l]() {
     cudaError_t e = cudaFuncSetAttribute(fit_sweep_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSweepMaxSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fit_sweep_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSweepRing);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fit_sweep_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(fit_sweep_kernel<false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     for (int cs = 1; cs <= BPC_MAX_CLUSTER && e == cudaSuccess; ++cs) {
@@ -901,7 +1085,7 @@ int sweep_cluster(const bpc_config* c, const SweepLimits* l) {
     const int nk = block_rows(c->n_max, cs);
     const int rounds = (nk / 128 + kSweepWarps - 1) / kSweepWarps;
     const int waves = (units + l->active[cs] - 1) / l->active[cs];
-    const double cost = waves * (rounds * ((size_t)nk * 4 > kSweepMaxSmem ? 1.5 : 1.0) + 4.0 + 0.1 * cs);
+    const double cost = waves * (rounds * (kSweepRing + (size_t)nk * 4 > kSweepMaxSmem ? 1.5 : 1.0) + 4.0 + 0.1 * cs);
     if (best_cost == 0.0 || cost < best_cost) { best_cost = cost; best = cs; }
   }
   return best;
@@ -919,14 +1103,14 @@ cudaError_t launch_project_tc(const bpc_ctx* ctx, const void* k_cache, const uin
   return cudaGetLastError();
 }
 
-template <int HALVES, int NBUF>
+template <int GROUPS>
 cudaError_t launch_gather_tc(const bpc_ctx* ctx, const void* k_cache, const uint32_t* hfit, double* wpart, int32_t* apart, int blk, int parts,
                              cudaStream_t stream) {
   const bpc_config& c = ctx->cfg;
-  const size_t smem = (size_t)kGatherGroups * (NBUF * kTileBytes + 128 * HALVES * kTileKeys * 2) + 1024;
-  cudaError_t e = cudaFuncSetAttribute(fit_gather_tc_kernel<HALVES, NBUF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const size_t smem = gather_smem(GROUPS, blk);
+  cudaError_t e = cudaFuncSetAttribute(fit_gather_tc_kernel<GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  fit_gather_tc_kernel<HALVES, NBUF><<<dim3(parts, ctx->units), kGroupThreads * kGatherGroups, smem, stream>>>(
+  fit_gather_tc_kernel<GROUPS><<<dim3(parts, ctx->units), kGroupThreads * GROUPS, smem, stream>>>(
       (const __nv_bfloat16*)k_cache, hfit, wpart, apart, ctx->unit_lens, ctx->dev_err, c.n_max, ctx->row_stride, c.code_bits, blk);
   return cudaGetLastError();
 }
@@ -948,12 +1132,16 @@ cudaError_t bpc_launch_fit_blocked(bpc_ctx* ctx, const void* k_cache, const floa
   const SweepLimits* lim = sweep_limits(ctx->device);
   if (lim == nullptr || lim->status != cudaSuccess) return lim == nullptr ? cudaErrorInvalidDevice : lim->status;
   const int cs = sweep_cluster(&c, lim);
-  const size_t words_bytes = (size_t)block_rows(c.n_max, cs) * 4;
+  const size_t sweep_smem = kSweepRing + (size_t)block_rows(c.n_max, cs) * 4;
   const bool tc = c.kv_dtype == BPC_BF16;
   const dim3 grid(parts, ctx->units);
   cudaError_t e = cudaSuccess;
   for (int blk = 0; blk < b / kBits && e == cudaSuccess; ++blk) {
-    if (blk > 0) fit_cross_kernel<<<dim3(blk, ctx->units), 256, 0, stream>>>(ctx->P, v_star, cross, b, blk);
+    if (blk > 0) {                                         // cross[j][l] = v_j . d_l for the bits so far and this block's columns
+      const size_t set = (size_t)b * BPC_D;
+      e = bpc_launch_dots(ctx->P, set, v_star + (size_t)kBits * blk * BPC_D, set, cross, (size_t)b * kBits, kBits, blk, 1, ctx->units, stream);
+      if (e != cudaSuccess) return e;
+    }
     if (tc) {
       // three warpgroups while the scalars of the earlier bits leave room for them (up to five earlier words)
       e = blk <= 5 ? launch_project_tc<3>(ctx, k_cache, hfit, v_star, cross, T, blk, parts, ts, stream)
@@ -964,27 +1152,30 @@ cudaError_t bpc_launch_fit_blocked(bpc_ctx* ctx, const void* k_cache, const floa
     }
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr;
-    if (words_bytes <= kSweepMaxSmem) {
-      cudaLaunchConfig_t cfg = sweep_config(&attr, ctx->units, cs, words_bytes, stream);
-      e = cudaLaunchKernelEx(&cfg, fit_sweep_kernel<true>, (const float*)T, hfit, words_g, (const int32_t*)ctx->unit_lens, (int)c.n_max, b, blk, ts, cs);
+    if (sweep_smem <= kSweepMaxSmem) {
+      cudaLaunchConfig_t cfg = sweep_config(&attr, ctx->units, cs, sweep_smem, stream);
+      e = cudaLaunchKernelEx(&cfg, fit_sweep_kernel<true>, (const float*)T, hfit, words_g, (const int32_t*)ctx->unit_lens, ctx->dev_err, (int)c.n_max, b, blk, ts, cs);
     } else {
-      cudaLaunchConfig_t cfg = sweep_config(&attr, ctx->units, cs, 0, stream);
-      e = cudaLaunchKernelEx(&cfg, fit_sweep_kernel<false>, (const float*)T, hfit, words_g, (const int32_t*)ctx->unit_lens, (int)c.n_max, b, blk, ts, cs);
+      cudaLaunchConfig_t cfg = sweep_config(&attr, ctx->units, cs, kSweepRing, stream);
+      e = cudaLaunchKernelEx(&cfg, fit_sweep_kernel<false>, (const float*)T, hfit, words_g, (const int32_t*)ctx->unit_lens, ctx->dev_err, (int)c.n_max, b, blk, ts, cs);
     }
     if (e != cudaSuccess) return e;
     if (tc) {
-      e = b <= 128 ? launch_gather_tc<1, 2>(ctx, k_cache, hfit, wpart, apart, blk, parts, stream)
-                   : launch_gather_tc<2, 1>(ctx, k_cache, hfit, wpart, apart, blk, parts, stream);
+      // as many warpgroups as their tile and sign buffers leave room for (four up to the third word, two from the sixth)
+      if (gather_smem(4, blk) <= kMaxSmem) e = launch_gather_tc<4>(ctx, k_cache, hfit, wpart, apart, blk, parts, stream);
+      else if (gather_smem(3, blk) <= kMaxSmem) e = launch_gather_tc<3>(ctx, k_cache, hfit, wpart, apart, blk, parts, stream);
+      else e = launch_gather_tc<2>(ctx, k_cache, hfit, wpart, apart, blk, parts, stream);
     } else {
       fit_gather_f32_kernel<<<grid, 256, 0, stream>>>((const float*)k_cache, hfit, wpart, apart, ctx->unit_lens, c.n_max, ctx->row_stride, b, blk);
     }
     if (e != cudaSuccess) return e;
-    const size_t rows_smem = (size_t)(kBits * kBits * (blk + 1) + kBits * BPC_D) * 8;
+    fit_sum_parts_kernel<<<dim3(16 + 4 * (blk + 1), ctx->units), 256, 0, stream>>>(wpart, apart, ctx->unit_lens, c.n_max, b, blk, parts);
+    const size_t rows_smem = (size_t)(kBits * kBits * (blk + 1) + kBits * blk * 32 + kBits * 32) * 8;
     e = cudaFuncSetAttribute(fit_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rows_smem);
     if (e != cudaSuccess) return e;
-    fit_rows_kernel<<<ctx->units, BPC_D * 4, rows_smem, stream>>>(wpart, apart, ctx->P, ctx->unit_lens, c.n_max, b, blk, parts);
+    fit_rows_kernel<<<dim3(4, ctx->units), 512, rows_smem, stream>>>(wpart, apart, ctx->P, ctx->unit_lens, c.n_max, b, blk, parts);
     e = cudaGetLastError();
-    *launches += blk > 0 ? 5 : 4;
+    *launches += blk > 0 ? 6 : 5;
   }
   return e;
 }

@@ -27,18 +27,51 @@ template <> __global__ void round_projection_kernel<__nv_bfloat16>(const float* 
   }
 }
 
-__global__ void gram_kernel(const float* __restrict__ Phf, float* __restrict__ gram, int b) {
-  // grid (b, hash_sets); thread j computes G[i][j] with fp64 accumulation
-  const int i = blockIdx.x, s = blockIdx.y;
-  const float* base = Phf + (size_t)s * b * BPC_D;
-  __shared__ float ri[BPC_D];
-  for (int c = threadIdx.x; c < BPC_D; c += blockDim.x) ri[c] = base[(size_t)i * BPC_D + c];
-  __syncthreads();
-  for (int j = threadIdx.x; j < b; j += blockDim.x) {
-    const float* rj = base + (size_t)j * BPC_D;
-    double acc = 0.0;
-    for (int c = 0; c < BPC_D; ++c) acc = fma((double)ri[c], (double)rj[c], acc);
-    gram[((size_t)s * b + i) * b + j] = (float)acc;
+// C[i][j] = A_i . B_j for 16 x 32 tiles of row pairs, fp64 products summed in channel order; grid (tiles of A, tiles of B,
+// sets).  Rows are converted to fp64 once on their way to shared memory and a thread keeps 2 x 2 sums.  fp64 issue bounds
+// it: small tiles spread few sets over more SMs, and a Gram matrix (A = B, `symmetric`) leaves the tiles left of the
+// diagonal to their mirror images.  (One thread per sum with a conversion per operand of each product: 266 us for the Gram
+// matrices of 32 sets of 128 bits.)
+constexpr int kDotThreads = 128;
+constexpr int kDotChannels = 64;
+__global__ void __launch_bounds__(kDotThreads)
+dots_kernel(const float* __restrict__ A, size_t a_set, const float* __restrict__ B, size_t b_set, float* __restrict__ C, size_t c_set, int ldc,
+            int symmetric) {
+  __shared__ double as[16][kDotChannels + 1], bs[32][kDotChannels + 1];
+  const int i0 = 16 * blockIdx.x, j0 = 32 * blockIdx.y;
+  if (symmetric && j0 + 31 < i0) return;
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const float* a = A + blockIdx.z * a_set + (size_t)i0 * BPC_D;
+  const float* b = B + blockIdx.z * b_set + (size_t)j0 * BPC_D;
+  double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+  for (int c0 = 0; c0 < BPC_D; c0 += kDotChannels) {
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 16 * kDotChannels / kDotThreads; ++k) {
+      const int e = tid + k * kDotThreads;
+      as[e / kDotChannels][e % kDotChannels] = (double)a[(size_t)(e / kDotChannels) * BPC_D + c0 + e % kDotChannels];
+    }
+#pragma unroll
+    for (int k = 0; k < 32 * kDotChannels / kDotThreads; ++k) {
+      const int e = tid + k * kDotThreads;
+      bs[e / kDotChannels][e % kDotChannels] = (double)b[(size_t)(e / kDotChannels) * BPC_D + c0 + e % kDotChannels];
+    }
+    __syncthreads();
+#pragma unroll 16
+    for (int c = 0; c < kDotChannels; ++c) {
+      const double b0 = bs[tx][c], b1 = bs[tx + 16][c], a0 = as[ty][c], a1 = as[ty + 8][c];
+      acc[0][0] = fma(a0, b0, acc[0][0]);
+      acc[0][1] = fma(a0, b1, acc[0][1]);
+      acc[1][0] = fma(a1, b0, acc[1][0]);
+      acc[1][1] = fma(a1, b1, acc[1][1]);
+    }
+  }
+  float* out = C + blockIdx.z * c_set;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int i = i0 + ty + 8 * (q >> 1), j = j0 + tx + 16 * (q & 1);
+    out[(size_t)i * ldc + j] = (float)acc[q >> 1][q & 1];
+    if (symmetric && j > i) out[(size_t)j * ldc + i] = (float)acc[q >> 1][q & 1];
   }
 }
 
@@ -644,6 +677,12 @@ build_eas_kernel(const float* __restrict__ key_err, const int32_t* __restrict__ 
 }  // namespace
 
 // =========================================================================== host launchers
+cudaError_t bpc_launch_dots(const float* A, size_t a_set, const float* B, size_t b_set, float* C, size_t c_set, int ldc, int tiles_a, int tiles_b,
+                            int sets, cudaStream_t stream) {
+  dots_kernel<<<dim3(2 * tiles_a, tiles_b, sets), kDotThreads, 0, stream>>>(A, a_set, B, b_set, C, c_set, ldc, A == B);
+  return cudaGetLastError();
+}
+
 cudaError_t bpc_launch_finalize_projection(bpc_ctx* ctx, cudaStream_t stream) {
   const bpc_config& c = ctx->cfg;
   const size_t n = (size_t)c.hash_sets * c.code_bits * BPC_D;
@@ -653,9 +692,10 @@ cudaError_t bpc_launch_finalize_projection(bpc_ctx* ctx, cudaStream_t stream) {
     round_projection_kernel<__nv_bfloat16><<<blocks, th, 0, stream>>>(ctx->P, (__nv_bfloat16*)ctx->P_h, ctx->P_hf, n);
   else
     round_projection_kernel<float><<<blocks, th, 0, stream>>>(ctx->P, (float*)ctx->P_h, ctx->P_hf, n);
-  gram_kernel<<<dim3(c.code_bits, c.hash_sets), 128, 0, stream>>>(ctx->P_hf, ctx->gram, c.code_bits);
   ctx->launches += 2;
-  return cudaGetLastError();
+  const size_t set = (size_t)c.code_bits * BPC_D;
+  return bpc_launch_dots(ctx->P_hf, set, ctx->P_hf, set, ctx->gram, (size_t)c.code_bits * c.code_bits, c.code_bits, c.code_bits / 32,
+                         c.code_bits / 32, c.hash_sets, stream);
 }
 
 cudaError_t bpc_launch_encode_simple(bpc_ctx* ctx, const void* k_cache, uint64_t* codes, cudaStream_t stream) {
