@@ -70,34 +70,45 @@ __device__ __forceinline__ void split3(float v, __nv_bfloat16 (&t)[3]) {   // v 
   t[2] = __float2bfloat16_rn(r1 - __bfloat162float(t[1]));
 }
 
-// 32 x 32 bit transpose across the lanes of a warp: lane i returns bit i of every lane
-__device__ __forceinline__ uint32_t warp_transpose(uint32_t x, int lane) {
-  uint32_t m = 0x0000FFFFu;
+// 32 x 32 bit transposes across the lanes of a warp, N words at once: lane i returns bit i of every lane.  Halves and bytes
+// move with one byte permute, smaller fields with a rotation and a merge.
+template <int N>
+__device__ __forceinline__ void warp_transpose(uint32_t (&x)[N], int lane) {
 #pragma unroll
-  for (int o = 16; o >= 1; o >>= 1) {
-    const uint32_t y = __shfl_xor_sync(0xffffffffu, x, o);
-    x = (lane & o) ? ((x & ~m) | ((y >> o) & m)) : ((x & m) | ((y & m) << o));
-    m ^= m << (o >> 1);
-  }
-  return x;
-}
-
-__device__ __forceinline__ void warp_transpose4(uint32_t (&x)[4], int lane) {   // four at once: the shuffles overlap
-  uint32_t m = 0x0000FFFFu;
-#pragma unroll
-  for (int o = 16; o >= 1; o >>= 1) {
+  for (int st = 0; st < 5; ++st) {
+    const int o = 16 >> st;
     const bool up = lane & o;
-    uint32_t y[4];
+    const uint32_t low = o == 16 ? 0u : o == 8 ? 0u : o == 4 ? 0x0F0F0F0Fu : o == 2 ? 0x33333333u : 0x55555555u;
+    const uint32_t keep = up ? ~low : low, sel = o == 16 ? (up ? 0x3276u : 0x5410u) : (up ? 0x3715u : 0x6240u);
+    const int rot = up ? 32 - o : o;
+    uint32_t y[N];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) y[k] = __shfl_xor_sync(0xffffffffu, x[k], o);
+    for (int k = 0; k < N; ++k) y[k] = __shfl_xor_sync(0xffffffffu, x[k], o);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) x[k] = up ? ((x[k] & ~m) | ((y[k] >> o) & m)) : ((x[k] & m) | ((y[k] << o) & ~m));
-    m ^= m << (o >> 1);
+    for (int k = 0; k < N; ++k)
+      x[k] = o >= 8 ? __byte_perm(x[k], y[k], sel) : ((x[k] & keep) | (__funnelshift_l(y[k], y[k], rot) & ~keep));
   }
+}
+__device__ __forceinline__ uint32_t warp_transpose(uint32_t x, int lane) {
+  uint32_t v[1] = {x};
+  warp_transpose<1>(v, lane);
+  return v[0];
 }
 
 // rows of a unit that block `blk` of `blocks` takes: equal shares of whole tiles
 __host__ __device__ inline int block_rows(int n, int blocks) { return ((n + blocks - 1) / blocks + kTileKeys - 1) / kTileKeys * kTileKeys; }
+
+// ---- sweep geometry (the projection fills the columns up to a whole group of keys)
+constexpr int kSweepThreads = 512;
+constexpr int kSweepWarps = kSweepThreads / 32;
+constexpr int kSweepPlanes = 8;
+constexpr int kSweepKeys = 8;                              // keys of a thread per round: two runs of four, 128 apart
+constexpr int kSweepGroup = 32 * kSweepKeys;               // keys of a warp per round
+constexpr int kSweepSlotBytes = 4 * kSweepThreads * 16;    // one round of two columns (two slots: in use, in flight)
+constexpr int kSweepRing = 2 * kSweepSlotBytes;
+constexpr int kSweepFlush = 30;                            // rounds of eight keys between flushes: 240 < 2^kSweepPlanes counts
+// keys of a sweep block: equal shares in whole groups (columns are zero up to a whole group past the last key)
+__host__ __device__ inline int sweep_share(int n, int blocks) { return ((n + blocks - 1) / blocks + kSweepGroup - 1) / kSweepGroup * kSweepGroup; }
 
 // --------------------------------------------------------------------------- project (tensor cores, bf16 caches)
 // T[l][key] for the 32 columns of block `blk`.  Per tile of 128 keys: eight MMAs K_tile x D (N = 96: three bf16 terms of
@@ -259,6 +270,9 @@ fit_project_tc_kernel(const __nv_bfloat16* __restrict__ k_cache, const uint32_t*
       dst[(size_t)l * t_stride] = live ? v + 0.f : 0.f;                // (never -0)
     }
   }
+  // the sweep reads whole groups of keys: zeros behind the unit's last tile where that ends half a group
+  for (int i = row0 + ntile * kTileKeys + tid; row_end == n && i < (n + kSweepGroup - 1) / kSweepGroup * kSweepGroup; i += kThreads)
+    for (int l = 0; l < kBits; ++l) T[((size_t)unit * kBits + l) * t_stride + i] = 0.f;
   if (timed_out_g[grp] && gtid == 0) atomicOr(err, BPC_DEVERR_TIMEOUT);
   cp_async_wait_all();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -275,7 +289,7 @@ fit_project_f32_kernel(const float* __restrict__ k_cache, const uint32_t* __rest
   const int unit = blockIdx.y, tid = threadIdx.x;
   const int n = min(unit_lens[unit], n_max);
   const int row = blockIdx.x * kTileKeys + tid;
-  if (blockIdx.x * kTileKeys >= n) return;
+  if (blockIdx.x * kTileKeys >= (n + kSweepGroup - 1) / kSweepGroup * kSweepGroup) return;   // (zeros up to a whole sweep group)
   const bool live = row < n;
   __shared__ __align__(16) float d_s[BPC_D][kBits];                    // directions, channel-major; then the scalars of 32 bits
   double acc[kBits];
@@ -564,13 +578,6 @@ fit_gather_f32_kernel(const float* __restrict__ k_cache, const uint32_t* __restr
 // bits), decide, and add the next column's entry to the running sums of the bits that are set (the sum over set bits
 // gives u_i^T T = 2 sum - total).  Agreements with the earlier bits are counted bit-sliced, 32 bits per operation.
 // The loop body is compiled for 8, 16, 24 and 32 bits in play.
-constexpr int kSweepThreads = 512;
-constexpr int kSweepWarps = kSweepThreads / 32;
-constexpr int kSweepPlanes = 8;
-constexpr int kSweepSlots = 3;                             // rounds of the two columns in flight or in use, per thread 32 bytes each
-constexpr int kSweepSlotBytes = 2 * kSweepThreads * 16;
-constexpr int kSweepRing = kSweepSlots * kSweepSlotBytes;
-constexpr int kSweepFlush = 60;                            // rounds of four keys between flushes: 240 < 2^kSweepPlanes counts
 
 struct SweepSums {                                         // lane i: bit i
   double s;                                                // u_i^T T over this warp's keys
@@ -589,8 +596,12 @@ struct SweepStream {
   __device__ __forceinline__ void request(unsigned char* slot) {      // (always a group, so that the waits can count)
     if (bit < kBits) {
       cp_async16(slot, next);
-      if (bit + 1 < kBits) cp_async16(slot + kSweepThreads * 16, next + t_stride);
-      next += kSweepWarps * 128;
+      cp_async16(slot + kSweepThreads * 16, next + 128);
+      if (bit + 1 < kBits) {
+        cp_async16(slot + 2 * kSweepThreads * 16, next + t_stride);
+        cp_async16(slot + 3 * kSweepThreads * 16, next + t_stride + 128);
+      }
+      next += kSweepWarps * kSweepGroup;
       if (++round == rounds) {
         round = 0;
         ++bit;
@@ -625,6 +636,23 @@ __device__ __forceinline__ void full_add(uint32_t a, uint32_t b, uint32_t c, uin
   s = a ^ b ^ c;
   cy = (a & b) | (c & (a | b));
 }
+// bit-sliced counters: adds the set bits of eight words to the planes
+__device__ __forceinline__ void count8(uint32_t (&pl)[kSweepPlanes], const uint32_t (&x)[8]) {
+  uint32_t s1, s2, s3, s4, c1, c2, c3, c4, d1, d2, e;
+  full_add(x[0], x[1], x[2], s1, c1);
+  full_add(x[3], x[4], x[5], s2, c2);
+  full_add(x[6], x[7], pl[0], s3, c3);
+  full_add(s1, s2, s3, pl[0], c4);
+  full_add(c1, c2, c3, s4, d1);
+  full_add(pl[1], s4, c4, pl[1], d2);
+  full_add(pl[2], d1, d2, pl[2], e);
+#pragma unroll
+  for (int k = 3; k < kSweepPlanes; ++k) {
+    const uint32_t nc = pl[k] & e;
+    pl[k] ^= e;
+    e = nc;
+  }
+}
 
 // acc += v where w has bit I set (written out so that the tests of a word become predicates, not selects)
 template <int I>
@@ -639,22 +667,26 @@ __device__ __forceinline__ void add_bits(float (&acc)[NS], float v, uint32_t w) 
     add_bits<I + 1, N>(acc, v, w);
   }
 }
-// entry (w >> 4 NB) & 15 of the look-up table's row NB; `base` is the table's shared-memory address, 512-byte aligned
+// entry (w >> 8 NB) & 255 of the look-up table's row NB; `base` is the table's shared-memory address, 1024-byte aligned.
+// (A byte per look-up: the lanes' bank conflicts cost the shared-memory pipe less than twice the address arithmetic of
+// conflict-free nibbles costs the integer pipe, which bounds the pass.)
 template <int NB>
 __device__ __forceinline__ float lut_at(unsigned base, uint32_t w) {
-  const uint32_t x = NB == 0 ? w << 2 : w >> (4 * NB - 2);
+  const uint32_t x = NB == 0 ? w << 2 : w >> (8 * NB - 2);
   float v;
-  asm volatile("ld.shared.f32 %0, [%1 + %2];" : "=f"(v) : "r"((x & 0x3Cu) | base), "n"(64 * NB));
+  asm volatile("ld.shared.f32 %0, [%1 + %2];" : "=f"(v) : "r"((x & 0x3FCu) | base), "n"(1024 * NB));
   return v;
 }
-template <int NB, int N>
-__device__ __forceinline__ float lut_sum(unsigned base, uint32_t w) {      // rows NB, NB + 2, ...
-  if constexpr (NB + 2 < N) return lut_at<NB>(base, w) + lut_sum<NB + 2, N>(base, w);
-  else return lut_at<NB>(base, w);
+template <int N>
+__device__ __forceinline__ float lut_sum(unsigned base, uint32_t w) {      // rows 0 .. N - 1
+  if constexpr (N == 1) return lut_at<0>(base, w);
+  else if constexpr (N == 2) return lut_at<0>(base, w) + lut_at<1>(base, w);
+  else if constexpr (N == 3) return (lut_at<0>(base, w) + lut_at<1>(base, w)) + lut_at<2>(base, w);
+  else return (lut_at<0>(base, w) + lut_at<1>(base, w)) + (lut_at<2>(base, w) + lut_at<3>(base, w));
 }
 
 // One pass over this block's keys: decides bit j; unless it is the block's last bit, also the sums for column j + 1.
-// Q4 = groups of four bits in play (j / 4 + 1).  Keys past the end (up to 127, all in the last group of the unit's last
+// Q4 = groups of four bits in play (j / 4 + 1).  Keys past the end (up to 255, all in the last group of the unit's last
 // block, entries zero) take part like any others and are subtracted at the end: they all carry the same code word.
 template <int Q4, bool LAST>
 __device__ __forceinline__ void sweep_pass(SweepStream& in, uint32_t* __restrict__ ws, unsigned lut, int j, int nk, int nkeys, int warp,
@@ -663,7 +695,7 @@ __device__ __forceinline__ void sweep_pass(SweepStream& in, uint32_t* __restrict
   out.s = 0.0;
   out.cnt = 0;
   const uint32_t bit = 1u << j;
-  const int ng = nk / 128;
+  const int ng = nk / kSweepGroup;
   for (int g0 = warp; g0 < ng; g0 += kSweepWarps * kSweepFlush) {
     float s[NS];
     float tot = 0.f;
@@ -673,56 +705,47 @@ __device__ __forceinline__ void sweep_pass(SweepStream& in, uint32_t* __restrict
 #pragma unroll
     for (int k = 0; k < kSweepPlanes; ++k) pl[k] = 0u;
     const int g1 = min(ng, g0 + kSweepWarps * kSweepFlush);
-    uint32_t* pw = ws + g0 * 128 + 4 * lane;
+    uint32_t* pw = ws + g0 * kSweepGroup + 4 * lane;
     for (int g = g0; g < g1; g += kSweepWarps) {
-      int ahead = in.at + 2 * kSweepSlotBytes;
-      if (ahead >= kSweepRing) ahead -= kSweepRing;
-      in.request(in.ring + ahead);
-      asm volatile("cp.async.wait_group 2;" ::: "memory");
-      const float4 t4 = *reinterpret_cast<const float4*>(in.ring + in.at);
-      const float4 n4 = *reinterpret_cast<const float4*>(in.ring + in.at + kSweepThreads * 16);
-      in.at += kSweepSlotBytes;
-      if (in.at == kSweepRing) in.at = 0;
-      const float t[4] = {t4.x, t4.y, t4.z, t4.w};
-      const float nx[4] = {n4.x, n4.y, n4.z, n4.w};
-      const uint4 w4 = *reinterpret_cast<const uint4*>(pw);
-      uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w}, x[4];
+      in.request(in.ring + (in.at ^ kSweepSlotBytes));
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+      const unsigned char* slot = in.ring + in.at;
+      in.at ^= kSweepSlotBytes;
+      uint32_t x[kSweepKeys];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float c = Q4 == 1 ? lut_at<0>(lut, w[e]) : lut_sum<0, Q4>(lut, w[e]) + lut_sum<1, Q4>(lut, w[e]);
-        const uint32_t neg = (uint32_t)((int)__float_as_uint(t[e] - c) >> 31);   // (never -0: columns hold no -0)
-        x[e] = w[e] ^ neg;                                 // bit i: agrees with the new bit
-        w[e] |= bit & ~neg;
-        if (!LAST) {
-          tot += nx[e];
-          add_bits<0, 4 * Q4>(s, nx[e], w[e]);
-        }
-      }
-      *reinterpret_cast<uint4*>(pw) = make_uint4(w[0], w[1], w[2], w[3]);
-      pw += kSweepWarps * 128;
-      if (!LAST) {
-        uint32_t s1, ca, cb, cc;
-        full_add(x[0], x[1], x[2], s1, ca);
-        full_add(pl[0], s1, x[3], pl[0], cb);
-        full_add(pl[1], ca, cb, pl[1], cc);
+      for (int h = 0; h < 2; ++h) {
+        const float4 t4 = *reinterpret_cast<const float4*>(slot + h * kSweepThreads * 16);
+        const float4 n4 = *reinterpret_cast<const float4*>(slot + (2 + h) * kSweepThreads * 16);
+        const uint4 w4 = *reinterpret_cast<const uint4*>(pw + 128 * h);
+        const float t[4] = {t4.x, t4.y, t4.z, t4.w};
+        const float nx[4] = {n4.x, n4.y, n4.z, n4.w};
+        uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w};
 #pragma unroll
-        for (int k = 2; k < kSweepPlanes; ++k) {
-          const uint32_t nc = pl[k] & cc;
-          pl[k] ^= cc;
-          cc = nc;
+        for (int e = 0; e < 4; ++e) {
+          const float c = lut_sum<(Q4 + 1) / 2>(lut, w[e]);
+          const uint32_t neg = (uint32_t)((int)__float_as_uint(t[e] - c) >> 31);   // (never -0: columns hold no -0)
+          x[4 * h + e] = w[e] ^ neg;                       // bit i: agrees with the new bit
+          w[e] |= bit & ~neg;
+          if (!LAST) {
+            tot += nx[e];
+            add_bits<0, 4 * Q4>(s, nx[e], w[e]);
+          }
         }
+        *reinterpret_cast<uint4*>(pw + 128 * h) = make_uint4(w[0], w[1], w[2], w[3]);
       }
+      pw += kSweepWarps * kSweepGroup;
+      if (!LAST) count8(pl, x);
     }
     if (!LAST) {
 #pragma unroll
       for (int o = 16; o >= 1; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
       out.s += 2.0 * (double)warp_sum_scatter<NS>(s, lane) - (double)tot;
-      const int keys_per_lane = 4 * ((g1 - g0 + kSweepWarps - 1) / kSweepWarps);
+      const int keys_per_lane = kSweepKeys * ((g1 - g0 + kSweepWarps - 1) / kSweepWarps);
 #pragma unroll
       for (int k0 = 0; k0 < kSweepPlanes; k0 += 4) {       // four independent transposes at a time
         if ((keys_per_lane >> k0) == 0) break;             // higher planes are empty
         uint32_t x[4] = {pl[k0], pl[k0 + 1], pl[k0 + 2], pl[k0 + 3]};
-        warp_transpose4(x, lane);
+        warp_transpose<4>(x, lane);
 #pragma unroll
         for (int k = 0; k < 4; ++k) out.cnt += __popc(x[k]) << (k0 + k);
       }
@@ -767,7 +790,8 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
 fit_sweep_kernel(const float* __restrict__ T, uint32_t* __restrict__ hfit, uint32_t* __restrict__ words_g,
                  const int32_t* __restrict__ unit_lens, int32_t* __restrict__ err, int n_max, int b, int blk, int t_stride, int cluster_size) {
   extern __shared__ __align__(16) unsigned char sweep_smem[];   // the copy ring, then (SMEM_WORDS) this block's code words
-  __shared__ __align__(512) float lut[8 * 16];             // lut[nibble][pattern] = sum of +-c over the nibble's bits
+  __shared__ __align__(1024) float lut[4 * 256];           // lut[byte][pattern] = sum of +-c over the byte's bits
+  __shared__ float nib[8 * 16];                            // the same by nibble
   __shared__ double red_s[kSweepWarps][32];
   __shared__ int red_c[kSweepWarps][32];
   __shared__ double slot_s[2][BPC_MAX_CLUSTER][32];        // the cluster's sums of bit i, by rank; two passes alternate
@@ -782,13 +806,13 @@ fit_sweep_kernel(const float* __restrict__ T, uint32_t* __restrict__ hfit, uint3
   const int rank = blockIdx.x % cluster_size, unit = blockIdx.x / cluster_size;
   const int n = min(unit_lens[unit], n_max);
   if (n <= 0) return;                                      // (the whole cluster)
-  const int share = block_rows(n, cluster_size);
+  const int share = sweep_share(n, cluster_size);
   const int row0 = rank * share;
-  const int nkeys = max(0, min(n - row0, share));          // keys of this block; nk = the same in whole groups of 128
-  const int nk = (nkeys + 127) / 128 * 128;
+  const int nkeys = max(0, min(n - row0, share));          // keys of this block; nk = the same in whole groups
+  const int nk = (nkeys + kSweepGroup - 1) / kSweepGroup * kSweepGroup;
   uint32_t* ws = SMEM_WORDS ? reinterpret_cast<uint32_t*>(sweep_smem + kSweepRing) : words_g + (size_t)unit * t_stride + row0;
   for (int i = tid; i < nk / 4; i += kSweepThreads) reinterpret_cast<uint4*>(ws)[i] = make_uint4(0u, 0u, 0u, 0u);
-  if (tid < 128) lut[tid] = 0.f;
+  for (int i = tid; i < 4 * 256; i += kSweepThreads) lut[i] = 0.f;
   if (tid < 32) c_s[tid] = 0.f;
   for (int i = tid; i < 32 * 33; i += kSweepThreads) (&inv_s[0][0])[i] = 0.0;
   if (tid == 0) {
@@ -811,15 +835,14 @@ fit_sweep_kernel(const float* __restrict__ T, uint32_t* __restrict__ hfit, uint3
       asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(Tu + (size_t)c * t_stride + 4 * at), "r"(16 * cnt) : "memory");
   };
   SweepStream in;
-  in.base = in.next = Tu + warp * 128 + 4 * lane;
+  in.base = in.next = Tu + warp * kSweepGroup + 4 * lane;
   in.t_stride = t_stride;
-  in.rounds = (nk / 128 - warp + kSweepWarps - 1) / kSweepWarps;
+  in.rounds = (nk / kSweepGroup - warp + kSweepWarps - 1) / kSweepWarps;
   in.bit = in.rounds > 0 ? 0 : kBits;                      // (a warp without keys requests nothing)
   in.round = 0;
   in.ring = sweep_smem + 16 * tid;
   in.at = 0;
   in.request(in.ring);
-  in.request(in.ring + kSweepSlotBytes);
   for (int j = 0; j < kBits; ++j) {
     SweepSums sums;
     if (j == kBits - 1) { sweep_pass<8, true>(in, ws, lut_a, j, nk, nkeys, warp, lane, sums); break; }
@@ -891,7 +914,7 @@ fit_sweep_kernel(const float* __restrict__ T, uint32_t* __restrict__ hfit, uint3
         for (int q = 0; q < 4; ++q) {
           const int e = lane + 32 * q;
           const float4 d = *reinterpret_cast<const float4*>(&c_s[4 * (e >> 4)]);
-          lut[e] = (((e & 1) ? d.x : -d.x) + ((e & 2) ? d.y : -d.y)) + (((e & 4) ? d.z : -d.z) + ((e & 8) ? d.w : -d.w));
+          nib[e] = (((e & 1) ? d.x : -d.x) + ((e & 2) ? d.y : -d.y)) + (((e & 4) ? d.z : -d.z) + ((e & 8) ? d.w : -d.w));
         }
       } else {
         agree_s[lane] = agree;
@@ -905,8 +928,11 @@ fit_sweep_kernel(const float* __restrict__ T, uint32_t* __restrict__ hfit, uint3
       }
     }
     __syncthreads();
+    for (int e = tid; e < 32 * (8 * (j >> 3) + 8); e += kSweepThreads)      // the bytes in play
+      lut[e] = nib[32 * (e >> 8) + (e & 15)] + nib[32 * (e >> 8) + 16 + ((e >> 4) & 15)];
     if (warp == 8) inv_s[j][lane] = new_row;               // (warp 0 has read the inverse; it reads it again two barriers on)
     if (tid == 0) mbar_expect(&bar_s[buf], (unsigned)cluster_size * 32u * 12u);   // arms the barrier for bit j + 2
+    __syncthreads();
   }
   cp_async_wait_all();
   __syncthreads();
@@ -992,7 +1018,7 @@ fit_rows_kernel(const double* __restrict__ wpart, const int32_t* __restrict__ ap
 
 // --------------------------------------------------------------------------- host side
 constexpr int kSms = 148;
-constexpr size_t kSweepMaxSmem = 196 * 1024;               // dynamic shared memory of a sweep block: copy ring and code words
+constexpr size_t kSweepMaxSmem = 194 * 1024;               // dynamic shared memory of a sweep block: copy ring and code words
 
 constexpr size_t kMaxSmem = 226 * 1024;                    // dynamic shared memory a block may ask for next to its static part
 // tiles, signs of 32 (blk + 1) bits, room for the last A operand (128 rows a half) to reach past its signs, and alignment
@@ -1001,7 +1027,7 @@ inline size_t gather_smem(int groups, int blk) {
 }
 
 inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
-inline int t_stride_of(const bpc_config* c) { return (c->n_max + kTileKeys - 1) / kTileKeys * kTileKeys; }
+inline int t_stride_of(const bpc_config* c) { return sweep_share(c->n_max, 1); }
 
 // Blocks per unit of project and gather (one block per SM): the first count from one wave up whose last wave is at least
 // 90 % full (32 units: 9, 8 units: 18, 128 units: 8), not below 384 keys per block.
@@ -1082,8 +1108,8 @@ int sweep_cluster(const bpc_config* c, const SweepLimits* l) {
   int best = 1;
   for (int cs = 1; cs <= BPC_MAX_CLUSTER; ++cs) {
     if (l->active[cs] < 1) continue;
-    const int nk = block_rows(c->n_max, cs);
-    const int rounds = (nk / 128 + kSweepWarps - 1) / kSweepWarps;
+    const int nk = sweep_share(c->n_max, cs);
+    const int rounds = (nk / kSweepGroup + kSweepWarps - 1) / kSweepWarps;
     const int waves = (units + l->active[cs] - 1) / l->active[cs];
     const double cost = waves * (rounds * (kSweepRing + (size_t)nk * 4 > kSweepMaxSmem ? 1.5 : 1.0) + 4.0 + 0.1 * cs);
     if (best_cost == 0.0 || cost < best_cost) { best_cost = cost; best = cs; }
@@ -1132,7 +1158,7 @@ cudaError_t bpc_launch_fit_blocked(bpc_ctx* ctx, const void* k_cache, const floa
   const SweepLimits* lim = sweep_limits(ctx->device);
   if (lim == nullptr || lim->status != cudaSuccess) return lim == nullptr ? cudaErrorInvalidDevice : lim->status;
   const int cs = sweep_cluster(&c, lim);
-  const size_t sweep_smem = kSweepRing + (size_t)block_rows(c.n_max, cs) * 4;
+  const size_t sweep_smem = kSweepRing + (size_t)sweep_share(c.n_max, cs) * 4;
   const bool tc = c.kv_dtype == BPC_BF16;
   const dim3 grid(parts, ctx->units);
   cudaError_t e = cudaSuccess;
@@ -1147,7 +1173,7 @@ cudaError_t bpc_launch_fit_blocked(bpc_ctx* ctx, const void* k_cache, const floa
       e = blk <= 5 ? launch_project_tc<3>(ctx, k_cache, hfit, v_star, cross, T, blk, parts, ts, stream)
                    : launch_project_tc<2>(ctx, k_cache, hfit, v_star, cross, T, blk, parts, ts, stream);
     } else {
-      fit_project_f32_kernel<<<dim3((c.n_max + kTileKeys - 1) / kTileKeys, ctx->units), kTileKeys, 0, stream>>>(
+      fit_project_f32_kernel<<<dim3(ts / kTileKeys, ctx->units), kTileKeys, 0, stream>>>(
           (const float*)k_cache, hfit, v_star, cross, T, ctx->unit_lens, c.n_max, ctx->row_stride, b, blk, ts);
     }
     if (e != cudaSuccess) return e;
