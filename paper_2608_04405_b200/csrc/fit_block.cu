@@ -48,21 +48,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// Signs as bf16 (bit 1 -> +1, 0 -> -1): nibble q of x as four values, from a table of the 16 patterns in shared memory
-// (address 128-byte aligned; one look-up replaces eight logic operations).
-__device__ __forceinline__ uint2 signs4(unsigned table, uint32_t x, int q) {
-  const uint32_t i = q == 0 ? x << 3 : x >> (4 * q - 3);
-  uint2 v;
-  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"((i & 0x78u) | table));
-  return v;
-}
-__device__ __forceinline__ void fill_sign_table(uint2* table, int tid) {
-  if (tid < 16) {
-    const uint32_t p[4] = {(tid & 1) ? 0x3F80u : 0xBF80u, (tid & 2) ? 0x3F80u : 0xBF80u, (tid & 4) ? 0x3F80u : 0xBF80u, (tid & 8) ? 0x3F80u : 0xBF80u};
-    table[tid] = make_uint2(p[0] | (p[1] << 16), p[2] | (p[3] << 16));
-  }
-}
-
 __device__ __forceinline__ void split3(float v, __nv_bfloat16 (&t)[3]) {   // v = t0 + t1 + t2 (24 mantissa bits)
   t[0] = __float2bfloat16_rn(v);
   const float r1 = v - __bfloat162float(t[0]);

@@ -76,76 +76,134 @@ dots_kernel(const float* __restrict__ A, size_t a_set, const float* __restrict__
 }
 
 // --------------------------------------------------------------------------- Algorithm 2 on CUDA cores
-// One thread per key.  Decision values t = k P_h^T are accumulated in fp64 and kept as fp32 in shared
-// memory ([bit][thread]); the greedy sweep u_i = sign(t_i), t_j -= u_i G_ij (j > i) then runs per thread.
-constexpr int kEncThreads = 128;
+// Blocks of 32 keys.  Decision values t = k P_h^T: a register-tiled product in fp64 (a thread owns 2 keys x 4 bits at a
+// time, four running sums per value), kept as fp32 in shared memory.  The greedy sweep u_i = sign(t_i), t_j -= u_i G_ij
+// (j > i) runs with one lane per column of a 32-bit block and four keys per warp: a decision is a shuffle, its corrections
+// one FMA per 32 columns.  fp64 issue bounds it; one thread per key with its own conversions and a column-by-column sweep
+// took 160 us at 4096 keys x 64 bits, where it filled 32 SMs.
+constexpr int kEncThreads = 256;
+constexpr int kEncKeys = 32;
+constexpr int kEncBits = 64;                                         // bits of a projection pass
+constexpr int kEncChannels = 32;                                     // channels of P staged at a time
+constexpr int kEncGramBits = 128;                                    // up to this code length the Gram matrix is kept in shared memory
 
-template <typename KV>
+struct EncSmem {
+  double k[kEncKeys][BPC_D + 1];
+  double p[kEncBits][kEncChannels + 1];
+  float t[kEncKeys][256 + 1];
+};
+
+template <typename KV, int NB>                                       // NB = code words per key
 __global__ void __launch_bounds__(kEncThreads)
 encode_simple_kernel(const KV* __restrict__ k_cache, const float* __restrict__ Phf, const float* __restrict__ gram,
                      const int32_t* __restrict__ unit_lens, uint64_t* __restrict__ codes, int n_kv_heads, int n_max,
-                     int row_stride, int b, int shared_sets, int residual_correction, float* __restrict__ key_err) {
+                     int row_stride, int shared_sets, int residual_correction, float* __restrict__ key_err) {
   extern __shared__ __align__(16) unsigned char smem[];
-  float* ps = reinterpret_cast<float*>(smem);                       // [128 rows of P][128]
-  float* ts = ps + 128 * BPC_D;                                      // [b][kEncThreads]
-  const int unit = blockIdx.y;
+  constexpr int b = 32 * NB;
+  EncSmem& sm = *reinterpret_cast<EncSmem*>(smem);
+  float* g_s = reinterpret_cast<float*>(smem + sizeof(EncSmem));     // [b][b] where it fits
+  const int unit = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n = min(unit_lens[unit], n_max);
-  const int key = blockIdx.x * kEncThreads + threadIdx.x;
-  if (blockIdx.x * kEncThreads >= n) return;                         // whole block beyond the unit: uniform
+  if (blockIdx.x * kEncKeys >= n) return;                            // uniform over the block
   const int set = shared_sets ? unit % n_kv_heads : unit;
   const float* Pset = Phf + (size_t)set * b * BPC_D;
   const float* Gset = gram + (size_t)set * b * b;
-  const bool live = key < n;
-  float kr[BPC_D];
-  {
-    const KV* row = k_cache + ((size_t)unit * n_max + (live ? key : 0)) * row_stride;
-#pragma unroll
-    for (int c = 0; c < BPC_D; ++c) kr[c] = to_float(row[c]);
-  }
-  for (int jb = 0; jb < b; jb += 128) {
-    const int rows = min(128, b - jb);
+  if (b <= kEncGramBits && residual_correction)
+    for (int i = tid; i < b * b / 4; i += kEncThreads) reinterpret_cast<float4*>(g_s)[i] = reinterpret_cast<const float4*>(Gset)[i];
+  for (int key0 = blockIdx.x * kEncKeys; key0 < n; key0 += gridDim.x * kEncKeys) {
     __syncthreads();
-    for (int i = threadIdx.x; i < rows * BPC_D; i += kEncThreads) ps[i] = Pset[(size_t)jb * BPC_D + i];
-    __syncthreads();
-    for (int j = 0; j < rows; ++j) {
-      const float4* pr = reinterpret_cast<const float4*>(ps + j * BPC_D);
-      double a0 = 0, a1 = 0, a2 = 0, a3 = 0;
+    for (int e = tid; e < kEncKeys * BPC_D; e += kEncThreads) {
+      const int r = e / BPC_D, c = e % BPC_D;
+      sm.k[r][c] = key0 + r < n ? (double)to_float(k_cache[((size_t)unit * n_max + key0 + r) * row_stride + c]) : 0.0;
+    }
+    const int tx = tid & 15, ty = tid >> 4;
+    for (int j0 = 0; j0 < b; j0 += kEncBits) {
+      constexpr int JN = (b < kEncBits ? b : kEncBits) / 16;         // bits of a thread: tx, tx + 16, ...
+      double acc[2][JN][4];
 #pragma unroll
-      for (int c4 = 0; c4 < BPC_D / 4; ++c4) {
-        const float4 pv = pr[c4];
-        a0 = fma((double)kr[4 * c4], (double)pv.x, a0);
-        a1 = fma((double)kr[4 * c4 + 1], (double)pv.y, a1);
-        a2 = fma((double)kr[4 * c4 + 2], (double)pv.z, a2);
-        a3 = fma((double)kr[4 * c4 + 3], (double)pv.w, a3);
+      for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int j = 0; j < JN; ++j)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) acc[r][j][q] = 0.0;
+      for (int c0 = 0; c0 < BPC_D; c0 += kEncChannels) {
+        __syncthreads();
+        for (int e = tid; e < 16 * JN * kEncChannels; e += kEncThreads)
+          sm.p[e / kEncChannels][e % kEncChannels] = (double)Pset[(size_t)(j0 + e / kEncChannels) * BPC_D + c0 + e % kEncChannels];
+        __syncthreads();
+#pragma unroll 2
+        for (int c = 0; c < kEncChannels; c += 4) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const double k0 = sm.k[ty][c0 + c + q], k1 = sm.k[ty + 16][c0 + c + q];
+#pragma unroll
+            for (int j = 0; j < JN; ++j) {
+              const double pv = sm.p[tx + 16 * j][c + q];
+              acc[0][j][q] = fma(k0, pv, acc[0][j][q]);
+              acc[1][j][q] = fma(k1, pv, acc[1][j][q]);
+            }
+          }
+        }
       }
-      ts[(size_t)(jb + j) * kEncThreads + threadIdx.x] = (float)((a0 + a1) + (a2 + a3));
-    }
-  }
-  uint32_t* dst = reinterpret_cast<uint32_t*>(codes) + ((size_t)unit * n_max + (live ? key : 0)) * (b / 32);
-  uint32_t word = 0;
-  double abs_sum = 0.0;                                              // sum of |t_i| at decision time
-  for (int i = 0; i < b; ++i) {
-    const float ti = ts[(size_t)i * kEncThreads + threadIdx.x];
-    const bool pos = ti >= 0.f;
-    abs_sum += (double)fabsf(ti);
-    word |= (pos ? 1u : 0u) << (i & 31);
-    if ((i & 31) == 31) {
-      if (live) dst[i >> 5] = word;
-      word = 0;
-    }
-    if (residual_correction) {
-      const float u = pos ? 1.f : -1.f;
-      const float* gi = Gset + (size_t)i * b;
-      for (int j = i + 1; j < b; ++j) ts[(size_t)j * kEncThreads + threadIdx.x] -= u * __ldg(gi + j);
-    }
-  }
-  if (key_err != nullptr && live) {
-    // squared reconstruction error (Eq. 8) from the sweep: ||k - hP||^2 = ||k||^2 - 2 sum|t_i| + trace(G)
-    double k2 = 0.0, trg = 0.0;
 #pragma unroll
-    for (int c = 0; c < BPC_D; ++c) k2 = fma((double)kr[c], (double)kr[c], k2);
-    for (int i = 0; i < b; ++i) trg += (double)__ldg(Gset + (size_t)i * b + i);
-    key_err[(size_t)unit * n_max + key] = (float)fmax(0.0, k2 - 2.0 * abs_sum + trg);
+      for (int j = 0; j < JN; ++j) {
+        sm.t[ty][j0 + tx + 16 * j] = (float)((acc[0][j][0] + acc[0][j][1]) + (acc[0][j][2] + acc[0][j][3]));
+        sm.t[ty + 16][j0 + tx + 16 * j] = (float)((acc[1][j][0] + acc[1][j][1]) + (acc[1][j][2] + acc[1][j][3]));
+      }
+    }
+    __syncthreads();
+    // sweep: keys 4 warp .. 4 warp + 3; lane = column of each 32-bit block
+    float t[4][NB];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int w = 0; w < NB; ++w) t[r][w] = sm.t[4 * warp + r][32 * w + lane];
+    double abs_sum[4] = {0.0, 0.0, 0.0, 0.0};                        // sums of |t_i| at decision time
+#pragma unroll
+    for (int cb = 0; cb < NB; ++cb) {
+      uint32_t word[4] = {0u, 0u, 0u, 0u};
+      for (int i = 0; i < 32; ++i) {
+        float g[NB];
+        if (residual_correction) {
+#pragma unroll
+          for (int w = cb; w < NB; ++w) {
+            const size_t at = (size_t)(32 * cb + i) * b + 32 * w + lane;
+            g[w] = b <= kEncGramBits ? g_s[at] : __ldg(Gset + at);
+          }
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const float ti = __shfl_sync(0xffffffffu, t[r][cb], i);
+          const bool pos = ti >= 0.f;
+          word[r] |= (pos ? 1u : 0u) << i;
+          if (key_err != nullptr) abs_sum[r] += (double)fabsf(ti);
+          if (residual_correction) {
+            const float u = pos ? 1.f : -1.f;
+            if (lane > i) t[r][cb] -= u * g[cb];
+#pragma unroll
+            for (int w = cb + 1; w < NB; ++w) t[r][w] -= u * g[w];
+          }
+        }
+      }
+      if (lane < 4 && key0 + 4 * warp + lane < n) {
+        const uint32_t v = lane == 0 ? word[0] : lane == 1 ? word[1] : lane == 2 ? word[2] : word[3];
+        (reinterpret_cast<uint32_t*>(codes) + ((size_t)unit * n_max + key0 + 4 * warp + lane) * NB)[cb] = v;
+      }
+    }
+    if (key_err != nullptr) {
+      // squared reconstruction error (Eq. 8) from the sweep: ||k - hP||^2 = ||k||^2 - 2 sum|t_i| + trace(G)
+      double trg = 0.0;
+      for (int i = lane; i < b; i += 32) trg += (double)__ldg(Gset + (size_t)i * b + i);
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        double v = trg;
+        for (int c = lane; c < BPC_D; c += 32) v = fma(sm.k[4 * warp + r][c], sm.k[4 * warp + r][c], v);
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0 && key0 + 4 * warp + r < n)
+          key_err[(size_t)unit * n_max + key0 + 4 * warp + r] = (float)fmax(0.0, v - 2.0 * abs_sum[r]);
+      }
+    }
   }
 }
 
@@ -698,28 +756,37 @@ cudaError_t bpc_launch_finalize_projection(bpc_ctx* ctx, cudaStream_t stream) {
                          c.code_bits / 32, c.hash_sets, stream);
 }
 
-cudaError_t bpc_launch_encode_simple(bpc_ctx* ctx, const void* k_cache, uint64_t* codes, cudaStream_t stream) {
+template <typename KV, int NB>
+static cudaError_t launch_encode_simple(bpc_ctx* ctx, const void* k_cache, uint64_t* codes, cudaStream_t stream) {
   const bpc_config& c = ctx->cfg;
-  const int b = c.code_bits;
-  const size_t smem = (size_t)128 * BPC_D * 4 + (size_t)b * kEncThreads * 4;
-  const dim3 grid((c.n_max + kEncThreads - 1) / kEncThreads, ctx->units);
-  const int shared_sets = c.hash_sets != ctx->units;
-  cudaError_t e;
-  if (c.kv_dtype == BPC_BF16) {
-    e = cudaFuncSetAttribute(encode_simple_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    encode_simple_kernel<__nv_bfloat16><<<grid, kEncThreads, smem, stream>>>(
-        (const __nv_bfloat16*)k_cache, ctx->P_hf, ctx->gram, ctx->unit_lens, codes, c.n_kv_heads, c.n_max, ctx->row_stride, b, shared_sets,
-        c.residual_correction, ctx->key_err);
-  } else {
-    e = cudaFuncSetAttribute(encode_simple_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    encode_simple_kernel<float><<<grid, kEncThreads, smem, stream>>>(
-        (const float*)k_cache, ctx->P_hf, ctx->gram, ctx->unit_lens, codes, c.n_kv_heads, c.n_max, ctx->row_stride, b, shared_sets,
-        c.residual_correction, ctx->key_err);
-  }
+  constexpr int b = 32 * NB;
+  const size_t smem = sizeof(EncSmem) + (b <= kEncGramBits ? (size_t)b * b * 4 : 0);
+  cudaError_t e = cudaFuncSetAttribute(encode_simple_kernel<KV, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  // a block per 32 keys up to about eight per SM over all units; longer units loop (the Gram matrix is staged once per block)
+  int blocks = (c.n_max + kEncKeys - 1) / kEncKeys;
+  const int most = (8 * ctx->sm_count + ctx->units - 1) / ctx->units;
+  if (blocks > most) blocks = most;
+  encode_simple_kernel<KV, NB><<<dim3(blocks, ctx->units), kEncThreads, smem, stream>>>(
+      (const KV*)k_cache, ctx->P_hf, ctx->gram, ctx->unit_lens, codes, c.n_kv_heads, c.n_max, ctx->row_stride, c.hash_sets != ctx->units,
+      c.residual_correction, ctx->key_err);
   ctx->launches += 1;
   return cudaGetLastError();
+}
+
+template <typename KV>
+static cudaError_t launch_encode_simple_bits(bpc_ctx* ctx, const void* k_cache, uint64_t* codes, cudaStream_t stream) {
+  switch (ctx->cfg.code_bits) {
+    case 32: return launch_encode_simple<KV, 1>(ctx, k_cache, codes, stream);
+    case 64: return launch_encode_simple<KV, 2>(ctx, k_cache, codes, stream);
+    case 128: return launch_encode_simple<KV, 4>(ctx, k_cache, codes, stream);
+    default: return launch_encode_simple<KV, 8>(ctx, k_cache, codes, stream);
+  }
+}
+
+cudaError_t bpc_launch_encode_simple(bpc_ctx* ctx, const void* k_cache, uint64_t* codes, cudaStream_t stream) {
+  return ctx->cfg.kv_dtype == BPC_BF16 ? launch_encode_simple_bits<__nv_bfloat16>(ctx, k_cache, codes, stream)
+                                       : launch_encode_simple_bits<float>(ctx, k_cache, codes, stream);
 }
 
 cudaError_t bpc_launch_append(bpc_ctx* ctx, const void* k_new, const void* v_new, void* k_cache, void* v_cache,

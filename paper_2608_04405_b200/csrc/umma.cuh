@@ -81,6 +81,29 @@ __device__ __forceinline__ size_t sw128_offset(int rows, int r, int ch) {
   return (size_t)(ch >> 3) * ((size_t)rows * 128) + (size_t)r * 128 + (size_t)(((ch & 7) ^ (r & 7)) << 4);
 }
 
+// Signs as bf16 (bit 1 -> +1, 0 -> -1): nibble q of x as four values, from a table of the 16 patterns in shared memory
+// (address 128-byte aligned; one look-up replaces eight logic operations).
+__device__ __forceinline__ uint2 signs4(unsigned table, uint32_t x, int q) {
+  const uint32_t i = q == 0 ? x << 3 : x >> (4 * q - 3);
+  uint2 v;
+  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"((i & 0x78u) | table));
+  return v;
+}
+__device__ __forceinline__ void fill_sign_table(uint2* table, int tid) {
+  if (tid < 16) {
+    const uint32_t p[4] = {(tid & 1) ? 0x3F80u : 0xBF80u, (tid & 2) ? 0x3F80u : 0xBF80u, (tid & 4) ? 0x3F80u : 0xBF80u, (tid & 8) ? 0x3F80u : 0xBF80u};
+    table[tid] = make_uint2(p[0] | (p[1] << 16), p[2] | (p[3] << 16));
+  }
+}
+
+// the same MMA with operand A in tensor memory: one row per lane, two consecutive K elements per column
+__device__ __forceinline__ void umma_bf16_ta(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n"
+      ::"r"(tmem_d), "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
+}
+
 constexpr uint32_t kIdescAMnMajor = 1u << 15;              // instruction descriptor: operand A is MN-major
 
 }  // namespace umma
