@@ -17,7 +17,7 @@
 //   * rows: v_i = (W_i - sum_{j<i} (u_i . u_j) v_j) / n in fp64, then the next block's scalars C = V D_next^T in fp64.
 // The keys are read twice per 32 bits instead of 32 times.  fp32 caches take CUDA-core versions of project and gather.
 #include <mutex>
-#include "umma.cuh"
+#include "tma.cuh"
 #include "fit_block.h"
 
 namespace {
@@ -105,9 +105,9 @@ constexpr int kProjN = 3 * kBits;
 
 template <int GROUPS>
 __global__ void __launch_bounds__(kGroupThreads * GROUPS, 1)
-fit_project_tc_kernel(const __nv_bfloat16* __restrict__ k_cache, const uint32_t* __restrict__ hfit, const float* __restrict__ v_star,
+fit_project_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* __restrict__ hfit, const float* __restrict__ v_star,
                       const float* __restrict__ cross, float* __restrict__ T, const int32_t* __restrict__ unit_lens,
-                      int32_t* __restrict__ err, int n_max, int row_stride, int b, int blk, int t_stride) {
+                      int32_t* __restrict__ err, int n_max, int b, int blk, int t_stride) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   constexpr int kThreads = kGroupThreads * GROUPS;
@@ -120,7 +120,7 @@ fit_project_tc_kernel(const __nv_bfloat16* __restrict__ k_cache, const uint32_t*
   unsigned char* u_s = b_s + kProjN * 256 + (size_t)grp * U_BYTES;     // this warpgroup's signs: [128 x 96], no swizzle
   unsigned char* c_s = b_s + kProjN * 256 + (size_t)GROUPS * U_BYTES;  // -C, three terms: [96 x 32 blk], no swizzle
   __shared__ __align__(128) uint2 sign_table[16];
-  __shared__ unsigned long long bar_s[GROUPS];
+  __shared__ unsigned long long bar_s[GROUPS], tile_bar_s[GROUPS];
   __shared__ uint32_t tmem_base_s;
   __shared__ int timed_out_g[GROUPS];
   const unsigned st_a = smem_u32(sign_table);
@@ -134,25 +134,15 @@ fit_project_tc_kernel(const __nv_bfloat16* __restrict__ k_cache, const uint32_t*
   const int words = b / 32;
 
   if (tid == 0) {
-    for (int g = 0; g < GROUPS; ++g) { mbar_init(&bar_s[g], 1); timed_out_g[g] = 0; }
+    for (int g = 0; g < GROUPS; ++g) { mbar_init(&bar_s[g], 1); mbar_init(&tile_bar_s[g], 1); timed_out_g[g] = 0; }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"(512) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  const unsigned char* kbase = reinterpret_cast<const unsigned char*>(k_cache) + (size_t)unit * n_max * (size_t)row_stride * 2;
-  auto load_tile = [&](int tile) {                                     // rows past the end are zero-filled
-    const int r0 = row0 + tile * kTileKeys;
-    for (int c = gtid; c < kTileKeys * 16; c += kGroupThreads) {
-      const int r = c >> 4, ch = c & 15;
-      unsigned char* d = a_t + sw128_offset(kTileKeys, r, ch);
-      if (r0 + r < row_end) cp_async16(d, kbase + (size_t)(r0 + r) * row_stride * 2 + ch * 16);
-      else *reinterpret_cast<uint4*>(d) = make_uint4(0u, 0u, 0u, 0u);
-    }
-    cp_async_commit();
-  };
-  if (grp < ntile) load_tile(grp);
+  unsigned long long* tile_bar = &tile_bar_s[grp];
+  auto load_tile = [&](int tile) { tma::load_key_tile(a_t, &kmap, unit * n_max + row0 + tile * kTileKeys, tile_bar); };   // (one thread)
   fill_sign_table(sign_table, tid);
   for (int c = tid; c < kBits * BPC_D; c += kThreads) {
     const int l = c >> 7, ch = c & 127;
@@ -179,7 +169,8 @@ fit_project_tc_kernel(const __nv_bfloat16* __restrict__ k_cache, const uint32_t*
   unsigned long long* bar = &bar_s[grp];
   const uint32_t idesc = umma_idesc_bf16(kTileKeys, kProjN);
 
-  unsigned ph = 0;
+  if (grp < ntile && gtid == 0) load_tile(grp);
+  unsigned ph = 0, tph = 0;
   uint32_t first[kSignCols / 32];                                      // the next tile's first code words of this thread's key
   auto load_words = [&](int tile) {
     const int r = row0 + tile * kTileKeys + gtid;
@@ -209,11 +200,14 @@ fit_project_tc_kernel(const __nv_bfloat16* __restrict__ k_cache, const uint32_t*
     for (int w = 0; w < kSignCols / 32; ++w)                           // (while the tile is on its way)
       if (w < w1) put_signs(w, first[w]);
     if (tl + GROUPS < ntile) load_words(tl + GROUPS);
-    cp_async_wait_all();
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    group_sync(grp);                                                   // tile and signs are there
-    if (timed_out_g[grp]) break;                                       // (set before a barrier, so all 128 threads agree)
+    group_sync(grp);                                                   // the signs are there
+    if (timed_out_g[grp]) {                                            // (set before a barrier, so all 128 threads agree)
+      if (gtid == 0) (void)mbar_wait(tile_bar, tph);                   // the copy in flight
+      break;
+    }
     if (gtid == 0) {
+      if (!mbar_wait(tile_bar, tph)) timed_out_g[grp] = 1;             // and the tile
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
       for (int ks = 0; ks < 8; ++ks) {
@@ -226,7 +220,8 @@ fit_project_tc_kernel(const __nv_bfloat16* __restrict__ k_cache, const uint32_t*
     }
     if (!mbar_wait(bar, ph)) timed_out_g[grp] = 1;
     ph ^= 1u;
-    if (tl + GROUPS < ntile) load_tile(tl + GROUPS);
+    tph ^= 1u;
+    if (tl + GROUPS < ntile && gtid == 0) load_tile(tl + GROUPS);
     for (int w0 = kSignCols / 32; w0 < blk; w0 += kSignCols / 32) {    // 256-bit codes: the words beyond the third
       const int wn = min(blk - w0, kSignCols / 32);
       const uint32_t* h = hfit + ((size_t)unit * n_max + (live ? row : row0)) * words + w0;
@@ -259,7 +254,6 @@ fit_project_tc_kernel(const __nv_bfloat16* __restrict__ k_cache, const uint32_t*
   for (int i = row0 + ntile * kTileKeys + tid; row_end == n && i < (n + kSweepGroup - 1) / kSweepGroup * kSweepGroup; i += kThreads)
     for (int l = 0; l < kBits; ++l) T[((size_t)unit * kBits + l) * t_stride + i] = 0.f;
   if (timed_out_g[grp] && gtid == 0) atomicOr(err, BPC_DEVERR_TIMEOUT);
-  cp_async_wait_all();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_all), "r"(512) : "memory");
@@ -331,9 +325,9 @@ constexpr int kFlushTiles = 8;
 
 template <int GROUPS>
 __global__ void __launch_bounds__(kGroupThreads * GROUPS, 1)
-fit_gather_tc_kernel(const __nv_bfloat16* __restrict__ k_cache, const uint32_t* __restrict__ hfit, double* __restrict__ wpart,
+fit_gather_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* __restrict__ hfit, double* __restrict__ wpart,
                      int32_t* __restrict__ apart, const int32_t* __restrict__ unit_lens, int32_t* __restrict__ err, int n_max,
-                     int row_stride, int b, int blk) {
+                     int b, int blk) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   constexpr int kThreads = kGroupThreads * GROUPS;
@@ -345,7 +339,7 @@ fit_gather_tc_kernel(const __nv_bfloat16* __restrict__ k_cache, const uint32_t* 
   unsigned char* a_t = smem + (size_t)grp * kTileBytes;
   unsigned char* u_s = smem + (size_t)GROUPS * kTileBytes + (size_t)grp * R * kTileKeys * 2;
   __shared__ __align__(128) uint2 sign_table[16];
-  __shared__ unsigned long long bar_s[GROUPS];
+  __shared__ unsigned long long bar_s[GROUPS], tile_bar_s[GROUPS];
   __shared__ uint32_t tmem_base_s;
   __shared__ int timed_out_g[GROUPS];
   const unsigned st_a = smem_u32(sign_table);
@@ -357,24 +351,15 @@ fit_gather_tc_kernel(const __nv_bfloat16* __restrict__ k_cache, const uint32_t* 
   const int row_end = min(n, row0 + rows);
   const int ntile = (row_end - row0 + kTileKeys - 1) / kTileKeys;
   if (tid == 0) {
-    for (int g = 0; g < GROUPS; ++g) { mbar_init(&bar_s[g], 1); timed_out_g[g] = 0; }
+    for (int g = 0; g < GROUPS; ++g) { mbar_init(&bar_s[g], 1); mbar_init(&tile_bar_s[g], 1); timed_out_g[g] = 0; }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"(512) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  const unsigned char* kbase = reinterpret_cast<const unsigned char*>(k_cache) + (size_t)unit * n_max * (size_t)row_stride * 2;
-  auto load_tile = [&](int tile) {                         // rows past the end are zero-filled
-    const int r0 = row0 + tile * kTileKeys;
-    for (int c = gtid; c < kTileKeys * 16; c += kGroupThreads) {
-      const int r = c >> 4, ch = c & 15;
-      unsigned char* d = a_t + sw128_offset(kTileKeys, r, ch);
-      if (r0 + r < row_end) cp_async16(d, kbase + (size_t)(r0 + r) * row_stride * 2 + ch * 16);
-      else *reinterpret_cast<uint4*>(d) = make_uint4(0u, 0u, 0u, 0u);
-    }
-    cp_async_commit();
-  };
+  unsigned long long* tile_bar = &tile_bar_s[grp];
+  auto load_tile = [&](int tile) { tma::load_key_tile(a_t, &kmap, unit * n_max + row0 + tile * kTileKeys, tile_bar); };   // (one thread)
   uint32_t nxt[kMaxWords];                                 // code words of this thread's key of the next tile
   auto load_words = [&](int tile) {
     const int r = row0 + tile * kTileKeys + gtid;
@@ -382,7 +367,7 @@ fit_gather_tc_kernel(const __nv_bfloat16* __restrict__ k_cache, const uint32_t* 
 #pragma unroll
     for (int w = 0; w < kMaxWords; ++w) nxt[w] = (w <= blk && r < row_end) ? h[w] : 0u;
   };
-  if (grp < ntile) { load_tile(grp); load_words(grp); }
+  if (grp < ntile) load_words(grp);
   fill_sign_table(sign_table, tid);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -395,7 +380,8 @@ fit_gather_tc_kernel(const __nv_bfloat16* __restrict__ k_cache, const uint32_t* 
   double acc[kBits];                                       // channel gtid
 #pragma unroll
   for (int i = 0; i < kBits; ++i) acc[i] = 0.0;
-  unsigned ph = 0;
+  if (grp < ntile && gtid == 0) load_tile(grp);
+  unsigned ph = 0, tph = 0;
   int since_flush = 0;
   bool first = true;
   for (int tl = grp; tl < ntile; tl += GROUPS) {
@@ -421,12 +407,23 @@ fit_gather_tc_kernel(const __nv_bfloat16* __restrict__ k_cache, const uint32_t* 
       }
     }
     if (tl + GROUPS < ntile) load_words(tl + GROUPS);
-    cp_async_wait_all();
+    const int tile_rows = min(row_end - (row0 + tl * kTileKeys), kTileKeys);
+    if (tile_rows < kTileKeys) {                           // the unit's last tile: what the cache holds past the end becomes zero
+      if (!mbar_wait(tile_bar, tph)) timed_out_g[grp] = 1;
+      if (gtid >= tile_rows) {
+#pragma unroll
+        for (int ch = 0; ch < 16; ++ch) *reinterpret_cast<uint4*>(a_t + sw128_offset(kTileKeys, gtid, ch)) = make_uint4(0u, 0u, 0u, 0u);
+      }
+    }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");   // (a flush's accumulator reads are done)
     group_sync(grp);
-    if (timed_out_g[grp]) break;                           // (set before a barrier, so all 128 threads agree)
+    if (timed_out_g[grp]) {                                // (set before a barrier, so all 128 threads agree)
+      if (gtid == 0) (void)mbar_wait(tile_bar, tph);       // the copy in flight
+      break;
+    }
     if (gtid == 0) {
+      if (!mbar_wait(tile_bar, tph)) timed_out_g[grp] = 1;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const unsigned char* ub = u_s + (size_t)(4 * blk) * 128;          // rows of this block's 32 bits
 #pragma unroll
@@ -444,7 +441,8 @@ fit_gather_tc_kernel(const __nv_bfloat16* __restrict__ k_cache, const uint32_t* 
     first = false;
     if (!mbar_wait(bar, ph)) timed_out_g[grp] = 1;
     ph ^= 1u;
-    if (tl + GROUPS < ntile) load_tile(tl + GROUPS);
+    tph ^= 1u;
+    if (tl + GROUPS < ntile && gtid == 0) load_tile(tl + GROUPS);
     ++since_flush;
     if (since_flush == kFlushTiles || tl + GROUPS >= ntile) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -460,7 +458,6 @@ fit_gather_tc_kernel(const __nv_bfloat16* __restrict__ k_cache, const uint32_t* 
     }
   }
   if (timed_out_g[grp] && gtid == 0) atomicOr(err, BPC_DEVERR_TIMEOUT);
-  cp_async_wait_all();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   __syncthreads();                                         // the tile buffers are free in all warpgroups
   double* red = reinterpret_cast<double*>(smem);           // [groups][32][128]
@@ -1103,26 +1100,26 @@ int sweep_cluster(const bpc_config* c, const SweepLimits* l) {
 }
 
 template <int GROUPS>
-cudaError_t launch_project_tc(const bpc_ctx* ctx, const void* k_cache, const uint32_t* hfit, const float* v_star, const float* cross, float* T,
+cudaError_t launch_project_tc(const bpc_ctx* ctx, const CUtensorMap& kmap, const uint32_t* hfit, const float* v_star, const float* cross, float* T,
                               int blk, int parts, int ts, cudaStream_t stream) {
   const bpc_config& c = ctx->cfg;
   const size_t smem = (size_t)GROUPS * (kTileBytes + kTileKeys * kSignCols * 2) + (size_t)kProjN * 256 + (size_t)blk * kProjN * 64 + 1024;
   cudaError_t e = cudaFuncSetAttribute(fit_project_tc_kernel<GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   fit_project_tc_kernel<GROUPS><<<dim3(parts, ctx->units), kGroupThreads * GROUPS, smem, stream>>>(
-      (const __nv_bfloat16*)k_cache, hfit, v_star, cross, T, ctx->unit_lens, ctx->dev_err, c.n_max, ctx->row_stride, c.code_bits, blk, ts);
+      kmap, hfit, v_star, cross, T, ctx->unit_lens, ctx->dev_err, c.n_max, c.code_bits, blk, ts);
   return cudaGetLastError();
 }
 
 template <int GROUPS>
-cudaError_t launch_gather_tc(const bpc_ctx* ctx, const void* k_cache, const uint32_t* hfit, double* wpart, int32_t* apart, int blk, int parts,
+cudaError_t launch_gather_tc(const bpc_ctx* ctx, const CUtensorMap& kmap, const uint32_t* hfit, double* wpart, int32_t* apart, int blk, int parts,
                              cudaStream_t stream) {
   const bpc_config& c = ctx->cfg;
   const size_t smem = gather_smem(GROUPS, blk);
   cudaError_t e = cudaFuncSetAttribute(fit_gather_tc_kernel<GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   fit_gather_tc_kernel<GROUPS><<<dim3(parts, ctx->units), kGroupThreads * GROUPS, smem, stream>>>(
-      (const __nv_bfloat16*)k_cache, hfit, wpart, apart, ctx->unit_lens, ctx->dev_err, c.n_max, ctx->row_stride, c.code_bits, blk);
+      kmap, hfit, wpart, apart, ctx->unit_lens, ctx->dev_err, c.n_max, c.code_bits, blk);
   return cudaGetLastError();
 }
 
@@ -1146,7 +1143,8 @@ cudaError_t bpc_launch_fit_blocked(bpc_ctx* ctx, const void* k_cache, const floa
   const size_t sweep_smem = kSweepRing + (size_t)sweep_share(c.n_max, cs) * 4;
   const bool tc = c.kv_dtype == BPC_BF16;
   const dim3 grid(parts, ctx->units);
-  cudaError_t e = cudaSuccess;
+  CUtensorMap kmap;
+  cudaError_t e = tc ? tma::make_key_map(&kmap, k_cache, (unsigned long long)ctx->units * c.n_max, ctx->row_stride) : cudaSuccess;
   for (int blk = 0; blk < b / kBits && e == cudaSuccess; ++blk) {
     if (blk > 0) {                                         // cross[j][l] = v_j . d_l for the bits so far and this block's columns
       const size_t set = (size_t)b * BPC_D;
@@ -1155,8 +1153,8 @@ cudaError_t bpc_launch_fit_blocked(bpc_ctx* ctx, const void* k_cache, const floa
     }
     if (tc) {
       // three warpgroups while the scalars of the earlier bits leave room for them (up to five earlier words)
-      e = blk <= 5 ? launch_project_tc<3>(ctx, k_cache, hfit, v_star, cross, T, blk, parts, ts, stream)
-                   : launch_project_tc<2>(ctx, k_cache, hfit, v_star, cross, T, blk, parts, ts, stream);
+      e = blk <= 5 ? launch_project_tc<3>(ctx, kmap, hfit, v_star, cross, T, blk, parts, ts, stream)
+                   : launch_project_tc<2>(ctx, kmap, hfit, v_star, cross, T, blk, parts, ts, stream);
     } else {
       fit_project_f32_kernel<<<dim3(ts / kTileKeys, ctx->units), kTileKeys, 0, stream>>>(
           (const float*)k_cache, hfit, v_star, cross, T, ctx->unit_lens, c.n_max, ctx->row_stride, b, blk, ts);
@@ -1173,9 +1171,9 @@ cudaError_t bpc_launch_fit_blocked(bpc_ctx* ctx, const void* k_cache, const floa
     if (e != cudaSuccess) return e;
     if (tc) {
       // as many warpgroups as their tile and sign buffers leave room for (four up to the third word, two from the sixth)
-      if (gather_smem(4, blk) <= kMaxSmem) e = launch_gather_tc<4>(ctx, k_cache, hfit, wpart, apart, blk, parts, stream);
-      else if (gather_smem(3, blk) <= kMaxSmem) e = launch_gather_tc<3>(ctx, k_cache, hfit, wpart, apart, blk, parts, stream);
-      else e = launch_gather_tc<2>(ctx, k_cache, hfit, wpart, apart, blk, parts, stream);
+      if (gather_smem(4, blk) <= kMaxSmem) e = launch_gather_tc<4>(ctx, kmap, hfit, wpart, apart, blk, parts, stream);
+      else if (gather_smem(3, blk) <= kMaxSmem) e = launch_gather_tc<3>(ctx, kmap, hfit, wpart, apart, blk, parts, stream);
+      else e = launch_gather_tc<2>(ctx, kmap, hfit, wpart, apart, blk, parts, stream);
     } else {
       fit_gather_f32_kernel<<<grid, 256, 0, stream>>>((const float*)k_cache, hfit, wpart, apart, ctx->unit_lens, c.n_max, ctx->row_stride, b, blk);
     }
