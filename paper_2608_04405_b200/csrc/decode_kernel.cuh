@@ -277,56 +277,54 @@ __device__ __forceinline__ int score_key<4, 2>(const uint32_t (&h)[4], const uin
   return __popc(s0) + __popc(x0[3]) + 2 * __popc(s2) + 4 * (__popc(c1) + __popc(c2));
 }
 
-// Weighted scores of U codes at once, planes in the outer loop.  The plane masks (up to ten planes of W32 words) are
-// read from shared memory one plane at a time (the whole warp reads one address: a broadcast) instead of living in
-// registers, which leaves the registers to the U codes and their carry words: U independent dependency chains per
-// thread instead of two, so that the logic and population-count pipes stay busy.  Same arithmetic as score_key.
-template <int W32, int NP, int U>
-__device__ __forceinline__ void score_keys_plane_outer(const uint32_t (&h)[U][W32], const uint32_t (&sg)[W32],
-                                                       const uint32_t (*mask)[8], int (&key)[U]) {
-  static_assert(W32 >= 2 && W32 % 2 == 0, "pairs of words");
-  constexpr int C = W32 / 2;
-  uint32_t x[U][W32], cy[U][C];
+// Weighted scores of U codes per lane on the warp-level integer tensor path (mma.sync m16n8k32, u8 x u8 -> s32, exact; two
+// cycles per SM and instruction on this part).  The score key of a code is sum_j x_j |A_j| with x = code agrees with the query's
+// sign.  Every lane keeps its own codes: row g of the A operand is made of the four codes of lanes 4g .. 4g + 3, each in its
+// lane's eight K slots, and the B operand gives every one of them two columns of its own (the low five and the high five
+// bits of |A_j|, zero in the other lanes' K slots), so that a lane's accumulators are the two sums of its own two codes.
+// A K slot holds one bit: (x & 0x01010101 << s) puts bits s, s + 8, s + 16, s + 24 of a word into four bytes of value 2^s,
+// and the weights carry the factor 2^(3 - s) that makes all slots count eight.  One logic operation per four bits (plus a
+// shift per word): 36 per 128-bit code, where counting ten masked planes took about 150 operations and kept the integer
+// pipe busy (scan of 32 x 128K keys at four heads: 31.7 us).
+constexpr int kWeightPair = 32 * 16;                        // bytes of the weight operands of two MMAs: 16 per lane
+__device__ __forceinline__ uint32_t xor_and(uint32_t a, uint32_t b, uint32_t m) {
+  uint32_t r;
+  asm("lop3.b32 %0, %1, %2, %3, 0x28;" : "=r"(r) : "r"(a), "r"(b), "r"(m));   // (a ^ b) & m
+  return r;
+}
+template <int W32, int U>
+__device__ __forceinline__ void weighted_keys(const uint32_t (&h)[U][W32], const uint32_t (&nsg)[W32], const unsigned (&base)[2], int (&key)[U]) {
+  static_assert(U % 2 == 0, "two codes of a lane share an MMA");
+  constexpr int TP = U / 2 < 2 ? U / 2 : 2;                 // tiles of two codes that share a read of the weights
 #pragma unroll
-  for (int u = 0; u < U; ++u) {
-    key[u] = 0;
+  for (int u0 = 0; u0 < U; u0 += 2 * TP) {
+    int c[TP][4];
 #pragma unroll
-    for (int f = 0; f < C; ++f) cy[u][f] = 0u;
+    for (int i = 0; i < TP; ++i) c[i][0] = c[i][1] = c[i][2] = c[i][3] = 0;
 #pragma unroll
-    for (int w = 0; w < W32; ++w) x[u][w] = ~(h[u][w] ^ sg[w]);
-  }
+    for (int pr = 0; pr < 2 * W32; ++pr) {                  // two MMAs: word pr / 2, bits s and s + 1 of every half byte
+      const int w = pr >> 1;
+      uint32_t bv[4];
+      asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(bv[0]), "=r"(bv[1]), "=r"(bv[2]), "=r"(bv[3])
+                   : "r"(base[pr >> 3] + (unsigned)((pr & 7) * kWeightPair)));
 #pragma unroll
-  for (int pl = 0; pl < NP; ++pl) {
-    uint32_t m[W32];
-    if constexpr (W32 % 4 == 0) {
+      for (int e = 0; e < 2; ++e) {
+        const uint32_t mask = 0x01010101u << (2 * (pr & 1) + e);
 #pragma unroll
-      for (int w = 0; w < W32; w += 4) {
-        const uint4 v = *reinterpret_cast<const uint4*>(&mask[pl][w]);
-        m[w] = v.x; m[w + 1] = v.y; m[w + 2] = v.z; m[w + 3] = v.w;
+        for (int i = 0; i < TP; ++i) {
+          const uint32_t x = h[u0 + 2 * i][w], y = h[u0 + 2 * i + 1][w];
+          asm volatile("mma.sync.aligned.m16n8k32.row.col.s32.u8.u8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                       : "+r"(c[i][0]), "+r"(c[i][1]), "+r"(c[i][2]), "+r"(c[i][3])
+                       : "r"(xor_and(x, nsg[w], mask)), "r"(xor_and(y, nsg[w], mask)), "r"(xor_and(x >> 4, nsg[w] >> 4, mask)),
+                         "r"(xor_and(y >> 4, nsg[w] >> 4, mask)), "r"(bv[2 * e]), "r"(bv[2 * e + 1]));
+        }
       }
-    } else {
-      const uint2 v = *reinterpret_cast<const uint2*>(&mask[pl][0]);
-      m[0] = v.x; m[1] = v.y;
     }
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      int c = 0;
-#pragma unroll
-      for (int f = 0; f < C; ++f) {
-        const uint32_t t = (x[u][2 * f] & m[2 * f]) ^ cy[u][f];
-        const uint32_t s2 = (x[u][2 * f + 1] & m[2 * f + 1]) ^ t;
-        cy[u][f] = cy[u][f] ^ (t & (s2 ^ t ^ cy[u][f]));
-        c += __popc(s2);
-      }
-      key[u] += c << pl;
+    for (int i = 0; i < TP; ++i) {
+      key[u0 + 2 * i] = (c[i][0] + 32 * c[i][1]) >> 3;
+      key[u0 + 2 * i + 1] = (c[i][2] + 32 * c[i][3]) >> 3;
     }
-  }
-#pragma unroll
-  for (int u = 0; u < U; ++u) {
-    int c = 0;
-#pragma unroll
-    for (int f = 0; f < C; ++f) c += __popc(cy[u][f]);
-    key[u] += c << NP;
   }
 }
 
@@ -506,10 +504,8 @@ bpc_decode_kernel(const DecodeParams p) {
   const int c1s = appender ? c1 - 1 : c1;
   const uint32_t* cu = reinterpret_cast<const uint32_t*>(p.codes) + (size_t)unit * (size_t)p.n_max * W32;
   int32_t* dbg = p.dbg_scores != nullptr ? p.dbg_scores + (size_t)unit * p.n_max : nullptr;
-  // codes in flight per thread and buffer: the Hamming scan is bound by memory latency and wants many; the weighted
-  // scan is bound by its arithmetic and scores a whole batch plane by plane (masks read from shared memory), so its
-  // batch is as large as the registers for the codes and their carry words allow
-  constexpr int U = MODE == 1 ? (W32 <= 1 ? 4 : W32 == 2 ? 8 : W32 == 4 ? 4 : 2) : (W32 <= 4 ? 8 : 4);
+  // codes in flight per thread and buffer: the scan is bound by memory latency and wants many
+  constexpr int U = W32 <= 4 ? 8 : 4;
   auto load_code = [&](uint32_t (&h)[W32], int i) {
     const uint32_t* src = cu + (size_t)i * W32;
     if (W32 == 1) {
@@ -543,7 +539,7 @@ bpc_decode_kernel(const DecodeParams p) {
   }
   if (tid < BPC_D)                                           // slot GP: the appended key (its decision values P_h k)
     qf_s[GP * BPC_D + tid] = appender ? to_float(reinterpret_cast<const KV*>(p.k_new)[(size_t)unit * BPC_D + tid]) : 0.f;
-  for (int i = tid; i < nbins; i += NT) hist[i] = 0u;
+  for (int i = tid; i < (MODE == 1 ? (nbins + 3) & ~3 : nbins); i += NT) hist[i] = 0u;   // (weighted: bins are read four at a time)
   if (tid < BPC_MAX_CLUSTER) { st->gt[tid] = 0u; st->eq[tid] = 0u; }
   if (tid == 0) { st->rsum = 0; st->T = 0; st->cnt_gt = 0; st->my_take = 0; st->my_base = 0; st->e0 = 0; st->e1 = 0; }
   // Safeguard keys inside this block's key range: the set is sorted, so their list positions [e0, e1) are the numbers
@@ -638,6 +634,7 @@ bpc_decode_kernel(const DecodeParams p) {
       }
       A += pv >= 0.0 ? a : -a;
     }
+    if (MODE == 1) reinterpret_cast<int*>(pd)[2 * tid] = A;  // (over this thread's own value of head 0, which nobody else reads)
     const int absA = A < 0 ? -A : A;
     const uint32_t sw = __ballot_sync(0xffffffffu, A >= 0);
     if (lane == 0) st->signw[warp] = sw;
@@ -675,25 +672,47 @@ bpc_decode_kernel(const DecodeParams p) {
     if (tid == 0) st->e0 = a; else st->e1 = a;              // read after the cluster barrier that ends the scan
   }
 
+  constexpr bool kWeighted = MODE == 1;
+  [[maybe_unused]] unsigned wbase[2] = {0u, 0u};
+  if constexpr (kWeighted) {
+    // weight operands of words 0 .. 3 in the index staging area, of words 4 .. 7 in the total histogram (both unused until
+    // the scan is over; each holds 4 KB at least: a weighted histogram has more than 1023 bins)
+    static_assert(8 * kWeightPair <= kIdxTile * 4, "");
+    wbase[0] = (unsigned)__cvta_generic_to_shared(idx_s) + 16u * (unsigned)lane;
+    wbase[1] = (unsigned)__cvta_generic_to_shared(tot) + 16u * (unsigned)lane;
+    const int* As = reinterpret_cast<const int*>(pd);
+    for (int m = warp; m < 4 * W32; m += NW) {               // MMA m: bits s, s + 4 of every byte of word m / 4; lane = column, K slots
+      const int w = m >> 2, sh = m & 3, col = lane >> 2;
+      uint32_t b0 = 0u, b1 = 0u;
+      if ((col >> 1) == (lane & 3)) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int A0 = abs(As[2 * (32 * w + sh + 8 * q)]), A1 = abs(As[2 * (32 * w + sh + 4 + 8 * q)]);
+          b0 |= (uint32_t)(((col & 1) ? A0 >> 5 : A0 & 31) << (3 - sh)) << (8 * q);
+          b1 |= (uint32_t)(((col & 1) ? A1 >> 5 : A1 & 31) << (3 - sh)) << (8 * q);
+        }
+      }
+      asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(wbase[m >> 4] + (unsigned)(((m >> 1) & 7) * kWeightPair + 8 * (m & 1))), "r"(b0), "r"(b1) : "memory");
+    }
+    __syncthreads();
+  }
   BPC_STAMP(1);
   // ------------------------------------------------------------------ phase 1: scan
   if (tid < nts) {
-    // weighted scores of codes of two or more words: the plane masks stay in shared memory (score_keys_plane_outer)
-    constexpr bool kPlaneOuter = MODE == 1 && W32 >= 2;
-    uint32_t sg[W32], mk[kPlaneOuter ? 1 : NP][W32];
+    uint32_t sg[W32], mk[kWeighted ? 1 : NP][W32];           // (weighted: sg holds the complement of the sign words)
 #pragma unroll
     for (int w = 0; w < W32; ++w) {
-      sg[w] = st->signw[w];
-      if constexpr (!kPlaneOuter) {
+      sg[w] = kWeighted ? ~st->signw[w] : st->signw[w];
+      if constexpr (!kWeighted) {
 #pragma unroll
         for (int pl = 0; pl < NP; ++pl) mk[pl][w] = st->mask[pl][w];
       }
     }
     const int rfull = st->rsum << cs;                       // sum_j |A_j|
     auto score_batch = [&](const uint32_t (&h)[U][W32], int base) {
-      if constexpr (kPlaneOuter) {
+      if constexpr (kWeighted) {
         int keys[U];
-        score_keys_plane_outer<W32, NP, U>(h, sg, st->mask, keys);
+        weighted_keys<W32, U>(h, sg, wbase, keys);
 #pragma unroll
         for (int u = 0; u < U; ++u) {
           sc[score_slot(base - c0 + u * nts + tid)] = (uint16_t)(keys[u] >> ksh);
@@ -715,7 +734,7 @@ bpc_decode_kernel(const DecodeParams p) {
       for (int i = c0 + tid; i < c1s; i += nts) {
         uint32_t h[W32];
         load_code(h, i);
-        if constexpr (kPlaneOuter) dbg[i] = ((2 * rescore_key<W32, NP>(h, st->signw, st->mask)) << cs) - rfull;
+        if constexpr (kWeighted) dbg[i] = ((2 * rescore_key<W32, NP>(h, st->signw, st->mask)) << cs) - rfull;
         else dbg[i] = ((2 * score_key<W32, NP>(h, sg, mk)) << cs) - rfull;
       }
     }
@@ -782,9 +801,9 @@ bpc_decode_kernel(const DecodeParams p) {
           for (int w = 0; w < W32; ++w) h[u][w] = 0u;
         }
       }
-      if constexpr (kPlaneOuter) {
+      if constexpr (kWeighted) {
         int keys[U];
-        score_keys_plane_outer<W32, NP, U>(h, sg, st->mask, keys);
+        weighted_keys<W32, U>(h, sg, wbase, keys);
 #pragma unroll
         for (int u = 0; u < U; ++u) {
           const int i = i0 + u * nts + tid;
@@ -940,22 +959,27 @@ bpc_decode_kernel(const DecodeParams p) {
   // With one bin per thread, every block first stores its finished histogram into a slot of every peer's shared memory
   // (behind the score keys), so that after the barrier all CS histograms are local reads.
   const bool fast_sel = kFastOnly || (nbins <= NT && hsh == 0);
+  // Weighted scores whose stored keys are exact (no shift): four bins per thread, then the low bits inside the threshold's
+  // bin; both levels are pushed to the peers like the one-bin-per-thread histograms.
+  const bool quad_sel = MODE == 1 && ksh == 0 && hsh > 0 && nbins <= 4 * NT && kh > 0;
+  const int bin_stride = quad_sel ? (nbins + 3) & ~3 : nbins;
   uint32_t* pushed = nullptr;
   {
     const size_t union_bytes = plan.total - plan.off_union;
     size_t push_off = STREAM ? (size_t)NW * nbins * 4 : L::score_bytes(p.chunk_cap, K8 ? 1 : 2);
     if (push_off < L::hashpart_bytes()) push_off = L::hashpart_bytes();   // a peer may still be hashing
     push_off = (push_off + 15) & ~(size_t)15;
-    if (fast_sel && CS > 1 && push_off + (size_t)CS * nbins * 4 + (size_t)B * B * 4 <= union_bytes)
+    if ((fast_sel || quad_sel) && CS > 1 && push_off + (size_t)CS * bin_stride * 4 + (size_t)B * B * 4 <= union_bytes)
       pushed = reinterpret_cast<uint32_t*>(uni + push_off);
   }
   if (pushed != nullptr) {
     __syncthreads();                                         // this block's histogram is complete
-    if (tid < nbins) {
-      const uint32_t v = hist[tid];
+    for (int i = tid; i < bin_stride; i += NT) {
+      const uint32_t v = hist[i];
 #pragma unroll
       for (int r = 0; r < BPC_MAX_CLUSTER; ++r)
-        if (r < CS) cluster.map_shared_rank(pushed, r)[rank * nbins + tid] = v;
+        if (r < CS) cluster.map_shared_rank(pushed, r)[rank * bin_stride + i] = v;
+      if (MODE == 0) break;                                  // (one bin per thread there)
     }
   }
   cluster.sync();                                            // every block's histogram is complete (and delivered)
@@ -1006,6 +1030,90 @@ bpc_decode_kernel(const DecodeParams p) {
     __syncthreads();
     T = st->T;
     BPC_STAMP(9);
+  } else if (quad_sel) {
+    if constexpr (MODE == 1) {
+    // Thread t owns bins 4q .. 4q + 3, q counted from the top; the block scan gives the keys above its bins (in the cluster and
+    // in the blocks of lower rank), and the thread whose bins hold the k-th key walks them.
+    const int q4 = ((nbins + 3) >> 2) - 1 - tid;
+    uint32_t c[4] = {0u, 0u, 0u, 0u}, low[4] = {0u, 0u, 0u, 0u};
+    if (q4 >= 0) {
+#pragma unroll 1
+      for (int r = 0; r < CS; ++r) {
+        const uint32_t* h = pushed != nullptr ? pushed + r * bin_stride : cluster.map_shared_rank(hist, r);
+        const uint4 v = *reinterpret_cast<const uint4*>(h + 4 * q4);
+        c[0] += v.x; c[1] += v.y; c[2] += v.z; c[3] += v.w;
+        if (r < rank) { low[0] += v.x; low[1] += v.y; low[2] += v.z; low[3] += v.w; }
+      }
+    }
+    uint32_t above, above_low;
+    const uint32_t s_all = (c[0] + c[1]) + (c[2] + c[3]);
+    block_excl_scan2<NT>(s_all, (low[0] + low[1]) + (low[2] + low[3]), st->wscan, scan_calls, above, above_low);
+    if (above < (uint32_t)kh && above + s_all >= (uint32_t)kh) {
+#pragma unroll
+      for (int i = 3; i >= 0; --i) {
+        if (above < (uint32_t)kh && above + c[i] >= (uint32_t)kh) { st->T = 4 * q4 + i; st->cnt_gt = (int)above; st->my_base = (int)above_low; }
+        above += c[i];
+        above_low += low[i];
+      }
+    }
+    if (tid < 32) tot[tid] = 0u;                             // this block's counts of the low bits
+    __syncthreads();
+    T = st->T;
+    BPC_STAMP(9);
+    // counts of the low bits of the keys in bin T, whole segments at a time: a half word whose high bits equal the bin's
+    // leaves a zero, which the subtraction carries into its top bit.  (A borrow from a zero low half can only raise a false
+    // alarm in the high half, so that half is compared once more.)
+    const int FB = 1 << hsh;
+    const uint32_t TT = (uint32_t)(T << hsh) * 0x10001u, HM = (uint32_t)(0xffff & ~(FB - 1)) * 0x10001u;
+    const int len = c1 - c0, nseg_f = (len + kSegKeys - 1) / kSegKeys;
+    for (int seg = tid; seg < nseg_f; seg += NT) {
+      const uint4* src = reinterpret_cast<const uint4*>(sc + (size_t)seg * kSegSlots);
+      const int valid = len - seg * kSegKeys;
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        const uint4 x4 = src[v];
+        const uint32_t kw[4] = {x4.x, x4.y, x4.z, x4.w};
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+          const uint32_t y = (kw[w] ^ TT) & HM;
+          const uint32_t z = (y - 0x00010001u) & ~y & 0x80008000u;
+          if (z) {
+            const int i = 8 * v + 2 * w;
+            if ((y & 0xffffu) == 0u && i < valid) atomicAdd(&tot[kw[w] & (FB - 1)], 1u);
+            if ((y >> 16) == 0u && i + 1 < valid) atomicAdd(&tot[(kw[w] >> 16) & (FB - 1)], 1u);
+          }
+        }
+      }
+    }
+    uint32_t* fine_in = reinterpret_cast<uint32_t*>(idx_s);  // [CS][32], written by the peers
+    __syncthreads();
+    for (int r = warp; r < CS; r += NW) cluster.map_shared_rank(fine_in, r)[rank * 32 + lane] = tot[lane];
+    cluster.sync();
+    if (warp == 0) {
+      uint32_t f = 0, f_low = 0, f_mine = 0;
+      for (int r = 0; r < CS; ++r) {
+        const uint32_t v = fine_in[r * 32 + lane];
+        f += v;
+        if (r < rank) f_low += v;
+        if (r == rank) f_mine = v;
+      }
+      uint32_t incl = f, incl_low = f_low;                   // suffix sums over lanes: keys of the bin with at least these low bits
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_down_sync(0xffffffffu, incl, o), vl = __shfl_down_sync(0xffffffffu, incl_low, o);
+        if (lane + o < 32) { incl += v; incl_low += vl; }
+      }
+      const uint32_t over = incl - f, need_c = (uint32_t)(kh - st->cnt_gt);   // keys still to take from the bin (>= 1)
+      if (over < need_c && over + f >= need_c) {             // one lane: the exact threshold's low bits
+        const int need = (int)(need_c - over), lower_take = min(need, (int)f_low);
+        st->T = (T << hsh) | lane;
+        st->cnt_gt += (int)over;
+        st->my_take = min(max(need - (int)f_low, 0), (int)f_mine);
+        st->my_base += (int)(incl_low - f_low) + lower_take;
+      }
+    }
+    __syncthreads();
+    }
   } else if constexpr (!kFastOnly) {
     // Total histogram through distributed shared memory.  With at most one bin per thread (the common case)
     // the per-block counts of that bin stay in registers and are reused for the per-block offsets below.
@@ -1068,8 +1176,8 @@ bpc_decode_kernel(const DecodeParams p) {
     }
     __syncthreads();
   }
-  int T_exact = T;
-  if (MODE == 1 && hsh > 0 && kh > 0) {
+  int T_exact = quad_sel ? st->T : T;
+  if (MODE == 1 && hsh > 0 && kh > 0 && !quad_sel) {
     // Weighted scores have more distinct values than histogram bins: the search above found the coarse bin
     // that holds the k-th score.  A second, small histogram over the low bits of the keys inside that bin (again
     // summed across the cluster) yields the exact threshold and corrects the per-block counts.
@@ -1178,7 +1286,7 @@ bpc_decode_kernel(const DecodeParams p) {
     __syncthreads();
     T_low = st->e0;
   }
-  if (!kFastOnly && !fast_sel && tid == 0) {
+  if (!kFastOnly && !fast_sel && !quad_sel && tid == 0) {
     const int need = kh - st->cnt_gt;                        // ties to take, cluster-wide (>= 1)
     int tie_base = 0, out_base = 0;
     for (int r = 0; r < CS; ++r) {
@@ -1189,7 +1297,7 @@ bpc_decode_kernel(const DecodeParams p) {
       tie_base += (int)st->eq[r];
     }
   }
-  if (!kFastOnly && !fast_sel) __syncthreads();                            // (the fast path published its values before its own barrier)
+  if (!kFastOnly && !fast_sel && !quad_sel) __syncthreads();               // (the fast paths published theirs before their own barrier)
   int32_t* sel_u = p.sel + (size_t)unit * p.n_max;
   BPC_STAMP(10);
   if constexpr (STREAM) {
