@@ -17,6 +17,8 @@ cudaError_t bpc_launch_decode_bf16_stream(bpc_ctx*, const DecodeParams&, cudaStr
 cudaError_t bpc_launch_decode_f32_stream(bpc_ctx*, const DecodeParams&, cudaStream_t);
 cudaError_t bpc_launch_decode_bf16_k8(bpc_ctx*, const DecodeParams&, cudaStream_t);
 cudaError_t bpc_launch_decode_f32_k8(bpc_ctx*, const DecodeParams&, cudaStream_t);
+cudaError_t bpc_launch_decode_bf16_short(bpc_ctx*, const DecodeParams&, cudaStream_t);
+cudaError_t bpc_launch_decode_f32_short(bpc_ctx*, const DecodeParams&, cudaStream_t);
 cudaError_t bpc_decode_limits_bf16_k8(const bpc_ctx*, int, int*, int*, size_t*);
 cudaError_t bpc_decode_limits_f32_k8(const bpc_ctx*, int, int*, int*, size_t*);
 cudaError_t bpc_launch_decode_bf16_w7(bpc_ctx*, const DecodeParams&, cudaStream_t);
@@ -497,6 +499,18 @@ bpc_status bpc_append(bpc_ctx* ctx, const void* k_new, const void* v_new, void* 
   return BPC_OK;
 }
 
+// Whether a step that appends a key takes the kernel with the deferred selection (Hamming scores in 16-bit keys; the same
+// results at any length).  Its sign sweep of the appended key runs beside the scan AND the threshold search: worth it while
+// the sweep (about 3 us) outlasts the scan, up to some 6K keys per block.  With 256-bit codes it also keeps the Gram matrix
+// in shared memory next to the scores of up to 20K keys per block (43 us of sweep from L2 otherwise).  Lengths are the host
+// shadow's: a captured step keeps the kernel that was chosen at capture.
+static bool short_ranges(const bpc_ctx* ctx) {
+  int longest = 0;
+  for (int i = 0; i < ctx->cfg.batch; ++i) longest = ctx->host_lens[i] > longest ? ctx->host_lens[i] : longest;
+  const int keys = ctx->cluster_size > 1 ? bpc_fused_chunk(longest + 1, ctx->cluster_size) : longest + 1;
+  return keys <= (ctx->cfg.code_bits == 256 ? 20480 : 6144);
+}
+
 static bpc_status decode_common(bpc_ctx* ctx, const void* k_new, const void* v_new, void* k_cache_w, void* v_cache_w,
                                 uint64_t* codes_w, const void* q, const void* k_cache, const void* v_cache,
                                 const uint64_t* codes, int32_t budget_ppm, int32_t budget_count, float* out,
@@ -589,6 +603,9 @@ static bpc_status decode_common(bpc_ctx* ctx, const void* k_new, const void* v_n
   else if (c.eas_ppm > 0)
     e = c.kv_dtype == BPC_BF16 ? bpc_launch_decode_bf16_eas(ctx, p, (cudaStream_t)stream)
                                : bpc_launch_decode_f32_eas(ctx, p, (cudaStream_t)stream);
+  else if (k_new != nullptr && short_ranges(ctx))
+    e = c.kv_dtype == BPC_BF16 ? bpc_launch_decode_bf16_short(ctx, p, (cudaStream_t)stream)
+                               : bpc_launch_decode_f32_short(ctx, p, (cudaStream_t)stream);
   else
     e = c.kv_dtype == BPC_BF16 ? bpc_launch_decode_bf16(ctx, p, (cudaStream_t)stream)
                                : bpc_launch_decode_f32(ctx, p, (cudaStream_t)stream);

@@ -64,7 +64,7 @@ struct bpc_ctx {
   int64_t launches;
   int chunk_cap_limit;      // keys one decode block can hold with all opt-in shared memory
   double sm_scale_d;        // softmax scale in double (exact 1/sqrt(head_dim) by default)
-  size_t decode_smem_set;   // non-zero once the decode kernel's function attributes have been set
+  size_t decode_smem_set;   // bit v: the function attributes of decode kernel variant v have been set
   // ---- work-item decode kernel (decode_sched.cuh): geometry and scratch, set up by bpc_create when the shape is covered
   bool sched_ok;            // the work-item kernel serves this context's decode calls
   int decode_path;          // 0 = automatic, 1 = cluster kernel, 2 = work-item kernel (diagnostic switch)

@@ -36,6 +36,7 @@ constexpr int kIdxTile = 1024;      // selected indices staged at a time (fp32 p
 constexpr int kMaxPlanes = 10;
 constexpr int kEasMax = 16384;      // largest error-aware safeguard set per unit
 constexpr int kUnrolledSweepKeys = 16384;   // key ranges shorter than this take the unrolled sign sweep of the appended key
+constexpr int kQuietKeys = 6144;    // key ranges of the appending block up to which only three quarters of its warps scan
 constexpr int kEasLocal = 1024;     // safeguard keys of one block kept in shared memory (larger slices stay in global)
 
 template <int GP, int MODE> struct PlaneCount {
@@ -51,11 +52,22 @@ struct SmallState {
   uint32_t wgt[32], weq[32];             // streaming selection: per-warp numbers of keys above / at the threshold
   uint32_t wscan[64];                    // block scans: two alternating buffers of 2 x 16 warp totals (16-byte aligned)
   double pmax[BPC_MAX_GROUP];
+  unsigned long long gram_bar;           // mbarrier: the appending block's Gram matrix is in shared memory (deferred selection)
   int T, cnt_gt, my_take, my_base, rsum, e0, e1, pad;
   uint32_t newcode[8];                   // code of the key appended by this launch
+  unsigned long long new_bar;            // mbarrier: the appended key's score has arrived (deferred selection)
+  int newkey, above_low, low, mine;      // ... that score; what the threshold search found for this block without it
   int32_t eas_s[kEasLocal];              // this block's slice of the safeguard set (when it fits)
   uint8_t stage_valid[32][4];            // per warp and gather stage: which of the 8 rows are real
 };
+
+// 256-bit Gram matrix in shared memory: 32 x 32 blocks on and right of the diagonal, padded to spread the banks; byte offset
+// of (row, column) inside the set
+constexpr int kGramBlock = 32 * 32 * 4 + 16;
+__device__ __forceinline__ int gram_tri(int row, int col) {
+  const int r = row >> 5, c = col >> 5;
+  return (r * 8 - r * (r - 1) / 2 + (c - r)) * kGramBlock + (row & 31) * 128 + (col & 31) * 4;
+}
 
 template <typename KV> struct IsBf16 { static constexpr bool value = false; };
 template <> struct IsBf16<__nv_bfloat16> { static constexpr bool value = true; };
@@ -137,9 +149,12 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t* wscan,
   return wbase + inc - v;
 }
 
-// the same for two values at once
-template <int NT>
-__device__ __forceinline__ void block_excl_scan2(uint32_t a, uint32_t b, uint32_t* wscan, int& ph, uint32_t& ea, uint32_t& eb) {
+// barrier among the first `threads` arriving threads of a block (hardware barrier 1; whole warps)
+__device__ __forceinline__ void partial_sync(int threads) { asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory"); }
+
+// the same for two values at once; with PARTIAL only `threads` threads take part (the others' totals are zero already)
+template <int NT, bool PARTIAL = false>
+__device__ __forceinline__ void block_excl_scan2(uint32_t a, uint32_t b, uint32_t* wscan, int& ph, uint32_t& ea, uint32_t& eb, int threads = NT) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t* buf = wscan + (ph & 1) * 32;
   ++ph;
@@ -151,7 +166,7 @@ __device__ __forceinline__ void block_excl_scan2(uint32_t a, uint32_t b, uint32_
     const uint32_t ta = __shfl_up_sync(0xffffffffu, ia, o), tb = __shfl_up_sync(0xffffffffu, ib, o);
     if (lane >= o) { ia += ta; ib += tb; }
   }
-  __syncthreads();
+  if (PARTIAL) partial_sync(threads); else __syncthreads();
   uint32_t ba = 0, bb = 0;
 #pragma unroll
   for (int w4 = 0; w4 < NT / 128; ++w4) {
@@ -360,14 +375,16 @@ __device__ __noinline__ int rescore_key(const uint32_t* code, const uint32_t* si
 // cluster's shared memory (no score is stored: the scan keeps one histogram per warp over that warp's contiguous key
 // range, and after the threshold is known every warp reads its codes a second time and emits its selection in order);
 // 3 = byte score keys: Hamming scores with at most 256 distinct keys are stored one byte per key, unpadded, so that a
-// block holds 2.5 times as many (contexts of a million keys and more in clusters that are all resident at once).
+// block holds 2.5 times as many (contexts of a million keys and more in clusters that are all resident at once);
+// 4 = the deferred selection for steps that append a key and whose blocks have few keys (see there).
 template <typename KV, int GP, int W32, int MODE, int VAR>
 __global__ void __launch_bounds__((DecodeSmem<KV, GP, W32>::NT), 1)
 bpc_decode_kernel(const DecodeParams p) {
   constexpr int EAS = VAR == 1 ? 1 : 0;
   constexpr bool STREAM = VAR == 2;
   constexpr bool K8 = VAR == 3;
-  static_assert(!K8 || MODE == 0, "byte keys are for Hamming scores");
+  constexpr bool kDefer = VAR == 4;
+  static_assert(!(K8 || kDefer) || MODE == 0, "byte keys and the deferred selection are for Hamming scores");
   typedef DecodeSmem<KV, GP, W32> L;
   typedef typename L::acc_t acc_t;
   constexpr int NT = L::NT, NW = L::NW, B = L::B;
@@ -414,6 +431,10 @@ bpc_decode_kernel(const DecodeParams p) {
     const int i = tid + v * NT;
     qreg[v] = (i < GP * BPC_D && (i >> 7) < G) ? qg[i] : (KV)0.f;
   }
+
+  // (deferred selection: the appended key too, before the length says which block needs it)
+  [[maybe_unused]] KV kreg = (KV)0.f;
+  if (kDefer && p.k_new != nullptr && tid < BPC_D) kreg = reinterpret_cast<const KV*>(p.k_new)[(size_t)unit * BPC_D + tid];
 
   int n = p.unit_lens[unit];
   n = max(0, min(n, p.n_max));
@@ -482,15 +503,24 @@ bpc_decode_kernel(const DecodeParams p) {
   // not reach (free until the gather ring starts), so that the sequential sign decisions of Algorithm 2 cost a
   // shuffle and a few FMAs each.  Shapes where it does not fit read it from global memory instead.
   const float* gsm = nullptr;
+  // (256 bits, deferred selection: the whole matrix does not fit, its 32 x 32 blocks on and right of the diagonal do)
+  constexpr bool kGramTri = kDefer && W32 == 8;
+  constexpr int kGramBytes = kGramTri ? W32 * (W32 + 1) / 2 * kGramBlock : B * B * 4;
   if (appender && p.residual_correction != 0) {
     const size_t union_bytes = plan.total - plan.off_union;
     const size_t score_bytes = STREAM ? (size_t)NW * nbins * 4      // (streaming: the per-warp histograms sit there)
                                       : L::score_bytes(p.chunk_cap, K8 ? 1 : 2);
-    constexpr size_t kGramPad = 0;
-    if (score_bytes + (size_t)B * B * 4 + kGramPad <= union_bytes && L::hashpart_bytes() + (size_t)B * B * 4 + kGramPad <= union_bytes) {
-      float* dstg = reinterpret_cast<float*>(uni + union_bytes - (size_t)B * B * 4 - kGramPad);
+    if (score_bytes + kGramBytes <= union_bytes && L::hashpart_bytes() + kGramBytes <= union_bytes) {
+      float* dstg = reinterpret_cast<float*>(uni + union_bytes - kGramBytes);
       const float* Gs = p.gram + (size_t)(p.shared_sets ? kvh : unit) * B * B;
-      for (int c = tid; c < B * B / 4; c += NT) cp_async16(dstg + 4 * c, Gs + 4 * c);
+      if constexpr (kGramTri) {
+        for (int c = tid; c < B * B / 4; c += NT) {          // row, four columns
+          const int r = c / (B / 4), q = c % (B / 4);
+          if (q / 8 >= r / 32) cp_async16(reinterpret_cast<unsigned char*>(dstg) + gram_tri(r, 4 * q), Gs + 4 * c);
+        }
+      } else {
+        for (int c = tid; c < B * B / 4; c += NT) cp_async16(dstg + 4 * c, Gs + 4 * c);
+      }
       gsm = dstg;
     }
   }
@@ -498,9 +528,25 @@ bpc_decode_kernel(const DecodeParams p) {
 
   // ---- scan set-up, hoisted above the query hash so that the first batch of codes is already in flight
   const int c0 = min(n, rank * chunk), c1 = min(n, c0 + chunk);
+  // Deferred selection.  The sign decisions of the appended key are a chain of some 3 us, which with short key ranges is
+  // longer than the scan; only the score at its end matters to the selection, and only in one way: ties at the threshold T
+  // of the OTHER keys go to the lowest index, so the appended key (the last one) is selected exactly if its score exceeds T,
+  // and then the last tie is not.  The clusters' histograms and the threshold search therefore leave it out, the appending
+  // warp takes no part in their barriers (it arrives at the cluster barrier before its sweep), and its score reaches every
+  // block through a store that completes on the block's mbarrier, awaited before the emission.  One sequence of 32K keys:
+  // 1.9 us of waiting at the histogram barrier less.
+  const bool deferred = kDefer && fused && kh < n && p.nbins <= NT - 32 && (kFastOnly || p.hist_shift == 0);
   // In the appending block the last warp codes the new key while the other warps scan; the new key's code is
   // not in memory yet, so the scan stops one key short and the key is scored separately below.
-  const int nts = appender ? NT - 32 : NT;
+  // With a short key range the other blocks wait for that warp, so the warps that share its scheduler do not scan (the
+  // sweep alone on its scheduler is a third faster; beyond kQuietKeys keys the scan is the longer one).  One sequence of 32K
+  // keys: 19.05 -> 18.5 us per step.
+  constexpr bool kQuiet = MODE == 0 && !STREAM && W32 <= 4 && GP <= 4;   // (the others' ranges take longer to scan than to sweep)
+  const bool quiet = kQuiet && appender && c1 - c0 <= kQuietKeys;
+  const int nts = appender ? (quiet ? NT - NT / 4 : NT - 32) : NT;
+  const bool appends = appender && warp == NW - 1;
+  const bool scans = quiet ? (warp & 3) != 3 : !appends;
+  const int stid = quiet ? tid - 32 * (warp >> 2) : tid;     // index among the scanning threads
   const int c1s = appender ? c1 - 1 : c1;
   const uint32_t* cu = reinterpret_cast<const uint32_t*>(p.codes) + (size_t)unit * (size_t)p.n_max * W32;
   int32_t* dbg = p.dbg_scores != nullptr ? p.dbg_scores + (size_t)unit * p.n_max : nullptr;
@@ -522,10 +568,10 @@ bpc_decode_kernel(const DecodeParams p) {
   };
   auto load_batch = [&](uint32_t (&h)[U][W32], int base) {
 #pragma unroll
-    for (int u = 0; u < U; ++u) load_code(h[u], base + u * nts + tid);
+    for (int u = 0; u < U; ++u) load_code(h[u], base + u * nts + stid);
   };
   uint32_t ha[U][W32], hb[U][W32];
-  const bool pipelined = tid < nts && c0 + nts * U <= c1s;   // at least one full batch
+  const bool pipelined = scans && c0 + nts * U <= c1s;   // at least one full batch
   if (!STREAM && pipelined) load_batch(ha, c0);
 
   // ------------------------------------------------------------------ phase 0: query hash
@@ -538,9 +584,18 @@ bpc_decode_kernel(const DecodeParams p) {
     if (i < GP * BPC_D) qf_s[i] = to_float(qreg[v]);
   }
   if (tid < BPC_D)                                           // slot GP: the appended key (its decision values P_h k)
-    qf_s[GP * BPC_D + tid] = appender ? to_float(reinterpret_cast<const KV*>(p.k_new)[(size_t)unit * BPC_D + tid]) : 0.f;
+    qf_s[GP * BPC_D + tid] = appender ? to_float(kDefer ? kreg : reinterpret_cast<const KV*>(p.k_new)[(size_t)unit * BPC_D + tid]) : 0.f;
   for (int i = tid; i < (MODE == 1 ? (nbins + 3) & ~3 : nbins); i += NT) hist[i] = 0u;   // (weighted: bins are read four at a time)
   if (tid < BPC_MAX_CLUSTER) { st->gt[tid] = 0u; st->eq[tid] = 0u; }
+  if (kDefer && tid == 0) {
+    if (gsm != nullptr)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"((unsigned)__cvta_generic_to_shared(&st->gram_bar)), "r"(NT) : "memory");
+    const unsigned bar = (unsigned)__cvta_generic_to_shared(&st->new_bar);
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], 4;" ::"r"(bar) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    st->wscan[NW - 1] = st->wscan[16 + NW - 1] = 0u;         // (the appending warp adds nothing to the threshold search)
+  }
   if (tid == 0) { st->rsum = 0; st->T = 0; st->cnt_gt = 0; st->my_take = 0; st->my_base = 0; st->e0 = 0; st->e1 = 0; }
   // Safeguard keys inside this block's key range: the set is sorted, so their list positions [e0, e1) are the numbers
   // of entries below the range's two ends.  A set of at most kEasLocal keys is copied to shared memory asynchronously
@@ -555,6 +610,8 @@ bpc_decode_kernel(const DecodeParams p) {
     cp_async_commit();
   }
   __syncthreads();
+  if (kDefer && gsm != nullptr)                              // (arrives when this thread's copies have landed)
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"((unsigned)__cvta_generic_to_shared(&st->gram_bar)) : "memory");
   if (EAS && me > kEasLocal) {
     const int lo_key = min(n, rank * chunk), hi_key = min(n, lo_key + chunk);
     int c_lo = 0, c_hi = 0;
@@ -650,7 +707,7 @@ bpc_decode_kernel(const DecodeParams p) {
     if (lane == 0) atomicAdd(&st->rsum, rs);
     if (p.dbg_qweights != nullptr && rank == 0) p.dbg_qweights[(size_t)unit * B + tid] = A;
   }
-  cp_async_wait<0>();                                        // Gram staging (appending block only) has landed
+  if (!kDefer) cp_async_wait<0>();                           // Gram staging (appending block only) has landed
   __syncthreads();
   // Weighted scores reach sum_j |A_j| <= 127 G b, which can exceed 16 bits (seven or eight query heads per KV head at
   // 128 bits, 256-bit codes).  The stored key is then the score key shifted right by ksh (0, 1 or 2, from this query's
@@ -699,7 +756,7 @@ bpc_decode_kernel(const DecodeParams p) {
   }
   BPC_STAMP(1);
   // ------------------------------------------------------------------ phase 1: scan
-  if (tid < nts) {
+  if (scans) {
     uint32_t sg[W32], mk[kWeighted ? 1 : NP][W32];           // (weighted: sg holds the complement of the sign words)
 #pragma unroll
     for (int w = 0; w < W32; ++w) {
@@ -716,15 +773,15 @@ bpc_decode_kernel(const DecodeParams p) {
         weighted_keys<W32, U>(h, sg, wbase, keys);
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          sc[score_slot(base - c0 + u * nts + tid)] = (uint16_t)(keys[u] >> ksh);
+          sc[score_slot(base - c0 + u * nts + stid)] = (uint16_t)(keys[u] >> ksh);
           atomicAdd(&hist[(keys[u] >> ksh) >> hsh], 1u);
         }
       } else {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
           const int key = score_key<W32, NP>(h[u], sg, mk);
-          if constexpr (K8) sc8[base - c0 + u * nts + tid] = (uint8_t)key;
-          else sc[score_slot(base - c0 + u * nts + tid)] = (uint16_t)(key >> ksh);
+          if constexpr (K8) sc8[base - c0 + u * nts + stid] = (uint8_t)key;
+          else sc[score_slot(base - c0 + u * nts + stid)] = (uint16_t)(key >> ksh);
           atomicAdd(&hist[(key >> ksh) >> hsh], 1u);
         }
       }
@@ -733,13 +790,13 @@ bpc_decode_kernel(const DecodeParams p) {
     // 256-bit codes: registers allow only four codes in flight per thread; every warp asks for its share of a later batch
     // to be brought into L2, which shortens the wait of the loads that follow (step of 16 x 16K-64K keys: 118 -> 99 us)
     auto prefetch_batch = [&](int base) {
-      const int first = base + warp * 32 * U;
+      const int first = base + (stid >> 5) * 32 * U;
       if (W32 == 8 && lane == 0 && first + 32 * U <= c1s)
         asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(cu + (size_t)first * W32), "n"(32 * U * W32 * 4) : "memory");
     };
     if (dbg != nullptr) {                                    // score export (tests): a plain loop, one key at a time
 #pragma unroll 1
-      for (int i = c0 + tid; i < c1s; i += nts) {
+      for (int i = c0 + stid; i < c1s; i += nts) {
         uint32_t h[W32];
         load_code(h, i);
         if constexpr (kWeighted) dbg[i] = ((2 * rescore_key<W32, NP>(h, st->signw, st->mask)) << cs) - rfull;
@@ -805,7 +862,7 @@ bpc_decode_kernel(const DecodeParams p) {
       uint32_t h[U][W32];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int i = i0 + u * nts + tid;
+        const int i = i0 + u * nts + stid;
         if (i < c1s) {
           load_code(h[u], i);
         } else {
@@ -818,7 +875,7 @@ bpc_decode_kernel(const DecodeParams p) {
         weighted_keys<W32, U>(h, sg, wbase, keys);
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          const int i = i0 + u * nts + tid;
+          const int i = i0 + u * nts + stid;
           if (i < c1s) {
             sc[score_slot(i - c0)] = (uint16_t)(keys[u] >> ksh);
             atomicAdd(&hist[(keys[u] >> ksh) >> hsh], 1u);
@@ -827,7 +884,7 @@ bpc_decode_kernel(const DecodeParams p) {
       } else {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          const int i = i0 + u * nts + tid;
+          const int i = i0 + u * nts + stid;
           if (i < c1s) {
             const int key = score_key<W32, NP>(h[u], sg, mk);
             if constexpr (K8) sc8[i - c0] = (uint8_t)key;
@@ -839,31 +896,41 @@ bpc_decode_kernel(const DecodeParams p) {
     }
     }
     if (p.dbg_times != nullptr && tid == 0) p.dbg_times[(size_t)blockIdx.x * 16 + 13] = (unsigned long long)clock64();
-  } else {
+  } else if (appends) {
+    if (deferred) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // (its part in the histogram barrier)
     // ---- appending warp (Algorithm 2 on the new key, Gram form): cache rows, sign sweep, code words.
-    // Lane l holds the decision values of bits l, 32+l, ...; bit i is decided by a shuffle from its owner
-    // lane and every later column is corrected with G[i][.].
     const size_t rstride_e = (size_t)p.row_stride;
     const KV* kn = reinterpret_cast<const KV*>(p.k_new) + (size_t)unit * BPC_D;
     const KV* vn = reinterpret_cast<const KV*>(p.v_new) + (size_t)unit * BPC_D;
     KV* krow = reinterpret_cast<KV*>(p.k_cache_w) + ((size_t)unit * p.n_max + (n - 1)) * rstride_e;
     KV* vrow = reinterpret_cast<KV*>(p.v_cache_w) + ((size_t)unit * p.n_max + (n - 1)) * rstride_e;
     constexpr int CPL = ROWB / 16 / 16;                      // 16-byte chunks per lane and row (1 bf16, 2 fp32)
+    uint4 kv_new[CPL];                                       // (deferred selection: requested here, stored after the sweep)
 #pragma unroll
-    for (int c = 0; c < CPL; ++c) {
-      const int chn = (lane & 15) * CPL + c;
-      if (lane < 16) reinterpret_cast<uint4*>(krow)[chn] = reinterpret_cast<const uint4*>(kn)[chn];
-      else           reinterpret_cast<uint4*>(vrow)[chn] = reinterpret_cast<const uint4*>(vn)[chn];
-    }
-    constexpr int NB = W32;                                  // 32-bit column blocks
-    float t[NB];
+    for (int c = 0; c < CPL; ++c) kv_new[c] = reinterpret_cast<const uint4*>(lane < 16 ? kn : vn)[(lane & 15) * CPL + c];
+    auto store_rows = [&]() {
 #pragma unroll
-    for (int c = 0; c < NB; ++c) t[c] = (float)pd[GP * B + 32 * c + lane] + 0.f;   // (never -0)
+      for (int c = 0; c < CPL; ++c) reinterpret_cast<uint4*>(lane < 16 ? krow : vrow)[(lane & 15) * CPL + c] = kv_new[c];
+    };
+    if (!kDefer) store_rows();
     const float* Gs = p.gram + (size_t)(p.shared_sets ? kvh : unit) * B * B;
     const bool rc = p.residual_correction != 0;
     uint32_t* code_dst = reinterpret_cast<uint32_t*>(p.codes_w) + ((size_t)unit * p.n_max + (n - 1)) * W32;
     if (p.dbg_times != nullptr && lane == 0) p.dbg_times[(size_t)blockIdx.x * 16 + 12] = (unsigned long long)clock64();
-    {
+    const float* gq = gsm != nullptr ? gsm : Gs;               // Gram matrix: staged in shared memory when it fits
+    if (kDefer && gsm != nullptr) {
+      int tries = 0;
+      uint32_t there = 0u;
+      while (!there && tries++ < 20000000)
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
+                     : "=r"(there) : "r"((unsigned)__cvta_generic_to_shared(&st->gram_bar)) : "memory");
+      if (!there && lane == 0) atomicOr(p.err, BPC_DEVERR_TIMEOUT);
+    }
+    if constexpr (kQuiet) {
+      constexpr int NB = W32;                                  // 32-bit column blocks
+      float t[NB];
+#pragma unroll
+      for (int c = 0; c < NB; ++c) t[c] = (float)pd[GP * B + 32 * c + lane] + 0.f;   // (never -0)
       // The b sign decisions are taken eight at a time: every lane collects the eight
       // decision values of the group and decides them on its own copy (their 8 x 8 Gram block is read at one address
       // by the whole warp: no cross-lane traffic inside the dependency chain), then the eight signs correct all later
@@ -875,7 +942,6 @@ bpc_decode_kernel(const DecodeParams p) {
       // block's key range is short and the other warps would wait for this one.  With a long range the scan outlasts
       // the sweep anyway, and the rolled loops (a quarter of the code, a lower issue rate) disturb the scanning warps
       // of the block less (config 2: 39.6 us per step against 39.9).
-      const float* gq = gsm != nullptr ? gsm : Gs;             // Gram matrix: staged in shared memory when it fits
       auto sweep = [&](auto unrolled_tag) {
       constexpr bool kUnrolled = decltype(unrolled_tag)::value;
 #pragma unroll (kUnrolled ? NB : 1)
@@ -923,59 +989,119 @@ bpc_decode_kernel(const DecodeParams p) {
         if (lane == 0) { st->newcode[bi] = wbits; code_dst[bi] = wbits; }
       }
       };
-      if constexpr (W32 == 8) {
-        // 256-bit codes: the Gram matrix (256 KB) stays in L2 and the scanning warps leave this one few issue slots, so the
-        // instructions count.  Lane l holds the eight columns 8l .. 8l + 7: a row of the Gram matrix is two 16-byte reads
-        // per lane, group g of eight bits is decided inside lane g (whose part of the group's rows is the 8 x 8 diagonal
-        // block; the other lanes run the same instructions on their own values, unused), and one shuffle hands the eight
-        // signs over.  About 5 400 instructions instead of 16 000 with one column of every word per lane.
-        float t8[8];
+      if (c1 - c0 < kUnrolledSweepKeys) sweep(std::true_type()); else sweep(std::false_type());
+    } else {
+      // Lane l holds the W32 columns W32 l .. W32 l + W32 - 1, so its part of a Gram row is one or two vector reads.  Group g
+      // of W32 bits is decided inside lane g (whose part of the group's rows is the diagonal block; the other lanes run the
+      // same instructions on their own values, unused), and one shuffle hands the signs over.  Slower alone than the form
+      // above but a third of its instructions, for the scans that keep the integer pipe or the issue slots busy: 256 bits
+      // took 16 000 instructions with one column of every word per lane (78 us beside a 60 us scan), 5 400 this way.
+      // Every value sees the same fp32 operations in the same order as a one-bit-at-a-time sweep.
+      float t[W32];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) t8[e] = (float)pd[GP * B + 8 * lane + e] + 0.f;   // (never -0)
-        uint32_t word = 0u;
-#pragma unroll 1
-        for (int g = 0; g < 32; ++g) {
-          float row[8][8];
+      for (int e = 0; e < W32; ++e) t[e] = (float)pd[GP * B + W32 * lane + e] + 0.f;   // (never -0)
+      [[maybe_unused]] const unsigned gram_s = (unsigned)__cvta_generic_to_shared(gsm);
+      constexpr int kBuf = W32 <= 4 ? 2 : 1;                   // rows of the next group are read ahead where registers allow
+      float row[kBuf][W32][W32];
+      auto load_rows = [&](float (&r)[W32][W32], int g) {
+        const int col = W32 * max(lane, g);                    // (columns before the group are never read again: those lanes repeat lane g's)
 #pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            float4 a = make_float4(0.f, 0.f, 0.f, 0.f), c = a;
-            if (rc && lane >= g) {
-              const float4* src = reinterpret_cast<const float4*>(gq + (size_t)(8 * g + e) * B + 8 * lane);
-              a = src[0]; c = src[1];
+        for (int e = 0; e < W32; ++e) {
+          if constexpr (W32 >= 4) {
+#pragma unroll
+            for (int f = 0; f < W32; f += 4) {
+              float4 v;
+              if (kGramTri && gsm != nullptr)
+                asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                             : "r"(gram_s + (unsigned)(gram_tri(W32 * g + e, col) + 4 * f)));
+              else
+                v = *reinterpret_cast<const float4*>(gq + (size_t)(W32 * g + e) * B + col + f);
+              r[e][f] = v.x; r[e][f + 1] = v.y; r[e][f + 2] = v.z; r[e][f + 3] = v.w;
             }
-            row[e][0] = a.x; row[e][1] = a.y; row[e][2] = a.z; row[e][3] = a.w;
-            row[e][4] = c.x; row[e][5] = c.y; row[e][6] = c.z; row[e][7] = c.w;
-          }
-          float w[8];
-          uint32_t bits = 0u;
+          } else {
 #pragma unroll
-          for (int e = 0; e < 8; ++e) w[e] = t8[e];
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            const uint32_t sb = __float_as_uint(w[e]) & 0x80000000u;
-            bits |= (sb >> (31 - e)) ^ (1u << e);
-            const float nu = __uint_as_float(sb ^ 0xBF800000u);
-#pragma unroll
-            for (int f = e + 1; f < 8; ++f) w[f] = fmaf(nu, row[e][f], w[f]);
-          }
-          bits = __shfl_sync(0xffffffffu, bits, g);
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            const float nu = __uint_as_float(0x3F800000u | ((bits << (31 - e)) & 0x80000000u));
-#pragma unroll
-            for (int f = 0; f < 8; ++f) t8[f] = fmaf(nu, row[e][f], t8[f]);
-          }
-          word |= bits << (8 * (g & 3));
-          if ((g & 3) == 3) {
-            if (lane == 0) { st->newcode[g >> 2] = word; code_dst[g >> 2] = word; }
-            word = 0u;
+            for (int f = 0; f < W32; ++f) r[e][f] = gq[(size_t)(W32 * g + e) * B + col + f];
           }
         }
+      };
+      uint32_t word = 0u;
+      auto group = [&](const float (&r)[W32][W32], int g) {
+        float w[W32];
+        uint32_t bits = 0u;
+#pragma unroll
+        for (int e = 0; e < W32; ++e) w[e] = t[e];
+#pragma unroll
+        for (int e = 0; e < W32; ++e) {
+          const uint32_t sb = __float_as_uint(w[e]) & 0x80000000u;
+          bits |= (sb >> (31 - e)) ^ (1u << e);
+          const float nu = __uint_as_float(sb ^ 0xBF800000u);
+#pragma unroll
+          for (int f = e + 1; f < W32; ++f) w[f] = fmaf(nu, r[e][f], w[f]);
+        }
+        bits = __shfl_sync(0xffffffffu, bits, g);
+#pragma unroll
+        for (int e = 0; e < W32; ++e) {
+          const float nu = __uint_as_float(0x3F800000u | ((bits << (31 - e)) & 0x80000000u));
+#pragma unroll
+          for (int f = 0; f < W32; ++f) t[f] = fmaf(nu, r[e][f], t[f]);
+        }
+        word |= bits << ((W32 * g) & 31);
+        if (((W32 * (g + 1)) & 31) == 0) {
+          if (lane == 0) { st->newcode[(W32 * g) >> 5] = word; code_dst[(W32 * g) >> 5] = word; }
+          word = 0u;
+        }
+      };
+      if (!rc) {                                               // plain signs
+        uint32_t mine = 0u;
+#pragma unroll
+        for (int e = 0; e < W32; ++e) mine |= (t[e] >= 0.f ? 1u : 0u) << e;
+        for (int w = 0; w < W32; ++w) {
+          uint32_t v = lane / (32 / W32) == w ? mine << (W32 * (lane & (32 / W32 - 1))) : 0u;
+          v = __reduce_or_sync(0xffffffffu, v);
+          if (lane == 0) { st->newcode[w] = v; code_dst[w] = v; }
+        }
+      } else if constexpr (kBuf == 2) {
+        load_rows(row[0], 0);
+#pragma unroll 1
+        for (int g = 0; g < 32; g += 2) {
+          load_rows(row[1], g + 1);
+          group(row[0], g);
+          if (g + 2 < 32) load_rows(row[0], g + 2);
+          group(row[1], g + 1);
+        }
       } else {
-        if (c1 - c0 < kUnrolledSweepKeys) sweep(std::true_type()); else sweep(std::false_type());
+#pragma unroll 1
+        for (int g = 0; g < 32; ++g) {
+          load_rows(row[0], g);
+          group(row[0], g);
+        }
       }
     }
     if (p.dbg_times != nullptr && lane == 0) p.dbg_times[(size_t)blockIdx.x * 16 + 11] = (unsigned long long)clock64();
+    if (kDefer) store_rows();
+    if (deferred) {
+      int key = 0;
+      if (lane == 0) {
+        uint32_t sg[W32], mk[NP][W32], h[W32];
+#pragma unroll
+        for (int w = 0; w < W32; ++w) {
+          sg[w] = st->signw[w]; h[w] = st->newcode[w];
+#pragma unroll
+          for (int pl = 0; pl < NP; ++pl) mk[pl][w] = st->mask[pl][w];
+        }
+        key = score_key<W32, NP>(h, sg, mk);
+        if constexpr (K8) sc8[n - 1 - c0] = (uint8_t)key;
+        else sc[score_slot(n - 1 - c0)] = (uint16_t)key;
+        if (p.dbg_scores != nullptr) p.dbg_scores[(size_t)unit * p.n_max + (n - 1)] = ((2 * key) << cs) - (st->rsum << cs);
+      }
+      key = __shfl_sync(0xffffffffu, key, 0);
+      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // (every block's mbarrier is set up)
+      if (lane < CS)
+        asm volatile("{\n\t.reg .b32 d, b;\n\tmapa.shared::cluster.u32 d, %0, %2;\n\tmapa.shared::cluster.u32 b, %1, %2;\n\t"
+                     "st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [d], %3, [b];\n\t}\n"
+                     ::"r"((unsigned)__cvta_generic_to_shared(&st->newkey)), "r"((unsigned)__cvta_generic_to_shared(&st->new_bar)), "r"(lane), "r"(key) : "memory");
+      __syncwarp();
+    }
   }
   int newkey = -1;                                           // streaming: score key of the key appended by this launch
   if constexpr (STREAM) {
@@ -999,7 +1125,7 @@ bpc_decode_kernel(const DecodeParams p) {
       hist[bin] = sum;
     }
   }
-  if (!STREAM && appender) {
+  if (!STREAM && appender && !deferred) {
     __syncthreads();                                         // the new code is in shared memory; the scan is done
     if (tid == 0) {
       uint32_t sg[W32], mk[NP][W32], h[W32];
@@ -1032,11 +1158,13 @@ bpc_decode_kernel(const DecodeParams p) {
     size_t push_off = STREAM ? (size_t)NW * nbins * 4 : L::score_bytes(p.chunk_cap, K8 ? 1 : 2);
     if (push_off < L::hashpart_bytes()) push_off = L::hashpart_bytes();   // a peer may still be hashing
     push_off = (push_off + 15) & ~(size_t)15;
-    if ((fast_sel || quad_sel) && CS > 1 && push_off + (size_t)CS * bin_stride * 4 + (size_t)B * B * 4 <= union_bytes)
+    if ((fast_sel || quad_sel) && CS > 1 && push_off + (size_t)CS * bin_stride * 4 + (size_t)kGramBytes <= union_bytes)
       pushed = reinterpret_cast<uint32_t*>(uni + push_off);
   }
-  if (pushed != nullptr) {
-    __syncthreads();                                         // this block's histogram is complete
+  const int sel_threads = deferred && appender ? NT - 32 : NT;   // threads of this block in the threshold search
+  const bool sits_out = deferred && appends;
+  if (pushed != nullptr && !sits_out) {
+    if (kDefer) partial_sync(sel_threads); else __syncthreads();   // this block's histogram is complete
     for (int i = tid; i < bin_stride; i += NT) {
       const uint32_t v = hist[i];
 #pragma unroll
@@ -1045,14 +1173,16 @@ bpc_decode_kernel(const DecodeParams p) {
       if (MODE == 0) break;                                  // (one bin per thread there)
     }
   }
-  cluster.sync();                                            // every block's histogram is complete (and delivered)
+  if (!sits_out) cluster.sync();                             // every block's histogram is complete (and delivered)
   BPC_STAMP(8);
   const int e0 = (EAS && me > 0) ? st->e0 : 0, e1 = (EAS && me > 0) ? st->e1 : 0;
   if (appender && tid == 0) p.unit_lens_w[unit] = n;         // every block of the cluster has read the old length
   // Threshold key T (the k-th largest score key) and this block's share of the output.
   int T;
   int scan_calls = 0;                                        // block scans so far (selects their buffer)
-  if (fast_sel) {
+  if (sits_out) {
+    scan_calls = 1;
+  } else if (fast_sel) {
     // Common case, one histogram bin per thread: thread t owns bin nbins-1-t, reads that bin from every block of
     // the cluster (distributed shared memory) and a two-value block scan yields, for every bin, the number of keys
     // in higher bins (cluster-wide, and in the blocks of lower rank).  The thread whose bin holds the k-th key
@@ -1081,7 +1211,7 @@ bpc_decode_kernel(const DecodeParams p) {
       }
     }
     uint32_t above_all, above_low;
-    block_excl_scan2<NT>(s_all, s_low, st->wscan, scan_calls, above_all, above_low);
+    block_excl_scan2<NT, kDefer>(s_all, s_low, st->wscan, scan_calls, above_all, above_low, sel_threads);
     if (bin >= 0 && above_all < (uint32_t)kh && above_all + s_all >= (uint32_t)kh) {
       const int need = kh - (int)above_all;                   // ties to take, cluster-wide (>= 1)
       const int lower_take = min(need, (int)s_low);          // ties granted to blocks of lower rank
@@ -1089,8 +1219,9 @@ bpc_decode_kernel(const DecodeParams p) {
       st->cnt_gt = (int)above_all;
       st->my_take = min(max(need - (int)s_low, 0), (int)mine);
       st->my_base = (int)above_low + lower_take;
+      if (kDefer) { st->above_low = (int)above_low; st->low = (int)s_low; st->mine = (int)mine; }
     }
-    __syncthreads();
+    if (!deferred) __syncthreads();
     T = st->T;
     BPC_STAMP(9);
   } else if (quad_sel) {
@@ -1238,6 +1369,16 @@ bpc_decode_kernel(const DecodeParams p) {
       if (tid < CS) st->eq[tid] = cluster.map_shared_rank(hist, tid)[T];
     }
     __syncthreads();
+  }
+  if (deferred) {
+    __syncthreads();                                         // the threshold is known, the appending warp is back
+    int tries = 0;
+    uint32_t there = 0u;
+    while (!there && tries++ < 20000000)
+      asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
+                   : "=r"(there) : "r"((unsigned)__cvta_generic_to_shared(&st->new_bar)) : "memory");
+    if (!there && tid == 0) atomicOr(p.err, BPC_DEVERR_TIMEOUT);
+    T = st->T;
   }
   int T_exact = quad_sel ? st->T : T;
   if (MODE == 1 && hsh > 0 && kh > 0 && !quad_sel) {
@@ -1434,7 +1575,12 @@ bpc_decode_kernel(const DecodeParams p) {
     // at again (re-read from shared memory) to tell "greater" from "tie".
     const int len = c1 - c0;
     const int nseg = (len + kSegKeys - 1) / kSegKeys;
-    const int my_take = st->my_take;
+    int my_take = st->my_take, my_base = st->my_base;
+    if (deferred && st->newkey > T_exact) {                  // the appended key is in: one tie less
+      const int need = kh - st->cnt_gt - 1;
+      my_take = min(max(need - st->low, 0), st->mine);
+      my_base = st->above_low + min(need, st->low);
+    }
     const int T = T_exact;                                   // shadows the coarse bin: from here on the exact key
     const uint32_t cge = (uint32_t)(0x8000 - T) * 0x10001u;
     constexpr int SPT = 4;                                   // most consecutive segments one thread takes per pass
@@ -1518,7 +1664,7 @@ bpc_decode_kernel(const DecodeParams p) {
       for (int q = 0; q < SPT; ++q) TK[q] = 0u;
       if (cgt | ceq) {
         int eqb = run_eq + (int)(ex >> 16);
-        int pos = st->my_base + run_gt + (int)(ex & 0xffffu) + min(eqb, my_take);
+        int pos = my_base + run_gt + (int)(ex & 0xffffu) + min(eqb, my_take);
 #pragma unroll
         for (int q = 0; q < SPT; ++q) {
           const int seg = s0 + tid * spt + q;

@@ -30,10 +30,10 @@ static cudaError_t launch_one(bpc_ctx* ctx, const DecodeParams& p_in, cudaStream
   p.stages = L(p.chunk_cap, p.nbins, 3, kKeyBytes).total <= (size_t)optin ? 3 : 2;
   const size_t smem = L(p.chunk_cap, p.nbins, p.stages, kKeyBytes).total;
   if (smem > (size_t)optin) return cudaErrorInvalidConfiguration;
-  if (ctx->decode_smem_set == 0) {                          // function attributes are sticky: set them once
+  if ((ctx->decode_smem_set & ((size_t)1 << EAS)) == 0) {   // function attributes are sticky: set them once per variant
     e = configure_kernel<KV, GP, W32, MODE, EAS>(ctx->device);
     if (e != cudaSuccess) return e;
-    ctx->decode_smem_set = 1;
+    ctx->decode_smem_set |= (size_t)1 << EAS;
   }
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3((unsigned)(ctx->units * ctx->cluster_size), 1, 1);
