@@ -585,7 +585,7 @@ bpc_decode_kernel(const DecodeParams p) {
   }
   if (tid < BPC_D)                                           // slot GP: the appended key (its decision values P_h k)
     qf_s[GP * BPC_D + tid] = appender ? to_float(kDefer ? kreg : reinterpret_cast<const KV*>(p.k_new)[(size_t)unit * BPC_D + tid]) : 0.f;
-  for (int i = tid; i < (MODE == 1 ? (nbins + 3) & ~3 : nbins); i += NT) hist[i] = 0u;   // (weighted: bins are read four at a time)
+  for (int i = tid; i < (kFastOnly ? nbins : (nbins + 3) & ~3); i += NT) hist[i] = 0u;   // (bins may be read four at a time)
   if (tid < BPC_MAX_CLUSTER) { st->gt[tid] = 0u; st->eq[tid] = 0u; }
   if (kDefer && tid == 0) {
     if (gsm != nullptr)
@@ -1148,9 +1148,10 @@ bpc_decode_kernel(const DecodeParams p) {
   // With one bin per thread, every block first stores its finished histogram into a slot of every peer's shared memory
   // (behind the score keys), so that after the barrier all CS histograms are local reads.
   const bool fast_sel = kFastOnly || (nbins <= NT && hsh == 0);
-  // Weighted scores whose stored keys are exact (no shift): four bins per thread, then the low bits inside the threshold's
-  // bin; both levels are pushed to the peers like the one-bin-per-thread histograms.
-  const bool quad_sel = MODE == 1 && ksh == 0 && hsh > 0 && nbins <= 4 * NT && kh > 0;
+  // More bins than threads and exact stored keys: four bins per thread, and where a bin holds several keys (weighted scores)
+  // the low bits inside the threshold's bin; both levels are pushed to the peers like the one-bin-per-thread histograms.
+  // (Histograms summed bin by bin through distributed shared memory took 3.1 us at 897 bins, 3.7 at 513.)
+  const bool quad_sel = !kFastOnly && !fast_sel && (MODE == 0 ? hsh == 0 : ksh == 0) && nbins <= 4 * NT && kh > 0;
   const int bin_stride = quad_sel ? (nbins + 3) & ~3 : nbins;
   uint32_t* pushed = nullptr;
   {
@@ -1170,7 +1171,7 @@ bpc_decode_kernel(const DecodeParams p) {
 #pragma unroll
       for (int r = 0; r < BPC_MAX_CLUSTER; ++r)
         if (r < CS) cluster.map_shared_rank(pushed, r)[rank * bin_stride + i] = v;
-      if (MODE == 0) break;                                  // (one bin per thread there)
+      if (kFastOnly) break;                                  // (one bin per thread there)
     }
   }
   if (!sits_out) cluster.sync();                             // every block's histogram is complete (and delivered)
@@ -1225,11 +1226,12 @@ bpc_decode_kernel(const DecodeParams p) {
     T = st->T;
     BPC_STAMP(9);
   } else if (quad_sel) {
-    if constexpr (MODE == 1) {
+    if constexpr (!kFastOnly) {
     // Thread t owns bins 4q .. 4q + 3, q counted from the top; the block scan gives the keys above its bins (in the cluster and
     // in the blocks of lower rank), and the thread whose bins hold the k-th key walks them.
     const int q4 = ((nbins + 3) >> 2) - 1 - tid;
     uint32_t c[4] = {0u, 0u, 0u, 0u}, low[4] = {0u, 0u, 0u, 0u};
+    [[maybe_unused]] uint32_t own[4] = {0u, 0u, 0u, 0u};
     if (q4 >= 0) {
 #pragma unroll 1
       for (int r = 0; r < CS; ++r) {
@@ -1237,6 +1239,7 @@ bpc_decode_kernel(const DecodeParams p) {
         const uint4 v = *reinterpret_cast<const uint4*>(h + 4 * q4);
         c[0] += v.x; c[1] += v.y; c[2] += v.z; c[3] += v.w;
         if (r < rank) { low[0] += v.x; low[1] += v.y; low[2] += v.z; low[3] += v.w; }
+        if (MODE == 0 && r == rank) { own[0] = v.x; own[1] = v.y; own[2] = v.z; own[3] = v.w; }
       }
     }
     uint32_t above, above_low;
@@ -1245,15 +1248,25 @@ bpc_decode_kernel(const DecodeParams p) {
     if (above < (uint32_t)kh && above + s_all >= (uint32_t)kh) {
 #pragma unroll
       for (int i = 3; i >= 0; --i) {
-        if (above < (uint32_t)kh && above + c[i] >= (uint32_t)kh) { st->T = 4 * q4 + i; st->cnt_gt = (int)above; st->my_base = (int)above_low; }
+        if (above < (uint32_t)kh && above + c[i] >= (uint32_t)kh) {
+          st->T = 4 * q4 + i;
+          st->cnt_gt = (int)above;
+          st->my_base = (int)above_low;
+          if (MODE == 0) {                                   // the bin is one key: ties go to the blocks in rank order
+            const int need = kh - (int)above, lower_take = min(need, (int)low[i]);
+            st->my_take = min(max(need - (int)low[i], 0), (int)own[i]);
+            st->my_base += lower_take;
+          }
+        }
         above += c[i];
         above_low += low[i];
       }
     }
-    if (tid < 32) tot[tid] = 0u;                             // this block's counts of the low bits
+    if (MODE == 1 && tid < 32) tot[tid] = 0u;                // this block's counts of the low bits
     __syncthreads();
     T = st->T;
     BPC_STAMP(9);
+    if constexpr (MODE == 1) {
     // counts of the low bits of the keys in bin T, whole segments at a time: a half word whose high bits equal the bin's
     // leaves a zero, which the subtraction carries into its top bit.  (A borrow from a zero low half can only raise a false
     // alarm in the high half, so that half is compared once more.)
@@ -1307,6 +1320,7 @@ bpc_decode_kernel(const DecodeParams p) {
       }
     }
     __syncthreads();
+    }
     }
   } else if constexpr (!kFastOnly) {
     // Total histogram through distributed shared memory.  With at most one bin per thread (the common case)
