@@ -401,6 +401,7 @@ bpc_status bpc_get_seq_lens(bpc_ctx* ctx, int32_t* host_out) {
 
 bpc_status bpc_set_projection(bpc_ctx* ctx, const float* P, void* stream) {
   if (ctx == nullptr || P == nullptr) return BPC_ERR_INVALID_ARG;
+  ctx->projection_settled = false;
   const bpc_config& c = ctx->cfg;
   cudaError_t e = cudaMemcpyAsync(ctx->P, P, (size_t)c.hash_sets * c.code_bits * BPC_D * 4, cudaMemcpyDeviceToDevice,
                                   (cudaStream_t)stream);
@@ -431,6 +432,7 @@ bpc_status bpc_fit(bpc_ctx* ctx, const void* k_cache, const float* v_star, void*
   if (ctx->cfg.hash_sets != ctx->units) return BPC_ERR_UNSUPPORTED;
   if (workspace_bytes < bpc_fit_workspace_bytes_impl(&ctx->cfg)) return BPC_ERR_INVALID_ARG;
   int launches = 0;
+  ctx->projection_settled = false;
   cudaError_t e = bpc_launch_fit(ctx, k_cache, v_star, workspace, (cudaStream_t)stream, &launches);
   ctx->launches += launches;
   if (e == cudaSuccess) e = bpc_launch_finalize_projection(ctx, (cudaStream_t)stream);
@@ -591,6 +593,7 @@ static bpc_status decode_common(bpc_ctx* ctx, const void* k_new, const void* v_n
   p.nbins = hist_bins(ctx);
   p.hist_shift = hist_shift(ctx);
   p.key_shift_min = ctx->key_shift_min;
+  p.early_projection = ctx->projection_settled && ctx->settled_stream == stream;
   if (ctx->streaming)
     e = c.kv_dtype == BPC_BF16 ? bpc_launch_decode_bf16_stream(ctx, p, (cudaStream_t)stream)
                                : bpc_launch_decode_f32_stream(ctx, p, (cudaStream_t)stream);
@@ -610,6 +613,8 @@ static bpc_status decode_common(bpc_ctx* ctx, const void* k_new, const void* v_n
     e = c.kv_dtype == BPC_BF16 ? bpc_launch_decode_bf16(ctx, p, (cudaStream_t)stream)
                                : bpc_launch_decode_f32(ctx, p, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(ctx, e);
+  ctx->projection_settled = true;
+  ctx->settled_stream = stream;
   ctx->launches += 1;
   return BPC_OK;
 }

@@ -35,6 +35,8 @@ struct bpc_ctx {
   int max_active[BPC_MAX_CLUSTER + 1];   // [cs]: clusters of size cs that can be resident at once (0 = not schedulable)
   int sm_count;
   bool fitted;
+  bool projection_settled;  // a decode step has been launched since the projection was last written ...
+  void* settled_stream;     // ... the last one on this stream
   bool use_pdl;             // launch the decode kernel with programmatic stream serialization
   bool streaming;           // the scores of a full unit do not fit the largest cluster: two-pass (streaming) selection
   float* P;                 // [hash_sets][b][D] float
@@ -123,6 +125,7 @@ struct DecodeParams {
   int chunk_cap;             // keys whose scores one thread block can hold
   int nbins;                 // histogram bins
   int hist_shift;            // histogram bin = stored score key >> hist_shift
+  int early_projection;      // the projection may be read before the programmatic dependency wait (see the kernel)
   int key_shift_min;         // weighted scores: smallest right shift of the stored 16-bit keys (diagnostic; normally 0)
 };
 

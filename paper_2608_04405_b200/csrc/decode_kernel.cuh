@@ -403,24 +403,29 @@ bpc_decode_kernel(const DecodeParams p) {
   const int kvh = unit % p.n_kv_heads;
   const int seq = unit / p.n_kv_heads;
 
+  // The rows of the projection are requested first of all.  Usually that is safe before the dependency wait below: if this
+  // context's previous launch was a decode step too (p.early_projection), whatever wrote the projection had completed before
+  // that step went past its own wait, and this grid starts after that.  Otherwise the kernel before this one in the stream may
+  // be the one that writes it (bpc_fit, bpc_set_projection).  Read at L2: this SM's L1 may hold lines from before.
+  constexpr int HPARTS = NT / B;                 // slices per projection row in the query hash
+  constexpr int HDS = BPC_D / HPARTS;            // channels per slice (a multiple of 8)
+  constexpr int HV = HDS * (int)sizeof(KV) / 16; // 16-byte vectors per slice
+  uint4 prow[HV];
+  const uint4* prow_src = reinterpret_cast<const uint4*>(reinterpret_cast<const KV*>(p.P_h) +
+                                                         ((size_t)(p.shared_sets ? kvh : unit) * B + tid % B) * BPC_D + (tid / B) * HDS);
+  if (p.early_projection) {
+#pragma unroll
+    for (int v = 0; v < HV; ++v) prow[v] = __ldcg(prow_src + v);
+  }
+
   // Programmatic dependent launch: when this grid was launched early (while its predecessor in the stream
   // was still running) nothing of the predecessor's output may be read before this point; afterwards the
   // successor's blocks may be scheduled as ours drain.  Both are no-ops for an ordinary launch.
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-
-  // The rows of the projection are requested first of all after the dependency wait (the kernel before this one in
-  // the stream may be the one that wrote them: bpc_fit, bpc_set_projection).
-  constexpr int HPARTS = NT / B;                 // slices per projection row in the query hash
-  constexpr int HDS = BPC_D / HPARTS;            // channels per slice (a multiple of 8)
-  constexpr int HV = HDS * (int)sizeof(KV) / 16; // 16-byte vectors per slice
-  uint4 prow[HV];
-  {
-    const int j = tid % B, part = tid / B;
-    const uint4* row = reinterpret_cast<const uint4*>(reinterpret_cast<const KV*>(p.P_h) +
-                                                      ((size_t)(p.shared_sets ? kvh : unit) * B + j) * BPC_D + part * HDS);
+  if (!p.early_projection) {
 #pragma unroll
-    for (int v = 0; v < HV; ++v) prow[v] = row[v];
+    for (int v = 0; v < HV; ++v) prow[v] = __ldcg(prow_src + v);
   }
 
   // The queries do not depend on the sequence length: their loads overlap the length read and the set-up below.
