@@ -416,6 +416,20 @@ bpc_decode_kernel(const DecodeParams p) {
   if (p.early_projection) {
 #pragma unroll
     for (int v = 0; v < HV; ++v) prow[v] = __ldcg(prow_src + v);
+    // Also from here on the first quarter of the block's codes is on its way to L2, by a length that may be one step old: a
+    // hint only.  (4 x 128K keys 40.1 -> 39.5 us, one sequence of 1M keys 42.8 -> 41.6, 256 bits ragged 91.4 -> 88.1; more of
+    // the codes, or all at once, gets in the way of the first batches.)
+    if (lane == 0) {
+      int n_e;
+      asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(n_e) : "l"(p.unit_lens + unit));
+      n_e = max(0, min(n_e, p.n_max));
+      const int ch_e = CS > 1 ? bpc_fused_chunk(n_e, CS) : n_e;
+      const int k0 = rank * ch_e, end = k0 + (min(n_e, k0 + ch_e) - k0) / 4;
+      constexpr int PIECE = 4096 / (W32 * 4);                // keys whose codes take 4 KB
+      for (int i = k0 + warp * PIECE; i + PIECE <= end; i += NW * PIECE)
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], 4096;"
+                     ::"l"(reinterpret_cast<const uint32_t*>(p.codes) + ((size_t)unit * p.n_max + i) * W32) : "memory");
+    }
   }
 
   // Programmatic dependent launch: when this grid was launched early (while its predecessor in the stream
