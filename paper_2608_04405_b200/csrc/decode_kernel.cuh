@@ -569,8 +569,9 @@ bpc_decode_kernel(const DecodeParams p) {
   const int c1s = appender ? c1 - 1 : c1;
   const uint32_t* cu = reinterpret_cast<const uint32_t*>(p.codes) + (size_t)unit * (size_t)p.n_max * W32;
   int32_t* dbg = p.dbg_scores != nullptr ? p.dbg_scores + (size_t)unit * p.n_max : nullptr;
-  // codes in flight per thread and buffer: the scan is bound by memory latency and wants many
-  constexpr int U = W32 <= 4 ? 8 : 4;
+  // codes in flight per thread and buffer: the scan is bound by memory latency and wants many; the weighted scan is bound by
+  // instruction fetches (its scoring code is long) and does better with few (4 x 128K keys: 52.4 us with eight, 51.6 with two)
+  constexpr int U = MODE == 1 ? (W32 <= 2 ? 4 : 2) : W32 <= 4 ? 8 : 4;
   auto load_code = [&](uint32_t (&h)[W32], int i) {
     const uint32_t* src = cu + (size_t)i * W32;
     if (W32 == 1) {

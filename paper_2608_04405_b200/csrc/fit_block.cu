@@ -670,9 +670,12 @@ __device__ __forceinline__ float lut_sum(unsigned base, uint32_t w) {      // ro
 // One pass over this block's keys: decides bit j; unless it is the block's last bit, also the sums for column j + 1.
 // Q4 = groups of four bits in play (j / 4 + 1).  Keys past the end (up to 255, all in the last group of the unit's last
 // block, entries zero) take part like any others and are subtracted at the end: they all carry the same code word.
-template <int Q4, bool LAST>
-__device__ __forceinline__ void sweep_pass(SweepStream& in, uint32_t* __restrict__ ws, unsigned lut, int j, int nk, int nkeys, int warp,
-                                           int lane, SweepSums& out) {
+// ONE = a warp has at most one group.  Lane i then keeps bit i of its warp's 256 keys as eight words (`rows`), and the
+// agreements are population counts against the new bit's ballots; the bit-sliced counters, whose transposition costs some
+// 900 cycles per bit, only pay with several groups (8 heads x 32K keys: 120 us per 32 bits with them).
+template <int Q4, bool LAST, bool ONE>
+__device__ __forceinline__ void sweep_pass(SweepStream& in, uint32_t* __restrict__ ws, uint32_t (&rows)[kSweepKeys], unsigned lut, int j,
+                                           int nk, int nkeys, int warp, int lane, SweepSums& out) {
   constexpr int NS = Q4 <= 2 ? 8 : Q4 <= 4 ? 16 : 32;      // running sums (a power of two for the warp reduction)
   out.s = 0.0;
   out.cnt = 0;
@@ -706,7 +709,8 @@ __device__ __forceinline__ void sweep_pass(SweepStream& in, uint32_t* __restrict
         for (int e = 0; e < 4; ++e) {
           const float c = lut_sum<(Q4 + 1) / 2>(lut, w[e]);
           const uint32_t neg = (uint32_t)((int)__float_as_uint(t[e] - c) >> 31);   // (never -0: columns hold no -0)
-          x[4 * h + e] = w[e] ^ neg;                       // bit i: agrees with the new bit
+          if (ONE) x[4 * h + e] = __ballot_sync(0xffffffffu, neg == 0u);
+          else x[4 * h + e] = w[e] ^ neg;                  // bit i: agrees with the new bit
           w[e] |= bit & ~neg;
           if (!LAST) {
             tot += nx[e];
@@ -716,12 +720,21 @@ __device__ __forceinline__ void sweep_pass(SweepStream& in, uint32_t* __restrict
         *reinterpret_cast<uint4*>(pw + 128 * h) = make_uint4(w[0], w[1], w[2], w[3]);
       }
       pw += kSweepWarps * kSweepGroup;
-      if (!LAST) count8(pl, x);
+      if (!LAST && !ONE) count8(pl, x);
+      if (!LAST && ONE) {
+#pragma unroll
+        for (int e = 0; e < kSweepKeys; ++e) {
+          out.cnt += __popc(~(rows[e] ^ x[e]));
+          if (lane == j) rows[e] = x[e];
+        }
+        break;
+      }
     }
     if (!LAST) {
 #pragma unroll
       for (int o = 16; o >= 1; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
       out.s += 2.0 * (double)warp_sum_scatter<NS>(s, lane) - (double)tot;
+      if (!ONE) {
       const int keys_per_lane = kSweepKeys * ((g1 - g0 + kSweepWarps - 1) / kSweepWarps);
 #pragma unroll
       for (int k0 = 0; k0 < kSweepPlanes; k0 += 4) {       // four independent transposes at a time
@@ -731,6 +744,7 @@ __device__ __forceinline__ void sweep_pass(SweepStream& in, uint32_t* __restrict
 #pragma unroll
         for (int k = 0; k < 4; ++k) out.cnt += __popc(x[k]) << (k0 + k);
       }
+      }
       if (g1 == ng && nkeys < nk && (ng - 1 - warp) % kSweepWarps == 0) {   // this warp took the group with keys past the end
         __syncwarp();
         const uint32_t wp = ws[nk - 1];
@@ -738,6 +752,7 @@ __device__ __forceinline__ void sweep_pass(SweepStream& in, uint32_t* __restrict
         out.cnt -= (nk - nkeys) * (int)((same >> lane) & 1u);
       }
     }
+    if (ONE) break;
   }
 }
 
@@ -767,7 +782,7 @@ __device__ __forceinline__ void send_b32(const void* dst, const void* bar, int r
                ::"r"(smem_u32(dst)), "r"(smem_u32(bar)), "r"(r), "r"(v) : "memory");
 }
 
-template <bool SMEM_WORDS>
+template <bool SMEM_WORDS, bool ONE>
 __global__ void __launch_bounds__(kSweepThreads, 1)
 fit_sweep_kernel(const float* __restrict__ T, uint32_t* __restrict__ hfit, uint32_t* __restrict__ words_g,
                  const int32_t* __restrict__ unit_lens, int32_t* __restrict__ err, int n_max, int b, int blk, int t_stride, int cluster_size) {
@@ -808,6 +823,7 @@ fit_sweep_kernel(const float* __restrict__ T, uint32_t* __restrict__ hfit, uint3
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");      // every rank's barriers are armed
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   double new_row = 0.0;
+  uint32_t rows[kSweepKeys] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
   const float* Tu = T + (size_t)unit * kBits * t_stride + row0;
   const double inv_n = 1.0 / (double)n;
   const unsigned lut_a = smem_u32(lut);
@@ -827,17 +843,17 @@ fit_sweep_kernel(const float* __restrict__ T, uint32_t* __restrict__ hfit, uint3
   in.request(in.ring);
   for (int j = 0; j < kBits; ++j) {
     SweepSums sums;
-    if (j == kBits - 1) { sweep_pass<8, true>(in, ws, lut_a, j, nk, nkeys, warp, lane, sums); break; }
+    if (j == kBits - 1) { sweep_pass<8, true, ONE>(in, ws, rows, lut_a, j, nk, nkeys, warp, lane, sums); break; }
     prefetch(j + 2);
     switch (j >> 2) {
-      case 0: sweep_pass<1, false>(in, ws, lut_a, j, nk, nkeys, warp, lane, sums); break;
-      case 1: sweep_pass<2, false>(in, ws, lut_a, j, nk, nkeys, warp, lane, sums); break;
-      case 2: sweep_pass<3, false>(in, ws, lut_a, j, nk, nkeys, warp, lane, sums); break;
-      case 3: sweep_pass<4, false>(in, ws, lut_a, j, nk, nkeys, warp, lane, sums); break;
-      case 4: sweep_pass<5, false>(in, ws, lut_a, j, nk, nkeys, warp, lane, sums); break;
-      case 5: sweep_pass<6, false>(in, ws, lut_a, j, nk, nkeys, warp, lane, sums); break;
-      case 6: sweep_pass<7, false>(in, ws, lut_a, j, nk, nkeys, warp, lane, sums); break;
-      default: sweep_pass<8, false>(in, ws, lut_a, j, nk, nkeys, warp, lane, sums); break;
+      case 0: sweep_pass<1, false, ONE>(in, ws, rows, lut_a, j, nk, nkeys, warp, lane, sums); break;
+      case 1: sweep_pass<2, false, ONE>(in, ws, rows, lut_a, j, nk, nkeys, warp, lane, sums); break;
+      case 2: sweep_pass<3, false, ONE>(in, ws, rows, lut_a, j, nk, nkeys, warp, lane, sums); break;
+      case 3: sweep_pass<4, false, ONE>(in, ws, rows, lut_a, j, nk, nkeys, warp, lane, sums); break;
+      case 4: sweep_pass<5, false, ONE>(in, ws, rows, lut_a, j, nk, nkeys, warp, lane, sums); break;
+      case 5: sweep_pass<6, false, ONE>(in, ws, rows, lut_a, j, nk, nkeys, warp, lane, sums); break;
+      case 6: sweep_pass<7, false, ONE>(in, ws, rows, lut_a, j, nk, nkeys, warp, lane, sums); break;
+      default: sweep_pass<8, false, ONE>(in, ws, rows, lut_a, j, nk, nkeys, warp, lane, sums); break;
     }
     red_s[warp][lane] = sums.s;
     red_c[warp][lane] = sums.cnt;
@@ -1065,14 +1081,16 @@ const SweepLimits* sweep_limits(int device) {
   if (device < 0 || device >= 64) return nullptr;
   SweepLimits* l = &g_sweep_limits[device];
   std::call_once(l->once, [l]() {
-    cudaError_t e = cudaFuncSetAttribute(fit_sweep_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSweepMaxSmem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fit_sweep_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSweepRing);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fit_sweep_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fit_sweep_kernel<false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaError_t e = cudaSuccess;
+    const void* kernels[3] = {(const void*)fit_sweep_kernel<true, true>, (const void*)fit_sweep_kernel<true, false>, (const void*)fit_sweep_kernel<false, false>};
+    for (const void* k : kernels) {
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSweepMaxSmem);
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    }
     for (int cs = 1; cs <= BPC_MAX_CLUSTER && e == cudaSuccess; ++cs) {
       cudaLaunchAttribute attr;
       cudaLaunchConfig_t cfg = sweep_config(&attr, 1, cs, kSweepMaxSmem, nullptr);
-      if (cudaOccupancyMaxActiveClusters(&l->active[cs], fit_sweep_kernel<true>, &cfg) != cudaSuccess) {
+      if (cudaOccupancyMaxActiveClusters(&l->active[cs], fit_sweep_kernel<true, false>, &cfg) != cudaSuccess) {
         (void)cudaGetLastError();
         l->active[cs] = 0;
       }
@@ -1161,13 +1179,10 @@ cudaError_t bpc_launch_fit_blocked(bpc_ctx* ctx, const void* k_cache, const floa
     }
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr;
-    if (sweep_smem <= kSweepMaxSmem) {
-      cudaLaunchConfig_t cfg = sweep_config(&attr, ctx->units, cs, sweep_smem, stream);
-      e = cudaLaunchKernelEx(&cfg, fit_sweep_kernel<true>, (const float*)T, hfit, words_g, (const int32_t*)ctx->unit_lens, ctx->dev_err, (int)c.n_max, b, blk, ts, cs);
-    } else {
-      cudaLaunchConfig_t cfg = sweep_config(&attr, ctx->units, cs, kSweepRing, stream);
-      e = cudaLaunchKernelEx(&cfg, fit_sweep_kernel<false>, (const float*)T, hfit, words_g, (const int32_t*)ctx->unit_lens, ctx->dev_err, (int)c.n_max, b, blk, ts, cs);
-    }
+    const bool words_fit = sweep_smem <= kSweepMaxSmem, one = sweep_share(c.n_max, cs) <= kSweepWarps * kSweepGroup;
+    cudaLaunchConfig_t cfg = sweep_config(&attr, ctx->units, cs, words_fit ? sweep_smem : kSweepRing, stream);
+    auto sweep = !words_fit ? fit_sweep_kernel<false, false> : one ? fit_sweep_kernel<true, true> : fit_sweep_kernel<true, false>;
+    e = cudaLaunchKernelEx(&cfg, sweep, (const float*)T, hfit, words_g, (const int32_t*)ctx->unit_lens, ctx->dev_err, (int)c.n_max, b, blk, ts, cs);
     if (e != cudaSuccess) return e;
     if (tc) {
       // as many warpgroups as their tile and sign buffers leave room for (four up to the third word, two from the sixth)
