@@ -1,0 +1,112 @@
+"""Kernel variants at the edges of their tiles, groups and dispatch rules, against the CPU checker."""
+import pytest
+import torch
+
+from paper_2608_04405_b200.inputs import CONFIGS
+
+pytestmark = pytest.mark.gpu
+
+
+def _harness():
+    from tests import gpu_harness as H
+    return H
+
+
+@pytest.mark.parametrize("dtype,bits,n,batch,n_min", [
+    ("bf16", 64, 1, 1, None), ("bf16", 32, 127, 1, None), ("bf16", 128, 129, 2, 1),     # a partial tile, a tile and one key
+    ("bf16", 64, 257, 1, None), ("bf16", 256, 4097, 1, None),                           # a sweep group and one key; all eight words
+    ("bf16", 64, 9000, 3, 200), ("bf16", 32, 70001, 1, None),                           # ragged; several groups per warp
+    ("f32", 32, 1, 1, None), ("f32", 128, 385, 2, 100), ("f32", 256, 2051, 1, None)])
+def test_blocked_fit_edges(dtype, bits, n, batch, n_min):
+    """Algorithm 1 in blocks of 32 bits at the edges of its tiles (128 keys), groups (256) and code words."""
+    H = _harness()
+    spec = CONFIGS[1].scaled(name="fitedge", wid=81, dtype=dtype, batch=batch, n_ctx=n, n_ctx_min=n_min, n_kv_heads=2, n_q_heads=2,
+                             code_bits=bits, steps=1)
+    sess = H.Session(spec, gen_device="cuda" if n > 20000 else "cpu")
+    rep = {}
+    sess.fit(dirty_workspace=True)
+    H.check_fit(sess, [0, batch * 2 - 1], rep)
+    assert sess.ctx.last_device_error() == 0
+    print(rep)
+
+
+def test_blocked_fit_code_words_outside_shared_memory():
+    """One unit of 800 000 keys: more than the largest cluster's shared memory keeps code words for.  Against the fit that
+    passes over the keys once per bit (the checker would need minutes)."""
+    H = _harness()
+    spec = CONFIGS[1].scaled(name="fitlong", wid=82, n_ctx=800000, n_kv_heads=1, n_q_heads=1, code_bits=32, steps=1)
+    sess = H.Session(spec, gen_device="cuda")
+    sess.fit(dirty_workspace=True)
+    blocked = sess.P.clone()
+    sess.ctx.debug_set_tensor_core_encode(False)
+    sess.fit()
+    sess.ctx.debug_set_tensor_core_encode(True)
+    assert sess.ctx.last_device_error() == 0
+    assert ((blocked - sess.P).norm() / sess.P.norm()).item() <= 1e-3
+    assert ((blocked[:, :4] - sess.P[:, :4]).norm() / sess.P[:, :4].norm()).item() <= 1e-4
+
+
+@pytest.mark.parametrize("dtype,bits,n", [("f32", 32, 1), ("f32", 64, 31), ("f32", 128, 33), ("f32", 256, 65), ("bf16", 32, 1),
+                                          ("bf16", 64, 127), ("bf16", 128, 129), ("bf16", 256, 515), ("bf16", 128, 2561)])
+def test_encode_edges(dtype, bits, n):
+    """Encode at the edges of its key tiles (128 keys on the tensor cores, 32 on the CUDA cores) and of a block's share."""
+    H = _harness()
+    spec = CONFIGS[1].scaled(name="encedge", wid=83, dtype=dtype, batch=2, n_ctx=n, n_ctx_min=max(1, n // 2), n_kv_heads=2, n_q_heads=2,
+                             code_bits=bits, steps=1)
+    sess = H.Session(spec)
+    rep = {}
+    sess.fit()
+    sess.encode()
+    H.check_encode(sess, [0, 3], rep)
+    assert sess.ctx.last_device_error() == 0
+
+
+@pytest.mark.parametrize("dtype,bits,group,n,cluster,budget", [
+    ("bf16", 128, 4, 3000, 0, {"budget_ppm": 20000}), ("bf16", 128, 4, 6143, 1, {"budget_ppm": 20000}),
+    ("bf16", 128, 4, 6144, 1, {"budget_ppm": 20000}),                                   # the last length of the short-range kernel, the first beyond
+    ("bf16", 64, 1, 1500, 3, {"budget_count": 64}), ("bf16", 32, 2, 200, 2, {"budget_ppm": 1000000}),   # every key: nothing to defer
+    ("bf16", 256, 4, 2500, 2, {"budget_ppm": 50000}), ("bf16", 256, 1, 2500, 4, {"budget_ppm": 50000}),
+    ("bf16", 128, 7, 5000, 3, {"budget_ppm": 20000}), ("f32", 64, 1, 4096, 4, {"budget_ppm": 20000}), ("f32", 128, 4, 700, 2, {"budget_count": 699})])
+def test_short_range_steps(dtype, bits, group, n, cluster, budget):
+    """Fused steps on short key ranges (deferred selection): the appended key once as the query itself, which selects it, and
+    once as its negative, which does not, and once like the others; index sets and outputs against the checker."""
+    H = _harness()
+    spec = CONFIGS[1].scaled(name="short", wid=84, dtype=dtype, n_ctx=n, n_kv_heads=2, n_q_heads=2 * group, code_bits=bits, steps=1)
+    sess = H.Session(spec, cluster_size=cluster, extra_rows=64)
+    sess.fit()
+    sess.encode()
+    rep = {}
+    budget = dict({"budget_ppm": 0}, **budget)
+    for sign in (1.0, -1.0, None):
+        k_new, v_new = sess.w.new_kv(sess.lens)
+        q, _ = sess.w.queries(sess.lens, k_cache=sess.k_cache.to(sess.w.device))
+        if sign is not None:
+            k_new = (sign * q.view(1, 2, group, -1).float().sum(2)).to(k_new.dtype)
+        H.check_decode(sess, q.cuda(), [0, 1], rep, append=(k_new.cuda(), v_new.cuda()), **budget)
+    assert sess.ctx.last_device_error() == 0
+
+
+def test_projection_update_between_steps():
+    """Steps that may read the projection early follow an update of it: every step has to use the projection of its moment."""
+    H = _harness()
+    spec = CONFIGS[1].scaled(name="settle", wid=85, n_ctx=4000, n_kv_heads=2, n_q_heads=8, steps=1)
+    sess = H.Session(spec)
+    sess.fit()
+    P = [sess.P.clone(), torch.flip(sess.P, dims=[1]).neg().contiguous()]
+    sess.encode()
+    q, _ = sess.w.queries(sess.lens)
+    q = q.cuda()
+    want, got = [], []
+    for p in P:                                              # one step each, waited for
+        sess.ctx.set_projection(p)
+        torch.cuda.synchronize()
+        want.append(sess.ctx.decode_attn(q, sess.k_cache, sess.v_cache, sess.codes))
+        torch.cuda.synchronize()
+    for i in range(6):                                       # queued back to back, two steps per projection
+        sess.ctx.set_projection(P[i % 2])
+        for _ in range(2):
+            got.append(sess.ctx.decode_attn(q, sess.k_cache, sess.v_cache, sess.codes))
+    torch.cuda.synchronize()
+    assert not torch.equal(want[0], want[1])
+    for i, o in enumerate(got):
+        assert torch.equal(o, want[(i // 2) % 2])
