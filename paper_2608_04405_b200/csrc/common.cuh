@@ -134,6 +134,22 @@ struct DecodeParams {
 // ---- launch geometry (api.cu): fills max_cluster, max_active, chunk_cap_limit and picks cluster_size (0 = none fits)
 cudaError_t bpc_plan_decode_geometry(bpc_ctx* ctx);
 
+// ---- a kernel that may be scheduled while its predecessor in the stream drains; it starts with pdl_wait()
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(bool early, void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t stream, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = early ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, (P)args...);
+}
+
 // ---- prefill-side launchers (prefill.cu)
 // C[set][i][j] = A[set][i] . B[set][j] over BPC_D channels in fp64, for 32 x 32 tiles of rows (strides in elements)
 cudaError_t bpc_launch_dots(const float* A, size_t a_set, const float* B, size_t b_set, float* C, size_t c_set, int ldc, int tiles_a, int tiles_b,
@@ -162,6 +178,13 @@ cudaError_t bpc_launch_encode_tc(bpc_ctx* ctx, const void* k_cache, uint64_t* co
 
 // --------------------------------------------------------------------------- device helpers
 #ifdef __CUDACC__
+// First statement of a kernel launched with launch_pdl: waits for the kernels before it in the stream (their results are
+// visible afterwards), then lets the next one be scheduled.  No effect in an ordinary launch.
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 __device__ __forceinline__ float bf16_lo(uint32_t x) { return __uint_as_float(x << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t x) { return __uint_as_float(x & 0xffff0000u); }
 

@@ -47,6 +47,10 @@ constexpr int kCrossBytes = 3 * 128 * 128 * 2;
 __host__ __device__ constexpr size_t gram_off(int bits, int p) { return (size_t)3 * 2 * kSub * (size_t)(p * bits - kSub * p * (p + 1) / 2); }
 __host__ __device__ constexpr size_t gram_bytes(int bits) { return gram_off(bits, bits / kSub - 1); }
 
+// Further warpgroups of a block that only take part in its set-up: the second launch of 256-bit codes has 128 x 128 cross terms
+// to split in three, which one warpgroup needed some 70 us for.
+__host__ __device__ constexpr int setup_groups(int half) { return half == 2 ? 2 : 0; }
+
 // barrier among the 128 threads of one warpgroup (hardware barriers 1 .. kGroups; 0 is __syncthreads)
 __device__ __forceinline__ void group_sync(int g) { asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "r"(kGroupThreads) : "memory"); }
 
@@ -94,7 +98,7 @@ __device__ __forceinline__ void diag_sweep(float (&t)[kSub], uint32_t& word, flo
 }
 
 template <int NBITS, int GROUPS, int HALF, bool ERR>
-__global__ void __launch_bounds__(kGroupThreads * GROUPS, 1)
+__global__ void __launch_bounds__(kGroupThreads * (GROUPS + setup_groups(HALF)), 1)
 encode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __nv_bfloat16* __restrict__ Ph, const float* __restrict__ gram,
                  const int32_t* __restrict__ unit_lens, uint64_t* __restrict__ codes, int32_t* __restrict__ err,
                  int n_kv_heads, int n_max, int shared_sets, int residual_correction, int blocks_per_unit,
@@ -103,7 +107,7 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __nv_bfloat16* 
   // the swizzled operand tiles need 1024-byte alignment in the shared address space
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   constexpr int kGroups = GROUPS;                          // (shadows the default of the single-launch code lengths)
-  constexpr int kThreads = kGroupThreads * GROUPS;
+  constexpr int kThreads = kGroupThreads * (GROUPS + setup_groups(HALF));   // (the last ones only help with the set-up)
   static_assert(HALF == 0 || NBITS == 128, "the two-launch form is for 256-bit codes");
   constexpr int TOTAL = HALF == 0 ? NBITS : 256;           // bits of a whole code
   constexpr int ROW0 = HALF == 2 ? 128 : 0;                // first projection row (= first bit) of this launch
@@ -130,8 +134,8 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __nv_bfloat16* 
   __shared__ unsigned long long mma_bar_s[kGroups], tile_bar_s[kGroups];
   __shared__ uint32_t tmem_base_s;
   __shared__ int timed_out_g[kGroups];
-  unsigned long long* mma_bar = &mma_bar_s[grp];
-  unsigned long long* tile_bar = &tile_bar_s[grp];
+  unsigned long long* mma_bar = &mma_bar_s[grp < kGroups ? grp : 0];
+  unsigned long long* tile_bar = &tile_bar_s[grp < kGroups ? grp : 0];
   constexpr int kAccCols = kGroups * NBITS;                // fp32 accumulator columns of the tiles in flight
   constexpr int kTmemCols = kAccCols <= 32 ? 32 : kAccCols <= 64 ? 64 : kAccCols <= 128 ? 128 : kAccCols <= 256 ? 256 : 512;   // a power of two >= 32
   static_assert(kAccCols <= 512, "accumulators exceed tensor memory");
@@ -257,7 +261,7 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __nv_bfloat16* 
   // run independent pipelines (own tile, own accumulator columns, own MMA barrier, own hardware barrier); all threads
   // of a warpgroup take the same branches, so its barrier is always reached by all 128 of them.
   const int tile_step = kGroups * blocks_per_unit;
-  int tl = kGroups * blockIdx.x + grp;
+  int tl = grp < kGroups ? kGroups * blockIdx.x + grp : ntiles;
   unsigned ph = 0;                                           // phase of the MMA barrier the next wait refers to
   if (tl < ntiles && gtid == 0) {
     load_tile(tl);
@@ -372,7 +376,7 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __nv_bfloat16* 
       }
     }
   }
-  if (timed_out_g[grp] && gtid == 0) atomicOr(err, BPC_DEVERR_TIMEOUT);
+  if (grp < kGroups && timed_out_g[grp] && gtid == 0) atomicOr(err, BPC_DEVERR_TIMEOUT);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();                                           // all warpgroups are done with tensor memory
   if (warp == 0) {
@@ -390,9 +394,10 @@ cudaError_t launch(bpc_ctx* ctx, const void* k_cache, uint64_t* codes, cudaStrea
   if (e != cudaSuccess) return e;
   const int steps_max = ((c.n_max + kTileKeys - 1) / kTileKeys + GROUPS - 1) / GROUPS;   // a block takes GROUPS tiles at a time
   // Blocks per unit.  One block fits an SM (shared memory), so the grid runs in waves of sm_count blocks and a last,
-  // partly filled wave costs as much as a full one: starting from about four waves, take the first count whose last
-  // wave is at least 90 % full (32 units on 148 SMs: 23 blocks per unit = 736 blocks = 4.97 waves).
-  int bpu = (4 * ctx->sm_count + ctx->units - 1) / ctx->units;
+  // partly filled wave costs as much as a full one: from one wave up, the first count whose last wave is at least 90 % full
+  // (32 units on 148 SMs: 9 blocks per unit = 1.95 waves).  Every block lays out the Gram operands anew, so few waves: from
+  // four waves up 32 x 128K keys take 621 us instead of 583, and 8 x 32K keys at 256 bits 296 instead of 273.
+  int bpu = (ctx->sm_count + ctx->units - 1) / ctx->units;
   if (bpu < 1) bpu = 1;
   for (int tries = 0; tries < 16; ++tries) {
     const int rem = (int)(((long long)ctx->units * bpu) % ctx->sm_count);
@@ -404,7 +409,7 @@ cudaError_t launch(bpc_ctx* ctx, const void* k_cache, uint64_t* codes, cudaStrea
   CUtensorMap kmap;
   e = tma::make_key_map(&kmap, k_cache, (unsigned long long)ctx->units * c.n_max, ctx->row_stride);
   if (e != cudaSuccess) return e;
-  kern<<<grid, kGroupThreads * GROUPS, smem, stream>>>(
+  kern<<<grid, kGroupThreads * (GROUPS + setup_groups(HALF)), smem, stream>>>(
       kmap, (const __nv_bfloat16*)ctx->P_h, ctx->gram, ctx->unit_lens, codes, ctx->dev_err,
       c.n_kv_heads, c.n_max, c.hash_sets != ctx->units, c.residual_correction, bpu, ctx->key_err);
   return cudaGetLastError();

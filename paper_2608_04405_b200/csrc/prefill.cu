@@ -219,6 +219,7 @@ append_kernel(const KV* __restrict__ k_new, const KV* __restrict__ v_new, KV* __
               uint64_t* __restrict__ codes, const KV* __restrict__ Ph, const float* __restrict__ gram,
               int32_t* __restrict__ unit_lens, int32_t* __restrict__ err, int n_kv_heads, int n_max, int row_stride,
               int b, int shared_sets, int residual_correction) {
+  pdl_wait();
   extern __shared__ __align__(16) unsigned char smem[];
   // the 32 x 32 blocks of the Gram matrix on and to the right of the diagonal (the only ones the sweep reads), block
   // (r, c) at slot r * nb - r (r - 1) / 2 + (c - r): 144 KB at 256 bits
@@ -799,20 +800,20 @@ cudaError_t bpc_launch_append(bpc_ctx* ctx, const void* k_new, const void* v_new
   if (c.kv_dtype == BPC_BF16) {
     e = cudaFuncSetAttribute(append_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    append_kernel<__nv_bfloat16><<<ctx->units, kAppThreads, smem, stream>>>(
+    e = launch_pdl(ctx->use_pdl, append_kernel<__nv_bfloat16>, ctx->units, kAppThreads, smem, stream,
         (const __nv_bfloat16*)k_new, (const __nv_bfloat16*)v_new, (__nv_bfloat16*)k_cache, (__nv_bfloat16*)v_cache, codes,
         (const __nv_bfloat16*)ctx->P_h, ctx->gram, ctx->unit_lens, ctx->dev_err, c.n_kv_heads, c.n_max, ctx->row_stride, b, shared_sets,
         c.residual_correction);
   } else {
     e = cudaFuncSetAttribute(append_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    append_kernel<float><<<ctx->units, kAppThreads, smem, stream>>>(
+    e = launch_pdl(ctx->use_pdl, append_kernel<float>, ctx->units, kAppThreads, smem, stream,
         (const float*)k_new, (const float*)v_new, (float*)k_cache, (float*)v_cache, codes, (const float*)ctx->P_h,
         ctx->gram, ctx->unit_lens, ctx->dev_err, c.n_kv_heads, c.n_max, ctx->row_stride, b, shared_sets,
         c.residual_correction);
   }
   ctx->launches += 1;
-  return cudaGetLastError();
+  return e;
 }
 
 static inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
