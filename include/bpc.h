@@ -120,7 +120,8 @@ bpc_status bpc_get_seq_lens(bpc_ctx* ctx, int32_t* host_lens_out);
  * its Gram matrix in the context.  With cfg.fit_power_iters = n > 0 the binary component comes from the power
  * iteration the same section starts from, u = sign((R R^T)^n R v*^T) = sign(R (R^T R)^n v*^T): the head_dim x head_dim
  * matrix R^T R is formed once (one extra pass over the keys) and then follows the residual by the rank-one change
- * -N v^T v per iteration, so the passes over R stay one per bit. */
+ * -N v^T v per iteration, so the passes over R stay one per bit; without it
+ * the keys are read twice per 32 bits. */
 bpc_status bpc_fit(bpc_ctx* ctx, const void* k_cache, const float* v_star,
                    void* workspace, size_t workspace_bytes, void* stream);
 
@@ -279,8 +280,9 @@ bpc_status bpc_debug_set_work_item_trace(bpc_ctx* ctx, uint64_t* trace);
  * context, number of kernels this context has launched so far.
  * Diagnostic switches (explicit calls; the library reads no environment variable): bpc_debug_set_pdl(ctx, 0) launches
  * the decode kernel without programmatic dependent launch; bpc_debug_set_tensor_core_encode(ctx, 0) makes
- * bpc_encode_keys and the passes of bpc_fit take the CUDA-core kernels instead of the tensor-core ones; bpc_debug_force_streaming(ctx, 1) selects the streaming selection at any
- * context length (Hamming scores without the safeguard only) and re-plans the launch geometry;
+ * bpc_encode_keys and bpc_fit take the CUDA-core kernels instead of the tensor-core ones (bpc_fit then makes one pass
+ * over the keys per bit); bpc_debug_force_streaming(ctx, 1) selects the streaming selection at any context length
+ * (Hamming scores without the safeguard only) and re-plans the launch geometry;
  * bpc_debug_force_key_shift(ctx, s) with s in 0..2 stores weighted score keys shifted right by at least s bits (the
  * library does that by itself only when a query's largest possible score exceeds 16 bits), so that the exact
  * re-scoring of the keys at the threshold can be exercised at any shape. */
