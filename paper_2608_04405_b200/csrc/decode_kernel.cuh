@@ -370,6 +370,28 @@ __device__ __noinline__ int rescore_key(const uint32_t* code, const uint32_t* si
   return score_key<W32, NP>(h, sg, mk);
 }
 
+// The sign sweep of the appended key once more where a decision value came out as NaN: that is bit 0 (not >= 0), which the sign
+// bit does not show, so one bit at a time by comparison.
+template <int W32>
+__device__ __noinline__ void careful_sweep(const double* t0, const float* gram, uint32_t* newcode, uint32_t* code_dst) {
+  const int lane = threadIdx.x & 31;
+  float t[W32];
+#pragma unroll
+  for (int c = 0; c < W32; ++c) t[c] = (float)t0[32 * c + lane];
+#pragma unroll
+  for (int w = 0; w < W32; ++w) {
+    uint32_t word = 0u;
+#pragma unroll 1
+    for (int i = 0; i < 32; ++i) {
+      const bool pos = __shfl_sync(0xffffffffu, t[w], i) >= 0.f;
+      word |= (pos ? 1u : 0u) << i;
+#pragma unroll
+      for (int c = w; c < W32; ++c) t[c] = fmaf(pos ? -1.f : 1.f, gram[(size_t)(32 * w + i) * (32 * W32) + 32 * c + lane], t[c]);
+    }
+    if (lane == 0) { newcode[w] = word; code_dst[w] = word; }
+  }
+}
+
 // VAR selects what is compiled in besides the plain path (VAR = 0): 1 = the error-aware safeguard (a static
 // hard-to-hash set that is always attended); 2 = the streaming selection for units whose scores do not fit the
 // cluster's shared memory (no score is stored: the scan keeps one histogram per warp over that warp's contiguous key
@@ -946,6 +968,7 @@ bpc_decode_kernel(const DecodeParams p) {
                      : "=r"(there) : "r"((unsigned)__cvta_generic_to_shared(&st->gram_bar)) : "memory");
       if (!there && lane == 0) atomicOr(p.err, BPC_DEVERR_TIMEOUT);
     }
+    bool nan = false;                                          // a decision value was NaN (it stays one)
     if constexpr (kQuiet) {
       constexpr int NB = W32;                                  // 32-bit column blocks
       float t[NB];
@@ -1010,6 +1033,8 @@ bpc_decode_kernel(const DecodeParams p) {
       }
       };
       if (c1 - c0 < kUnrolledSweepKeys) sweep(std::true_type()); else sweep(std::false_type());
+#pragma unroll
+      for (int c = 0; c < NB; ++c) nan = nan || t[c] != t[c];
     } else {
       // Lane l holds the W32 columns W32 l .. W32 l + W32 - 1, so its part of a Gram row is one or two vector reads.  Group g
       // of W32 bits is decided inside lane g (whose part of the group's rows is the diagonal block; the other lanes run the
@@ -1096,7 +1121,10 @@ bpc_decode_kernel(const DecodeParams p) {
           group(row[0], g);
         }
       }
+#pragma unroll
+      for (int e = 0; e < W32; ++e) nan = nan || t[e] != t[e];
     }
+    if (rc && __any_sync(0xffffffffu, nan)) careful_sweep<W32>(pd + GP * B, Gs, st->newcode, code_dst);
     if (p.dbg_times != nullptr && lane == 0) p.dbg_times[(size_t)blockIdx.x * 16 + 11] = (unsigned long long)clock64();
     if (kDefer) store_rows();
     if (deferred) {

@@ -64,7 +64,7 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&t)[kSub]) {
         "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr) : "memory");
 #pragma unroll
-  for (int i = 0; i < kSub; ++i) t[i] = __uint_as_float(r[i]) + 0.f;         // (-0 becomes 0)
+  for (int i = 0; i < kSub; ++i) t[i] = __uint_as_float(r[i]) + 0.f;   // (-0 becomes 0)
 }
 __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8]) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};\n\ttcgen05.wait::st.sync.aligned;"
@@ -73,11 +73,12 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8])
 
 // Greedy sweep of one 16-bit column block held in registers (every index a compile-time constant).  On entry t already
 // carries the corrections of all earlier blocks (no value is -0); on exit bit I of `word` is 1 where decision I came out
-// positive or zero.
+// positive or zero.  A NaN is not >= 0: the addition carries the canonical NaN, and nothing else, over into the sign bit
+// (comparisons instead cost 1 % of the encode, NaN replaced on the way out of tensor memory 7 %).
 template <int I, bool ERR>
 __device__ __forceinline__ void diag_sweep(float (&t)[kSub], uint32_t& word, float& abs_sum, const float* g_diag) {
   if constexpr (I < kSub) {
-    const uint32_t v = __float_as_uint(t[I]);
+    const uint32_t v = __float_as_uint(t[I]) + 0x007FFFFFu;
     word = __funnelshift_l(v, word, 1);                        // collects the sign bits, first decision on top
     if (ERR) abs_sum += fabsf(t[I]);
     const float nu = __uint_as_float((v & 0x80000000u) ^ 0xBF800000u);       // -u
@@ -331,7 +332,7 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __nv_bfloat16* 
         diag_sweep<0, ERR>(t, word, abs_sum, gd_s + (size_t)cb * kSub * kSub);
       } else {
 #pragma unroll
-        for (int i = 0; i < kSub; ++i) word |= ((__float_as_uint(t[i]) >> 31) ^ 1u) << i;
+        for (int i = 0; i < kSub; ++i) word |= (((__float_as_uint(t[i]) + 0x007FFFFFu) >> 31) ^ 1u) << i;
       }
       if (cb & 1) words[cb / 2] |= word << 16;
       else words[cb / 2] = word;

@@ -110,3 +110,61 @@ def test_projection_update_between_steps():
     assert not torch.equal(want[0], want[1])
     for i, o in enumerate(got):
         assert torch.equal(o, want[(i // 2) % 2])
+
+
+def _codes_of(sess, call, k, v, row):
+    """Codes of unit 0's row after one bpc_append ("append") or one fused step ("step") that brings k[:, :, row] at position 900."""
+    H = _harness()
+    sess.ctx.set_seq_lens([900])
+    kc, vc, codes = k.clone(), v.clone(), sess.codes.clone()
+    kn, vn = k[:, :, row].contiguous(), v[:, :, row].contiguous()
+    if call == "append":
+        sess.ctx.append(kn, vn, kc, vc, codes)
+    else:
+        sess.ctx.append_decode_attn(kn, vn, kc, vc, codes, torch.ones(1, sess.spec.n_q_heads, 128, dtype=k.dtype, device="cuda"), budget_ppm=20000)
+    torch.cuda.synchronize()
+    return H.codes_to_bits(codes[0, 0, 900:901], sess.spec.code_bits)[0]
+
+
+@pytest.mark.parametrize("dtype,bits,group,score_mode,cluster", [
+    ("bf16", 32, 1, 0, 0), ("bf16", 64, 4, 0, 2), ("bf16", 128, 4, 0, 1), ("bf16", 128, 8, 0, 2), ("bf16", 256, 4, 0, 2),
+    ("bf16", 128, 4, 1, 2), ("f32", 64, 1, 0, 1), ("f32", 256, 2, 1, 0)])
+def test_decisions_that_are_not_numbers(dtype, bits, group, score_mode, cluster):
+    """A bit is 1 where the decision value is >= 0, so a NaN decision is 0: keys with a NaN, an infinity or both infinities, and a
+    projection with a NaN in one row, coded alike by encode, append and the fused step (none of these decisions is close)."""
+    import numpy as np
+    from oracle import bpc_oracle as O
+    H = _harness()
+    spec = CONFIGS[1].scaled(name="nan", wid=86, dtype=dtype, n_ctx=1000, n_kv_heads=2, n_q_heads=2 * group, code_bits=bits, steps=1)
+    sess = H.Session(spec, score_mode=score_mode, cluster_size=cluster)
+    sess.fit()
+    sess.encode()
+    k, v = sess.k_cache.clone(), sess.v_cache
+    inf = float("inf")
+    for row, put in ((5, {7: float("nan")}), (6, {7: inf}), (7, {7: inf, 9: -inf}), (8, {3: -inf})):
+        for c, x in put.items():
+            k[0, 0, row, c] = x
+    Pbad = sess.P.clone()
+    Pbad[0, 21, 3] = float("nan")
+    Pbad[0, 21] *= -1.0                                      # (the decisions before it are those of the good projection)
+    for P, rows in ((sess.P, (5, 6, 7, 8)), (Pbad, (20,))):
+        sess.ctx.set_projection(P)
+        sess.ctx.set_seq_lens([1000])
+        sess.ctx.encode_keys(k, sess.codes)
+        torch.cuda.synchronize()
+        with np.errstate(invalid="ignore"):
+            want, _ = O.encode(H._np64(k[0, 0, list(rows)]), H._np64(sess.ctx.get_projection()[1][0]))
+        got = H.codes_to_bits(sess.codes[0, 0, list(rows)], bits)
+        assert np.array_equal(got, want)
+        for i, row in enumerate(rows):
+            for call in ("append", "step"):
+                assert np.array_equal(_codes_of(sess, call, k, v, row), want[i]), (call, row)
+    assert sess.ctx.last_device_error() == 0
+    sess.ctx = H.B.Context(H.B.make_config(1, spec.n_q_heads, 2, sess.w.n_max, bits, spec.torch_dtype, score_mode=score_mode,
+                                           residual_correction=False))   # plain signs
+    sess.ctx.set_projection(sess.P)
+    sess.ctx.set_seq_lens([1000])
+    sess.ctx.encode_keys(k, sess.codes)
+    torch.cuda.synchronize()
+    assert not H.codes_to_bits(sess.codes[0, 0, 5:6], bits).any()
+    assert not _codes_of(sess, "append", k, v, 5).any() and not _codes_of(sess, "step", k, v, 5).any()
