@@ -49,17 +49,22 @@ struct SmallState {
   uint32_t mask[kMaxPlanes][8];
   uint32_t gt[BPC_MAX_CLUSTER];
   uint32_t eq[BPC_MAX_CLUSTER];
-  uint32_t wgt[32], weq[32];             // streaming selection: per-warp numbers of keys above / at the threshold
+  union {
+    struct { uint32_t wgt[32], weq[32]; };                   // streaming selection: per-warp numbers of keys above / at the threshold
+    struct {                                                 // deferred selection:
+      unsigned long long gram_bar, new_bar;                  // mbarriers: the Gram matrix is in shared memory; the appended key's score is here
+      int newkey, above_low, low, mine;                      // that score; what the threshold search found for this block without it
+    };
+  };
   uint32_t wscan[64];                    // block scans: two alternating buffers of 2 x 16 warp totals (16-byte aligned)
   double pmax[BPC_MAX_GROUP];
-  unsigned long long gram_bar;           // mbarrier: the appending block's Gram matrix is in shared memory (deferred selection)
   int T, cnt_gt, my_take, my_base, rsum, e0, e1, pad;
   uint32_t newcode[8];                   // code of the key appended by this launch
-  unsigned long long new_bar;            // mbarrier: the appended key's score has arrived (deferred selection)
-  int newkey, above_low, low, mine;      // ... that score; what the threshold search found for this block without it
   int32_t eas_s[kEasLocal];              // this block's slice of the safeguard set (when it fits)
   uint8_t stage_valid[32][4];            // per warp and gather stage: which of the 8 rows are real
 };
+// (what is added here is taken from the score keys a block holds, and so from the longest context)
+static_assert(sizeof(SmallState) == 5344, "");
 
 // 256-bit Gram matrix in shared memory: 32 x 32 blocks on and right of the diagonal, padded to spread the banks; byte offset
 // of (row, column) inside the set

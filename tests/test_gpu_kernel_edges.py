@@ -168,3 +168,12 @@ def test_decisions_that_are_not_numbers(dtype, bits, group, score_mode, cluster)
     torch.cuda.synchronize()
     assert not H.codes_to_bits(sess.codes[0, 0, 5:6], bits).any()
     assert not _codes_of(sess, "append", k, v, 5).any() and not _codes_of(sess, "step", k, v, 5).any()
+
+
+@pytest.mark.parametrize("dtype,bits,group,keys", [("bf16", 128, 1, 81152), ("bf16", 64, 2, 80896), ("f32", 128, 2, 79744)])
+def test_longest_weighted_context(dtype, bits, group, keys):
+    """Weighted scores are kept by a cluster of 16 blocks whose shared memory holds `keys` 16-bit scores each next to the kernel's
+    other arrays: 232 448 bytes less the fixed part, in steps of 64 keys."""
+    H = _harness()
+    ctx = H.B.Context(H.B.make_config(1, group, 1, 1024, bits, torch.bfloat16 if dtype == "bf16" else torch.float32, score_mode=1))
+    assert ctx.max_context() == 16 * keys
