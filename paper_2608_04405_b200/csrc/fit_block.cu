@@ -260,7 +260,8 @@ fit_project_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* 
 }
 
 // --------------------------------------------------------------------------- project (CUDA cores, fp32 caches)
-// One thread per key: dot products in fp32 over 16 channels (or 32 earlier bits) at a time, added in fp64.
+// One thread per key.  Both sums run in fp64 and are rounded once, on their way to the column (sums of 16 channels and of 32
+// earlier bits in fp32 left the decisions less precise than one pass per bit has them).
 __global__ void __launch_bounds__(kTileKeys)
 fit_project_f32_kernel(const float* __restrict__ k_cache, const uint32_t* __restrict__ hfit, const float* __restrict__ v_star,
                        const float* __restrict__ cross, float* __restrict__ T, const int32_t* __restrict__ unit_lens,
@@ -270,41 +271,31 @@ fit_project_f32_kernel(const float* __restrict__ k_cache, const uint32_t* __rest
   const int row = blockIdx.x * kTileKeys + tid;
   if (blockIdx.x * kTileKeys >= (n + kSweepGroup - 1) / kSweepGroup * kSweepGroup) return;   // (zeros up to a whole sweep group)
   const bool live = row < n;
-  __shared__ __align__(16) float d_s[BPC_D][kBits];                    // directions, channel-major; then the scalars of 32 bits
+  __shared__ __align__(16) double d_s[BPC_D][kBits];                   // directions, channel-major; then the scalars of 32 bits
   double acc[kBits];
 #pragma unroll
   for (int l = 0; l < kBits; ++l) acc[l] = 0.0;
-  for (int c = tid; c < kBits * BPC_D; c += kTileKeys) d_s[c & 127][c >> 7] = v_star[((size_t)unit * b + kBits * blk + (c >> 7)) * BPC_D + (c & 127)];
+  for (int c = tid; c < kBits * BPC_D; c += kTileKeys) d_s[c & 127][c >> 7] = (double)v_star[((size_t)unit * b + kBits * blk + (c >> 7)) * BPC_D + (c & 127)];
   __syncthreads();
   const float4* kr = reinterpret_cast<const float4*>(k_cache + ((size_t)unit * n_max + (live ? row : 0)) * row_stride);
-  for (int c0 = 0; c0 < BPC_D; c0 += 16) {
-    float x[16], p[kBits];
+  for (int c0 = 0; c0 < BPC_D; c0 += 4) {
+    const float4 q = kr[c0 / 4];
+    const double x[4] = {(double)q.x, (double)q.y, (double)q.z, (double)q.w};
 #pragma unroll
-    for (int v = 0; v < 4; ++v) { const float4 q = kr[c0 / 4 + v]; x[4 * v] = q.x; x[4 * v + 1] = q.y; x[4 * v + 2] = q.z; x[4 * v + 3] = q.w; }
+    for (int c = 0; c < 4; ++c)
 #pragma unroll
-    for (int l = 0; l < kBits; ++l) p[l] = 0.f;
-#pragma unroll
-    for (int c = 0; c < 16; ++c)
-#pragma unroll
-      for (int l = 0; l < kBits; ++l) p[l] = fmaf(x[c], d_s[c0 + c][l], p[l]);
-#pragma unroll
-    for (int l = 0; l < kBits; ++l) acc[l] += (double)p[l];
+      for (int l = 0; l < kBits; ++l) acc[l] = fma(x[c], d_s[c0 + c][l], acc[l]);
   }
   for (int w = 0; w < blk; ++w) {
     __syncthreads();
-    for (int c = tid; c < kBits * kBits; c += kTileKeys) d_s[c >> 5][c & 31] = cross[((size_t)unit * b + 32 * w + (c >> 5)) * kBits + (c & 31)];
+    for (int c = tid; c < kBits * kBits; c += kTileKeys) d_s[c >> 5][c & 31] = (double)cross[((size_t)unit * b + 32 * w + (c >> 5)) * kBits + (c & 31)];
     __syncthreads();
     const uint32_t x = hfit[((size_t)unit * n_max + (live ? row : 0)) * (b / 32) + w];
-    float p[kBits];
-#pragma unroll
-    for (int l = 0; l < kBits; ++l) p[l] = 0.f;
     for (int j = 0; j < 32; ++j) {
-      const float u = ((x >> j) & 1u) ? 1.f : -1.f;
+      const double u = ((x >> j) & 1u) ? 1.0 : -1.0;
 #pragma unroll
-      for (int l = 0; l < kBits; ++l) p[l] = fmaf(u, d_s[j][l], p[l]);
+      for (int l = 0; l < kBits; ++l) acc[l] = fma(-u, d_s[j][l], acc[l]);
     }
-#pragma unroll
-    for (int l = 0; l < kBits; ++l) acc[l] -= (double)p[l];
   }
   float* dst = T + (size_t)unit * kBits * t_stride + row;
 #pragma unroll
@@ -317,11 +308,12 @@ fit_project_f32_kernel(const float* __restrict__ k_cache, const uint32_t* __rest
 // transposes its 32 keys' code words across lanes, one lane then writes one bit's 32 keys); then eight MMAs K_tile^T
 // (channel-major view of the tile, M = 128 channels) x U_blk (N = 32) and eight per 128 bits U x U_blk.  An A operand of 128
 // rows reaches past the R rows of U into whatever follows; those accumulator rows are not read.  Channel sums move to fp64
-// registers every kFlushTiles tiles (1024 rows); the inner products are integers below 2^24 and stay exact in fp32.
+// registers every kFlushTiles tiles (the tensor cores' fp32 sums lose with their length: 5.0e-8 of a row over 1024 keys, 3.0e-8
+// over 512; the pass per bit sums at least 384); the inner products are integers below 2^24 and stay exact in fp32.
 // A tile occupies its buffer from the start of its load to the end of its MMAs and the load is most of that, so as many
 // warpgroups with one buffer each as shared memory holds beat fewer with two (two groups of two buffers: 261 to 372 us at
 // 32 x 128K keys).
-constexpr int kFlushTiles = 8;
+constexpr int kFlushTiles = 3;
 
 template <int GROUPS>
 __global__ void __launch_bounds__(kGroupThreads * GROUPS, 1)
@@ -498,8 +490,10 @@ fit_gather_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* _
 }
 
 // --------------------------------------------------------------------------- gather (CUDA cores, fp32 caches)
-// Thread (half, channel) adds +-K over at most 1024 rows in fp32; the inner products come from ballots: lane i holds bit i of
+// Thread (half, channel) adds +-K over kGatherRows rows in fp32 and the sums in fp64; the inner products come from ballots: lane i holds bit i of
 // the block over a warp's 32 keys, every earlier bit's 32 keys are one broadcast word.
+constexpr int kGatherRows = 32;
+
 __global__ void __launch_bounds__(256)
 fit_gather_f32_kernel(const float* __restrict__ k_cache, const uint32_t* __restrict__ hfit, double* __restrict__ wpart,
                       int32_t* __restrict__ apart, const int32_t* __restrict__ unit_lens, int n_max, int row_stride, int b, int blk) {
@@ -516,11 +510,11 @@ fit_gather_f32_kernel(const float* __restrict__ k_cache, const uint32_t* __restr
 #pragma unroll
   for (int i = 0; i < kBits; ++i) acc64[i] = 0.0;
   const uint32_t* h = hfit + (size_t)unit * n_max * words;
-  for (int r0 = row0; r0 < row_end; r0 += 1024) {
+  for (int r0 = row0; r0 < row_end; r0 += 2 * kGatherRows) {
     float acc[kBits];
 #pragma unroll
     for (int i = 0; i < kBits; ++i) acc[i] = 0.f;
-    for (int r = r0 + half; r < min(row_end, r0 + 1024); r += 2) {
+    for (int r = r0 + half; r < min(row_end, r0 + 2 * kGatherRows); r += 2) {
       const float x = k_cache[((size_t)unit * n_max + r) * row_stride + c];
       const uint32_t w = h[(size_t)r * words + blk];
 #pragma unroll

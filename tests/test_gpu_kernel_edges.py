@@ -177,3 +177,27 @@ def test_longest_weighted_context(dtype, bits, group, keys):
     H = _harness()
     ctx = H.B.Context(H.B.make_config(1, group, 1, 1024, bits, torch.bfloat16 if dtype == "bf16" else torch.float32, score_mode=1))
     assert ctx.max_context() == 16 * keys
+
+
+@pytest.mark.parametrize("dtype,bits,n,batch,bound", [("f32", 128, 300, 2, 2.0 ** -23), ("bf16", 32, 8192, 37, 1.5 * 2.4e-8)])
+def test_fitted_rows_precision(dtype, bits, n, batch, bound):
+    """Rows of P against fp64 with the library's signs.  Rounding a row to fp32 costs 2^-23 / sqrt(12) / 1.44 = 2.4e-8 of its norm
+    on average; the sums over the keys may add half of that where rows keep their size.  With more bits than the keys need the
+    rows shrink against what is summed (measured 8.3e-8 in both forms of the fit): 2^-23 there."""
+    import numpy as np
+    H = _harness()
+    spec = CONFIGS[1].scaled(name="rows", wid=87, dtype=dtype, batch=batch, n_ctx=n, n_kv_heads=4, n_q_heads=4, code_bits=bits, steps=1)
+    sess = H.Session(spec, gen_device="cuda")
+    sess.fit()
+    err = ref = 0.0
+    for u in (0, 5):
+        bi, h, _ = sess.unit_views(u)
+        R = H._np64(sess.k_cache[bi, h, :n])
+        signs = 2.0 * sess.hfit_bits(u) - 1.0
+        P = H._np64(sess.P[u])
+        for i in range(bits):
+            v = signs[:, i] @ R / n
+            R -= np.outer(signs[:, i], v)
+            err += float(((P[i] - v) ** 2).sum())
+            ref += float((v ** 2).sum())
+    assert (err / ref) ** 0.5 <= bound, (err / ref) ** 0.5
