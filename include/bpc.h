@@ -287,6 +287,9 @@ bpc_status bpc_debug_set_work_item_trace(bpc_ctx* ctx, uint64_t* trace);
  * library does that by itself only when a query's largest possible score exceeds 16 bits), so that the exact
  * re-scoring of the keys at the threshold can be exercised at any shape. */
 bpc_status bpc_status_of_device_error(int32_t error_word);
+/* Tries after which the kernels of bpc_fit and of the fused step stop waiting for the other blocks of their cluster and raise
+ * bit 2 of the device error word (their result is then not valid); 0 gives up at once, -1 restores the default. */
+bpc_status bpc_debug_set_wait_limit(bpc_ctx* ctx, int32_t tries);
 bpc_status bpc_debug_set_pdl(bpc_ctx* ctx, int32_t on);
 bpc_status bpc_debug_force_key_shift(bpc_ctx* ctx, int32_t shift);
 bpc_status bpc_debug_set_tensor_core_encode(bpc_ctx* ctx, int32_t on);

@@ -280,6 +280,7 @@ bpc_status bpc_create(const bpc_config* cfg, bpc_ctx** out) {
   ctx->units = cfg->batch * cfg->n_kv_heads;
   ctx->group = cfg->n_q_heads / cfg->n_kv_heads;
   ctx->use_pdl = true;
+  ctx->wait_tries = BPC_WAIT_TRIES;
   ctx->row_stride = cfg->kv_row_stride == 0 ? cfg->head_dim : cfg->kv_row_stride;
   cudaError_t e = cudaGetDevice(&ctx->device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, ctx->device);
@@ -593,6 +594,7 @@ static bpc_status decode_common(bpc_ctx* ctx, const void* k_new, const void* v_n
   p.nbins = hist_bins(ctx);
   p.hist_shift = hist_shift(ctx);
   p.key_shift_min = ctx->key_shift_min;
+  p.wait_tries = ctx->wait_tries;
   p.early_projection = ctx->projection_settled && ctx->settled_stream == stream;
   if (ctx->streaming)
     e = c.kv_dtype == BPC_BF16 ? bpc_launch_decode_bf16_stream(ctx, p, (cudaStream_t)stream)
@@ -656,6 +658,12 @@ bpc_status bpc_debug_set_phase_timer(bpc_ctx* ctx, uint64_t* stamps) {
 bpc_status bpc_debug_set_pdl(bpc_ctx* ctx, int32_t on) {
   if (ctx == nullptr) return BPC_ERR_INVALID_ARG;
   ctx->use_pdl = on != 0;
+  return BPC_OK;
+}
+
+bpc_status bpc_debug_set_wait_limit(bpc_ctx* ctx, int32_t tries) {
+  if (ctx == nullptr || tries < -1) return BPC_ERR_INVALID_ARG;
+  ctx->wait_tries = tries < 0 ? BPC_WAIT_TRIES : tries;
   return BPC_OK;
 }
 

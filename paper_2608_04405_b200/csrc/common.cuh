@@ -14,6 +14,7 @@
 #define BPC_DEVERR_CHUNK_CAP   1   // a unit does not fit the cluster's score storage
 #define BPC_DEVERR_APPEND_CAP  2   // append at n_max
 #define BPC_DEVERR_TIMEOUT     4   // a bounded wait gave up
+#define BPC_WAIT_TRIES 20000000    // tries after which a wait inside a kernel gives up
 
 // In a launch that also appends, the block that codes the new key scans with fewer resources (one warp runs
 // Algorithm 2's sign sweep); it is given (16 - BPC_APPEND_LOSS16)/16 of the other blocks' key share.
@@ -37,6 +38,7 @@ struct bpc_ctx {
   bool fitted;
   bool projection_settled;  // a decode step has been launched since the projection was last written ...
   void* settled_stream;     // ... the last one on this stream
+  int wait_tries;           // tries after which waits for other blocks of a cluster give up
   bool use_pdl;             // launch the decode kernel with programmatic stream serialization
   bool streaming;           // the scores of a full unit do not fit the largest cluster: two-pass (streaming) selection
   float* P;                 // [hash_sets][b][D] float
@@ -125,6 +127,7 @@ struct DecodeParams {
   int chunk_cap;             // keys whose scores one thread block can hold
   int nbins;                 // histogram bins
   int hist_shift;            // histogram bin = stored score key >> hist_shift
+  int wait_tries;            // tries after which the wait for the appended key's score gives up
   int early_projection;      // the projection may be read before the programmatic dependency wait (see the kernel)
   int key_shift_min;         // weighted scores: smallest right shift of the stored 16-bit keys (diagnostic; normally 0)
 };

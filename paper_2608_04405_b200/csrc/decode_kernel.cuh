@@ -641,6 +641,7 @@ bpc_decode_kernel(const DecodeParams p) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], 4;" ::"r"(bar) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    st->newkey = -1;                                         // (below every threshold, should the wait for it give up)
     st->wscan[NW - 1] = st->wscan[16 + NW - 1] = 0u;         // (the appending warp adds nothing to the threshold search)
   }
   if (tid == 0) { st->rsum = 0; st->T = 0; st->cnt_gt = 0; st->my_take = 0; st->my_base = 0; st->e0 = 0; st->e1 = 0; }
@@ -968,7 +969,7 @@ bpc_decode_kernel(const DecodeParams p) {
     if (kDefer && gsm != nullptr) {
       int tries = 0;
       uint32_t there = 0u;
-      while (!there && tries++ < 20000000)
+      while (!there && tries++ < BPC_WAIT_TRIES)
         asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
                      : "=r"(there) : "r"((unsigned)__cvta_generic_to_shared(&st->gram_bar)) : "memory");
       if (!there && lane == 0) atomicOr(p.err, BPC_DEVERR_TIMEOUT);
@@ -1441,7 +1442,7 @@ bpc_decode_kernel(const DecodeParams p) {
     __syncthreads();                                         // the threshold is known, the appending warp is back
     int tries = 0;
     uint32_t there = 0u;
-    while (!there && tries++ < 20000000)
+    while (!there && tries++ < p.wait_tries)
       asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
                    : "=r"(there) : "r"((unsigned)__cvta_generic_to_shared(&st->new_bar)) : "memory");
     if (!there && tid == 0) atomicOr(p.err, BPC_DEVERR_TIMEOUT);

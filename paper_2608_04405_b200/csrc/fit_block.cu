@@ -755,8 +755,8 @@ __device__ __forceinline__ void mbar_expect(unsigned long long* bar, unsigned by
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
 }
 // bounded wait for a phase whose data other blocks of the cluster sent; false when the iteration budget runs out
-__device__ __forceinline__ bool mbar_wait_cluster(unsigned long long* bar, unsigned parity) {
-  for (int it = 0; it < 20000000; ++it) {
+__device__ __forceinline__ bool mbar_wait_cluster(unsigned long long* bar, unsigned parity, int tries) {
+  for (int it = 0; it < tries; ++it) {
     unsigned ok;
     asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
                  : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
@@ -779,7 +779,8 @@ __device__ __forceinline__ void send_b32(const void* dst, const void* bar, int r
 template <bool SMEM_WORDS, bool ONE>
 __global__ void __launch_bounds__(kSweepThreads, 1)
 fit_sweep_kernel(const float* __restrict__ T, uint32_t* __restrict__ hfit, uint32_t* __restrict__ words_g,
-                 const int32_t* __restrict__ unit_lens, int32_t* __restrict__ err, int n_max, int b, int blk, int t_stride, int cluster_size) {
+                 const int32_t* __restrict__ unit_lens, int32_t* __restrict__ err, int n_max, int b, int blk, int t_stride, int cluster_size,
+                 int wait_tries) {
   extern __shared__ __align__(16) unsigned char sweep_smem[];   // the copy ring, then (SMEM_WORDS) this block's code words
   __shared__ __align__(1024) float lut[4 * 256];           // lut[byte][pattern] = sum of +-c over the byte's bits
   __shared__ float nib[8 * 16];                            // the same by nibble
@@ -837,7 +838,11 @@ fit_sweep_kernel(const float* __restrict__ T, uint32_t* __restrict__ hfit, uint3
   in.request(in.ring);
   for (int j = 0; j < kBits; ++j) {
     SweepSums sums;
-    if (j == kBits - 1) { sweep_pass<8, true, ONE>(in, ws, rows, lut_a, j, nk, nkeys, warp, lane, sums); break; }
+    if (j == kBits - 1) {
+      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // (this block sends no more: see the end)
+      sweep_pass<8, true, ONE>(in, ws, rows, lut_a, j, nk, nkeys, warp, lane, sums);
+      break;
+    }
     prefetch(j + 2);
     switch (j >> 2) {
       case 0: sweep_pass<1, false, ONE>(in, ws, rows, lut_a, j, nk, nkeys, warp, lane, sums); break;
@@ -849,6 +854,7 @@ fit_sweep_kernel(const float* __restrict__ T, uint32_t* __restrict__ hfit, uint3
       case 6: sweep_pass<7, false, ONE>(in, ws, rows, lut_a, j, nk, nkeys, warp, lane, sums); break;
       default: sweep_pass<8, false, ONE>(in, ws, rows, lut_a, j, nk, nkeys, warp, lane, sums); break;
     }
+    int stop = timed_out;                                  // (last set between the previous bit's barriers)
     red_s[warp][lane] = sums.s;
     red_c[warp][lane] = sums.cnt;
     __syncthreads();
@@ -856,7 +862,10 @@ fit_sweep_kernel(const float* __restrict__ T, uint32_t* __restrict__ hfit, uint3
     const unsigned phase = (unsigned)(j >> 1) & 1u;
     // Exchange within the cluster: warps 0..3 send the block's sums, 4..7 its counts, each to every fourth rank; the sends
     // complete on the receiver's barrier of this parity (a rank sends bit j + 2 only after it has everybody's bit j + 1).
-    if (warp < 4) {
+    // A block that gave up a wait sends no more (its peers then miss its sums and give up in turn: every wait is bounded) and
+    // runs to the end on what it has.
+    if (stop) {
+    } else if (warp < 4) {
       double v[kSweepWarps];
 #pragma unroll
       for (int w = 0; w < kSweepWarps; ++w) v[w] = red_s[w][lane];
@@ -875,7 +884,7 @@ fit_sweep_kernel(const float* __restrict__ T, uint32_t* __restrict__ hfit, uint3
     // n c_{i,j+1} = u_i^T T - sum_{m<i} (u_i . u_m) c_{m,j+1}: c_i for i < j are rows of the triangle's inverse times the
     // sums, c_j follows from them (warp 0); the new bit's row of the inverse (warp 8) is needed one bit later.
     if (warp == 0 || warp == 8) {
-      if (!timed_out && !mbar_wait_cluster(&bar_s[buf], phase)) timed_out = 1;
+      if (!stop && !mbar_wait_cluster(&bar_s[buf], phase, wait_tries)) stop = timed_out = 1;
       int c = 0;
 #pragma unroll
       for (int r = 0; r < BPC_MAX_CLUSTER; ++r) c += r < cluster_size ? slot_c[buf][r][lane] : 0;
@@ -923,14 +932,20 @@ fit_sweep_kernel(const float* __restrict__ T, uint32_t* __restrict__ hfit, uint3
     for (int e = tid; e < 32 * (8 * (j >> 3) + 8); e += kSweepThreads)      // the bytes in play
       lut[e] = nib[32 * (e >> 8) + (e & 15)] + nib[32 * (e >> 8) + 16 + ((e >> 4) & 15)];
     if (warp == 8) inv_s[j][lane] = new_row;               // (warp 0 has read the inverse; it reads it again two barriers on)
-    if (tid == 0) mbar_expect(&bar_s[buf], (unsigned)cluster_size * 32u * 12u);   // arms the barrier for bit j + 2
+    if (tid == 0 && !stop) mbar_expect(&bar_s[buf], (unsigned)cluster_size * 32u * 12u);   // arms the barrier for bit j + 2
     __syncthreads();
   }
   cp_async_wait_all();
   __syncthreads();
   uint32_t* h = hfit + ((size_t)unit * n_max + row0) * (b / 32) + blk;
   for (int i = tid; i < nkeys; i += kSweepThreads) h[(size_t)i * (b / 32)] = ws[i];
-  if (timed_out && tid == 0) atomicOr(err, BPC_DEVERR_TIMEOUT);
+  // No block leaves while a peer may still send to it.  With all sums received nothing is under way; a block that gave up a wait
+  // leaves what was sent to it before this barrier the time to land (microseconds).
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (timed_out) {
+    if (tid == 0) atomicOr(err, BPC_DEVERR_TIMEOUT);
+    for (int i = 0; i < 100; ++i) __nanosleep(1000);
+  }
 }
 
 // --------------------------------------------------------------------------- rows and scalars
@@ -1176,7 +1191,8 @@ cudaError_t bpc_launch_fit_blocked(bpc_ctx* ctx, const void* k_cache, const floa
     const bool words_fit = sweep_smem <= kSweepMaxSmem, one = sweep_share(c.n_max, cs) <= kSweepWarps * kSweepGroup;
     cudaLaunchConfig_t cfg = sweep_config(&attr, ctx->units, cs, words_fit ? sweep_smem : kSweepRing, stream);
     auto sweep = !words_fit ? fit_sweep_kernel<false, false> : one ? fit_sweep_kernel<true, true> : fit_sweep_kernel<true, false>;
-    e = cudaLaunchKernelEx(&cfg, sweep, (const float*)T, hfit, words_g, (const int32_t*)ctx->unit_lens, ctx->dev_err, (int)c.n_max, b, blk, ts, cs);
+    e = cudaLaunchKernelEx(&cfg, sweep, (const float*)T, hfit, words_g, (const int32_t*)ctx->unit_lens, ctx->dev_err, (int)c.n_max, b, blk, ts, cs,
+                           ctx->wait_tries);
     if (e != cudaSuccess) return e;
     if (tc) {
       // as many warpgroups as their tile and sign buffers leave room for (four up to the third word, two from the sixth)

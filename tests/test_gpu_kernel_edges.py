@@ -201,3 +201,35 @@ def test_fitted_rows_precision(dtype, bits, n, batch, bound):
             err += float(((P[i] - v) ** 2).sum())
             ref += float((v ** 2).sum())
     assert (err / ref) ** 0.5 <= bound, (err / ref) ** 0.5
+
+
+@pytest.mark.parametrize("bits", [32, 128])
+def test_waits_that_give_up(bits):
+    """A wait for another block of the cluster that runs out of tries ends in the device error word, and the context works on: the fit
+    (all ranks of every cluster give up at the first bit) and the fused step (every block goes on without the new key's score)."""
+    H = _harness()
+    spec = CONFIGS[1].scaled(name="giveup", wid=88, n_ctx=30000, n_kv_heads=4, n_q_heads=16, code_bits=bits, steps=1)
+    sess = H.Session(spec, extra_rows=64)
+    sess.fit()
+    sess.encode()
+    good = sess.P.clone()
+    k_new, v_new = sess.w.new_kv(sess.lens)
+    q, _ = sess.w.queries(sess.lens)
+    args = (k_new.cuda(), v_new.cuda(), sess.k_cache, sess.v_cache, sess.codes, q.cuda())
+    want = sess.ctx.append_decode_attn(*args, budget_ppm=20000)
+    assert sess.ctx.last_device_error() == 0
+    for call in ("fit", "step"):
+        ctx = H.B.Context(sess.cfg)
+        ctx.set_seq_lens(sess.lens)
+        ctx.set_projection(good)
+        ctx.debug_set_wait_limit(0)
+        if call == "fit":
+            ctx.fit(sess.k_cache, sess.v_star, sess.fit_ws)
+        else:
+            ctx.append_decode_attn(*args, budget_ppm=20000)
+        assert ctx.last_device_error() == 4
+        ctx.debug_set_wait_limit(-1)
+        ctx.set_seq_lens(sess.lens)
+        ctx.fit(sess.k_cache, sess.v_star, sess.fit_ws)
+        assert torch.equal(ctx.get_projection()[0], good)
+        assert torch.equal(ctx.append_decode_attn(*args, budget_ppm=20000), want)
