@@ -1028,6 +1028,10 @@ constexpr int kSms = 148;
 constexpr size_t kSweepMaxSmem = 194 * 1024;               // dynamic shared memory of a sweep block: copy ring and code words
 
 constexpr size_t kMaxSmem = 226 * 1024;                    // dynamic shared memory a block may ask for next to its static part
+// The limit of a kernel belongs to the process: one value for every launch, whatever it needs, so that a thread's launch does
+// not fall between another's lower limit and that one's launch.
+template <typename K>
+cudaError_t allow_smem(K* kernel) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem); }
 // tiles, signs of 32 (blk + 1) bits, room for the last A operand (128 rows a half) to reach past its signs, and alignment
 inline size_t gather_smem(int groups, int blk) {
   return (size_t)groups * (kTileBytes + (size_t)kBits * (blk + 1) * kTileKeys * 2) + (size_t)(2048 * (blk / 4 + 1) - 512 * (blk + 1)) + 1024;
@@ -1064,11 +1068,11 @@ struct Layout {
 };
 
 // Resident sweep clusters by size on a device (the kernel takes a whole SM per block, so this depends on nothing else);
-// asked for once per device.
+// asked for until it succeeds, then kept.
 struct SweepLimits {
-  std::once_flag once;
+  std::mutex lock;
+  bool known;
   int active[BPC_MAX_CLUSTER + 1];
-  cudaError_t status;
 };
 SweepLimits g_sweep_limits[64];
 
@@ -1086,27 +1090,28 @@ cudaLaunchConfig_t sweep_config(cudaLaunchAttribute* attr, int units, int cs, si
   return cfg;
 }
 
-const SweepLimits* sweep_limits(int device) {
-  if (device < 0 || device >= 64) return nullptr;
+cudaError_t sweep_limits(int device, const SweepLimits** out) {
+  if (device < 0 || device >= 64) return cudaErrorInvalidDevice;
   SweepLimits* l = &g_sweep_limits[device];
-  std::call_once(l->once, [l]() {
-    cudaError_t e = cudaSuccess;
-    const void* kernels[3] = {(const void*)fit_sweep_kernel<true, true>, (const void*)fit_sweep_kernel<true, false>, (const void*)fit_sweep_kernel<false, false>};
-    for (const void* k : kernels) {
-      if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSweepMaxSmem);
-      if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  *out = l;
+  std::lock_guard<std::mutex> hold(l->lock);
+  if (l->known) return cudaSuccess;
+  const void* kernels[3] = {(const void*)fit_sweep_kernel<true, true>, (const void*)fit_sweep_kernel<true, false>, (const void*)fit_sweep_kernel<false, false>};
+  for (const void* k : kernels) {
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSweepMaxSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+  }
+  for (int cs = 1; cs <= BPC_MAX_CLUSTER; ++cs) {
+    cudaLaunchAttribute attr;
+    cudaLaunchConfig_t cfg = sweep_config(&attr, 1, cs, kSweepMaxSmem, nullptr);
+    if (cudaOccupancyMaxActiveClusters(&l->active[cs], fit_sweep_kernel<true, false>, &cfg) != cudaSuccess) {
+      (void)cudaGetLastError();
+      l->active[cs] = 0;
     }
-    for (int cs = 1; cs <= BPC_MAX_CLUSTER && e == cudaSuccess; ++cs) {
-      cudaLaunchAttribute attr;
-      cudaLaunchConfig_t cfg = sweep_config(&attr, 1, cs, kSweepMaxSmem, nullptr);
-      if (cudaOccupancyMaxActiveClusters(&l->active[cs], fit_sweep_kernel<true, false>, &cfg) != cudaSuccess) {
-        (void)cudaGetLastError();
-        l->active[cs] = 0;
-      }
-    }
-    l->status = e;
-  });
-  return l;
+    l->known = l->known || l->active[cs] > 0;
+  }
+  return l->known ? cudaSuccess : cudaErrorInvalidConfiguration;
 }
 
 // Cluster size of the sweep: the smallest estimate of waves x (rounds of 128 keys per warp + the exchange of a bit), in
@@ -1131,7 +1136,7 @@ cudaError_t launch_project_tc(const bpc_ctx* ctx, const CUtensorMap& kmap, const
                               int blk, int parts, int ts, cudaStream_t stream) {
   const bpc_config& c = ctx->cfg;
   const size_t smem = (size_t)GROUPS * (kTileBytes + kTileKeys * kSignCols * 2) + (size_t)kProjN * 256 + (size_t)blk * kProjN * 64 + 1024;
-  cudaError_t e = cudaFuncSetAttribute(fit_project_tc_kernel<GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(fit_project_tc_kernel<GROUPS>);
   if (e != cudaSuccess) return e;
   fit_project_tc_kernel<GROUPS><<<dim3(parts, ctx->units), kGroupThreads * GROUPS, smem, stream>>>(
       kmap, hfit, v_star, cross, T, ctx->unit_lens, ctx->dev_err, c.n_max, c.code_bits, blk, ts);
@@ -1143,7 +1148,7 @@ cudaError_t launch_gather_tc(const bpc_ctx* ctx, const CUtensorMap& kmap, const 
                              cudaStream_t stream) {
   const bpc_config& c = ctx->cfg;
   const size_t smem = gather_smem(GROUPS, blk);
-  cudaError_t e = cudaFuncSetAttribute(fit_gather_tc_kernel<GROUPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(fit_gather_tc_kernel<GROUPS>);
   if (e != cudaSuccess) return e;
   fit_gather_tc_kernel<GROUPS><<<dim3(parts, ctx->units), kGroupThreads * GROUPS, smem, stream>>>(
       kmap, hfit, wpart, apart, ctx->unit_lens, ctx->dev_err, c.n_max, c.code_bits, blk);
@@ -1164,14 +1169,15 @@ cudaError_t bpc_launch_fit_blocked(bpc_ctx* ctx, const void* k_cache, const floa
   int32_t* apart = (int32_t*)(ws + lay.apart);
   float* cross = (float*)(ws + lay.cross);
   const int ts = t_stride_of(&c), parts = parts_of(&c), b = c.code_bits;
-  const SweepLimits* lim = sweep_limits(ctx->device);
-  if (lim == nullptr || lim->status != cudaSuccess) return lim == nullptr ? cudaErrorInvalidDevice : lim->status;
+  const SweepLimits* lim = nullptr;
+  cudaError_t e = sweep_limits(ctx->device, &lim);
+  if (e != cudaSuccess) return e;
   const int cs = sweep_cluster(&c, lim);
   const size_t sweep_smem = kSweepRing + (size_t)sweep_share(c.n_max, cs) * 4;
   const bool tc = c.kv_dtype == BPC_BF16;
   const dim3 grid(parts, ctx->units);
   CUtensorMap kmap;
-  cudaError_t e = tc ? tma::make_key_map(&kmap, k_cache, (unsigned long long)ctx->units * c.n_max, ctx->row_stride) : cudaSuccess;
+  if (tc) e = tma::make_key_map(&kmap, k_cache, (unsigned long long)ctx->units * c.n_max, ctx->row_stride);
   for (int blk = 0; blk < b / kBits && e == cudaSuccess; ++blk) {
     if (blk > 0) {                                         // cross[j][l] = v_j . d_l for the bits so far and this block's columns
       const size_t set = (size_t)b * BPC_D;
@@ -1205,7 +1211,7 @@ cudaError_t bpc_launch_fit_blocked(bpc_ctx* ctx, const void* k_cache, const floa
     if (e != cudaSuccess) return e;
     fit_sum_parts_kernel<<<dim3(16 + 4 * (blk + 1), ctx->units), 256, 0, stream>>>(wpart, apart, ctx->unit_lens, c.n_max, b, blk, parts);
     const size_t rows_smem = (size_t)(kBits * kBits * (blk + 1) + kBits * blk * 32 + kBits * 32) * 8;
-    e = cudaFuncSetAttribute(fit_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rows_smem);
+    e = allow_smem(fit_rows_kernel);
     if (e != cudaSuccess) return e;
     fit_rows_kernel<<<dim3(4, ctx->units), 512, rows_smem, stream>>>(wpart, apart, ctx->P, ctx->unit_lens, c.n_max, b, blk, parts);
     e = cudaGetLastError();

@@ -795,17 +795,18 @@ cudaError_t bpc_launch_append(bpc_ctx* ctx, const void* k_new, const void* v_new
   const bpc_config& c = ctx->cfg;
   const int b = c.code_bits;
   const size_t smem = (size_t)(b / 32) * (b / 32 + 1) / 2 * 4096;   // Gram blocks on and right of the diagonal
+  const int smem_limit = 8 * 9 / 2 * 4096;                 // (for every code length: the limit is shared by all threads' contexts)
   const int shared_sets = c.hash_sets != ctx->units;
   cudaError_t e;
   if (c.kv_dtype == BPC_BF16) {
-    e = cudaFuncSetAttribute(append_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(append_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit);
     if (e != cudaSuccess) return e;
     e = launch_pdl(ctx->use_pdl, append_kernel<__nv_bfloat16>, ctx->units, kAppThreads, smem, stream,
         (const __nv_bfloat16*)k_new, (const __nv_bfloat16*)v_new, (__nv_bfloat16*)k_cache, (__nv_bfloat16*)v_cache, codes,
         (const __nv_bfloat16*)ctx->P_h, ctx->gram, ctx->unit_lens, ctx->dev_err, c.n_kv_heads, c.n_max, ctx->row_stride, b, shared_sets,
         c.residual_correction);
   } else {
-    e = cudaFuncSetAttribute(append_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(append_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit);
     if (e != cudaSuccess) return e;
     e = launch_pdl(ctx->use_pdl, append_kernel<float>, ctx->units, kAppThreads, smem, stream,
         (const float*)k_new, (const float*)v_new, (float*)k_cache, (float*)v_cache, codes, (const float*)ctx->P_h,

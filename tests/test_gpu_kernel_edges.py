@@ -233,3 +233,39 @@ def test_waits_that_give_up(bits):
         ctx.fit(sess.k_cache, sess.v_star, sess.fit_ws)
         assert torch.equal(ctx.get_projection()[0], good)
         assert torch.equal(ctx.append_decode_attn(*args, budget_ppm=20000), want)
+
+
+def test_fits_and_appends_of_several_threads():
+    """Contexts of several threads share the kernels' shared-memory limits, whatever code length and block of bits they are at."""
+    import threading
+    H = _harness()
+    jobs = []
+    for bits in (32, 64, 128, 256):
+        spec = CONFIGS[1].scaled(name="threads", wid=89, n_ctx=600, n_kv_heads=1, n_q_heads=1, code_bits=bits, steps=1)
+        sess = H.Session(spec, extra_rows=200)
+        sess.fit()
+        sess.encode()
+        jobs.append((sess, sess.P.clone()))
+    failed = []
+
+    def work(sess):
+        k_new, v_new = (x.cuda() for x in sess.w.new_kv(sess.lens))
+        with torch.cuda.stream(torch.cuda.Stream()):
+            try:
+                for _ in range(150):
+                    sess.ctx.fit(sess.k_cache, sess.v_star, sess.fit_ws)
+                    sess.ctx.append(k_new, v_new, sess.k_cache, sess.v_cache, sess.codes)
+                    sess.ctx.set_seq_lens(sess.lens)
+            except H.B.BpcError as e:
+                failed.append((sess.spec.code_bits, str(e)))
+            torch.cuda.current_stream().synchronize()
+
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=work, args=(sess,)) for sess, _ in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed, failed
+    for sess, P in jobs:
+        assert torch.equal(sess.ctx.get_projection()[0], P) and sess.ctx.last_device_error() == 0
