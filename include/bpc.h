@@ -291,6 +291,9 @@ bpc_status bpc_status_of_device_error(int32_t error_word);
  * bit 2 of the device error word (their result is then not valid); 0 gives up at once, -1 restores the default. */
 bpc_status bpc_debug_set_wait_limit(bpc_ctx* ctx, int32_t tries);
 bpc_status bpc_debug_set_pdl(bpc_ctx* ctx, int32_t on);
+/* 1 when the last decode step may have read the projection while the kernel before it on the stream was still running: the
+ * context's launch before it there was a decode step as well, and no call that writes the projection has been captured. */
+int32_t    bpc_step_read_early(bpc_ctx* ctx);
 bpc_status bpc_debug_force_key_shift(bpc_ctx* ctx, int32_t shift);
 bpc_status bpc_debug_set_tensor_core_encode(bpc_ctx* ctx, int32_t on);
 bpc_status bpc_debug_force_streaming(bpc_ctx* ctx, int32_t on);

@@ -63,6 +63,25 @@ bpc_status cuda_fail(bpc_ctx* ctx, cudaError_t e) {
   return BPC_ERR_CUDA;
 }
 
+// The capture that `stream` is part of (0: none), false when it cannot be told (a legacy stream beside another's capture).
+bool capture_of(void* stream, unsigned long long* id) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  *id = 0;
+  if (cudaStreamGetCaptureInfo((cudaStream_t)stream, &status, id) != cudaSuccess) { (void)cudaGetLastError(); return false; }
+  if (status == cudaStreamCaptureStatusNone) *id = 0;
+  return true;
+}
+
+// A decode step may read the projection ahead of its dependency wait if the launch before it on the stream that touches the
+// projection is a step too: what wrote the projection had completed before that step went past its own wait.  Calls only count
+// among calls of the same kind: a captured step has not run when the next call follows, and a captured write runs whenever its
+// graph does, with no call of the library (no step reads early any more then).
+void projection_written(bpc_ctx* ctx, void* stream) {
+  unsigned long long id = 0;
+  if (!capture_of(stream, &id) || id != 0) ctx->projection_captured = true;
+  ctx->projection_settled = false;
+}
+
 // Largest score key (sum of |A_j| after removing the common factor), the shift that maps keys to at most 2048
 // histogram bins, and the number of bins.
 int max_score_key(const bpc_ctx* ctx) {
@@ -402,7 +421,7 @@ bpc_status bpc_get_seq_lens(bpc_ctx* ctx, int32_t* host_out) {
 
 bpc_status bpc_set_projection(bpc_ctx* ctx, const float* P, void* stream) {
   if (ctx == nullptr || P == nullptr) return BPC_ERR_INVALID_ARG;
-  ctx->projection_settled = false;
+  projection_written(ctx, stream);
   const bpc_config& c = ctx->cfg;
   cudaError_t e = cudaMemcpyAsync(ctx->P, P, (size_t)c.hash_sets * c.code_bits * BPC_D * 4, cudaMemcpyDeviceToDevice,
                                   (cudaStream_t)stream);
@@ -433,7 +452,7 @@ bpc_status bpc_fit(bpc_ctx* ctx, const void* k_cache, const float* v_star, void*
   if (ctx->cfg.hash_sets != ctx->units) return BPC_ERR_UNSUPPORTED;
   if (workspace_bytes < bpc_fit_workspace_bytes_impl(&ctx->cfg)) return BPC_ERR_INVALID_ARG;
   int launches = 0;
-  ctx->projection_settled = false;
+  projection_written(ctx, stream);
   cudaError_t e = bpc_launch_fit(ctx, k_cache, v_star, workspace, (cudaStream_t)stream, &launches);
   ctx->launches += launches;
   if (e == cudaSuccess) e = bpc_launch_finalize_projection(ctx, (cudaStream_t)stream);
@@ -595,7 +614,10 @@ static bpc_status decode_common(bpc_ctx* ctx, const void* k_new, const void* v_n
   p.hist_shift = hist_shift(ctx);
   p.key_shift_min = ctx->key_shift_min;
   p.wait_tries = ctx->wait_tries;
-  p.early_projection = ctx->projection_settled && ctx->settled_stream == stream;
+  unsigned long long capture = 0;
+  const bool known = capture_of(stream, &capture);
+  p.early_projection = known && !ctx->projection_captured && ctx->projection_settled && ctx->settled_stream == stream &&
+                       ctx->settled_capture == capture;
   if (ctx->streaming)
     e = c.kv_dtype == BPC_BF16 ? bpc_launch_decode_bf16_stream(ctx, p, (cudaStream_t)stream)
                                : bpc_launch_decode_f32_stream(ctx, p, (cudaStream_t)stream);
@@ -615,8 +637,10 @@ static bpc_status decode_common(bpc_ctx* ctx, const void* k_new, const void* v_n
     e = c.kv_dtype == BPC_BF16 ? bpc_launch_decode_bf16(ctx, p, (cudaStream_t)stream)
                                : bpc_launch_decode_f32(ctx, p, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(ctx, e);
-  ctx->projection_settled = true;
+  ctx->projection_settled = known;
   ctx->settled_stream = stream;
+  ctx->settled_capture = capture;
+  ctx->read_early = p.early_projection != 0;
   ctx->launches += 1;
   return BPC_OK;
 }
@@ -701,6 +725,8 @@ bpc_status bpc_debug_force_byte_keys(bpc_ctx* ctx, int32_t mode) {
 }
 
 int32_t bpc_uses_byte_keys(bpc_ctx* ctx) { return (ctx != nullptr && ctx->byte_keys) ? 1 : 0; }
+
+int32_t bpc_step_read_early(bpc_ctx* ctx) { return (ctx != nullptr && ctx->read_early) ? 1 : 0; }
 
 bpc_status bpc_status_of_device_error(int32_t error_word) { return error_word == 0 ? BPC_OK : BPC_ERR_DEVICE; }
 

@@ -430,10 +430,10 @@ bpc_decode_kernel(const DecodeParams p) {
   const int kvh = unit % p.n_kv_heads;
   const int seq = unit / p.n_kv_heads;
 
-  // The rows of the projection are requested first of all.  Usually that is safe before the dependency wait below: if this
-  // context's previous launch was a decode step too (p.early_projection), whatever wrote the projection had completed before
-  // that step went past its own wait, and this grid starts after that.  Otherwise the kernel before this one in the stream may
-  // be the one that writes it (bpc_fit, bpc_set_projection).  Read at L2: this SM's L1 may hold lines from before.
+  // The rows of the projection are requested first of all, before the dependency wait below where p.early_projection says that
+  // whatever wrote them had completed before this grid could start.  That is work moved under the tail of the step before, and
+  // a gain only between adjacent steps: behind another kernel that does not release its dependents early nothing is running yet.
+  // Read at L2: this SM's L1 may hold lines from before.
   constexpr int HPARTS = NT / B;                 // slices per projection row in the query hash
   constexpr int HDS = BPC_D / HPARTS;            // channels per slice (a multiple of 8)
   constexpr int HV = HDS * (int)sizeof(KV) / 16; // 16-byte vectors per slice

@@ -269,3 +269,80 @@ def test_fits_and_appends_of_several_threads():
     assert not failed, failed
     for sess, P in jobs:
         assert torch.equal(sess.ctx.get_projection()[0], P) and sess.ctx.last_device_error() == 0
+
+
+@pytest.mark.parametrize("bits,n,cluster", [(128, 4000, 0), (128, 9000, 1), (256, 30000, 1)])   # short ranges; plain; 256 bits, plain
+def test_steps_around_captured_calls(bits, n, cluster):
+    """Which steps read the projection early, and that all of them use the projection of their moment: behind writes, on another
+    stream, around a captured step that has not run, and around replays of captured writes (fused and plain steps)."""
+    H = _harness()
+    spec = CONFIGS[1].scaled(name="captured", wid=90, n_ctx=n, n_kv_heads=2, n_q_heads=8, code_bits=bits, steps=1)
+    sess = H.Session(spec, cluster_size=cluster, extra_rows=64)
+    sess.fit()
+    P = [sess.P.clone(), torch.flip(sess.P, dims=[1]).neg().contiguous()]
+    sess.encode()
+    q = sess.w.queries(sess.lens)[0].cuda()
+    k_new, v_new = (x.cuda() for x in sess.w.new_kv(sess.lens))
+    ctx, early = sess.ctx, []
+    saved = [x.clone() for x in (sess.k_cache, sess.v_cache, sess.codes)]
+
+    def step(fused):
+        if fused:
+            out = ctx.append_decode_attn(k_new, v_new, sess.k_cache, sess.v_cache, sess.codes, q, budget_ppm=20000)
+        else:
+            out = ctx.decode_attn(q, sess.k_cache, sess.v_cache, sess.codes, budget_ppm=20000)
+        early.append(ctx.step_read_early())
+        return out
+
+    def sequence(write, wait):
+        """From the same caches: writes of the two projections in turn, each before a fused step, a plain one and another fused one."""
+        torch.cuda.synchronize()
+        for x, y in zip((sess.k_cache, sess.v_cache, sess.codes), saved):
+            x.copy_(y)
+        ctx.set_seq_lens(sess.lens)
+        torch.cuda.synchronize()
+        outs = []
+        for i in range(4):
+            write(i % 2)
+            for fused in (True, False, True):
+                wait()
+                outs.append(step(fused))
+        torch.cuda.synchronize()
+        return outs
+
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        want = sequence(lambda i: ctx.set_projection(P[i]), torch.cuda.synchronize)
+        got = sequence(lambda i: ctx.set_projection(P[i]), lambda: None)
+        assert early == 8 * [False, True, True]
+        assert not torch.equal(want[1], want[4])
+        assert all(torch.equal(a, b) for a, b in zip(want, got))
+        del early[:]
+        step(False)
+        with torch.cuda.stream(torch.cuda.Stream()):         # ordered, but not the stream of the step before
+            torch.cuda.current_stream().wait_stream(stream)
+            step(False)
+            stream.wait_stream(torch.cuda.current_stream())
+        assert early == [True, False]
+        del early[:]
+        ctx.set_projection(P[0])
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):         # the second captured step follows one of its own kind
+            out0, out1 = step(False), step(False)
+        step(False)                                          # no step has run since the write
+        step(False)
+        assert early == [False, True, False, True]
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(out0, out1)
+        graphs = []
+        for p in P:                                          # writes that run with no call: no early read from here on
+            graphs.append(torch.cuda.CUDAGraph())
+            with torch.cuda.graph(graphs[-1], stream=stream):
+                ctx.set_projection(p)
+        del early[:]
+        got = sequence(lambda i: graphs[i].replay(), lambda: None)
+        assert early == 12 * [False]
+        assert all(torch.equal(a, b) for a, b in zip(want, got))
+    assert ctx.last_device_error() == 0
