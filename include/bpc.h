@@ -98,6 +98,10 @@ bpc_status bpc_destroy(bpc_ctx* ctx);
  * and reads the codes twice (n_max up to 2^26); the weighted score mode and the safeguard keep the cluster limit. */
 size_t  bpc_codes_bytes(const bpc_config* host_cfg);
 size_t  bpc_fit_workspace_bytes(const bpc_config* host_cfg);
+/* The smallest workspace bpc_fit takes: the codes and the block sums of one pass over the keys per bit.  With less than
+ * bpc_fit_workspace_bytes the fit makes those passes instead of working on 32 bits at a time (32 x 128K keys, 128 bits: 0.07
+ * instead of 0.64 GB, 31 instead of 3.6 ms; the same signs up to rounding). */
+size_t  bpc_fit_workspace_min_bytes(const bpc_config* host_cfg);
 /* Byte offset inside the fit workspace at which bpc_fit leaves the codes H that Algorithm 1 itself
  * assigns to the fitted keys ([units][n_max][code_bits/64] uint64, same bit layout as `codes`).  They are a
  * diagnostic: the cache codes always come from Algorithm 2 (bpc_encode_keys). */
@@ -115,8 +119,8 @@ bpc_status bpc_get_seq_lens(bpc_ctx* ctx, int32_t* host_lens_out);
 /* Algorithm 1 (Section 3.2, "Binary Principal Components Finding"): for every unit, run code_bits
  * greedy iterations on its first seq_len keys of k_cache.  v_star [hash_sets][code_bits][head_dim]
  * float are the Gaussian directions the algorithm samples (supplied by the caller so that a run is
- * reproducible).  workspace must hold bpc_fit_workspace_bytes(cfg).  Requires hash_sets ==
- * batch*n_kv_heads.  Leaves P, P rounded to the cache precision (the hash function proper) and
+ * reproducible).  workspace must hold bpc_fit_workspace_bytes(cfg), or at least bpc_fit_workspace_min_bytes(cfg).
+ * Requires hash_sets == batch*n_kv_heads.  Leaves P, P rounded to the cache precision (the hash function proper) and
  * its Gram matrix in the context.  With cfg.fit_power_iters = n > 0 the binary component comes from the power
  * iteration the same section starts from, u = sign((R R^T)^n R v*^T) = sign(R (R^T R)^n v*^T): the head_dim x head_dim
  * matrix R^T R is formed once (one extra pass over the keys) and then follows the residual by the rank-one change

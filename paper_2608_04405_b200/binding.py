@@ -47,6 +47,7 @@ def _load() -> ctypes.CDLL:
         "bpc_destroy": (i32, [vp]),
         "bpc_codes_bytes": (sz, [cfgp]),
         "bpc_fit_workspace_bytes": (sz, [cfgp]),
+        "bpc_fit_workspace_min_bytes": (sz, [cfgp]),
         "bpc_fit_codes_offset": (sz, [cfgp]),
         "bpc_max_context": (i64, [cfgp]),
         "bpc_set_seq_lens": (i32, [vp, ctypes.POINTER(i32), vp]),
@@ -98,7 +99,7 @@ def _load() -> ctypes.CDLL:
 
 
 lib = _load()
-EXPORTS = ["bpc_create", "bpc_destroy", "bpc_codes_bytes", "bpc_fit_workspace_bytes", "bpc_fit_codes_offset",
+EXPORTS = ["bpc_create", "bpc_destroy", "bpc_codes_bytes", "bpc_fit_workspace_bytes", "bpc_fit_workspace_min_bytes", "bpc_fit_codes_offset",
            "bpc_max_context",
            "bpc_set_seq_lens", "bpc_get_seq_lens", "bpc_fit", "bpc_set_projection", "bpc_get_projection",
            "bpc_encode_keys", "bpc_build_eas", "bpc_get_eas", "bpc_eas_capacity", "bpc_exact_topk", "bpc_append", "bpc_decode_attn", "bpc_append_decode_attn", "bpc_decode_attn_static", "bpc_static_scratch_entries", "bpc_static_last_device_error",
@@ -188,6 +189,9 @@ class Context:
 
     def fit_workspace_bytes(self) -> int:
         return lib.bpc_fit_workspace_bytes(ctypes.byref(self.cfg))
+
+    def fit_workspace_min_bytes(self) -> int:
+        return lib.bpc_fit_workspace_min_bytes(ctypes.byref(self.cfg))
 
     def fit_codes_offset(self) -> int:
         return lib.bpc_fit_codes_offset(ctypes.byref(self.cfg))

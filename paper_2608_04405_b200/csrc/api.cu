@@ -269,6 +269,11 @@ size_t bpc_fit_workspace_bytes(const bpc_config* c) {
   return bpc_fit_workspace_bytes_impl(c);
 }
 
+size_t bpc_fit_workspace_min_bytes(const bpc_config* c) {
+  if (check_cfg(c) != BPC_OK) return 0;
+  return bpc_fit_workspace_min_bytes_impl(c);
+}
+
 size_t bpc_fit_codes_offset(const bpc_config* c) {
   if (check_cfg(c) != BPC_OK) return 0;
   return bpc_fit_codes_offset_impl(c);
@@ -450,10 +455,10 @@ bpc_status bpc_fit(bpc_ctx* ctx, const void* k_cache, const float* v_star, void*
   if (ctx == nullptr || k_cache == nullptr || v_star == nullptr || workspace == nullptr) return BPC_ERR_INVALID_ARG;
   if (!aligned16(k_cache) || !aligned16(v_star) || !aligned16(workspace)) return BPC_ERR_INVALID_ARG;
   if (ctx->cfg.hash_sets != ctx->units) return BPC_ERR_UNSUPPORTED;
-  if (workspace_bytes < bpc_fit_workspace_bytes_impl(&ctx->cfg)) return BPC_ERR_INVALID_ARG;
+  if (workspace_bytes < bpc_fit_workspace_min_bytes_impl(&ctx->cfg)) return BPC_ERR_INVALID_ARG;
   int launches = 0;
   projection_written(ctx, stream);
-  cudaError_t e = bpc_launch_fit(ctx, k_cache, v_star, workspace, (cudaStream_t)stream, &launches);
+  cudaError_t e = bpc_launch_fit(ctx, k_cache, v_star, workspace, workspace_bytes, (cudaStream_t)stream, &launches);
   ctx->launches += launches;
   if (e == cudaSuccess) e = bpc_launch_finalize_projection(ctx, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(ctx, e);

@@ -164,9 +164,10 @@ cudaError_t bpc_launch_finalize_projection(bpc_ctx* ctx, cudaStream_t stream);
 cudaError_t bpc_launch_encode_simple(bpc_ctx* ctx, const void* k_cache, uint64_t* codes, cudaStream_t stream);
 cudaError_t bpc_launch_append(bpc_ctx* ctx, const void* k_new, const void* v_new, void* k_cache, void* v_cache,
                               uint64_t* codes, cudaStream_t stream);
-cudaError_t bpc_launch_fit(bpc_ctx* ctx, const void* k_cache, const float* v_star, void* workspace,
+cudaError_t bpc_launch_fit(bpc_ctx* ctx, const void* k_cache, const float* v_star, void* workspace, size_t workspace_bytes,
                            cudaStream_t stream, int* launches);
 size_t bpc_fit_workspace_bytes_impl(const bpc_config* cfg);
+size_t bpc_fit_workspace_min_bytes_impl(const bpc_config* cfg);
 // tensor-core pass of Algorithm 1 (fit_tc.cu)
 bool bpc_fit_tc_covers(const bpc_ctx* ctx);
 void bpc_fit_tc_geometry(const bpc_ctx* ctx, int* blocks_per_unit, int* rows_per_block);

@@ -848,8 +848,10 @@ static size_t fit_off_power(const bpc_config* c) {
   return fit_off_dir(c) + align256(units * BPC_D * 4) + align256(units * c->code_bits * 4);
 }
 
+size_t bpc_fit_workspace_min_bytes_impl(const bpc_config* c) { return fit_off_power(c) + fit_power_bytes(c); }
+
 size_t bpc_fit_workspace_bytes_impl(const bpc_config* c) {
-  const size_t passes = fit_off_power(c) + fit_power_bytes(c);
+  const size_t passes = bpc_fit_workspace_min_bytes_impl(c);
   if (!bpc_fit_blocked_covers(c)) return passes;
   const size_t blocked = fit_off_partials(c) + bpc_fit_blocked_bytes(c);   // (either path: the diagnostic switch changes it per call)
   return blocked > passes ? blocked : passes;
@@ -857,11 +859,12 @@ size_t bpc_fit_workspace_bytes_impl(const bpc_config* c) {
 
 size_t bpc_fit_codes_offset_impl(const bpc_config* c) { (void)c; return 0; }
 
-cudaError_t bpc_launch_fit(bpc_ctx* ctx, const void* k_cache, const float* v_star, void* workspace,
+cudaError_t bpc_launch_fit(bpc_ctx* ctx, const void* k_cache, const float* v_star, void* workspace, size_t workspace_bytes,
                            cudaStream_t stream, int* launches) {
   const bpc_config& c = ctx->cfg;
-  // without power iterations the fit runs in blocks of 32 bits; one pass over the keys per bit otherwise
-  if (bpc_fit_blocked_covers(&c) && !ctx->no_tc_encode)
+  // without power iterations the fit runs in blocks of 32 bits where the workspace has room for their columns (132 B per key:
+  // 0.55 of 0.64 GB at 32 x 128K keys); one pass over the keys per bit otherwise
+  if (bpc_fit_blocked_covers(&c) && !ctx->no_tc_encode && workspace_bytes >= bpc_fit_workspace_bytes_impl(&c))
     return bpc_launch_fit_blocked(ctx, k_cache, v_star, (uint32_t*)workspace, (unsigned char*)workspace + fit_off_partials(&c), stream, launches);
   const size_t units = (size_t)ctx->units;
   int bpu = (c.n_max + kFitRowsPerBlock - 1) / kFitRowsPerBlock;

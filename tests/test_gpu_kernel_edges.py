@@ -346,3 +346,22 @@ def test_steps_around_captured_calls(bits, n, cluster):
         assert early == 12 * [False]
         assert all(torch.equal(a, b) for a, b in zip(want, got))
     assert ctx.last_device_error() == 0
+
+
+@pytest.mark.parametrize("dtype,bits,n", [("bf16", 128, 3000), ("bf16", 256, 700), ("f32", 64, 2000)])
+def test_fit_in_the_smallest_workspace(dtype, bits, n):
+    """The workspace of one pass per bit, full of ones: per unit n_max codes, and per 1024 keys 128 sums and `bits` counts."""
+    H = _harness()
+    spec = CONFIGS[1].scaled(name="smallws", wid=91, dtype=dtype, n_ctx=n, n_kv_heads=2, n_q_heads=2, code_bits=bits, steps=1)
+    sess = H.Session(spec)
+    n_max, up = sess.w.n_max, lambda x: (x + 255) // 256 * 256
+    tiles = -(-n_max // 1024)
+    size = up(2 * n_max * bits // 8) + up(2 * tiles * 128 * 4) + up(2 * tiles * bits * 4) + up(2 * 128 * 4) + up(2 * bits * 4)
+    assert sess.ctx.fit_workspace_min_bytes() == size < sess.ctx.fit_workspace_bytes()
+    sess.fit_ws = torch.full((size,), 255, dtype=torch.uint8, device="cuda")
+    sess.ctx.fit(sess.k_cache, sess.v_star, sess.fit_ws)
+    sess.P, sess.Ph, sess.gram = sess.ctx.get_projection()
+    H.check_fit(sess, [0, 1], {})
+    with pytest.raises(H.B.BpcError):
+        sess.ctx.fit(sess.k_cache, sess.v_star, sess.fit_ws[:-1])
+    assert sess.ctx.last_device_error() == 0
