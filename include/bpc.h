@@ -298,6 +298,9 @@ bpc_status bpc_debug_set_pdl(bpc_ctx* ctx, int32_t on);
 /* 1 when the last decode step may have read the projection while the kernel before it on the stream was still running: the
  * context's launch before it there was a decode step as well, and no call that writes the projection has been captured. */
 int32_t    bpc_step_read_early(bpc_ctx* ctx);
+/* 1 when the last decode step took the kernel variant for short key ranges (the appended key is selected after the threshold of
+ * the others is known; with 256-bit codes its Gram matrix may be kept in shared memory).  The results are the same. */
+int32_t    bpc_step_deferred(bpc_ctx* ctx);
 bpc_status bpc_debug_force_key_shift(bpc_ctx* ctx, int32_t shift);
 bpc_status bpc_debug_set_tensor_core_encode(bpc_ctx* ctx, int32_t on);
 bpc_status bpc_debug_force_streaming(bpc_ctx* ctx, int32_t on);

@@ -526,18 +526,6 @@ bpc_status bpc_append(bpc_ctx* ctx, const void* k_new, const void* v_new, void* 
   return BPC_OK;
 }
 
-// Whether a step that appends a key takes the kernel with the deferred selection (Hamming scores in 16-bit keys; the same
-// results at any length).  Its sign sweep of the appended key runs beside the scan AND the threshold search: worth it while
-// the sweep (about 3 us) outlasts the scan, up to some 6K keys per block.  With 256-bit codes it also keeps the Gram matrix
-// in shared memory next to the scores of up to 20K keys per block (43 us of sweep from L2 otherwise).  Lengths are the host
-// shadow's: a captured step keeps the kernel that was chosen at capture.
-static bool short_ranges(const bpc_ctx* ctx) {
-  int longest = 0;
-  for (int i = 0; i < ctx->cfg.batch; ++i) longest = ctx->host_lens[i] > longest ? ctx->host_lens[i] : longest;
-  const int keys = ctx->cluster_size > 1 ? bpc_fused_chunk(longest + 1, ctx->cluster_size) : longest + 1;
-  return keys <= (ctx->cfg.code_bits == 256 ? 20480 : 6144);
-}
-
 static bpc_status decode_common(bpc_ctx* ctx, const void* k_new, const void* v_new, void* k_cache_w, void* v_cache_w,
                                 uint64_t* codes_w, const void* q, const void* k_cache, const void* v_cache,
                                 const uint64_t* codes, int32_t budget_ppm, int32_t budget_count, float* out,
@@ -623,6 +611,7 @@ static bpc_status decode_common(bpc_ctx* ctx, const void* k_new, const void* v_n
   const bool known = capture_of(stream, &capture);
   p.early_projection = known && !ctx->projection_captured && ctx->projection_settled && ctx->settled_stream == stream &&
                        ctx->settled_capture == capture;
+  bool deferred = false;
   if (ctx->streaming)
     e = c.kv_dtype == BPC_BF16 ? bpc_launch_decode_bf16_stream(ctx, p, (cudaStream_t)stream)
                                : bpc_launch_decode_f32_stream(ctx, p, (cudaStream_t)stream);
@@ -635,17 +624,22 @@ static bpc_status decode_common(bpc_ctx* ctx, const void* k_new, const void* v_n
   else if (c.eas_ppm > 0)
     e = c.kv_dtype == BPC_BF16 ? bpc_launch_decode_bf16_eas(ctx, p, (cudaStream_t)stream)
                                : bpc_launch_decode_f32_eas(ctx, p, (cudaStream_t)stream);
-  else if (k_new != nullptr && short_ranges(ctx))
-    e = c.kv_dtype == BPC_BF16 ? bpc_launch_decode_bf16_short(ctx, p, (cudaStream_t)stream)
-                               : bpc_launch_decode_f32_short(ctx, p, (cudaStream_t)stream);
-  else
-    e = c.kv_dtype == BPC_BF16 ? bpc_launch_decode_bf16(ctx, p, (cudaStream_t)stream)
-                               : bpc_launch_decode_f32(ctx, p, (cudaStream_t)stream);
+  else {
+    e = cudaErrorNotSupported;                               // the deferred selection, for steps that append a key to short ranges
+    if (k_new != nullptr)
+      e = c.kv_dtype == BPC_BF16 ? bpc_launch_decode_bf16_short(ctx, p, (cudaStream_t)stream)
+                                 : bpc_launch_decode_f32_short(ctx, p, (cudaStream_t)stream);
+    deferred = e != cudaErrorNotSupported;
+    if (!deferred)
+      e = c.kv_dtype == BPC_BF16 ? bpc_launch_decode_bf16(ctx, p, (cudaStream_t)stream)
+                                 : bpc_launch_decode_f32(ctx, p, (cudaStream_t)stream);
+  }
   if (e != cudaSuccess) return cuda_fail(ctx, e);
   ctx->projection_settled = known;
   ctx->settled_stream = stream;
   ctx->settled_capture = capture;
   ctx->read_early = p.early_projection != 0;
+  ctx->step_deferred = deferred;
   ctx->launches += 1;
   return BPC_OK;
 }
@@ -731,6 +725,7 @@ bpc_status bpc_debug_force_byte_keys(bpc_ctx* ctx, int32_t mode) {
 
 int32_t bpc_uses_byte_keys(bpc_ctx* ctx) { return (ctx != nullptr && ctx->byte_keys) ? 1 : 0; }
 
+int32_t bpc_step_deferred(bpc_ctx* ctx) { return (ctx != nullptr && ctx->step_deferred) ? 1 : 0; }
 int32_t bpc_step_read_early(bpc_ctx* ctx) { return (ctx != nullptr && ctx->read_early) ? 1 : 0; }
 
 bpc_status bpc_status_of_device_error(int32_t error_word) { return error_word == 0 ? BPC_OK : BPC_ERR_DEVICE; }

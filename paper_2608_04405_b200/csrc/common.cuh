@@ -41,6 +41,7 @@ struct bpc_ctx {
   unsigned long long settled_capture;   // ... into this capture (0: not captured)
   bool projection_captured; // a call that writes the projection is part of a graph, which may run at any time
   bool read_early;          // the last decode step read the projection ahead of its dependency wait
+  bool step_deferred;       // the last decode step took the variant with the deferred selection
   int wait_tries;           // tries after which waits for other blocks of a cluster give up
   bool use_pdl;             // launch the decode kernel with programmatic stream serialization
   bool streaming;           // the scores of a full unit do not fit the largest cluster: two-pass (streaming) selection

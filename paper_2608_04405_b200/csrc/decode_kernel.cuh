@@ -69,6 +69,7 @@ static_assert(sizeof(SmallState) == 5344, "");
 // 256-bit Gram matrix in shared memory: 32 x 32 blocks on and right of the diagonal, padded to spread the banks; byte offset
 // of (row, column) inside the set
 constexpr int kGramBlock = 32 * 32 * 4 + 16;
+constexpr int kGramTriBytes = 8 * 9 / 2 * kGramBlock;
 __device__ __forceinline__ int gram_tri(int row, int col) {
   const int r = row >> 5, c = col >> 5;
   return (r * 8 - r * (r - 1) / 2 + (c - r)) * kGramBlock + (row & 31) * 128 + (col & 31) * 4;
@@ -101,6 +102,12 @@ struct DecodeSmem {
     return key_bytes == 1 ? (size_t)((chunk_cap + kSegKeys - 1) / kSegKeys) * kSegKeys
                           : (size_t)((chunk_cap + kSegKeys - 1) / kSegKeys) * kSegSlots * 2;
   }
+  // room for `bytes` in the union behind what the scan and the query hash use of it
+  __host__ __device__ bool union_room(int chunk_cap, int key_bytes, size_t bytes) const {
+    return score_bytes(chunk_cap, key_bytes) + bytes <= total - off_union && hashpart_bytes() + bytes <= total - off_union;
+  }
+  // steps that append a key take the threshold without it (see the deferred selection)
+  __host__ __device__ static constexpr bool can_defer(int nbins, int hist_shift) { return nbins <= NT - 32 && hist_shift == 0; }
   __host__ __device__ DecodeSmem(int chunk_cap, int nbins, int stages, int key_bytes = 2) {
     const size_t nb = a16((size_t)nbins * 4);
     off_hist = 0;
@@ -551,12 +558,12 @@ bpc_decode_kernel(const DecodeParams p) {
   const float* gsm = nullptr;
   // (256 bits, deferred selection: the whole matrix does not fit, its 32 x 32 blocks on and right of the diagonal do)
   constexpr bool kGramTri = kDefer && W32 == 8;
-  constexpr int kGramBytes = kGramTri ? W32 * (W32 + 1) / 2 * kGramBlock : B * B * 4;
+  constexpr int kGramBytes = kGramTri ? kGramTriBytes : B * B * 4;
   if (appender && p.residual_correction != 0) {
     const size_t union_bytes = plan.total - plan.off_union;
-    const size_t score_bytes = STREAM ? (size_t)NW * nbins * 4      // (streaming: the per-warp histograms sit there)
-                                      : L::score_bytes(p.chunk_cap, K8 ? 1 : 2);
-    if (score_bytes + kGramBytes <= union_bytes && L::hashpart_bytes() + kGramBytes <= union_bytes) {
+    const bool room = STREAM ? (size_t)NW * nbins * 4 + kGramBytes <= union_bytes && L::hashpart_bytes() + kGramBytes <= union_bytes
+                             : plan.union_room(p.chunk_cap, K8 ? 1 : 2, kGramBytes);   // (streaming: the per-warp histograms sit there)
+    if (room) {
       float* dstg = reinterpret_cast<float*>(uni + union_bytes - kGramBytes);
       const float* Gs = p.gram + (size_t)(p.shared_sets ? kvh : unit) * B * B;
       if constexpr (kGramTri) {
@@ -581,7 +588,7 @@ bpc_decode_kernel(const DecodeParams p) {
   // warp takes no part in their barriers (it arrives at the cluster barrier before its sweep), and its score reaches every
   // block through a store that completes on the block's mbarrier, awaited before the emission.  One sequence of 32K keys:
   // 1.9 us of waiting at the histogram barrier less.
-  const bool deferred = kDefer && fused && kh < n && p.nbins <= NT - 32 && (kFastOnly || p.hist_shift == 0);
+  const bool deferred = kDefer && fused && kh < n && L::can_defer(p.nbins, p.hist_shift);
   // In the appending block the last warp codes the new key while the other warps scan; the new key's code is
   // not in memory yet, so the scan stops one key short and the key is scored separately below.
   // With a short key range the other blocks wait for that warp, so the warps that share its scheduler do not scan (the

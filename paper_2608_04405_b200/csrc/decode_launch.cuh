@@ -19,6 +19,24 @@ static cudaError_t configure_kernel(int device) {
   return cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
 }
 
+// Whether a step that appends a key is faster with the deferred selection (variant 4; the same results at any length).  That
+// variant does two things.  The sign sweep of the appended key runs beside the threshold search as well as beside the scan: worth it
+// while the sweep (about 3 us, 43 us at 256 bits from L2) outlasts the scan, up to some 6K keys per block and 20K at 256 bits, and
+// only where every bin of the histogram has a thread that is not the sweep's (not with more than 480 bins: seven and eight heads
+// at 128 bits, more than two at 256; 224 in the blocks of fp32 caches with more than two heads).  And at 256 bits the sweep finds
+// the Gram matrix in shared memory, if the score keys of a block filled to n_max leave it room (bf16 caches, up to 19K keys).
+// With neither the plain variant is faster: seven heads, 8K keys 21.7 -> 21.1 us; 256 bits, 16 x 8K keys in caches of 64K 42.5 -> 41.3.
+// Lengths are the host shadow's: a captured step keeps the kernel that was chosen at capture.
+template <typename KV, int GP, int W32>
+static bool defers(const bpc_ctx* ctx, const DecodeParams& p, const DecodeSmem<KV, GP, W32>& plan) {
+  int longest = 0;
+  for (int i = 0; i < ctx->cfg.batch; ++i) longest = ctx->host_lens[i] > longest ? ctx->host_lens[i] : longest;
+  const int keys = ctx->cluster_size > 1 ? bpc_fused_chunk(longest + 1, ctx->cluster_size) : longest + 1;
+  if (keys > (W32 == 8 ? 20480 : 6144)) return false;
+  return DecodeSmem<KV, GP, W32>::can_defer(p.nbins, p.hist_shift) ||
+         (W32 == 8 && p.residual_correction != 0 && plan.union_room(p.chunk_cap, 2, kGramTriBytes));
+}
+
 template <typename KV, int GP, int W32, int MODE, int EAS>
 static cudaError_t launch_one(bpc_ctx* ctx, const DecodeParams& p_in, cudaStream_t stream) {
   typedef DecodeSmem<KV, GP, W32> L;
@@ -30,6 +48,8 @@ static cudaError_t launch_one(bpc_ctx* ctx, const DecodeParams& p_in, cudaStream
   p.stages = L(p.chunk_cap, p.nbins, 3, kKeyBytes).total <= (size_t)optin ? 3 : 2;
   const size_t smem = L(p.chunk_cap, p.nbins, p.stages, kKeyBytes).total;
   if (smem > (size_t)optin) return cudaErrorInvalidConfiguration;
+  if constexpr (EAS == 4)
+    if (!defers<KV, GP, W32>(ctx, p, L(p.chunk_cap, p.nbins, p.stages, kKeyBytes))) return cudaErrorNotSupported;   // (the plain variant serves)
   if ((ctx->decode_smem_set & ((size_t)1 << EAS)) == 0) {   // function attributes are sticky: set them once per variant
     e = configure_kernel<KV, GP, W32, MODE, EAS>(ctx->device);
     if (e != cudaSuccess) return e;

@@ -365,3 +365,24 @@ def test_fit_in_the_smallest_workspace(dtype, bits, n):
     with pytest.raises(H.B.BpcError):
         sess.ctx.fit(sess.k_cache, sess.v_star, sess.fit_ws[:-1])
     assert sess.ctx.last_device_error() == 0
+
+
+@pytest.mark.parametrize("dtype,bits,group,n,n_max,deferred", [
+    ("bf16", 128, 4, 6143, 8192, True), ("bf16", 128, 4, 6144, 8192, False),            # by the length
+    ("bf16", 128, 7, 3000, 8192, False), ("bf16", 64, 8, 3000, 8192, True),             # 897 bins, 257 bins
+    ("f32", 64, 4, 3000, 8192, True), ("f32", 128, 4, 3000, 8192, False),               # 129 and 257 bins in a block of 256 threads
+    ("bf16", 256, 2, 20479, 24576, True), ("bf16", 256, 2, 20480, 24576, False),
+    ("bf16", 256, 4, 8000, 19328, True), ("bf16", 256, 4, 8000, 24576, False), ("f32", 256, 4, 3000, 8192, False)])   # room for the Gram matrix
+def test_rule_of_the_deferred_selection(dtype, bits, group, n, n_max, deferred):
+    """One block per unit: which steps take the variant for short ranges, and their results."""
+    H = _harness()
+    spec = CONFIGS[1].scaled(name="rule", wid=92, dtype=dtype, n_ctx=n, n_kv_heads=1, n_q_heads=group, code_bits=bits, steps=1)
+    sess = H.Session(spec, cluster_size=1, extra_rows=n_max - n)
+    sess.fit()
+    sess.encode()
+    k_new, v_new = (x.cuda() for x in sess.w.new_kv(sess.lens))
+    q = sess.w.queries(sess.lens)[0].cuda()
+    sess.ctx.append_decode_attn(k_new, v_new, sess.k_cache, sess.v_cache, sess.codes, q, budget_ppm=20000)
+    assert sess.ctx.step_deferred() == deferred
+    sess.ctx.set_seq_lens(sess.lens)
+    H.check_decode(sess, q, [0], {}, budget_ppm=20000, append=(k_new, v_new))
