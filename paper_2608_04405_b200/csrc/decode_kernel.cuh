@@ -1151,8 +1151,7 @@ bpc_decode_kernel(const DecodeParams p) {
           for (int pl = 0; pl < NP; ++pl) mk[pl][w] = st->mask[pl][w];
         }
         key = score_key<W32, NP>(h, sg, mk);
-        if constexpr (K8) sc8[n - 1 - c0] = (uint8_t)key;
-        else sc[score_slot(n - 1 - c0)] = (uint16_t)key;
+        sc[score_slot(n - 1 - c0)] = (uint16_t)key;
         if (p.dbg_scores != nullptr) p.dbg_scores[(size_t)unit * p.n_max + (n - 1)] = ((2 * key) << cs) - (st->rsum << cs);
       }
       key = __shfl_sync(0xffffffffu, key, 0);
@@ -1384,26 +1383,11 @@ bpc_decode_kernel(const DecodeParams p) {
     }
     }
   } else if constexpr (!kFastOnly) {
-    // Total histogram through distributed shared memory.  With at most one bin per thread (the common case)
-    // the per-block counts of that bin stay in registers and are reused for the per-block offsets below.
-    const bool one_bin = nbins <= NT;
-    uint32_t myv[BPC_MAX_CLUSTER];
-#pragma unroll
-    for (int r = 0; r < BPC_MAX_CLUSTER; ++r) myv[r] = 0u;
-    if (one_bin) {
-      if (tid < nbins) {
-        uint32_t s = 0;
-#pragma unroll
-        for (int r = 0; r < BPC_MAX_CLUSTER; ++r)
-          if (r < CS) { myv[r] = cluster.map_shared_rank(hist, r)[tid]; s += myv[r]; }
-        tot[tid] = s;
-      }
-    } else {
-      for (int bin = tid; bin < nbins; bin += NT) {
-        uint32_t s = 0;
-        for (int r = 0; r < CS; ++r) s += cluster.map_shared_rank(hist, r)[bin];
-        tot[bin] = s;
-      }
+    // Total histogram through distributed shared memory (more bins than threads, whose stored keys are not exact)
+    for (int bin = tid; bin < nbins; bin += NT) {
+      uint32_t s = 0;
+      for (int r = 0; r < CS; ++r) s += cluster.map_shared_rank(hist, r)[bin];
+      tot[bin] = s;
     }
     __syncthreads();
     {
@@ -1423,26 +1407,14 @@ bpc_decode_kernel(const DecodeParams p) {
     __syncthreads();
     T = st->T;
     BPC_STAMP(9);
-    if (one_bin) {
-      if (tid < nbins && tid >= T) {
-#pragma unroll
-        for (int r = 0; r < BPC_MAX_CLUSTER; ++r) {
-          if (r < CS) {
-            if (tid == T) st->eq[r] = myv[r];
-            else if (myv[r]) atomicAdd(&st->gt[r], myv[r]);
-          }
-        }
+    for (int bin = T + 1 + tid; bin < nbins; bin += NT) {
+      if (tot[bin] == 0u) continue;
+      for (int r = 0; r < CS; ++r) {
+        const uint32_t v = cluster.map_shared_rank(hist, r)[bin];
+        if (v) atomicAdd(&st->gt[r], v);
       }
-    } else {
-      for (int bin = T + 1 + tid; bin < nbins; bin += NT) {
-        if (tot[bin] == 0u) continue;
-        for (int r = 0; r < CS; ++r) {
-          const uint32_t v = cluster.map_shared_rank(hist, r)[bin];
-          if (v) atomicAdd(&st->gt[r], v);
-        }
-      }
-      if (tid < CS) st->eq[tid] = cluster.map_shared_rank(hist, tid)[T];
     }
+    if (tid < CS) st->eq[tid] = cluster.map_shared_rank(hist, tid)[T];
     __syncthreads();
   }
   if (deferred) {

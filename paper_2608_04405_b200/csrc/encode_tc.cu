@@ -173,15 +173,10 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __nv_bfloat16* 
       // -G[i][128 + j] for the first half's bits i, as three bf16 terms; operand rows j, K index i, [128 x 128] each
       for (int c = tid; c < 128 * 128; c += kThreads) {
         const int i = c >> 7, j = c & 127;
-        const float g = -gfull[(size_t)i * TOTAL + 128 + j];
-        const __nv_bfloat16 t1 = __float2bfloat16_rn(g);
-        const float r1 = g - __bfloat162float(t1);
-        const __nv_bfloat16 t2 = __float2bfloat16_rn(r1);
-        const __nv_bfloat16 t3 = __float2bfloat16_rn(r1 - __bfloat162float(t2));
-        unsigned char* base = x_s + nosw_offset(128, j, i);
-        *reinterpret_cast<__nv_bfloat16*>(base) = t1;
-        *reinterpret_cast<__nv_bfloat16*>(base + 32768) = t2;
-        *reinterpret_cast<__nv_bfloat16*>(base + 65536) = t3;
+        __nv_bfloat16 t3[3];
+        split3(-gfull[(size_t)i * TOTAL + 128 + j], t3);
+#pragma unroll
+        for (int p = 0; p < 3; ++p) *reinterpret_cast<__nv_bfloat16*>(x_s + nosw_offset(128, j, i) + 32768 * p) = t3[p];
       }
     }
     // -G[16 pb + i][j], j after block pb, as three bf16 terms (g = t1 + t2 + t3 up to 2^-24 |g|); operand rows j, K index i
@@ -189,16 +184,11 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __nv_bfloat16* 
       const int pb = c / (kSub * NBITS), i = (c / NBITS) % kSub, j = c % NBITS;
       const int j0 = kSub * (pb + 1);
       if (j < j0) continue;
-      const float g = -gsrc[(size_t)(kSub * pb + i) * TOTAL + j];
-      const __nv_bfloat16 t1 = __float2bfloat16_rn(g);
-      const float r1 = g - __bfloat162float(t1);
-      const __nv_bfloat16 t2 = __float2bfloat16_rn(r1);
-      const __nv_bfloat16 t3 = __float2bfloat16_rn(r1 - __bfloat162float(t2));
-      const size_t part = (size_t)gb_cols(pb) * kSub * 2;
+      __nv_bfloat16 t3[3];
+      split3(-gsrc[(size_t)(kSub * pb + i) * TOTAL + j], t3);
       unsigned char* base = gb_s + gb_off(pb) + nosw_offset(gb_cols(pb), j - j0, i);
-      *reinterpret_cast<__nv_bfloat16*>(base) = t1;
-      *reinterpret_cast<__nv_bfloat16*>(base + part) = t2;
-      *reinterpret_cast<__nv_bfloat16*>(base + 2 * part) = t3;
+#pragma unroll
+      for (int p = 0; p < 3; ++p) *reinterpret_cast<__nv_bfloat16*>(base + (size_t)p * gb_cols(pb) * kSub * 2) = t3[p];
     }
   }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy writes -> visible to the tensor core

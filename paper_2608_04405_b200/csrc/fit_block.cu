@@ -9,9 +9,10 @@
 //     run on the tensor cores (directions and scalars as three bf16 terms each: 24 mantissa bits, products exact).
 //   * sweep: the 32 sequential bits on T alone.  A key costs 4 bytes of new data per bit (its entry of the next column)
 //     where the row pass costs 272.  Pass j decides bit j from column j and already sums u_i T[:, j+1] for all i <= j;
-//     those sums and the agreement counts u_j . u_i give c_{i,j+1} by forward substitution in fp64, because
-//     n c_{i,l} = u_i^T T_l - sum_{m<i} (u_i . u_m) c_{m,l}.  One thread block cluster per unit: the exchange per bit is a
-//     few hundred bytes through distributed shared memory and one cluster barrier.
+//     those sums and the agreement counts u_j . u_i give c_{i,j+1} in fp64, because
+//     n c_{i,l} = u_i^T T_l - sum_{m<i} (u_i . u_m) c_{m,l}: a triangular system, whose inverse grows by one row per bit.  One
+//     thread block cluster per unit: the exchange per bit is a few hundred bytes per block, stored asynchronously into the
+//     peers' shared memory and counted on their mbarriers.
 //   * gather: W = U_blk^T K and the agreement counts of the block's bits with all bits so far (tensor cores again, the key
 //     tile read channel-major).
 //   * rows: v_i = (W_i - sum_{j<i} (u_i . u_j) v_j) / n in fp64, then the next block's scalars C = V D_next^T in fp64.
@@ -47,13 +48,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
                : "r"(taddr));
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
-__device__ __forceinline__ void split3(float v, __nv_bfloat16 (&t)[3]) {   // v = t0 + t1 + t2 (24 mantissa bits)
-  t[0] = __float2bfloat16_rn(v);
-  const float r1 = v - __bfloat162float(t[0]);
-  t[1] = __float2bfloat16_rn(r1);
-  t[2] = __float2bfloat16_rn(r1 - __bfloat162float(t[1]));
-}
 
 // 32 x 32 bit transposes across the lanes of a warp, N words at once: lane i returns bit i of every lane.  Halves and bytes
 // move with one byte permute, smaller fields with a rotation and a merge.
@@ -550,10 +544,13 @@ fit_gather_f32_kernel(const float* __restrict__ k_cache, const uint32_t* __restr
 
 // --------------------------------------------------------------------------- sweep
 // The 32 sequential bits of a block on the columns T.  Block r of the unit's cluster owns an equal share of the keys; a
-// thread takes four consecutive keys at a time.  Per key and bit: subtract sum_i u_i c_i (two table look-ups per eight
+// thread takes eight keys at a time, two runs of four.  Per key and bit: subtract sum_i u_i c_i (one table look-up per eight
 // bits), decide, and add the next column's entry to the running sums of the bits that are set (the sum over set bits
 // gives u_i^T T = 2 sum - total).  Agreements with the earlier bits are counted bit-sliced, 32 bits per operation.
-// The loop body is compiled for 8, 16, 24 and 32 bits in play.
+// The loop body is compiled for every four bits in play.
+// Precision: the running sums are fp32 over at most 30 rounds of eight keys and the 32 lanes of a warp, fp64 above.  Their error
+// enters c_i, one scalar for all keys, where it averages over the n keys (about 4 * 2^-24 / sqrt(n) of a typical T, against
+// 0.3 * 2^-24 for the rounding of a key's own T).
 
 struct SweepSums {                                         // lane i: bit i
   double s;                                                // u_i^T T over this warp's keys
@@ -729,15 +726,15 @@ __device__ __forceinline__ void sweep_pass(SweepStream& in, uint32_t* __restrict
       for (int o = 16; o >= 1; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
       out.s += 2.0 * (double)warp_sum_scatter<NS>(s, lane) - (double)tot;
       if (!ONE) {
-      const int keys_per_lane = kSweepKeys * ((g1 - g0 + kSweepWarps - 1) / kSweepWarps);
+        const int keys_per_lane = kSweepKeys * ((g1 - g0 + kSweepWarps - 1) / kSweepWarps);
 #pragma unroll
-      for (int k0 = 0; k0 < kSweepPlanes; k0 += 4) {       // four independent transposes at a time
-        if ((keys_per_lane >> k0) == 0) break;             // higher planes are empty
-        uint32_t x[4] = {pl[k0], pl[k0 + 1], pl[k0 + 2], pl[k0 + 3]};
-        warp_transpose<4>(x, lane);
+        for (int k0 = 0; k0 < kSweepPlanes; k0 += 4) {     // four independent transposes at a time
+          if ((keys_per_lane >> k0) == 0) break;           // higher planes are empty
+          uint32_t x[4] = {pl[k0], pl[k0 + 1], pl[k0 + 2], pl[k0 + 3]};
+          warp_transpose<4>(x, lane);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) out.cnt += __popc(x[k]) << (k0 + k);
-      }
+          for (int k = 0; k < 4; ++k) out.cnt += __popc(x[k]) << (k0 + k);
+        }
       }
       if (g1 == ng && nkeys < nk && (ng - 1 - warp) % kSweepWarps == 0) {   // this warp took the group with keys past the end
         __syncwarp();

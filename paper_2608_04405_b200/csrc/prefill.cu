@@ -87,10 +87,11 @@ constexpr int kEncBits = 64;                                         // bits of 
 constexpr int kEncChannels = 32;                                     // channels of P staged at a time
 constexpr int kEncGramBits = 128;                                    // up to this code length the Gram matrix is kept in shared memory
 
+template <int NB>
 struct EncSmem {
   double k[kEncKeys][BPC_D + 1];
   double p[kEncBits][kEncChannels + 1];
-  float t[kEncKeys][256 + 1];
+  float t[kEncKeys][32 * NB + 1];
 };
 
 template <typename KV, int NB>                                       // NB = code words per key
@@ -100,8 +101,8 @@ encode_simple_kernel(const KV* __restrict__ k_cache, const float* __restrict__ P
                      int row_stride, int shared_sets, int residual_correction, float* __restrict__ key_err) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int b = 32 * NB;
-  EncSmem& sm = *reinterpret_cast<EncSmem*>(smem);
-  float* g_s = reinterpret_cast<float*>(smem + sizeof(EncSmem));     // [b][b] where it fits
+  EncSmem<NB>& sm = *reinterpret_cast<EncSmem<NB>*>(smem);
+  float* g_s = reinterpret_cast<float*>(smem + sizeof(EncSmem<NB>));     // [b][b] where it fits
   const int unit = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n = min(unit_lens[unit], n_max);
   if (blockIdx.x * kEncKeys >= n) return;                            // uniform over the block
@@ -761,7 +762,7 @@ template <typename KV, int NB>
 static cudaError_t launch_encode_simple(bpc_ctx* ctx, const void* k_cache, uint64_t* codes, cudaStream_t stream) {
   const bpc_config& c = ctx->cfg;
   constexpr int b = 32 * NB;
-  const size_t smem = sizeof(EncSmem) + (b <= kEncGramBits ? (size_t)b * b * 4 : 0);
+  const size_t smem = sizeof(EncSmem<NB>) + (b <= kEncGramBits ? (size_t)b * b * 4 : 0);
   cudaError_t e = cudaFuncSetAttribute(encode_simple_kernel<KV, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   // a block per 32 keys up to about eight per SM over all units; longer units loop (the Gram matrix is staged once per block)

@@ -96,6 +96,14 @@ __device__ __forceinline__ void fill_sign_table(uint2* table, int tid) {
   }
 }
 
+// v = t0 + t1 + t2 in bf16 (24 mantissa bits)
+__device__ __forceinline__ void split3(float v, __nv_bfloat16 (&t)[3]) {
+  t[0] = __float2bfloat16_rn(v);
+  const float r1 = v - __bfloat162float(t[0]);
+  t[1] = __float2bfloat16_rn(r1);
+  t[2] = __float2bfloat16_rn(r1 - __bfloat162float(t[1]));
+}
+
 // the same MMA with operand A in tensor memory: one row per lane, two consecutive K elements per column
 __device__ __forceinline__ void umma_bf16_ta(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
