@@ -1111,18 +1111,21 @@ cudaError_t sweep_limits(int device, const SweepLimits** out) {
   return l->known ? cudaSuccess : cudaErrorInvalidConfiguration;
 }
 
-// Cluster size of the sweep: the smallest estimate of waves x (rounds of 128 keys per warp + the exchange of a bit), in
-// units of one round.
+// Cluster size of the sweep: the smallest estimate, in microseconds per 32 bits, of waves x (groups of keys per block, at
+// issue-bound 2.1 each and never less than one per scheduler, + the exchanges, which cost less where no warp has two groups).
+// Against every size from 1 to 16 on fourteen shapes of 1 to 128 units and 4K to 512K keys the estimate picks the fastest or one
+// within 1 %.  Whole rounds of 16 groups as the unit were too coarse: per 32 bits of a fit, 1 x 16K keys 144 -> 122 us, 8 x 8K
+// 146 -> 121, 16 x 32K 265 -> 245, 8 x 128K 380 -> 359.
 int sweep_cluster(const bpc_config* c, const SweepLimits* l) {
   const int units = c->batch * c->n_kv_heads;
   double best_cost = 0.0;
   int best = 1;
   for (int cs = 1; cs <= BPC_MAX_CLUSTER; ++cs) {
     if (l->active[cs] < 1) continue;
-    const int nk = sweep_share(c->n_max, cs);
-    const int rounds = (nk / kSweepGroup + kSweepWarps - 1) / kSweepWarps;
+    const int nk = sweep_share(c->n_max, cs), groups = nk / kSweepGroup;
     const int waves = (units + l->active[cs] - 1) / l->active[cs];
-    const double cost = waves * (rounds * (kSweepRing + (size_t)nk * 4 > kSweepMaxSmem ? 1.5 : 1.0) + 4.0 + 0.1 * cs);
+    const double words = kSweepRing + (size_t)nk * 4 > kSweepMaxSmem ? 1.5 : 1.0;       // (code words in global memory)
+    const double cost = waves * (2.1 * words * (groups < 4 ? 4 : groups) + (groups <= kSweepWarps ? 70.0 : 100.0) + 0.2 * cs);
     if (best_cost == 0.0 || cost < best_cost) { best_cost = cost; best = cs; }
   }
   return best;
