@@ -1,5 +1,6 @@
 // Tensor-core pass of Algorithm 1 (bf16 caches): one pass over the keys per bit.  Taken when the binary components come from
-// power iterations, whose directions depend on the signs so far; without them the bits are fitted 32 at a time.
+// power iterations, whose directions depend on the signs so far, and in workspaces without room for the columns of 32 bits;
+// otherwise the bits are fitted 32 at a time.
 //
 // Per bit i the pass needs, for every key row, the decision value
 //     t = R_row . d = K_row . d - sum_{j<i} u_j (v_j . d)
