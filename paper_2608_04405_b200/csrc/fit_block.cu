@@ -12,7 +12,7 @@
 //     those sums and the agreement counts u_j . u_i give c_{i,j+1} in fp64, because
 //     n c_{i,l} = u_i^T T_l - sum_{m<i} (u_i . u_m) c_{m,l}: a triangular system, whose inverse grows by one row per bit.  One
 //     thread block cluster per unit: the exchange per bit is a few hundred bytes per block, stored asynchronously into the
-//     peers' shared memory and counted on their mbarriers.
+//     peers' shared memory (added there) and counted on their mbarriers.
 //   * gather: W = U_blk^T K and the agreement counts of the block's bits with all bits so far (tensor cores again, the key
 //     tile read channel-major).
 //   * rows: v_i = (W_i - sum_{j<i} (u_i . u_j) v_j) / n in fp64, then the next block's scalars C = V D_next^T in fp64.
@@ -74,18 +74,20 @@ __device__ __forceinline__ uint32_t warp_transpose(uint32_t x, int lane) {
   return v[0];
 }
 
+// larger of a and |v|; a NaN stays one (as an unsigned word it is above everything else)
+__device__ __forceinline__ float max_abs(float a, float v) {
+  asm("max.NaN.f32 %0, %0, %1;" : "+f"(a) : "f"(fabsf(v)));
+  return a;
+}
+
 // rows of a unit that block `blk` of `blocks` takes: equal shares of whole tiles
 __host__ __device__ inline int block_rows(int n, int blocks) { return ((n + blocks - 1) / blocks + kTileKeys - 1) / kTileKeys * kTileKeys; }
 
 // ---- sweep geometry (the projection fills the columns up to a whole group of keys)
 constexpr int kSweepThreads = 512;
 constexpr int kSweepWarps = kSweepThreads / 32;
-constexpr int kSweepPlanes = 8;
 constexpr int kSweepKeys = 8;                              // keys of a thread per round: two runs of four, 128 apart
 constexpr int kSweepGroup = 32 * kSweepKeys;               // keys of a warp per round
-constexpr int kSweepSlotBytes = 4 * kSweepThreads * 16;    // one round of two columns (two slots: in use, in flight)
-constexpr int kSweepRing = 2 * kSweepSlotBytes;
-constexpr int kSweepFlush = 30;                            // rounds of eight keys between flushes: 240 < 2^kSweepPlanes counts
 // keys of a sweep block: equal shares in whole groups (columns are zero up to a whole group past the last key)
 __host__ __device__ inline int sweep_share(int n, int blocks) { return ((n + blocks - 1) / blocks + kSweepGroup - 1) / kSweepGroup * kSweepGroup; }
 
@@ -100,8 +102,8 @@ constexpr int kProjN = 3 * kBits;
 template <int GROUPS>
 __global__ void __launch_bounds__(kGroupThreads * GROUPS, 1)
 fit_project_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* __restrict__ hfit, const float* __restrict__ v_star,
-                      const float* __restrict__ cross, float* __restrict__ T, const int32_t* __restrict__ unit_lens,
-                      int32_t* __restrict__ err, int n_max, int b, int blk, int t_stride) {
+                      const float* __restrict__ cross, float* __restrict__ T, uint32_t* __restrict__ t_max,
+                      const int32_t* __restrict__ unit_lens, int32_t* __restrict__ err, int n_max, int b, int blk, int t_stride) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   constexpr int kThreads = kGroupThreads * GROUPS;
@@ -115,13 +117,14 @@ fit_project_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* 
   unsigned char* c_s = b_s + kProjN * 256 + (size_t)GROUPS * U_BYTES;  // -C, three terms: [96 x 32 blk], no swizzle
   __shared__ __align__(128) uint2 sign_table[16];
   __shared__ unsigned long long bar_s[GROUPS], tile_bar_s[GROUPS];
-  __shared__ uint32_t tmem_base_s;
+  __shared__ uint32_t tmem_base_s, max_s;
   __shared__ int timed_out_g[GROUPS];
   const unsigned st_a = smem_u32(sign_table);
-  const int unit = blockIdx.y;
+  // The keys that the gather before read last come first: some of them are still in L2 (32 x 128K keys 273 -> 262 us a launch).
+  const int unit = gridDim.y - 1 - blockIdx.y, part = gridDim.x - 1 - blockIdx.x;
   const int n = min(unit_lens[unit], n_max);
   const int rows = block_rows(n, gridDim.x);
-  const int row0 = blockIdx.x * rows;
+  const int row0 = part * rows;
   if (row0 >= n) return;                                               // uniform over the block, nothing set up yet
   const int row_end = min(n, row0 + rows);
   const int ntile = (row_end - row0 + kTileKeys - 1) / kTileKeys;
@@ -129,6 +132,7 @@ fit_project_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* 
 
   if (tid == 0) {
     for (int g = 0; g < GROUPS; ++g) { mbar_init(&bar_s[g], 1); mbar_init(&tile_bar_s[g], 1); timed_out_g[g] = 0; }
+    max_s = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
@@ -136,7 +140,7 @@ fit_project_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* 
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   unsigned long long* tile_bar = &tile_bar_s[grp];
-  auto load_tile = [&](int tile) { tma::load_key_tile(a_t, &kmap, unit * n_max + row0 + tile * kTileKeys, tile_bar); };   // (one thread)
+  auto load_tile = [&](int tile) { tma::load_key_tile(a_t, &kmap, unit * n_max + row0 + (ntile - 1 - tile) * kTileKeys, tile_bar); };   // (one thread)
   fill_sign_table(sign_table, tid);
   for (int c = tid; c < kBits * BPC_D; c += kThreads) {
     const int l = c >> 7, ch = c & 127;
@@ -167,7 +171,7 @@ fit_project_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* 
   unsigned ph = 0, tph = 0;
   uint32_t first[kSignCols / 32];                                      // the next tile's first code words of this thread's key
   auto load_words = [&](int tile) {
-    const int r = row0 + tile * kTileKeys + gtid;
+    const int r = row0 + (ntile - 1 - tile) * kTileKeys + gtid;
     const uint32_t* h = hfit + ((size_t)unit * n_max + r) * words;
 #pragma unroll
     for (int w = 0; w < kSignCols / 32; ++w) first[w] = (w < blk && r < row_end) ? h[w] : 0u;
@@ -186,8 +190,9 @@ fit_project_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* 
                 umma_desc_nosw(c_s + (size_t)(4 * w0 + 2 * ks) * C_LBO, C_LBO, 128), idesc, 1u);
   };
   if (grp < ntile) load_words(grp);
+  float t_abs = 0.f;                                                   // largest |T| of this thread's keys
   for (int tl = grp; tl < ntile; tl += GROUPS) {
-    const int row = row0 + tl * kTileKeys + gtid;
+    const int row = row0 + (ntile - 1 - tl) * kTileKeys + gtid;
     const bool live = row < row_end;
     const int w1 = min(blk, kSignCols / 32);
 #pragma unroll
@@ -241,8 +246,14 @@ fit_project_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* 
 #pragma unroll
     for (int l = 0; l < kBits; ++l) {
       const float v = (__uint_as_float(r0[l]) + __uint_as_float(r1[l])) + __uint_as_float(r2[l]);
-      dst[(size_t)l * t_stride] = live ? v + 0.f : 0.f;                // (never -0)
+      const float tv = live ? v + 0.f : 0.f;                           // (never -0)
+      dst[(size_t)l * t_stride] = tv;
+      t_abs = max_abs(t_abs, tv);
     }
+  }
+  {
+    const uint32_t m = __reduce_max_sync(0xffffffffu, __float_as_uint(t_abs));
+    if ((tid & 31) == 0) atomicMax(&max_s, m);
   }
   // the sweep reads whole groups of keys: zeros behind the unit's last tile where that ends half a group
   for (int i = row0 + ntile * kTileKeys + tid; row_end == n && i < (n + kSweepGroup - 1) / kSweepGroup * kSweepGroup; i += kThreads)
@@ -250,6 +261,7 @@ fit_project_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* 
   if (timed_out_g[grp] && gtid == 0) atomicOr(err, BPC_DEVERR_TIMEOUT);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
+  if (tid == 0) t_max[(size_t)unit * b * kBits + part] = max_s;
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_all), "r"(512) : "memory");
 }
 
@@ -258,8 +270,8 @@ fit_project_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* 
 // earlier bits in fp32 left the decisions less precise than one pass per bit has them).
 __global__ void __launch_bounds__(kTileKeys)
 fit_project_f32_kernel(const float* __restrict__ k_cache, const uint32_t* __restrict__ hfit, const float* __restrict__ v_star,
-                       const float* __restrict__ cross, float* __restrict__ T, const int32_t* __restrict__ unit_lens,
-                       int n_max, int row_stride, int b, int blk, int t_stride) {
+                       const float* __restrict__ cross, float* __restrict__ T, uint32_t* __restrict__ t_max,
+                       const int32_t* __restrict__ unit_lens, int n_max, int row_stride, int b, int blk, int t_stride) {
   const int unit = blockIdx.y, tid = threadIdx.x;
   const int n = min(unit_lens[unit], n_max);
   const int row = blockIdx.x * kTileKeys + tid;
@@ -292,8 +304,15 @@ fit_project_f32_kernel(const float* __restrict__ k_cache, const uint32_t* __rest
     }
   }
   float* dst = T + (size_t)unit * kBits * t_stride + row;
+  float t_abs = 0.f;
 #pragma unroll
-  for (int l = 0; l < kBits; ++l) dst[(size_t)l * t_stride] = live ? (float)acc[l] + 0.f : 0.f;   // (never -0)
+  for (int l = 0; l < kBits; ++l) {
+    const float tv = live ? (float)acc[l] + 0.f : 0.f;                 // (never -0)
+    dst[(size_t)l * t_stride] = tv;
+    t_abs = max_abs(t_abs, tv);
+  }
+  const uint32_t m = __reduce_max_sync(0xffffffffu, __float_as_uint(t_abs));
+  if ((tid & 31) == 0) atomicMax(&t_max[(size_t)unit * b * kBits], m);
 }
 
 // --------------------------------------------------------------------------- gather (tensor cores, bf16 caches)
@@ -545,205 +564,237 @@ fit_gather_f32_kernel(const float* __restrict__ k_cache, const uint32_t* __restr
 // --------------------------------------------------------------------------- sweep
 // The 32 sequential bits of a block on the columns T.  Block r of the unit's cluster owns an equal share of the keys; a
 // thread takes eight keys at a time, two runs of four.  Per key and bit: subtract sum_i u_i c_i (one table look-up per eight
-// bits), decide, and add the next column's entry to the running sums of the bits that are set (the sum over set bits
-// gives u_i^T T = 2 sum - total).  Agreements with the earlier bits are counted bit-sliced, 32 bits per operation.
-// The loop body is compiled for every four bits in play.
-// Precision: the running sums are fp32 over at most 30 rounds of eight keys and the 32 lanes of a warp, fp64 above.  Their error
-// enters c_i, one scalar for all keys, where it averages over the n keys (about 4 * 2^-24 / sqrt(n) of a typical T, against
-// 0.3 * 2^-24 for the rounding of a key's own T).
+// bits) and decide; then the next column's sums over the keys whose bit i is set (u_i^T T = 2 sum - total).
+// Those sums and the agreements with the earlier bits are one contraction over the keys and run on the warp-level integer
+// tensor path (mma.sync m16n8k32, u8 x u8 -> s32, exact): rows = the block's bits, columns = the four bytes of T in 32-bit
+// fixed point, a column of ones (keys set) and the new bit itself (keys set in both).  A warp keeps its keys' bits a second
+// time for that, bit-major: lane (g, t) holds bits g, g + 8, g + 16, g + 24 of the keys of lanes 8t .. 8t + 7, bit 8b + s of
+// word h being key (lane 8t + s, entry 4h + b), so that (word & 0x01010101 << s) is an operand register of four keys and a new
+// bit costs six byte permutes of its ballots.  The bytes of T are transposed by byte permutes and pass through the warp's
+// part of the copy slot it has just consumed.  One logic operation per 128 (bit, key) pairs, where predicated adds took two
+// instructions per 32.  Per 32 bits, against sums in fp32 with the agreements counted bit-sliced, byte tables for sum_i u_i c_i, 16-way
+// exchange slots and a copy ring: 8 x 32K keys 102 -> 77 us, 32 x 128K 372 -> 342.  With one group per warp a bit takes 2.4 us, half of
+// it the exchange (send 0.2, transit 0.2, scalars 0.4, tables 0.2) and the rest a chain of latencies; with several, the integer pipe
+// and the shared-memory pipe (shuffles and operand staging) share the bound at 2.1 us per group of keys and 32 bits.
+// The bit-major words stay in registers where a warp has one group of keys, in tensor memory (a scratchpad here: the kernel
+// issues no tcgen05.mma) beside key-major words in shared memory, and over column 0 of T, which is dead after bit 0, where a block
+// has more keys than fit on chip.
+// Precision: T enters the sums as a 32-bit integer with a power-of-two scale, 2^-30 or finer of the largest |T| of the unit's block
+// of columns; everything after that is exact up to the fp64 scalars.  A key's own T stays the fp32 value.
 
-struct SweepSums {                                         // lane i: bit i
-  double s;                                                // u_i^T T over this warp's keys
-  int cnt;                                                 // keys whose new bit agrees with bit i
+constexpr int kOneGroup = 0, kWordsOnChip = 1, kWordsGlobal = 2;
+
+// one round of a warp: this lane's entries of a column, keys 4 lane .. + 3 and 128 + 4 lane .. + 3 of a group
+__device__ __forceinline__ void load_entries(float4 (&v)[2], const float* src) {
+  v[0] = __ldcg(reinterpret_cast<const float4*>(src));
+  v[1] = __ldcg(reinterpret_cast<const float4*>(src + 128));
+}
+
+__device__ __forceinline__ void mma_u8(int (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k32.row.col.s32.u8.u8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+               : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// Operand B of a round, per warp: five rows (the bytes of T, least significant first, and the new bit), each 32 lanes x 2 words;
+// 80 bytes per eight lanes and 320 per row keep the 16-byte reads of a quarter warp (two rows, all four parts) on different banks.
+constexpr int kStagePart = 80, kStageRow = 320, kStageWarp = 5 * kStageRow;
+// sums of a block: six columns (bytes 0 .. 3, keys set, keys set in both) of 32 bits; a stride of 36 spreads the lanes' banks
+constexpr int kSumStride = 36;
+constexpr int kTabBits = 5, kTabs = 7;                     // sum_i u_i c_i: five bits per look-up
+
+// What a warp carries from pass to pass.
+struct SweepWarp {
+  float tab[kTabs];                                        // entry `lane` of the look-up tables
+  float4 t[2], nx[2];                                      // this lane's entries of columns j and j + 1, requested a round ahead
+  uint32_t aw[4][2];                                       // bit-major words (of the warp's only group, or of the one at hand)
+  uint32_t w[kSweepKeys];                                  // the same key-major
 };
-
-// The columns on their way to a warp: round after round and pass after pass without a break, so that the first entries of
-// a pass arrive while the block still exchanges the previous one's sums.
-struct SweepStream {
-  const float* base;                                       // this lane's entry of column 0, round 0
-  const float* next;                                       // ... of the next request
-  int t_stride, rounds;                                    // rounds of this warp per pass
-  int bit, round;                                          // of the next request
-  unsigned char* ring;                                     // this thread's slots
-  int at;                                                  // offset of the slot to be read next
-  __device__ __forceinline__ void request(unsigned char* slot) {      // (always a group, so that the waits can count)
-    if (bit < kBits) {
-      cp_async16(slot, next);
-      cp_async16(slot + kSweepThreads * 16, next + 128);
-      if (bit + 1 < kBits) {
-        cp_async16(slot + 2 * kSweepThreads * 16, next + t_stride);
-        cp_async16(slot + 3 * kSweepThreads * 16, next + t_stride + 128);
-      }
-      next += kSweepWarps * kSweepGroup;
-      if (++round == rounds) {
-        round = 0;
-        ++bit;
-        next = base + (size_t)bit * t_stride;
-      }
-    }
-    cp_async_commit();
-  }
-};
-
-// values v[0..N-1] of every lane summed over the warp: lane l returns the sum of v[l] (l & (N - 1) for N < 32)
-template <int N>
-__device__ __forceinline__ float warp_sum_scatter(float (&v)[N], int lane) {
-  static_assert(N == 8 || N == 16 || N == 32, "");
-#pragma unroll
-  for (int o = 16; o >= N; o >>= 1)
-#pragma unroll
-    for (int i = 0; i < N; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
-#pragma unroll
-  for (int o = N / 2; o >= 1; o >>= 1) {
-    const bool up = lane & o;
-#pragma unroll
-    for (int i = 0; i < o; ++i) {
-      const float keep = up ? v[i + o] : v[i], give = up ? v[i] : v[i + o];
-      v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
-    }
-  }
-  return v[0];
-}
-
-__device__ __forceinline__ void full_add(uint32_t a, uint32_t b, uint32_t c, uint32_t& s, uint32_t& cy) {
-  s = a ^ b ^ c;
-  cy = (a & b) | (c & (a | b));
-}
-// bit-sliced counters: adds the set bits of eight words to the planes
-__device__ __forceinline__ void count8(uint32_t (&pl)[kSweepPlanes], const uint32_t (&x)[8]) {
-  uint32_t s1, s2, s3, s4, c1, c2, c3, c4, d1, d2, e;
-  full_add(x[0], x[1], x[2], s1, c1);
-  full_add(x[3], x[4], x[5], s2, c2);
-  full_add(x[6], x[7], pl[0], s3, c3);
-  full_add(s1, s2, s3, pl[0], c4);
-  full_add(c1, c2, c3, s4, d1);
-  full_add(pl[1], s4, c4, pl[1], d2);
-  full_add(pl[2], d1, d2, pl[2], e);
-#pragma unroll
-  for (int k = 3; k < kSweepPlanes; ++k) {
-    const uint32_t nc = pl[k] & e;
-    pl[k] ^= e;
-    e = nc;
-  }
-}
-
-// acc += v where w has bit I set (written out so that the tests of a word become predicates, not selects)
-template <int I>
-__device__ __forceinline__ void add_if(float& acc, float v, uint32_t w) {
-  asm("{\n\t.reg .pred p;\n\t.reg .b32 q;\n\tand.b32 q, %1, %2;\n\tsetp.ne.b32 p, q, 0;\n\t@p add.f32 %0, %0, %3;\n\t}\n"
-      : "+f"(acc) : "r"(w), "n"(1u << I), "f"(v));
-}
-template <int I, int N, int NS>
-__device__ __forceinline__ void add_bits(float (&acc)[NS], float v, uint32_t w) {
-  if constexpr (I < N) {
-    add_if<I>(acc[I], v, w);
-    add_bits<I + 1, N>(acc, v, w);
-  }
-}
-// entry (w >> 8 NB) & 255 of the look-up table's row NB; `base` is the table's shared-memory address, 1024-byte aligned.
-// (A byte per look-up: the lanes' bank conflicts cost the shared-memory pipe less than twice the address arithmetic of
-// conflict-free nibbles costs the integer pipe, which bounds the pass.)
-template <int NB>
-__device__ __forceinline__ float lut_at(unsigned base, uint32_t w) {
-  const uint32_t x = NB == 0 ? w << 2 : w >> (8 * NB - 2);
-  float v;
-  asm volatile("ld.shared.f32 %0, [%1 + %2];" : "=f"(v) : "r"((x & 0x3FCu) | base), "n"(1024 * NB));
-  return v;
-}
-template <int N>
-__device__ __forceinline__ float lut_sum(unsigned base, uint32_t w) {      // rows 0 .. N - 1
-  if constexpr (N == 1) return lut_at<0>(base, w);
-  else if constexpr (N == 2) return lut_at<0>(base, w) + lut_at<1>(base, w);
-  else if constexpr (N == 3) return (lut_at<0>(base, w) + lut_at<1>(base, w)) + lut_at<2>(base, w);
-  else return (lut_at<0>(base, w) + lut_at<1>(base, w)) + (lut_at<2>(base, w) + lut_at<3>(base, w));
-}
 
 // One pass over this block's keys: decides bit j; unless it is the block's last bit, also the sums for column j + 1.
-// Q4 = groups of four bits in play (j / 4 + 1).  Keys past the end (up to 255, all in the last group of the unit's last
-// block, entries zero) take part like any others and are subtracted at the end: they all carry the same code word.
-// ONE = a warp has at most one group.  Lane i then keeps bit i of its warp's 256 keys as eight words (`rows`), and the
-// agreements are population counts against the new bit's ballots; the bit-sliced counters, whose transposition costs some
-// 900 cycles per bit, only pay with several groups (8 heads x 32K keys: 120 us per 32 bits with them).
-template <int Q4, bool LAST, bool ONE>
-__device__ __forceinline__ void sweep_pass(SweepStream& in, uint32_t* __restrict__ ws, uint32_t (&rows)[kSweepKeys], unsigned lut, int j,
-                                           int nk, int nkeys, int warp, int lane, SweepSums& out) {
-  constexpr int NS = Q4 <= 2 ? 8 : Q4 <= 4 ? 16 : 32;      // running sums (a power of two for the warp reduction)
-  out.s = 0.0;
-  out.cnt = 0;
+// TILES = tiles of 16 bits in play.  The last row of the last tile is all ones (the totals) until its own bit is
+// decided, so bit 15 already takes two tiles.  Keys past the end (up to 255, all in the last group of the unit's last
+// block, entries zero) take part like any others and are subtracted by the sender: they all carry the same code word.
+// sum_i u_i c_i comes from tables of 32 sums held by the lanes of the warp, one shuffle per five bits: no address arithmetic and
+// no bank conflicts (byte tables in shared memory: 3.4 wavefronts a look-up, which bounded the pass).
+template <int TILES, bool LAST, int WORDS>
+__device__ __forceinline__ void sweep_pass(SweepWarp& st, uint32_t* __restrict__ ws, const float* __restrict__ Tw, int t_stride,
+                                           uint32_t aw_tmem, uint32_t* __restrict__ aw_g, int j, int nk, float scale, int warp, int lane,
+                                           unsigned stage, unsigned ones, unsigned* __restrict__ sums) {
   const uint32_t bit = 1u << j;
-  const int ng = nk / kSweepGroup;
-  for (int g0 = warp; g0 < ng; g0 += kSweepWarps * kSweepFlush) {
-    float s[NS];
-    float tot = 0.f;
-    uint32_t pl[kSweepPlanes];
+  const int ng = nk / kSweepGroup, g = lane >> 2, t = lane & 3;
+  const int nl = (j + kTabBits - 1) / kTabBits;            // tables in play
+  uint32_t (&aw)[4][2] = st.aw;
+  int acc[TILES][4][4];                                    // [tile][s & 3]: counts times 2^(s & 3)
 #pragma unroll
-    for (int i = 0; i < NS; ++i) s[i] = 0.f;
+  for (int r = 0; r < TILES; ++r)
 #pragma unroll
-    for (int k = 0; k < kSweepPlanes; ++k) pl[k] = 0u;
-    const int g1 = min(ng, g0 + kSweepWarps * kSweepFlush);
-    uint32_t* pw = ws + g0 * kSweepGroup + 4 * lane;
-    for (int g = g0; g < g1; g += kSweepWarps) {
-      in.request(in.ring + (in.at ^ kSweepSlotBytes));
-      asm volatile("cp.async.wait_group 1;" ::: "memory");
-      const unsigned char* slot = in.ring + in.at;
-      in.at ^= kSweepSlotBytes;
-      uint32_t x[kSweepKeys];
+    for (int s = 0; s < 4; ++s) acc[r][s][0] = acc[r][s][1] = acc[r][s][2] = acc[r][s][3] = 0;
+  const unsigned sel = (unsigned)t | ((unsigned)(t + 4) << 4);
+  // operand B: lane g reads row g of the bytes, the column of ones, the new bit (columns 6 and 7 are not used)
+  const unsigned b_src = (g < 4 || g == 5 ? stage + (unsigned)((g == 5 ? 4 : g) * kStageRow) : ones) + (unsigned)(t * kStagePart);
+  const unsigned st_dst = stage + (unsigned)((lane >> 3) * kStagePart + (lane & 7) * 8);
+  const float* col = Tw + (size_t)j * t_stride + 4 * lane;
+#pragma unroll 1
+  for (int gr = warp; gr < ng; gr += kSweepWarps) {
+    uint32_t* pw = ws + gr * kSweepGroup + 4 * lane;
+    if constexpr (!LAST && WORDS == kWordsOnChip) {
+      const uint32_t a = aw_tmem + (uint32_t)(gr / kSweepWarps) * 8u;
+      if (TILES == 1 || j == 15) {
+        if (j > 0) asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                                : "=r"(aw[0][0]), "=r"(aw[0][1]), "=r"(aw[1][0]), "=r"(aw[1][1]) : "r"(a));
+      } else {
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                     : "=r"(aw[0][0]), "=r"(aw[0][1]), "=r"(aw[1][0]), "=r"(aw[1][1]), "=r"(aw[2][0]), "=r"(aw[2][1]), "=r"(aw[3][0]), "=r"(aw[3][1]) : "r"(a));
+      }
+    }
+    uint32_t (&w)[kSweepKeys] = st.w;
+    if (WORDS != kOneGroup) {
+      const uint4 wl = *reinterpret_cast<const uint4*>(pw), wh = *reinterpret_cast<const uint4*>(pw + 128);
+      w[0] = wl.x; w[1] = wl.y; w[2] = wl.z; w[3] = wl.w; w[4] = wh.x; w[5] = wh.y; w[6] = wh.z; w[7] = wh.w;
+    }
+    float c[kSweepKeys];
+#pragma unroll
+    for (int e = 0; e < kSweepKeys; ++e) c[e] = __shfl_sync(0xffffffffu, st.tab[0], w[e]);
+#pragma unroll
+    for (int q = 1; q < kTabs; ++q) {
+      if (q < nl) {
+#pragma unroll
+        for (int e = 0; e < kSweepKeys; ++e) c[e] += __shfl_sync(0xffffffffu, st.tab[q], w[e] >> (kTabBits * q));
+      }
+    }
+    uint32_t f[2] = {0u, 0u};                              // the new bit, a byte per key
+    [[maybe_unused]] uint32_t x[kSweepKeys];
+    {
+      const float tv[kSweepKeys] = {st.t[0].x, st.t[0].y, st.t[0].z, st.t[0].w, st.t[1].x, st.t[1].y, st.t[1].z, st.t[1].w};
+#pragma unroll
+      for (int e = 0; e < kSweepKeys; ++e) {
+        const bool set = !(tv[e] < c[e]);
+        if (set) w[e] |= bit;
+        if (!LAST) {
+          if (set) f[e >> 2] |= 1u << (8 * (e & 3));
+          x[e] = __ballot_sync(0xffffffffu, set);
+        }
+      }
+    }
+    if (WORDS != kOneGroup || LAST) {
+      *reinterpret_cast<uint4*>(pw) = make_uint4(w[0], w[1], w[2], w[3]);
+      *reinterpret_cast<uint4*>(pw + 128) = make_uint4(w[4], w[5], w[6], w[7]);
+    } else if (lane == 31) {
+      pw[131] = w[7];                                      // (the last key's: the sender may need it)
+    }
+    // The registers just used take the next round's entries, or the next pass's first.
+    const bool more = WORDS != kOneGroup && gr + kSweepWarps < ng;
+    const float* next = more ? col + (gr + kSweepWarps) * kSweepGroup : col + t_stride + warp * kSweepGroup;
+    if (WORDS != kOneGroup && (!LAST || more)) load_entries(st.t, next);
+    if constexpr (!LAST) {
+      // the next column in fixed point, its bytes and the new bit to the warp's staging rows
+      uint32_t v[kSweepKeys], z[5][2];
+      {
+        const float nv[kSweepKeys] = {st.nx[0].x, st.nx[0].y, st.nx[0].z, st.nx[0].w, st.nx[1].x, st.nx[1].y, st.nx[1].z, st.nx[1].w};
+#pragma unroll
+        for (int e = 0; e < kSweepKeys; ++e) v[e] = (uint32_t)__float2int_rn(nv[e] * scale);
+      }
+      if (WORDS == kOneGroup) { st.t[0] = st.nx[0]; st.t[1] = st.nx[1]; }
+      if (more || j + 2 < kBits) load_entries(st.nx, next + t_stride);
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const float4 t4 = *reinterpret_cast<const float4*>(slot + h * kSweepThreads * 16);
-        const float4 n4 = *reinterpret_cast<const float4*>(slot + (2 + h) * kSweepThreads * 16);
-        const uint4 w4 = *reinterpret_cast<const uint4*>(pw + 128 * h);
-        const float t[4] = {t4.x, t4.y, t4.z, t4.w};
-        const float nx[4] = {n4.x, n4.y, n4.z, n4.w};
-        uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w};
+        const uint32_t p0 = __byte_perm(v[4 * h], v[4 * h + 1], 0x5140), p1 = __byte_perm(v[4 * h + 2], v[4 * h + 3], 0x5140);
+        const uint32_t q0 = __byte_perm(v[4 * h], v[4 * h + 1], 0x7362), q1 = __byte_perm(v[4 * h + 2], v[4 * h + 3], 0x7362);
+        z[0][h] = __byte_perm(p0, p1, 0x5410);
+        z[1][h] = __byte_perm(p0, p1, 0x7632);
+        z[2][h] = __byte_perm(q0, q1, 0x5410);
+        z[3][h] = __byte_perm(q0, q1, 0x7632) ^ 0x80808080u;         // (the integer plus 2^31)
+        z[4][h] = f[h];
+      }
+      __syncwarp();                                        // every lane has read the rows of the round before
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const float c = lut_sum<(Q4 + 1) / 2>(lut, w[e]);
-          const uint32_t neg = (uint32_t)((int)__float_as_uint(t[e] - c) >> 31);   // (never -0: columns hold no -0)
-          if (ONE) x[4 * h + e] = __ballot_sync(0xffffffffu, neg == 0u);
-          else x[4 * h + e] = w[e] ^ neg;                  // bit i: agrees with the new bit
-          w[e] |= bit & ~neg;
-          if (!LAST) {
-            tot += nx[e];
-            add_bits<0, 4 * Q4>(s, nx[e], w[e]);
+      for (int d = 0; d < 5; ++d)
+        asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(st_dst + (unsigned)(d * kStageRow)), "r"(z[d][0]), "r"(z[d][1]) : "memory");
+      // the new bit joins the bit-major words
+      if constexpr (WORDS == kWordsOnChip) {
+        if (TILES == 1)
+          asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(aw[0][0]), "+r"(aw[0][1]), "+r"(aw[1][0]), "+r"(aw[1][1]) :: "memory");
+        else
+          asm volatile("tcgen05.wait::ld.sync.aligned;"
+                       : "+r"(aw[0][0]), "+r"(aw[0][1]), "+r"(aw[1][0]), "+r"(aw[1][1]), "+r"(aw[2][0]), "+r"(aw[2][1]), "+r"(aw[3][0]), "+r"(aw[3][1]) :: "memory");
+      }
+      [[maybe_unused]] uint4* ag = reinterpret_cast<uint4*>(aw_g + gr * kSweepGroup + 8 * lane);
+      if constexpr (WORDS == kWordsGlobal) {
+        if (j > 0) {
+          const uint4 lo = ag[0];
+          aw[0][0] = lo.x; aw[0][1] = lo.y; aw[1][0] = lo.z; aw[1][1] = lo.w;
+          if (TILES == 2 && j > 15) {
+            const uint4 hi = ag[1];
+            aw[2][0] = hi.x; aw[2][1] = hi.y; aw[3][0] = hi.z; aw[3][1] = hi.w;
           }
         }
-        *reinterpret_cast<uint4*>(pw + 128 * h) = make_uint4(w[0], w[1], w[2], w[3]);
       }
-      pw += kSweepWarps * kSweepGroup;
-      if (!LAST && !ONE) count8(pl, x);
-      if (!LAST && ONE) {
+      if (TILES == 1 && j == 0) {
+        aw[0][0] = aw[0][1] = 0u;
+        aw[1][0] = aw[1][1] = g == 7 ? ~0u : 0u;
+      }
+      if (TILES == 2 && j == 15) {
+        aw[2][0] = aw[2][1] = 0u;
+        aw[3][0] = aw[3][1] = g == 7 ? ~0u : 0u;
+      }
+      {
+        uint32_t nw[2];
 #pragma unroll
-        for (int e = 0; e < kSweepKeys; ++e) {
-          out.cnt += __popc(~(rows[e] ^ x[e]));
-          if (lane == j) rows[e] = x[e];
+        for (int h = 0; h < 2; ++h)
+          nw[h] = __byte_perm(__byte_perm(x[4 * h], x[4 * h + 1], sel), __byte_perm(x[4 * h + 2], x[4 * h + 3], sel), 0x5410);
+#pragma unroll
+        for (int q = 0; q < 2 * TILES; ++q)
+          if (lane >> 2 == j - 8 * q) { aw[q][0] = nw[0]; aw[q][1] = nw[1]; }
+      }
+      if constexpr (WORDS == kWordsOnChip) {
+        const uint32_t a = aw_tmem + (uint32_t)(gr / kSweepWarps) * 8u;
+        if (TILES == 1)
+          asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(a), "r"(aw[0][0]), "r"(aw[0][1]), "r"(aw[1][0]), "r"(aw[1][1]) : "memory");
+        else
+          asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
+                       ::"r"(a), "r"(aw[0][0]), "r"(aw[0][1]), "r"(aw[1][0]), "r"(aw[1][1]), "r"(aw[2][0]), "r"(aw[2][1]), "r"(aw[3][0]), "r"(aw[3][1]) : "memory");
+      }
+      __syncwarp();                                        // the bytes are there
+      if constexpr (WORDS == kWordsGlobal) {               // (over column 0, whose entries every lane has used)
+        ag[0] = make_uint4(aw[0][0], aw[0][1], aw[1][0], aw[1][1]);
+        if (TILES == 2) ag[1] = make_uint4(aw[2][0], aw[2][1], aw[3][0], aw[3][1]);
+      }
+      uint32_t lo[TILES][4], hi[TILES][4];                 // (operand A's registers of bits g, g + 8, word 0, 1; low and high half bytes)
+#pragma unroll
+      for (int r = 0; r < TILES; ++r) {
+        lo[r][0] = aw[2 * r][0]; lo[r][1] = aw[2 * r + 1][0]; lo[r][2] = aw[2 * r][1]; lo[r][3] = aw[2 * r + 1][1];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) hi[r][q] = lo[r][q] >> 4;
+      }
+#pragma unroll
+      for (int s2 = 0; s2 < 4; ++s2) {                     // keys of lanes 8t + 2 s2, 8t + 2 s2 + 1
+        uint32_t b[4];
+        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3]) : "r"(b_src + 16u * s2) : "memory");
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int s = (2 * s2 + e) & 3;
+          const uint32_t m = 0x01010101u << s;
+#pragma unroll
+          for (int r = 0; r < TILES; ++r) {
+            const uint32_t* a = s2 < 2 ? lo[r] : hi[r];
+            mma_u8(acc[r][s], a[0] & m, a[1] & m, a[2] & m, a[3] & m, b[2 * e], b[2 * e + 1]);
+          }
         }
-        break;
       }
     }
-    if (!LAST) {
+    if (WORDS == kOneGroup) break;
+  }
+  if constexpr (!LAST) {
+    if (WORDS == kWordsOnChip) asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    if (warp < ng && t < 3) {                              // lane (g, t): columns 2t, 2t + 1 of bits g, g + 8 of a tile
 #pragma unroll
-      for (int o = 16; o >= 1; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
-      out.s += 2.0 * (double)warp_sum_scatter<NS>(s, lane) - (double)tot;
-      if (!ONE) {
-        const int keys_per_lane = kSweepKeys * ((g1 - g0 + kSweepWarps - 1) / kSweepWarps);
+      for (int r = 0; r < TILES; ++r)
 #pragma unroll
-        for (int k0 = 0; k0 < kSweepPlanes; k0 += 4) {     // four independent transposes at a time
-          if ((keys_per_lane >> k0) == 0) break;           // higher planes are empty
-          uint32_t x[4] = {pl[k0], pl[k0 + 1], pl[k0 + 2], pl[k0 + 3]};
-          warp_transpose<4>(x, lane);
-#pragma unroll
-          for (int k = 0; k < 4; ++k) out.cnt += __popc(x[k]) << (k0 + k);
+        for (int q = 0; q < 4; ++q) {
+          const unsigned v = (8u * (unsigned)acc[r][0][q] + 4u * (unsigned)acc[r][1][q] + 2u * (unsigned)acc[r][2][q] + (unsigned)acc[r][3][q]) >> 3;
+          atomicAdd(&sums[(2 * t + (q & 1)) * kSumStride + 16 * r + g + 8 * (q >> 1)], v);
         }
-      }
-      if (g1 == ng && nkeys < nk && (ng - 1 - warp) % kSweepWarps == 0) {   // this warp took the group with keys past the end
-        __syncwarp();
-        const uint32_t wp = ws[nk - 1];
-        const uint32_t same = (wp & bit) ? wp : ~wp;
-        out.cnt -= (nk - nkeys) * (int)((same >> lane) & 1u);
-      }
     }
-    if (ONE) break;
   }
 }
 
@@ -761,36 +812,38 @@ __device__ __forceinline__ bool mbar_wait_cluster(unsigned long long* bar, unsig
   }
   return false;
 }
-// asynchronous store into rank r's copy of `dst`, counted on rank r's copy of `bar`
-__device__ __forceinline__ void send_b64(const void* dst, const void* bar, int r, unsigned long long v) {
+// asynchronous addition to rank r's copy of `dst`, counted on rank r's copy of `bar`
+__device__ __forceinline__ void add_b64(const void* dst, const void* bar, int r, unsigned long long v) {
   asm volatile("{\n\t.reg .b32 d, b;\n\tmapa.shared::cluster.u32 d, %0, %2;\n\tmapa.shared::cluster.u32 b, %1, %2;\n\t"
-               "st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [d], %3, [b];\n\t}\n"
+               "red.async.relaxed.cluster.shared::cluster.mbarrier::complete_tx::bytes.add.u64 [d], %3, [b];\n\t}\n"
                ::"r"(smem_u32(dst)), "r"(smem_u32(bar)), "r"(r), "l"(v) : "memory");
 }
-__device__ __forceinline__ void send_b32(const void* dst, const void* bar, int r, uint32_t v) {
+__device__ __forceinline__ void add_b32(const void* dst, const void* bar, int r, uint32_t v) {
   asm volatile("{\n\t.reg .b32 d, b;\n\tmapa.shared::cluster.u32 d, %0, %2;\n\tmapa.shared::cluster.u32 b, %1, %2;\n\t"
-               "st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [d], %3, [b];\n\t}\n"
+               "red.async.relaxed.cluster.shared::cluster.mbarrier::complete_tx::bytes.add.u32 [d], %3, [b];\n\t}\n"
                ::"r"(smem_u32(dst)), "r"(smem_u32(bar)), "r"(r), "r"(v) : "memory");
 }
 
-template <bool SMEM_WORDS, bool ONE>
+template <int WORDS>
 __global__ void __launch_bounds__(kSweepThreads, 1)
-fit_sweep_kernel(const float* __restrict__ T, uint32_t* __restrict__ hfit, uint32_t* __restrict__ words_g,
-                 const int32_t* __restrict__ unit_lens, int32_t* __restrict__ err, int n_max, int b, int blk, int t_stride, int cluster_size,
-                 int wait_tries) {
-  extern __shared__ __align__(16) unsigned char sweep_smem[];   // the copy ring, then (SMEM_WORDS) this block's code words
-  __shared__ __align__(1024) float lut[4 * 256];           // lut[byte][pattern] = sum of +-c over the byte's bits
-  __shared__ float nib[8 * 16];                            // the same by nibble
-  __shared__ double red_s[kSweepWarps][32];
-  __shared__ int red_c[kSweepWarps][32];
-  __shared__ double slot_s[2][BPC_MAX_CLUSTER][32];        // the cluster's sums of bit i, by rank; two passes alternate
-  __shared__ int slot_c[2][BPC_MAX_CLUSTER][32];
+fit_sweep_kernel(float* __restrict__ T, uint32_t* __restrict__ hfit, uint32_t* __restrict__ words_g, const uint32_t* __restrict__ t_max,
+                 const int32_t* __restrict__ unit_lens, int32_t* __restrict__ err, int n_max, int b, int blk, int t_stride, int parts,
+                 int cluster_size, int wait_tries) {
+  extern __shared__ __align__(16) unsigned char sweep_smem[];   // this block's code words (unless global)
+  __shared__ __align__(16) unsigned char stage_s[kSweepWarps * kStageWarp];
+  __shared__ __align__(16) uint32_t ones_s[kStageRow / 4]; // operand B's column of ones
+  __shared__ unsigned sum_s[2][6 * kSumStride];            // this block's sums; two passes alternate
+  // the cluster's u_i^T T (fixed point) and keys whose new bit agrees with bit i; of four passes, so that a buffer is cleared two
+  // exchanges before anyone adds to it again
+  __shared__ unsigned long long slot_s[4][32];
+  __shared__ int slot_c[4][32];
   __shared__ unsigned long long bar_s[2];                  // the cluster's sums of this parity have arrived
-  __shared__ double sum_s[32];
+  __shared__ double tot_s[32];
   __shared__ double inv_s[32][33];                         // c = inv_s * sums: the inverse of the triangle n I + (u_i . u_m), m < i
   __shared__ double agree_s[32];                           // u_j . u_m of the newest bit
-  __shared__ __align__(16) float c_s[32];
+  __shared__ __align__(16) float c_s[kTabs][8];            // the scalars of the next column, five to a row
   __shared__ int timed_out;
+  __shared__ uint32_t tmem_base_s, max_s;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int rank = blockIdx.x % cluster_size, unit = blockIdx.x / cluster_size;
   const int n = min(unit_lens[unit], n_max);
@@ -799,11 +852,34 @@ fit_sweep_kernel(const float* __restrict__ T, uint32_t* __restrict__ hfit, uint3
   const int row0 = rank * share;
   const int nkeys = max(0, min(n - row0, share));          // keys of this block; nk = the same in whole groups
   const int nk = (nkeys + kSweepGroup - 1) / kSweepGroup * kSweepGroup;
-  uint32_t* ws = SMEM_WORDS ? reinterpret_cast<uint32_t*>(sweep_smem + kSweepRing) : words_g + (size_t)unit * t_stride + row0;
+  uint32_t* ws = WORDS != kWordsGlobal ? reinterpret_cast<uint32_t*>(sweep_smem) : words_g + (size_t)unit * t_stride + row0;
+  float* Tu = T + (size_t)unit * kBits * t_stride + row0;
+  SweepWarp st;
+  if (warp * kSweepGroup < nk) {
+    load_entries(st.t, Tu + warp * kSweepGroup + 4 * lane);
+    load_entries(st.nx, Tu + t_stride + warp * kSweepGroup + 4 * lane);
+  }
+#pragma unroll
+  for (int q = 0; q < kTabs; ++q) st.tab[q] = 0.f;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) st.aw[q][0] = st.aw[q][1] = st.w[2 * q] = st.w[2 * q + 1] = 0u;
   for (int i = tid; i < nk / 4; i += kSweepThreads) reinterpret_cast<uint4*>(ws)[i] = make_uint4(0u, 0u, 0u, 0u);
-  for (int i = tid; i < 4 * 256; i += kSweepThreads) lut[i] = 0.f;
-  if (tid < 32) c_s[tid] = 0.f;
+  if (tid < kTabs * 8) (&c_s[0][0])[tid] = 0.f;
+  if (tid < kStageRow / 4) ones_s[tid] = 0x01010101u;
+  for (int i = tid; i < 2 * 6 * kSumStride; i += kSweepThreads) (&sum_s[0][0])[i] = 0u;
   for (int i = tid; i < 32 * 33; i += kSweepThreads) (&inv_s[0][0])[i] = 0.0;
+  if (tid < 4 * 32) { (&slot_s[0][0])[tid] = 0ull; (&slot_c[0][0])[tid] = 0; }
+  if (warp == 0) {                                         // largest |T| of the unit's columns, by block of the projection
+    const int used = parts > 0 ? (n + block_rows(n, parts) - 1) / block_rows(n, parts) : 1;
+    uint32_t m = 0u;
+    for (int i = lane; i < used; i += 32) m = max(m, t_max[(size_t)unit * b * kBits + i]);
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0) max_s = m;
+  }
+  if (WORDS == kWordsOnChip && warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"(512) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
   if (tid == 0) {
     timed_out = 0;
     for (int q = 0; q < 2; ++q) {
@@ -812,108 +888,81 @@ fit_sweep_kernel(const float* __restrict__ T, uint32_t* __restrict__ hfit, uint3
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  if (WORDS == kWordsOnChip) asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");      // every rank's barriers are armed
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (WORDS == kWordsOnChip) asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   double new_row = 0.0;
-  uint32_t rows[kSweepKeys] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-  const float* Tu = T + (size_t)unit * kBits * t_stride + row0;
+  const uint32_t aw_tmem = WORDS == kWordsOnChip ? tmem_base_s + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(warp >> 2) * 128u : 0u;
+  uint32_t* aw_g = reinterpret_cast<uint32_t*>(Tu);        // (column 0)
+  // Fixed point: 2^(156 - e) for a largest |T| below 2^(e - 126), so that every entry is below 2^30.  Infinities and NaN among the
+  // entries make the scalars NaN.
+  const int e_max = max((int)(max_s >> 23), 32);
+  const float scale = e_max == 255 ? 0.f : __uint_as_float((uint32_t)(283 - e_max) << 23);
+  const double unscale = e_max == 255 ? __longlong_as_double(0x7ff8000000000000ll) : __longlong_as_double((long long)(1023 - 156 + e_max) << 52);
   const double inv_n = 1.0 / (double)n;
-  const unsigned lut_a = smem_u32(lut);
-  auto prefetch = [&](int c) {                             // column c of this block's keys into L2, a part per warp
-    const int part = (nk / 4 + kSweepWarps - 1) / kSweepWarps, at = warp * part, cnt = min(part, nk / 4 - at);
-    if (c < kBits && lane == 0 && cnt > 0)
-      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(Tu + (size_t)c * t_stride + 4 * at), "r"(16 * cnt) : "memory");
-  };
-  SweepStream in;
-  in.base = in.next = Tu + warp * kSweepGroup + 4 * lane;
-  in.t_stride = t_stride;
-  in.rounds = (nk / kSweepGroup - warp + kSweepWarps - 1) / kSweepWarps;
-  in.bit = in.rounds > 0 ? 0 : kBits;                      // (a warp without keys requests nothing)
-  in.round = 0;
-  in.ring = sweep_smem + 16 * tid;
-  in.at = 0;
-  in.request(in.ring);
+  const unsigned ones_a = smem_u32(ones_s), stage_a = smem_u32(stage_s) + (unsigned)(warp * kStageWarp);
+  float sgn[kTabBits];                                     // of the five bits of this lane's table entries
+#pragma unroll
+  for (int k = 0; k < kTabBits; ++k) sgn[k] = ((lane >> k) & 1) ? 1.f : -1.f;
   for (int j = 0; j < kBits; ++j) {
-    SweepSums sums;
+    const int buf = j & 1;
+#define BPC_SWEEP(TILES, LAST) sweep_pass<TILES, LAST, WORDS>(st, ws, Tu, t_stride, aw_tmem, aw_g, j, nk, scale, warp, lane, stage_a, ones_a, sum_s[buf])
     if (j == kBits - 1) {
       asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // (this block sends no more: see the end)
-      sweep_pass<8, true, ONE>(in, ws, rows, lut_a, j, nk, nkeys, warp, lane, sums);
+      BPC_SWEEP(1, true);
       break;
     }
-    prefetch(j + 2);
-    switch (j >> 2) {
-      case 0: sweep_pass<1, false, ONE>(in, ws, rows, lut_a, j, nk, nkeys, warp, lane, sums); break;
-      case 1: sweep_pass<2, false, ONE>(in, ws, rows, lut_a, j, nk, nkeys, warp, lane, sums); break;
-      case 2: sweep_pass<3, false, ONE>(in, ws, rows, lut_a, j, nk, nkeys, warp, lane, sums); break;
-      case 3: sweep_pass<4, false, ONE>(in, ws, rows, lut_a, j, nk, nkeys, warp, lane, sums); break;
-      case 4: sweep_pass<5, false, ONE>(in, ws, rows, lut_a, j, nk, nkeys, warp, lane, sums); break;
-      case 5: sweep_pass<6, false, ONE>(in, ws, rows, lut_a, j, nk, nkeys, warp, lane, sums); break;
-      case 6: sweep_pass<7, false, ONE>(in, ws, rows, lut_a, j, nk, nkeys, warp, lane, sums); break;
-      default: sweep_pass<8, false, ONE>(in, ws, rows, lut_a, j, nk, nkeys, warp, lane, sums); break;
-    }
+    if (j < 15) BPC_SWEEP(1, false);
+    else BPC_SWEEP(2, false);
+#undef BPC_SWEEP
     int stop = timed_out;                                  // (last set between the previous bit's barriers)
-    red_s[warp][lane] = sums.s;
-    red_c[warp][lane] = sums.cnt;
     __syncthreads();
-    const int buf = j & 1;
     const unsigned phase = (unsigned)(j >> 1) & 1u;
-    // Exchange within the cluster: warps 0..3 send the block's sums, 4..7 its counts, each to every fourth rank; the sends
-    // complete on the receiver's barrier of this parity (a rank sends bit j + 2 only after it has everybody's bit j + 1).
-    // A block that gave up a wait sends no more (its peers then miss its sums and give up in turn: every wait is bounded) and
-    // runs to the end on what it has.
-    if (stop) {
-    } else if (warp < 4) {
-      double v[kSweepWarps];
-#pragma unroll
-      for (int w = 0; w < kSweepWarps; ++w) v[w] = red_s[w][lane];
-#pragma unroll
-      for (int o = kSweepWarps / 2; o >= 1; o >>= 1)
-#pragma unroll
-        for (int w = 0; w < o; ++w) v[w] += v[w + o];
-      for (int r = warp; r < cluster_size; r += 4)
-        send_b64(&slot_s[buf][rank][lane], &bar_s[buf], r, (unsigned long long)__double_as_longlong(v[0]));
-    } else if (warp < 8) {
-      int c = 0;
-#pragma unroll
-      for (int w = 0; w < kSweepWarps; ++w) c += red_c[w][lane];
-      for (int r = warp - 4; r < cluster_size; r += 4) send_b32(&slot_c[buf][rank][lane], &bar_s[buf], r, (uint32_t)c);
+    // Exchange within the cluster: warp r sends the block's sums to rank r; the sends complete on the receiver's barrier of this
+    // parity (a rank sends bit j + 2 only after it has everybody's bit j + 1).  A block that gave up a wait sends no more (its
+    // peers then miss its sums and give up in turn: every wait is bounded) and runs to the end on what it has.
+    if (!stop && warp < cluster_size) {
+      const unsigned* s = sum_s[buf];
+      const int all = j < 15 ? 15 : 31;                    // the row of ones
+      auto fixed = [&](int i) {
+        return (long long)(s[i] + ((unsigned long long)s[kSumStride + i] << 8) + ((unsigned long long)s[2 * kSumStride + i] << 16) +
+                           ((unsigned long long)s[3 * kSumStride + i] << 24)) - ((long long)s[4 * kSumStride + i] << 31);
+      };
+      int agree = nk - (int)s[4 * kSumStride + j] - (int)s[4 * kSumStride + lane] + 2 * (int)s[5 * kSumStride + lane];
+      if (nkeys < nk) {                                    // take off the keys past the end
+        const uint32_t wp = ws[nk - 1], same = ((wp >> j) & 1u) ? wp : ~wp;
+        agree -= (nk - nkeys) * (int)((same >> lane) & 1u);
+      }
+      add_b64(&slot_s[j & 3][lane], &bar_s[buf], warp, (unsigned long long)(2 * fixed(lane) - fixed(all)));
+      add_b32(&slot_c[j & 3][lane], &bar_s[buf], warp, (uint32_t)agree);
+    }
+    if (warp == 15) {                                      // (what was read before the last barrier, or two passes ago)
+      for (int i = lane; i < 6 * kSumStride; i += 32) sum_s[buf ^ 1][i] = 0u;
+      slot_s[(j + 2) & 3][lane] = 0ull;
+      slot_c[(j + 2) & 3][lane] = 0;
     }
     // n c_{i,j+1} = u_i^T T - sum_{m<i} (u_i . u_m) c_{m,j+1}: c_i for i < j are rows of the triangle's inverse times the
     // sums, c_j follows from them (warp 0); the new bit's row of the inverse (warp 8) is needed one bit later.
     if (warp == 0 || warp == 8) {
       if (!stop && !mbar_wait_cluster(&bar_s[buf], phase, wait_tries)) stop = timed_out = 1;
-      int c = 0;
-#pragma unroll
-      for (int r = 0; r < BPC_MAX_CLUSTER; ++r) c += r < cluster_size ? slot_c[buf][r][lane] : 0;
+      const int c = slot_c[j & 3][lane];
       const double agree = lane < j ? (double)(2 * c - n) : 0.0;         // u_j . u_lane
       if (warp == 0) {
-        double v[BPC_MAX_CLUSTER];
-#pragma unroll
-        for (int r = 0; r < BPC_MAX_CLUSTER; ++r) v[r] = r < cluster_size ? slot_s[buf][r][lane] : 0.0;
-#pragma unroll
-        for (int o = BPC_MAX_CLUSTER / 2; o >= 1; o >>= 1)
-#pragma unroll
-          for (int r = 0; r < o; ++r) v[r] += v[r + o];
-        sum_s[lane] = v[0];
+        const double sum = (double)(long long)slot_s[j & 3][lane] * unscale;
+        tot_s[lane] = sum;
         __syncwarp();
         double a[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll 2
         for (int m = 0; m < j; m += 4)
 #pragma unroll
-          for (int q = 0; q < 4; ++q) a[q] += inv_s[lane][m + q] * sum_s[m + q];   // (zero beyond the row's own bit)
+          for (int q = 0; q < 4; ++q) a[q] += inv_s[lane][m + q] * tot_s[m + q];   // (zero beyond the row's own bit)
         double ci = (a[0] + a[1]) + (a[2] + a[3]);
         double x = lane < j ? agree * ci : 0.0;
 #pragma unroll
         for (int o = 16; o >= 1; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        if (lane == j) ci = (v[0] - x) * inv_n;
-        c_s[lane] = lane <= j ? (float)ci : 0.f;
-        __syncwarp();
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int e = lane + 32 * q;
-          const float4 d = *reinterpret_cast<const float4*>(&c_s[4 * (e >> 4)]);
-          nib[e] = (((e & 1) ? d.x : -d.x) + ((e & 2) ? d.y : -d.y)) + (((e & 4) ? d.z : -d.z) + ((e & 8) ? d.w : -d.w));
-        }
+        if (lane == j) ci = (sum - x) * inv_n;
+        c_s[lane / kTabBits][lane % kTabBits] = lane <= j ? (float)ci : 0.f;
       } else {
         agree_s[lane] = agree;
         __syncwarp();
@@ -925,15 +974,24 @@ fit_sweep_kernel(const float* __restrict__ T, uint32_t* __restrict__ hfit, uint3
         new_row = lane == j ? inv_n : -((a[0] + a[1]) + (a[2] + a[3])) * inv_n;
       }
     }
-    __syncthreads();
-    for (int e = tid; e < 32 * (8 * (j >> 3) + 8); e += kSweepThreads)      // the bytes in play
-      lut[e] = nib[32 * (e >> 8) + (e & 15)] + nib[32 * (e >> 8) + 16 + ((e >> 4) & 15)];
-    if (warp == 8) inv_s[j][lane] = new_row;               // (warp 0 has read the inverse; it reads it again two barriers on)
     if (tid == 0 && !stop) mbar_expect(&bar_s[buf], (unsigned)cluster_size * 32u * 12u);   // arms the barrier for bit j + 2
     __syncthreads();
+    if (warp == 8) inv_s[j][lane] = new_row;               // (read again behind the next pass's barrier)
+    // this lane's entries of the tables in play
+#pragma unroll
+    for (int q = 0; q < kTabs; ++q) {
+      if (kTabBits * q <= j) {
+        const float4 cv = *reinterpret_cast<const float4*>(c_s[q]);
+        st.tab[q] = fmaf(sgn[4], c_s[q][4], fmaf(sgn[1], cv.y, sgn[0] * cv.x) + fmaf(sgn[3], cv.w, sgn[2] * cv.z));
+      }
+    }
   }
-  cp_async_wait_all();
+  if (WORDS == kWordsOnChip) asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
+  if (WORDS == kWordsOnChip && warp == 1) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base_s), "r"(512) : "memory");
+  }
   uint32_t* h = hfit + ((size_t)unit * n_max + row0) * (b / 32) + blk;
   for (int i = tid; i < nkeys; i += kSweepThreads) h[(size_t)i * (b / 32)] = ws[i];
   // No block leaves while a peer may still send to it.  With all sums received nothing is under way; a block that gave up a wait
@@ -1022,7 +1080,7 @@ fit_rows_kernel(const double* __restrict__ wpart, const int32_t* __restrict__ ap
 
 // --------------------------------------------------------------------------- host side
 constexpr int kSms = 148;
-constexpr size_t kSweepMaxSmem = 194 * 1024;               // dynamic shared memory of a sweep block: copy ring and code words
+constexpr size_t kSweepMaxSmem = 186 * 1024;               // dynamic shared memory of a sweep block: its code words
 
 constexpr size_t kMaxSmem = 226 * 1024;                    // dynamic shared memory a block may ask for next to its static part
 // The limit of a kernel belongs to the process: one value for every launch, whatever it needs, so that a thread's launch does
@@ -1093,7 +1151,7 @@ cudaError_t sweep_limits(int device, const SweepLimits** out) {
   *out = l;
   std::lock_guard<std::mutex> hold(l->lock);
   if (l->known) return cudaSuccess;
-  const void* kernels[3] = {(const void*)fit_sweep_kernel<true, true>, (const void*)fit_sweep_kernel<true, false>, (const void*)fit_sweep_kernel<false, false>};
+  const void* kernels[3] = {(const void*)fit_sweep_kernel<kOneGroup>, (const void*)fit_sweep_kernel<kWordsOnChip>, (const void*)fit_sweep_kernel<kWordsGlobal>};
   for (const void* k : kernels) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSweepMaxSmem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -1102,7 +1160,7 @@ cudaError_t sweep_limits(int device, const SweepLimits** out) {
   for (int cs = 1; cs <= BPC_MAX_CLUSTER; ++cs) {
     cudaLaunchAttribute attr;
     cudaLaunchConfig_t cfg = sweep_config(&attr, 1, cs, kSweepMaxSmem, nullptr);
-    if (cudaOccupancyMaxActiveClusters(&l->active[cs], fit_sweep_kernel<true, false>, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&l->active[cs], fit_sweep_kernel<kWordsOnChip>, &cfg) != cudaSuccess) {
       (void)cudaGetLastError();
       l->active[cs] = 0;
     }
@@ -1111,11 +1169,11 @@ cudaError_t sweep_limits(int device, const SweepLimits** out) {
   return l->known ? cudaSuccess : cudaErrorInvalidConfiguration;
 }
 
-// Cluster size of the sweep: the smallest estimate, in microseconds per 32 bits, of waves x (groups of keys per block, at
-// issue-bound 2.1 each and never less than one per scheduler, + the exchanges, which cost less where no warp has two groups).
-// Against every size from 1 to 16 on fourteen shapes of 1 to 128 units and 4K to 512K keys the estimate picks the fastest or one
-// within 1 %.  Whole rounds of 16 groups as the unit were too coarse: per 32 bits of a fit, 1 x 16K keys 144 -> 122 us, 8 x 8K
-// 146 -> 121, 16 x 32K 265 -> 245, 8 x 128K 380 -> 359.
+// Cluster size of the sweep: the smallest estimate, in microseconds per 32 bits, of waves x (groups of keys per block + the exchanges,
+// which grow with the ranks).  With at most one group per warp the first groups hide behind each other's latencies (1.3 each to two
+// per scheduler, 3.1 from there); several groups per warp are issue-bound at 2.13 each, half as much again with the words in global
+// memory.  Measured against every size from 1 to 16 on fifteen shapes of 1 to 128 units and 4K to 256K keys: the estimate picks the
+// fastest or one within 3 %.
 int sweep_cluster(const bpc_config* c, const SweepLimits* l) {
   const int units = c->batch * c->n_kv_heads;
   double best_cost = 0.0;
@@ -1124,8 +1182,10 @@ int sweep_cluster(const bpc_config* c, const SweepLimits* l) {
     if (l->active[cs] < 1) continue;
     const int nk = sweep_share(c->n_max, cs), groups = nk / kSweepGroup;
     const int waves = (units + l->active[cs] - 1) / l->active[cs];
-    const double words = kSweepRing + (size_t)nk * 4 > kSweepMaxSmem ? 1.5 : 1.0;       // (code words in global memory)
-    const double cost = waves * (2.1 * words * (groups < 4 ? 4 : groups) + (groups <= kSweepWarps ? 70.0 : 100.0) + 0.2 * cs);
+    const double words = (size_t)nk * 4 > kSweepMaxSmem ? 1.5 : 1.0;
+    const double keys = groups > kSweepWarps ? 2.13 * words * groups + 56.0
+                                             : 1.3 * (groups < 4 ? 4 : groups) + 1.8 * (groups < 8 ? 0 : groups - 8) + 50.0;
+    const double cost = waves * (keys + 0.7 * cs);
     if (best_cost == 0.0 || cost < best_cost) { best_cost = cost; best = cs; }
   }
   return best;
@@ -1133,13 +1193,13 @@ int sweep_cluster(const bpc_config* c, const SweepLimits* l) {
 
 template <int GROUPS>
 cudaError_t launch_project_tc(const bpc_ctx* ctx, const CUtensorMap& kmap, const uint32_t* hfit, const float* v_star, const float* cross, float* T,
-                              int blk, int parts, int ts, cudaStream_t stream) {
+                              uint32_t* t_max, int blk, int parts, int ts, cudaStream_t stream) {
   const bpc_config& c = ctx->cfg;
   const size_t smem = (size_t)GROUPS * (kTileBytes + kTileKeys * kSignCols * 2) + (size_t)kProjN * 256 + (size_t)blk * kProjN * 64 + 1024;
   cudaError_t e = allow_smem(fit_project_tc_kernel<GROUPS>);
   if (e != cudaSuccess) return e;
   fit_project_tc_kernel<GROUPS><<<dim3(parts, ctx->units), kGroupThreads * GROUPS, smem, stream>>>(
-      kmap, hfit, v_star, cross, T, ctx->unit_lens, ctx->dev_err, c.n_max, c.code_bits, blk, ts);
+      kmap, hfit, v_star, cross, T, t_max, ctx->unit_lens, ctx->dev_err, c.n_max, c.code_bits, blk, ts);
   return cudaGetLastError();
 }
 
@@ -1168,12 +1228,13 @@ cudaError_t bpc_launch_fit_blocked(bpc_ctx* ctx, const void* k_cache, const floa
   double* wpart = (double*)(ws + lay.wpart);
   int32_t* apart = (int32_t*)(ws + lay.apart);
   float* cross = (float*)(ws + lay.cross);
+  uint32_t* t_max = (uint32_t*)cross + (size_t)(c.code_bits - kBits) * kBits;   // (the last 32 rows of a unit's scalars are never used; 1024 words)
   const int ts = t_stride_of(&c), parts = parts_of(&c), b = c.code_bits;
   const SweepLimits* lim = nullptr;
   cudaError_t e = sweep_limits(ctx->device, &lim);
   if (e != cudaSuccess) return e;
   const int cs = sweep_cluster(&c, lim);
-  const size_t sweep_smem = kSweepRing + (size_t)sweep_share(c.n_max, cs) * 4;
+  const size_t sweep_smem = (size_t)sweep_share(c.n_max, cs) * 4;
   const bool tc = c.kv_dtype == BPC_BF16;
   const dim3 grid(parts, ctx->units);
   CUtensorMap kmap;
@@ -1186,19 +1247,21 @@ cudaError_t bpc_launch_fit_blocked(bpc_ctx* ctx, const void* k_cache, const floa
     }
     if (tc) {
       // three warpgroups while the scalars of the earlier bits leave room for them (up to five earlier words)
-      e = blk <= 5 ? launch_project_tc<3>(ctx, kmap, hfit, v_star, cross, T, blk, parts, ts, stream)
-                   : launch_project_tc<2>(ctx, kmap, hfit, v_star, cross, T, blk, parts, ts, stream);
+      e = blk <= 5 ? launch_project_tc<3>(ctx, kmap, hfit, v_star, cross, T, t_max, blk, parts, ts, stream)
+                   : launch_project_tc<2>(ctx, kmap, hfit, v_star, cross, T, t_max, blk, parts, ts, stream);
     } else {
+      e = cudaMemset2DAsync(t_max, (size_t)b * kBits * 4, 0, 4, ctx->units, stream);
+      if (e != cudaSuccess) return e;
       fit_project_f32_kernel<<<dim3(ts / kTileKeys, ctx->units), kTileKeys, 0, stream>>>(
-          (const float*)k_cache, hfit, v_star, cross, T, ctx->unit_lens, c.n_max, ctx->row_stride, b, blk, ts);
+          (const float*)k_cache, hfit, v_star, cross, T, t_max, ctx->unit_lens, c.n_max, ctx->row_stride, b, blk, ts);
     }
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr;
     const bool words_fit = sweep_smem <= kSweepMaxSmem, one = sweep_share(c.n_max, cs) <= kSweepWarps * kSweepGroup;
-    cudaLaunchConfig_t cfg = sweep_config(&attr, ctx->units, cs, words_fit ? sweep_smem : kSweepRing, stream);
-    auto sweep = !words_fit ? fit_sweep_kernel<false, false> : one ? fit_sweep_kernel<true, true> : fit_sweep_kernel<true, false>;
-    e = cudaLaunchKernelEx(&cfg, sweep, (const float*)T, hfit, words_g, (const int32_t*)ctx->unit_lens, ctx->dev_err, (int)c.n_max, b, blk, ts, cs,
-                           ctx->wait_tries);
+    cudaLaunchConfig_t cfg = sweep_config(&attr, ctx->units, cs, words_fit ? sweep_smem : 0, stream);
+    auto sweep = !words_fit ? fit_sweep_kernel<kWordsGlobal> : one ? fit_sweep_kernel<kOneGroup> : fit_sweep_kernel<kWordsOnChip>;
+    e = cudaLaunchKernelEx(&cfg, sweep, T, hfit, words_g, (const uint32_t*)t_max, (const int32_t*)ctx->unit_lens, ctx->dev_err, (int)c.n_max, b, blk,
+                           ts, tc ? parts : 0, cs, ctx->wait_tries);
     if (e != cudaSuccess) return e;
     if (tc) {
       // as many warpgroups as their tile and sign buffers leave room for (four up to the third word, two from the sixth)

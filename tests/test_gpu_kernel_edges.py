@@ -16,6 +16,7 @@ def _harness():
     ("bf16", 64, 1, 1, None), ("bf16", 32, 127, 1, None), ("bf16", 128, 129, 2, 1),     # a partial tile, a tile and one key
     ("bf16", 64, 257, 1, None), ("bf16", 256, 4097, 1, None),                           # a sweep group and one key; all eight words
     ("bf16", 64, 9000, 3, 200), ("bf16", 32, 70001, 1, None),                           # ragged; several groups per warp
+    ("bf16", 64, 8449, 64, None),                                                       # clusters of one, three rounds, a group of one key
     ("f32", 32, 1, 1, None), ("f32", 128, 385, 2, 100), ("f32", 256, 2051, 1, None)])
 def test_blocked_fit_edges(dtype, bits, n, batch, n_min):
     """Algorithm 1 in blocks of 32 bits at the edges of its tiles (128 keys), groups (256) and code words."""
@@ -28,6 +29,20 @@ def test_blocked_fit_edges(dtype, bits, n, batch, n_min):
     H.check_fit(sess, [0, batch * 2 - 1], rep)
     assert sess.ctx.last_device_error() == 0
     print(rep)
+
+
+def test_fit_with_infinities():
+    """An infinite key makes its own unit's rows NaN or infinite and leaves the other units alone."""
+    H = _harness()
+    spec = CONFIGS[1].scaled(name="fitinf", wid=91, n_ctx=3000, n_kv_heads=2, n_q_heads=2, code_bits=64, steps=1)
+    sess = H.Session(spec)
+    sess.fit(dirty_workspace=True)
+    want = sess.P.clone()
+    sess.k_cache[0, 1, 1234, 5] = float("inf")
+    sess.fit(dirty_workspace=True)
+    assert sess.ctx.last_device_error() == 0
+    assert torch.equal(sess.P[0], want[0])
+    assert not torch.isfinite(sess.P[1]).all()
 
 
 def test_blocked_fit_code_words_outside_shared_memory():
