@@ -301,6 +301,9 @@ int32_t    bpc_step_read_early(bpc_ctx* ctx);
 /* 1 when the last decode step took the kernel variant for short key ranges (the appended key is selected after the threshold of
  * the others is known; with 256-bit codes its Gram matrix may be kept in shared memory).  The results are the same. */
 int32_t    bpc_step_deferred(bpc_ctx* ctx);
+/* 1 when the last decode step ran blocks of half the size, two to an SM (batches of unequal lengths, longest units paired with
+ * shortest; not with a cluster size set by the caller).  The selection is the same, the sums are taken in another order. */
+int32_t    bpc_step_two_per_sm(bpc_ctx* ctx);
 bpc_status bpc_debug_force_key_shift(bpc_ctx* ctx, int32_t shift);
 bpc_status bpc_debug_set_tensor_core_encode(bpc_ctx* ctx, int32_t on);
 bpc_status bpc_debug_force_streaming(bpc_ctx* ctx, int32_t on);

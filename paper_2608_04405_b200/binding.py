@@ -77,6 +77,7 @@ def _load() -> ctypes.CDLL:
         "bpc_debug_set_wait_limit": (i32, [vp, i32]),
         "bpc_step_read_early": (i32, [vp]),
         "bpc_step_deferred": (i32, [vp]),
+        "bpc_step_two_per_sm": (i32, [vp]),
         "bpc_debug_force_key_shift": (i32, [vp, i32]),
         "bpc_debug_set_tensor_core_encode": (i32, [vp, i32]),
         "bpc_debug_force_streaming": (i32, [vp, i32]),
@@ -106,7 +107,7 @@ EXPORTS = ["bpc_create", "bpc_destroy", "bpc_codes_bytes", "bpc_fit_workspace_by
            "bpc_encode_keys", "bpc_build_eas", "bpc_get_eas", "bpc_eas_capacity", "bpc_exact_topk", "bpc_append", "bpc_decode_attn", "bpc_append_decode_attn", "bpc_decode_attn_static", "bpc_static_scratch_entries", "bpc_static_last_device_error",
            "bpc_debug_set_buffers", "bpc_debug_set_phase_timer",
            "bpc_set_cluster_size", "bpc_plan_cluster_size",
-           "bpc_get_cluster_size", "bpc_uses_streaming", "bpc_status_of_device_error", "bpc_debug_set_pdl", "bpc_debug_set_wait_limit", "bpc_step_read_early", "bpc_step_deferred", "bpc_debug_force_key_shift",
+           "bpc_get_cluster_size", "bpc_uses_streaming", "bpc_status_of_device_error", "bpc_debug_set_pdl", "bpc_debug_set_wait_limit", "bpc_step_read_early", "bpc_step_deferred", "bpc_step_two_per_sm", "bpc_debug_force_key_shift",
            "bpc_debug_set_tensor_core_encode", "bpc_debug_force_streaming", "bpc_debug_force_byte_keys", "bpc_uses_byte_keys", "bpc_uses_work_items", "bpc_work_item_grid", "bpc_debug_set_decode_path",
            "bpc_debug_set_work_item_geometry", "bpc_debug_set_work_item_trace", "bpc_last_device_error", "bpc_last_cuda_error", "bpc_launch_count", "bpc_version"]
 
@@ -329,6 +330,9 @@ class Context:
 
     def step_read_early(self) -> bool:
         return bool(lib.bpc_step_read_early(self._h))
+
+    def step_two_per_sm(self) -> bool:
+        return bool(lib.bpc_step_two_per_sm(self._h))
 
     def step_deferred(self) -> bool:
         return bool(lib.bpc_step_deferred(self._h))

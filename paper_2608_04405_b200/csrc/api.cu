@@ -19,6 +19,10 @@ cudaError_t bpc_launch_decode_bf16_k8(bpc_ctx*, const DecodeParams&, cudaStream_
 cudaError_t bpc_launch_decode_f32_k8(bpc_ctx*, const DecodeParams&, cudaStream_t);
 cudaError_t bpc_launch_decode_bf16_short(bpc_ctx*, const DecodeParams&, cudaStream_t);
 cudaError_t bpc_launch_decode_f32_short(bpc_ctx*, const DecodeParams&, cudaStream_t);
+cudaError_t bpc_launch_decode_bf16_duo(bpc_ctx*, const DecodeParams&, cudaStream_t);
+cudaError_t bpc_launch_decode_bf16_w7_duo(bpc_ctx*, const DecodeParams&, cudaStream_t);
+cudaError_t bpc_decode_limits_bf16_duo(const bpc_ctx*, int, int*, int*, size_t*);
+cudaError_t bpc_decode_limits_bf16_w7_duo(const bpc_ctx*, int, int*, int*, size_t*);
 cudaError_t bpc_decode_limits_bf16_k8(const bpc_ctx*, int, int*, int*, size_t*);
 cudaError_t bpc_decode_limits_f32_k8(const bpc_ctx*, int, int*, int*, size_t*);
 cudaError_t bpc_launch_decode_bf16_w7(bpc_ctx*, const DecodeParams&, cudaStream_t);
@@ -251,7 +255,49 @@ cudaError_t bpc_plan_decode_geometry(bpc_ctx* ctx) {
     ctx->cluster_size = cs;
     ctx->streaming = true;
   }
+  ctx->duo_cap = 0;
+  if (ctx->cfg.batch > 1 && ctx->cfg.batch <= BPC_DUO_MAX_BATCH && ctx->cfg.kv_dtype == BPC_BF16 && ctx->cfg.eas_ppm == 0 && !ctx->streaming &&
+      !ctx->byte_keys) {
+    auto limits = ctx->cfg.score_mode == BPC_SCORE_WEIGHTED7 ? bpc_decode_limits_bf16_w7_duo : bpc_decode_limits_bf16_duo;
+    e = limits(ctx, hist_bins(ctx), ctx->duo_active, &ctx->duo_cap, nullptr);
+    if (e != cudaSuccess) return e;
+  }
   return cudaSuccess;
+}
+
+// Two blocks of half the size per SM for batches of unequal lengths.  With one block per SM a launch takes as long as its longest
+// unit, whose SMs work at what one SM can load while those of the short units are idle; here the work of an SM is one of the longest
+// units or one long and one short.  Step, 16 sequences of 16K to 64K keys x 8 heads, 2 %: 128 bits 56.9 -> 49.0 to 52.6 us by the lengths
+// drawn, 256 bits 90.2 -> 83.0 (there the sign sweep of the appended key, from L2, holds up the short units).  The variant costs some 8 us (no overlap with the kernels around it, half the gather ring), so it is taken where the busiest SM saves as many keys
+// as take that long to scan and gather: 0.25 us per 1000 keys for the gather at 2 %, and for the scan 0.4 at 128 bits (0.64 with
+// weighted scores) in proportion to the code length.
+bool bpc_plan_duo(const bpc_ctx* ctx, const int32_t* lens, bpc_duo_plan* plan) {
+  const int batch = ctx->cfg.batch, heads = ctx->cfg.n_kv_heads, units = ctx->units;
+  if (ctx->duo_cap <= 0 || batch < 2 || batch > BPC_DUO_MAX_BATCH) return false;
+  int cs = 0;
+  for (int c = 1; c <= BPC_MAX_CLUSTER; ++c)
+    if (ctx->duo_active[c] >= units && chunk_for(ctx->cfg.n_max, c) <= ctx->duo_cap) cs = c;
+  if (cs == 0) return false;
+  const int first = ctx->duo_active[cs] / 2, pairs = units - first;
+  if (pairs <= 0) return false;
+  for (int i = 0; i < batch; ++i) {                         // longest first
+    int j = i;
+    for (; j > 0 && lens[plan->order[j - 1]] < lens[i]; --j) plan->order[j] = plan->order[j - 1];
+    plan->order[j] = (uint8_t)i;
+  }
+  auto len = [&](int rank) { return (long long)lens[plan->order[rank / heads]]; };
+  const int alone = first - pairs;
+  long long load = alone > 0 ? len(0) : 0;
+  for (int i = 0; i < pairs; ++i) {
+    const long long both = len(alone + i) + len(units - 1 - i);
+    load = both > load ? both : load;
+  }
+  plan->cluster = cs;
+  plan->chunk = chunk_for(ctx->cfg.n_max, cs);
+  plan->first = first;
+  plan->pairs = pairs;
+  const double scan = (ctx->cfg.score_mode == BPC_SCORE_WEIGHTED7 ? 0.64 : 0.4) * ctx->cfg.code_bits / 128;
+  return (double)len(0) / ctx->cluster_size - (double)load / cs > 9500.0 / (0.25 + scan);
 }
 
 extern "C" {
@@ -369,11 +415,13 @@ bpc_status bpc_set_cluster_size(bpc_ctx* ctx, int32_t cs) {
     cs = choose_cluster(ctx, cap, mc);
     if (cs < 1) return BPC_ERR_UNSUPPORTED;
     ctx->cluster_size = cs;
+    ctx->cluster_forced = false;
     return BPC_OK;
   }
   if (cs < 1 || cs > mc || ctx->max_active[cs] < 1) return BPC_ERR_UNSUPPORTED;
   if (!ctx->streaming && chunk_for(ctx->cfg.n_max, cs) > cap) return BPC_ERR_UNSUPPORTED;
   ctx->cluster_size = cs;
+  ctx->cluster_forced = true;
   return BPC_OK;
 }
 
@@ -612,7 +660,13 @@ static bpc_status decode_common(bpc_ctx* ctx, const void* k_new, const void* v_n
   p.early_projection = known && !ctx->projection_captured && ctx->projection_settled && ctx->settled_stream == stream &&
                        ctx->settled_capture == capture;
   bool deferred = false;
-  if (ctx->streaming)
+  e = cudaErrorNotSupported;                                 // batches of unequal lengths: two blocks per SM
+  if (ctx->duo_cap > 0 && !ctx->cluster_forced && ctx->dbg_times == nullptr)   // (a caller's time stamps are sized for the plain grid)
+    e = c.score_mode == BPC_SCORE_WEIGHTED7 ? bpc_launch_decode_bf16_w7_duo(ctx, p, (cudaStream_t)stream)
+                                            : bpc_launch_decode_bf16_duo(ctx, p, (cudaStream_t)stream);
+  const bool duo = e != cudaErrorNotSupported;
+  if (duo) {
+  } else if (ctx->streaming)
     e = c.kv_dtype == BPC_BF16 ? bpc_launch_decode_bf16_stream(ctx, p, (cudaStream_t)stream)
                                : bpc_launch_decode_f32_stream(ctx, p, (cudaStream_t)stream);
   else if (ctx->byte_keys)
@@ -640,6 +694,7 @@ static bpc_status decode_common(bpc_ctx* ctx, const void* k_new, const void* v_n
   ctx->settled_capture = capture;
   ctx->read_early = p.early_projection != 0;
   ctx->step_deferred = deferred;
+  ctx->step_duo = duo;
   ctx->launches += 1;
   return BPC_OK;
 }
@@ -725,6 +780,7 @@ bpc_status bpc_debug_force_byte_keys(bpc_ctx* ctx, int32_t mode) {
 
 int32_t bpc_uses_byte_keys(bpc_ctx* ctx) { return (ctx != nullptr && ctx->byte_keys) ? 1 : 0; }
 
+int32_t bpc_step_two_per_sm(bpc_ctx* ctx) { return (ctx != nullptr && ctx->step_duo) ? 1 : 0; }
 int32_t bpc_step_deferred(bpc_ctx* ctx) { return (ctx != nullptr && ctx->step_deferred) ? 1 : 0; }
 int32_t bpc_step_read_early(bpc_ctx* ctx) { return (ctx != nullptr && ctx->read_early) ? 1 : 0; }
 

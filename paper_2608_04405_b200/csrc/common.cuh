@@ -19,6 +19,7 @@
 // In a launch that also appends, the block that codes the new key scans with fewer resources (one warp runs
 // Algorithm 2's sign sweep); it is given (16 - BPC_APPEND_LOSS16)/16 of the other blocks' key share.
 #define BPC_APPEND_LOSS16 2
+#define BPC_DUO_MAX_BATCH 64       // sequences a launch with two blocks per SM can rank
 __host__ __device__ inline int bpc_fused_chunk(int n, int cs) {
   // n <= 2^26 (bpc_create rejects larger n_max), so 32-bit arithmetic is exact here; a 64-bit division by a run-time
   // divisor would cost every thread of the kernel some hundred instructions
@@ -42,8 +43,12 @@ struct bpc_ctx {
   bool projection_captured; // a call that writes the projection is part of a graph, which may run at any time
   bool read_early;          // the last decode step read the projection ahead of its dependency wait
   bool step_deferred;       // the last decode step took the variant with the deferred selection
+  bool step_duo;            // the last decode step ran two blocks per SM
+  bool cluster_forced;      // the caller has set a cluster size
   int wait_tries;           // tries after which waits for other blocks of a cluster give up
   bool use_pdl;             // launch the decode kernel with programmatic stream serialization
+  int duo_active[BPC_MAX_CLUSTER + 1];   // [cs]: resident clusters with two blocks per SM (0 = variant not used)
+  int duo_cap;              // keys such a block can hold
   bool streaming;           // the scores of a full unit do not fit the largest cluster: two-pass (streaming) selection
   float* P;                 // [hash_sets][b][D] float
   void*  P_h;               // [hash_sets][b][D] cache dtype (the hash function)
@@ -134,12 +139,23 @@ struct DecodeParams {
   int wait_tries;            // tries after which the wait for the appended key's score gives up
   int early_projection;      // the projection may be read before the programmatic dependency wait (see the kernel)
   int key_shift_min;         // weighted scores: smallest right shift of the stored 16-bit keys (diagnostic; normally 0)
+  // two blocks per SM (batches of unequal lengths): clusters in the first layer, those that share their SMs, sequences by length
+  int duo_first, duo_pairs;
+  uint8_t duo_order[BPC_DUO_MAX_BATCH];
 };
 
 // ---- launchers implemented in the per-dtype translation units
 
 // ---- launch geometry (api.cu): fills max_cluster, max_active, chunk_cap_limit and picks cluster_size (0 = none fits)
 cudaError_t bpc_plan_decode_geometry(bpc_ctx* ctx);
+
+// ---- batches of unequal lengths: plan of a launch with two blocks per SM (api.cu)
+struct bpc_duo_plan {
+  int cluster, chunk;       // blocks per unit, keys they are sized for
+  int first, pairs;         // clusters in the first layer, those that share their SMs with one of the second
+  uint8_t order[BPC_DUO_MAX_BATCH];   // sequences, longest first
+};
+bool bpc_plan_duo(const bpc_ctx* ctx, const int32_t* lens, bpc_duo_plan* plan);
 
 // ---- a kernel that may be scheduled while its predecessor in the stream drains; it starts with pdl_wait()
 template <typename... P, typename... A>

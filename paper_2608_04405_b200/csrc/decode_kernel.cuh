@@ -79,11 +79,11 @@ template <typename KV> struct IsBf16 { static constexpr bool value = false; };
 template <> struct IsBf16<__nv_bfloat16> { static constexpr bool value = true; };
 
 // Shared-memory plan of one block, computed identically on host and device.
-template <typename KV, int GP, int W32>
+template <typename KV, int GP, int W32, int DUO = 0>      // DUO: 1 = two blocks per SM, 2 = the same with weighted scores
 struct DecodeSmem {
   typedef typename KvTraits<KV>::acc_t acc_t;
   static constexpr bool kMma = IsBf16<KV>::value;
-  static constexpr int NT = kMma ? 512 : (GP <= 2 ? 512 : 256);
+  static constexpr int NT = DUO ? 256 : kMma ? 512 : (GP <= 2 ? 512 : 256);
   static constexpr int NW = NT / 32;
   static constexpr int B = W32 * 32;
   static constexpr int kRowBytes = BPC_D * (int)sizeof(KV);
@@ -115,7 +115,7 @@ struct DecodeSmem {
     off_qf = off_tot + nb;                                           // float[GP+1][128]
     off_pd = off_qf + (size_t)GV * BPC_D * 4;                        // double[GP+1][B]
     off_idx = off_pd + (size_t)GV * B * 8;                           // int32[kIdxTile]
-    off_cta = off_idx + kIdxTile * 4;                                // merge inbox: acc_t[GP * (128 + 2 * 16) + 16]
+    off_cta = off_idx + (DUO == 1 ? 0 : kIdxTile * 4);                                // merge inbox: acc_t[GP * (128 + 2 * 16) + 16]
     off_small = a16(off_cta + ((size_t)GP * (BPC_D + 2 * BPC_MAX_CLUSTER) + BPC_MAX_CLUSTER) * sizeof(acc_t));
     off_union = a16(off_small + sizeof(SmallState));
     size_t u = score_bytes(chunk_cap, key_bytes);                                  // score keys
@@ -404,22 +404,35 @@ __device__ __noinline__ void careful_sweep(const double* t0, const float* gram, 
   }
 }
 
+// Which unit the cluster at a position of the grid works on (batches of unequal lengths, two blocks per SM).  Clusters fill
+// an empty device breadth-first (which is why this variant is launched, and lets its successor be launched, only when the kernel
+// before has gone: on a device that is still draining long units end up side by side, 56 us instead of 49), so with A of them in the first layer the cluster at position A + i shares its SMs with the one at
+// position i.  Units are ranked by length; the longest have their SMs to themselves, each next one is paired with the shortest left.
+__device__ __forceinline__ int duo_unit(const DecodeParams& p, int pos) {
+  const int units = gridDim.x / cg::this_cluster().num_blocks(), alone = p.duo_first - p.duo_pairs;
+  const int r = pos < p.duo_pairs ? alone + pos : pos < p.duo_first ? pos - p.duo_pairs : units - 1 - (pos - p.duo_first);
+  return p.duo_order[r / p.n_kv_heads] * p.n_kv_heads + r % p.n_kv_heads;
+}
+
 // VAR selects what is compiled in besides the plain path (VAR = 0): 1 = the error-aware safeguard (a static
 // hard-to-hash set that is always attended); 2 = the streaming selection for units whose scores do not fit the
 // cluster's shared memory (no score is stored: the scan keeps one histogram per warp over that warp's contiguous key
 // range, and after the threshold is known every warp reads its codes a second time and emits its selection in order);
 // 3 = byte score keys: Hamming scores with at most 256 distinct keys are stored one byte per key, unpadded, so that a
 // block holds 2.5 times as many (contexts of a million keys and more in clusters that are all resident at once);
-// 4 = the deferred selection for steps that append a key and whose blocks have few keys (see there).
+// 4 = the deferred selection for steps that append a key and whose blocks have few keys (see there);
+// 5 = blocks of half the size, two to an SM, for batches of unequal lengths: long units share their SMs with short ones.
 template <typename KV, int GP, int W32, int MODE, int VAR>
-__global__ void __launch_bounds__((DecodeSmem<KV, GP, W32>::NT), 1)
+__global__ void __launch_bounds__((DecodeSmem<KV, GP, W32, VAR == 5 ? MODE + 1 : 0>::NT), VAR == 5 ? 2 : 1)
 bpc_decode_kernel(const DecodeParams p) {
   constexpr int EAS = VAR == 1 ? 1 : 0;
   constexpr bool STREAM = VAR == 2;
   constexpr bool K8 = VAR == 3;
   constexpr bool kDefer = VAR == 4;
   static_assert(!(K8 || kDefer) || MODE == 0, "byte keys and the deferred selection are for Hamming scores");
-  typedef DecodeSmem<KV, GP, W32> L;
+  constexpr bool kDuo = VAR == 5;
+  static_assert(!kDuo || IsBf16<KV>::value, "");             // (the index tile that Hamming scores leave out is the fp32 path's)
+  typedef DecodeSmem<KV, GP, W32, kDuo ? MODE + 1 : 0> L;
   typedef typename L::acc_t acc_t;
   constexpr int NT = L::NT, NW = L::NW, B = L::B;
   constexpr int NP = PlaneCount<GP, MODE>::value;
@@ -431,7 +444,7 @@ bpc_decode_kernel(const DecodeParams p) {
   cg::cluster_group cluster = cg::this_cluster();
   const int CS = (int)cluster.num_blocks();
   const int rank = (int)cluster.block_rank();
-  const int unit = blockIdx.x / CS;
+  const int unit = kDuo ? duo_unit(p, blockIdx.x / CS) : blockIdx.x / CS;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int G = p.group;
   const int kvh = unit % p.n_kv_heads;
@@ -470,7 +483,7 @@ bpc_decode_kernel(const DecodeParams p) {
   // was still running) nothing of the predecessor's output may be read before this point; afterwards the
   // successor's blocks may be scheduled as ours drain.  Both are no-ops for an ordinary launch.
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (!kDuo) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (!p.early_projection) {
 #pragma unroll
     for (int v = 0; v < HV; ++v) prow[v] = __ldcg(prow_src + v);

@@ -19,6 +19,18 @@ static cudaError_t configure_kernel(int device) {
   return cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
 }
 
+// Batches of unequal lengths, two blocks of half the size per SM (variant 5): see bpc_plan_duo.
+inline bool plan_duo(const bpc_ctx* ctx, DecodeParams* p, int* cluster) {
+  bpc_duo_plan d;
+  if (!bpc_plan_duo(ctx, ctx->host_lens, &d)) return false;
+  p->duo_first = d.first;
+  p->duo_pairs = d.pairs;
+  for (int i = 0; i < ctx->cfg.batch; ++i) p->duo_order[i] = d.order[i];
+  p->chunk_cap = d.chunk;
+  *cluster = d.cluster;
+  return true;
+}
+
 // Whether a step that appends a key is faster with the deferred selection (variant 4; the same results at any length).  That
 // variant does two things.  The sign sweep of the appended key runs beside the threshold search as well as beside the scan: worth it
 // while the sweep (about 3 us, 43 us at 256 bits from L2) outlasts the scan, up to some 6K keys per block and 20K at 256 bits, and
@@ -37,13 +49,28 @@ static bool defers(const bpc_ctx* ctx, const DecodeParams& p, const DecodeSmem<K
          (W32 == 8 && p.residual_correction != 0 && plan.union_room(p.chunk_cap, 2, kGramTriBytes));
 }
 
+// Shared memory a block may ask for: the device's opt-in maximum, or half an SM's where two blocks share one.
+template <int EAS>
+static cudaError_t block_smem(int device, int* bytes) {
+  if (EAS != 5) return cudaDeviceGetAttribute(bytes, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
+  int sm = 0, reserved = 0;
+  cudaError_t e = cudaDeviceGetAttribute(&sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, device);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, device);
+  *bytes = sm / 2 - reserved;
+  return e;
+}
+
 template <typename KV, int GP, int W32, int MODE, int EAS>
 static cudaError_t launch_one(bpc_ctx* ctx, const DecodeParams& p_in, cudaStream_t stream) {
-  typedef DecodeSmem<KV, GP, W32> L;
+  typedef DecodeSmem<KV, GP, W32, EAS == 5 ? MODE + 1 : 0> L;
   DecodeParams p = p_in;
   int optin = 0;
-  cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, ctx->device);
+  cudaError_t e = block_smem<EAS>(ctx->device, &optin);
   if (e != cudaSuccess) return e;
+  int cluster = ctx->cluster_size;
+  if constexpr (EAS == 5) {
+    if (!plan_duo(ctx, &p, &cluster)) return cudaErrorNotSupported;   // (the plain variant serves)
+  }
   constexpr int kKeyBytes = EAS == 3 ? 1 : 2;               // (variant 3 stores byte score keys)
   p.stages = L(p.chunk_cap, p.nbins, 3, kKeyBytes).total <= (size_t)optin ? 3 : 2;
   const size_t smem = L(p.chunk_cap, p.nbins, p.stages, kKeyBytes).total;
@@ -56,13 +83,13 @@ static cudaError_t launch_one(bpc_ctx* ctx, const DecodeParams& p_in, cudaStream
     ctx->decode_smem_set |= (size_t)1 << EAS;
   }
   cudaLaunchConfig_t lc = {};
-  lc.gridDim = dim3((unsigned)(ctx->units * ctx->cluster_size), 1, 1);
+  lc.gridDim = dim3((unsigned)(ctx->units * cluster), 1, 1);
   lc.blockDim = dim3(L::NT, 1, 1);
   lc.dynamicSmemBytes = smem;
   lc.stream = stream;
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)ctx->cluster_size;
+  at[0].val.clusterDim.x = (unsigned)cluster;
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
   // let the grid be scheduled while the previous kernel of the stream drains (the kernel waits for that
@@ -70,7 +97,7 @@ static cudaError_t launch_one(bpc_ctx* ctx, const DecodeParams& p_in, cudaStream
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[1].val.programmaticStreamSerializationAllowed = 1;
   lc.attrs = at;
-  lc.numAttrs = ctx->use_pdl ? 2 : 1;
+  lc.numAttrs = ctx->use_pdl && EAS != 5 ? 2 : 1;
   return cudaLaunchKernelEx(&lc, bpc_decode_kernel<KV, GP, W32, MODE, EAS>, p);
 }
 
@@ -78,9 +105,9 @@ static cudaError_t launch_one(bpc_ctx* ctx, const DecodeParams& p_in, cudaStream
 // hold next to a two-stage gather ring.
 template <typename KV, int GP, int W32, int MODE, int EAS>
 static cudaError_t limits_one(const bpc_ctx* ctx, int nbins, int* max_cluster, int* chunk_cap, size_t* smem_bytes) {
-  typedef DecodeSmem<KV, GP, W32> L;
+  typedef DecodeSmem<KV, GP, W32, EAS == 5 ? MODE + 1 : 0> L;
   int dev = ctx->device, optin = 0;
-  cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  cudaError_t e = block_smem<EAS>(dev, &optin);
   if (e != cudaSuccess) return e;
   const size_t fixed = L(0, nbins, 2).off_union;
   const size_t avail = (size_t)optin > fixed + 64 ? (size_t)optin - fixed - 64 : 0;

@@ -401,3 +401,49 @@ def test_rule_of_the_deferred_selection(dtype, bits, group, n, n_max, deferred):
     assert sess.ctx.step_deferred() == deferred
     sess.ctx.set_seq_lens(sess.lens)
     H.check_decode(sess, q, [0], {}, budget_ppm=20000, append=(k_new, v_new))
+
+
+@pytest.mark.parametrize("bits,group,batch,score,long", [
+    (128, 4, 16, 0, 40000), (256, 1, 16, 0, 40000), (256, 4, 17, 0, 32001), (128, 7, 16, 0, 40000), (64, 2, 16, 0, 60000),
+    (128, 4, 16, 1, 30000), (256, 2, 16, 1, 25000), (32, 4, 16, 0, 60000)])
+def test_two_blocks_per_sm(bits, group, batch, score, long):
+    """Batches of unequal lengths (down to empty ones) on blocks of half the size, against one block per SM: the same selection, codes
+    and cache rows; outputs that differ by the order of fp32 sums (averages of some hundred values of order one: 2^-24 each)."""
+    H = _harness()
+    heads, room = 8, 8
+    n_max = (long + room + 7) // 8 * 8
+    g = torch.Generator(device="cuda").manual_seed(7 * bits + batch)
+    kv, k, v = H.B.interleaved_kv(batch, heads, n_max, 128, torch.bfloat16)
+    for i in range(batch):
+        kv[i].normal_(generator=g)
+    P = torch.randn(batch * heads, bits, 128, device="cuda", generator=g) / 16
+    few = [0, 1, 31, 64, 900, 2047, 2048, 5000]
+    lens = [long if i % 5 == 2 else long - 777 * i if i % 5 == 4 else few[i % 8] for i in range(batch)]
+    new = [torch.randn(batch, n, 128, device="cuda", generator=g).to(torch.bfloat16) for n in (heads, heads, heads * group)]
+    got = []
+    for forced in (0, 1):
+        ctx = H.B.Context(H.B.make_config(batch, heads * group, heads, n_max, bits, torch.bfloat16, kv_row_stride=256, score_mode=score))
+        plain = ctx.get_cluster_size()
+        if forced:
+            H.B._check(H.B.lib.bpc_set_cluster_size(ctx._h, plain), "bpc_set_cluster_size")
+        ctx.set_projection(P)
+        ctx.set_seq_lens(lens)
+        codes = ctx.alloc_codes()
+        ctx.encode_keys(k, codes)
+        kv_c, kc, vc = H.B.interleaved_kv(batch, heads, n_max, 128, torch.bfloat16)
+        kv_c.copy_(kv)
+        sel = torch.zeros(batch * heads, n_max, dtype=torch.int32, device="cuda")
+        outs = []
+        for step in range(2):
+            outs.append(ctx.append_decode_attn(new[0], new[1], kc, vc, codes, new[2], budget_ppm=20000, sel_idx=sel).clone())
+            assert ctx.step_two_per_sm() == (not forced)
+        outs.append(ctx.decode_attn(new[2], kc, vc, codes, budget_ppm=0, budget_count=700, sel_idx=sel).clone())
+        assert ctx.last_device_error() == 0
+        got.append((outs, sel, codes, kv_c))
+    (outs0, sel0, codes0, kv0), (outs1, sel1, codes1, kv1) = got
+    assert torch.equal(codes0, codes1) and torch.equal(kv0, kv1)
+    for i in range(batch):
+        n = min(lens[i] + 2, 700)
+        assert torch.equal(sel0[i * heads:(i + 1) * heads, :n], sel1[i * heads:(i + 1) * heads, :n])
+    for a, b in zip(outs0, outs1):
+        assert torch.isfinite(a).all() and (a - b).abs().max().item() <= 64 * 2.0 ** -24 * max(1.0, b.abs().max().item())
