@@ -79,8 +79,11 @@ dots_kernel(const float* __restrict__ A, size_t a_set, const float* __restrict__
 // Blocks of 32 keys.  Decision values t = k P_h^T: a register-tiled product in fp64 (a thread owns 2 keys x 4 bits at a
 // time, four running sums per value), kept as fp32 in shared memory.  The greedy sweep u_i = sign(t_i), t_j -= u_i G_ij
 // (j > i) runs with one lane per column of a 32-bit block and four keys per warp: a decision is a shuffle, its corrections
-// one FMA per 32 columns.  fp64 issue bounds it; one thread per key with its own conversions and a column-by-column sweep
-// took 160 us at 4096 keys x 64 bits, where it filled 32 SMs.
+// one FMA per 32 columns, and a block's word is one ballot at its end, because a decided column keeps its decision value.  The
+// chunks of the projection are requested one ahead and the Gram matrix arrives by asynchronous copies, so that no global latency but
+// the first is waited for.  Bound by the product's fp64 issue and shared-memory reads (two channels a read) and by the chain of
+// decisions, with eight warps per SM to hide it.  4096 keys x 64 bits: 18.4 -> 12.3 us with those (160 with one thread per key, its
+// own conversions and a column-by-column sweep, which filled 32 SMs).
 constexpr int kEncThreads = 256;
 constexpr int kEncKeys = 32;
 constexpr int kEncBits = 64;                                         // bits of a projection pass
@@ -89,8 +92,8 @@ constexpr int kEncGramBits = 128;                                    // up to th
 
 template <int NB>
 struct EncSmem {
-  double k[kEncKeys][BPC_D + 1];
-  double p[kEncBits][kEncChannels + 1];
+  double k[kEncKeys][BPC_D + 2];                                     // (even strides: read two channels at a time)
+  double p[kEncBits][kEncChannels + 2];
   float t[kEncKeys][32 * NB + 1];
 };
 
@@ -104,13 +107,28 @@ encode_simple_kernel(const KV* __restrict__ k_cache, const float* __restrict__ P
   EncSmem<NB>& sm = *reinterpret_cast<EncSmem<NB>*>(smem);
   float* g_s = reinterpret_cast<float*>(smem + sizeof(EncSmem<NB>));     // [b][b] where it fits
   const int unit = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  pdl_wait();
   const int n = min(unit_lens[unit], n_max);
   if (blockIdx.x * kEncKeys >= n) return;                            // uniform over the block
   const int set = shared_sets ? unit % n_kv_heads : unit;
   const float* Pset = Phf + (size_t)set * b * BPC_D;
   const float* Gset = gram + (size_t)set * b * b;
   if (b <= kEncGramBits && residual_correction)
-    for (int i = tid; i < b * b / 4; i += kEncThreads) reinterpret_cast<float4*>(g_s)[i] = reinterpret_cast<const float4*>(Gset)[i];
+    for (int i = tid; i < b * b / 4; i += kEncThreads)               // (lands during the product)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(g_s + 4 * i)), "l"(Gset + 4 * i) : "memory");
+  // the rows of the projection one chunk ahead, in registers: chunk s holds channels 32 (s % 4) .. of bits 64 (s / 4) ..
+  constexpr int JN = (b < kEncBits ? b : kEncBits) / 16;             // bits of a thread: tx, tx + 16, ...
+  constexpr int kChunks = BPC_D / kEncChannels, kSteps = (b + kEncBits - 1) / kEncBits * kChunks;
+  constexpr int kAhead = 16 * JN * kEncChannels / kEncThreads;
+  float ahead[kAhead];
+  auto fetch = [&](int s) {
+#pragma unroll
+    for (int m = 0; m < kAhead; ++m) {
+      const int e = tid + m * kEncThreads;
+      ahead[m] = Pset[(size_t)(kEncBits * (s / kChunks) + e / kEncChannels) * BPC_D + kEncChannels * (s % kChunks) + e % kEncChannels];
+    }
+  };
+  fetch(0);
   for (int key0 = blockIdx.x * kEncKeys; key0 < n; key0 += gridDim.x * kEncKeys) {
     __syncthreads();
     for (int e = tid; e < kEncKeys * BPC_D; e += kEncThreads) {
@@ -119,7 +137,6 @@ encode_simple_kernel(const KV* __restrict__ k_cache, const float* __restrict__ P
     }
     const int tx = tid & 15, ty = tid >> 4;
     for (int j0 = 0; j0 < b; j0 += kEncBits) {
-      constexpr int JN = (b < kEncBits ? b : kEncBits) / 16;         // bits of a thread: tx, tx + 16, ...
       double acc[2][JN][4];
 #pragma unroll
       for (int r = 0; r < 2; ++r)
@@ -129,19 +146,25 @@ encode_simple_kernel(const KV* __restrict__ k_cache, const float* __restrict__ P
           for (int q = 0; q < 4; ++q) acc[r][j][q] = 0.0;
       for (int c0 = 0; c0 < BPC_D; c0 += kEncChannels) {
         __syncthreads();
-        for (int e = tid; e < 16 * JN * kEncChannels; e += kEncThreads)
-          sm.p[e / kEncChannels][e % kEncChannels] = (double)Pset[(size_t)(j0 + e / kEncChannels) * BPC_D + c0 + e % kEncChannels];
+#pragma unroll
+        for (int m = 0; m < kAhead; ++m) {
+          const int e = tid + m * kEncThreads;
+          sm.p[e / kEncChannels][e % kEncChannels] = (double)ahead[m];
+        }
+        fetch((j0 / kEncBits * kChunks + c0 / kEncChannels + 1) % kSteps);   // (behind the last chunk: the next keys' first)
         __syncthreads();
 #pragma unroll 2
         for (int c = 0; c < kEncChannels; c += 4) {
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const double k0 = sm.k[ty][c0 + c + q], k1 = sm.k[ty + 16][c0 + c + q];
+          for (int q = 0; q < 4; q += 2) {
+            const double2 k0 = *reinterpret_cast<const double2*>(&sm.k[ty][c0 + c + q]), k1 = *reinterpret_cast<const double2*>(&sm.k[ty + 16][c0 + c + q]);
 #pragma unroll
             for (int j = 0; j < JN; ++j) {
-              const double pv = sm.p[tx + 16 * j][c + q];
-              acc[0][j][q] = fma(k0, pv, acc[0][j][q]);
-              acc[1][j][q] = fma(k1, pv, acc[1][j][q]);
+              const double2 pv = *reinterpret_cast<const double2*>(&sm.p[tx + 16 * j][c + q]);
+              acc[0][j][q] = fma(k0.x, pv.x, acc[0][j][q]);
+              acc[1][j][q] = fma(k1.x, pv.x, acc[1][j][q]);
+              acc[0][j][q + 1] = fma(k0.y, pv.y, acc[0][j][q + 1]);
+              acc[1][j][q + 1] = fma(k1.y, pv.y, acc[1][j][q + 1]);
             }
           }
         }
@@ -152,6 +175,7 @@ encode_simple_kernel(const KV* __restrict__ k_cache, const float* __restrict__ P
         sm.t[ty + 16][j0 + tx + 16 * j] = (float)((acc[1][j][0] + acc[1][j][1]) + (acc[1][j][2] + acc[1][j][3]));
       }
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");                 // (the Gram matrix)
     __syncthreads();
     // sweep: keys 4 warp .. 4 warp + 3; lane = column of each 32-bit block
     float t[4][NB];
@@ -159,32 +183,33 @@ encode_simple_kernel(const KV* __restrict__ k_cache, const float* __restrict__ P
     for (int r = 0; r < 4; ++r)
 #pragma unroll
       for (int w = 0; w < NB; ++w) t[r][w] = sm.t[4 * warp + r][32 * w + lane];
-    double abs_sum[4] = {0.0, 0.0, 0.0, 0.0};                        // sums of |t_i| at decision time
+    double abs_sum[4] = {0.0, 0.0, 0.0, 0.0};                        // this lane's part of the sums of |t_i| at decision time
 #pragma unroll
     for (int cb = 0; cb < NB; ++cb) {
-      uint32_t word[4] = {0u, 0u, 0u, 0u};
-      for (int i = 0; i < 32; ++i) {
-        float g[NB];
-        if (residual_correction) {
+      // (a column takes no more corrections once it is decided: after the block lane i still holds decision value i)
+      if (residual_correction) {
+#pragma unroll 8
+        for (int i = 0; i < 32; ++i) {
+          float g[NB];
 #pragma unroll
           for (int w = cb; w < NB; ++w) {
             const size_t at = (size_t)(32 * cb + i) * b + 32 * w + lane;
             g[w] = b <= kEncGramBits ? g_s[at] : __ldg(Gset + at);
           }
-        }
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          const float ti = __shfl_sync(0xffffffffu, t[r][cb], i);
-          const bool pos = ti >= 0.f;
-          word[r] |= (pos ? 1u : 0u) << i;
-          if (key_err != nullptr) abs_sum[r] += (double)fabsf(ti);
-          if (residual_correction) {
-            const float u = pos ? 1.f : -1.f;
-            if (lane > i) t[r][cb] -= u * g[cb];
+          for (int r = 0; r < 4; ++r) {
+            const float nu = __shfl_sync(0xffffffffu, t[r][cb], i) >= 0.f ? -1.f : 1.f;
+            if (lane > i) t[r][cb] = fmaf(nu, g[cb], t[r][cb]);
 #pragma unroll
-            for (int w = cb + 1; w < NB; ++w) t[r][w] -= u * g[w];
+            for (int w = cb + 1; w < NB; ++w) t[r][w] = fmaf(nu, g[w], t[r][w]);
           }
         }
+      }
+      uint32_t word[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        word[r] = __ballot_sync(0xffffffffu, t[r][cb] >= 0.f);
+        if (key_err != nullptr) abs_sum[r] += (double)fabsf(t[r][cb]);       // (this lane's columns)
       }
       if (lane < 4 && key0 + 4 * warp + lane < n) {
         const uint32_t v = lane == 0 ? word[0] : lane == 1 ? word[1] : lane == 2 ? word[2] : word[3];
@@ -197,12 +222,12 @@ encode_simple_kernel(const KV* __restrict__ k_cache, const float* __restrict__ P
       for (int i = lane; i < b; i += 32) trg += (double)__ldg(Gset + (size_t)i * b + i);
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
-        double v = trg;
+        double v = trg - 2.0 * abs_sum[r];
         for (int c = lane; c < BPC_D; c += 32) v = fma(sm.k[4 * warp + r][c], sm.k[4 * warp + r][c], v);
 #pragma unroll
         for (int o = 16; o >= 1; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         if (lane == 0 && key0 + 4 * warp + r < n)
-          key_err[(size_t)unit * n_max + key0 + 4 * warp + r] = (float)fmax(0.0, v - 2.0 * abs_sum[r]);
+          key_err[(size_t)unit * n_max + key0 + 4 * warp + r] = (float)fmax(0.0, v);
       }
     }
   }
@@ -769,11 +794,11 @@ static cudaError_t launch_encode_simple(bpc_ctx* ctx, const void* k_cache, uint6
   int blocks = (c.n_max + kEncKeys - 1) / kEncKeys;
   const int most = (8 * ctx->sm_count + ctx->units - 1) / ctx->units;
   if (blocks > most) blocks = most;
-  encode_simple_kernel<KV, NB><<<dim3(blocks, ctx->units), kEncThreads, smem, stream>>>(
+  e = launch_pdl(ctx->use_pdl, encode_simple_kernel<KV, NB>, dim3(blocks, ctx->units), kEncThreads, smem, stream,
       (const KV*)k_cache, ctx->P_hf, ctx->gram, ctx->unit_lens, codes, c.n_kv_heads, c.n_max, ctx->row_stride, c.hash_sets != ctx->units,
       c.residual_correction, ctx->key_err);
   ctx->launches += 1;
-  return cudaGetLastError();
+  return e;
 }
 
 template <typename KV>
