@@ -268,24 +268,33 @@ cudaError_t bpc_plan_decode_geometry(bpc_ctx* ctx) {
 // Two blocks of half the size per SM for batches of unequal lengths.  With one block per SM a launch takes as long as its longest
 // unit, whose SMs work at what one SM can load while those of the short units are idle; here the work of an SM is one of the longest
 // units or one long and one short.  Step, 16 sequences of 16K to 64K keys x 8 heads, 2 %: 128 bits 56.9 -> 49.0 to 52.6 us by the lengths
-// drawn, 256 bits 90.2 -> 83.0 (there the sign sweep of the appended key, from L2, holds up the short units).  The variant costs some 8 us (no overlap with the kernels around it, half the gather ring), so it is taken where the busiest SM saves as many keys
-// as take that long to scan and gather: 0.25 us per 1000 keys for the gather at 2 %, and for the scan 0.4 at 128 bits (0.64 with
-// weighted scores) in proportion to the code length.
+// drawn, 256 bits 90.2 -> 83.0 (there the sign sweep of the appended key, from L2, holds up the short units).  The variant costs some
+// 8 us (no overlap with the kernels around it, half the gather ring), so it is taken where the busiest SM saves as many keys as take
+// that long to scan and gather: 0.25 us per 1000 keys for the gather at 2 %, and for the scan 0.4 at 128 bits (0.64 with weighted
+// scores) in proportion to the code length.
 bool bpc_plan_duo(const bpc_ctx* ctx, const int32_t* lens, bpc_duo_plan* plan) {
   const int batch = ctx->cfg.batch, heads = ctx->cfg.n_kv_heads, units = ctx->units;
   if (ctx->duo_cap <= 0 || batch < 2 || batch > BPC_DUO_MAX_BATCH) return false;
+  const double scan = (ctx->cfg.score_mode == BPC_SCORE_WEIGHTED7 ? 0.64 : 0.4) * ctx->cfg.code_bits / 128;
+  const double least = 9500.0 / (0.25 + scan);              // keys of an SM that pay for the variant
+  int longest = 0;
+  for (int i = 0; i < batch; ++i) longest = lens[i] > longest ? lens[i] : longest;
+  if (longest <= least * ctx->cluster_size) return false;   // (most steps end here)
   int cs = 0;
   for (int c = 1; c <= BPC_MAX_CLUSTER; ++c)
     if (ctx->duo_active[c] >= units && chunk_for(ctx->cfg.n_max, c) <= ctx->duo_cap) cs = c;
   if (cs == 0) return false;
   const int first = ctx->duo_active[cs] / 2, pairs = units - first;
-  if (pairs <= 0) return false;
+  if (pairs <= 0 || pairs > first || units > 65535) return false;
+  uint8_t order[BPC_DUO_MAX_BATCH];
   for (int i = 0; i < batch; ++i) {                         // longest first
     int j = i;
-    for (; j > 0 && lens[plan->order[j - 1]] < lens[i]; --j) plan->order[j] = plan->order[j - 1];
-    plan->order[j] = (uint8_t)i;
+    for (; j > 0 && lens[order[j - 1]] < lens[i]; --j) order[j] = order[j - 1];
+    order[j] = (uint8_t)i;
   }
-  auto len = [&](int rank) { return (long long)lens[plan->order[rank / heads]]; };
+  plan->order = 0;
+  for (int i = 0; i < batch; ++i) plan->order |= (unsigned long long)order[i] << (4 * i);
+  auto len = [&](int rank) { return (long long)lens[order[rank / heads]]; };
   const int alone = first - pairs;
   long long load = alone > 0 ? len(0) : 0;
   for (int i = 0; i < pairs; ++i) {
@@ -296,8 +305,7 @@ bool bpc_plan_duo(const bpc_ctx* ctx, const int32_t* lens, bpc_duo_plan* plan) {
   plan->chunk = chunk_for(ctx->cfg.n_max, cs);
   plan->first = first;
   plan->pairs = pairs;
-  const double scan = (ctx->cfg.score_mode == BPC_SCORE_WEIGHTED7 ? 0.64 : 0.4) * ctx->cfg.code_bits / 128;
-  return (double)len(0) / ctx->cluster_size - (double)load / cs > 9500.0 / (0.25 + scan);
+  return (double)len(0) / ctx->cluster_size - (double)load / cs > least;
 }
 
 extern "C" {

@@ -19,7 +19,7 @@
 // In a launch that also appends, the block that codes the new key scans with fewer resources (one warp runs
 // Algorithm 2's sign sweep); it is given (16 - BPC_APPEND_LOSS16)/16 of the other blocks' key share.
 #define BPC_APPEND_LOSS16 2
-#define BPC_DUO_MAX_BATCH 64       // sequences a launch with two blocks per SM can rank
+#define BPC_DUO_MAX_BATCH 16       // sequences a launch with two blocks per SM can rank
 __host__ __device__ inline int bpc_fused_chunk(int n, int cs) {
   // n <= 2^26 (bpc_create rejects larger n_max), so 32-bit arithmetic is exact here; a 64-bit division by a run-time
   // divisor would cost every thread of the kernel some hundred instructions
@@ -140,8 +140,9 @@ struct DecodeParams {
   int early_projection;      // the projection may be read before the programmatic dependency wait (see the kernel)
   int key_shift_min;         // weighted scores: smallest right shift of the stored 16-bit keys (diagnostic; normally 0)
   // two blocks per SM (batches of unequal lengths): clusters in the first layer, those that share their SMs, sequences by length
-  int duo_first, duo_pairs;
-  uint8_t duo_order[BPC_DUO_MAX_BATCH];
+  // (four bits each)
+  unsigned long long duo_order;
+  uint16_t duo_first, duo_pairs;
 };
 
 // ---- launchers implemented in the per-dtype translation units
@@ -153,7 +154,7 @@ cudaError_t bpc_plan_decode_geometry(bpc_ctx* ctx);
 struct bpc_duo_plan {
   int cluster, chunk;       // blocks per unit, keys they are sized for
   int first, pairs;         // clusters in the first layer, those that share their SMs with one of the second
-  uint8_t order[BPC_DUO_MAX_BATCH];   // sequences, longest first
+  unsigned long long order; // sequences, longest first (the longest in the lowest four bits)
 };
 bool bpc_plan_duo(const bpc_ctx* ctx, const int32_t* lens, bpc_duo_plan* plan);
 

@@ -411,7 +411,7 @@ __device__ __noinline__ void careful_sweep(const double* t0, const float* gram, 
 __device__ __forceinline__ int duo_unit(const DecodeParams& p, int pos) {
   const int units = gridDim.x / cg::this_cluster().num_blocks(), alone = p.duo_first - p.duo_pairs;
   const int r = pos < p.duo_pairs ? alone + pos : pos < p.duo_first ? pos - p.duo_pairs : units - 1 - (pos - p.duo_first);
-  return p.duo_order[r / p.n_kv_heads] * p.n_kv_heads + r % p.n_kv_heads;
+  return (int)((p.duo_order >> (4 * (r / p.n_kv_heads))) & 15u) * p.n_kv_heads + r % p.n_kv_heads;
 }
 
 // VAR selects what is compiled in besides the plain path (VAR = 0): 1 = the error-aware safeguard (a static

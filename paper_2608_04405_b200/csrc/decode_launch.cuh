@@ -23,9 +23,9 @@ static cudaError_t configure_kernel(int device) {
 inline bool plan_duo(const bpc_ctx* ctx, DecodeParams* p, int* cluster) {
   bpc_duo_plan d;
   if (!bpc_plan_duo(ctx, ctx->host_lens, &d)) return false;
-  p->duo_first = d.first;
-  p->duo_pairs = d.pairs;
-  for (int i = 0; i < ctx->cfg.batch; ++i) p->duo_order[i] = d.order[i];
+  p->duo_first = (uint16_t)d.first;
+  p->duo_pairs = (uint16_t)d.pairs;
+  p->duo_order = d.order;
   p->chunk_cap = d.chunk;
   *cluster = d.cluster;
   return true;

@@ -404,7 +404,7 @@ def test_rule_of_the_deferred_selection(dtype, bits, group, n, n_max, deferred):
 
 
 @pytest.mark.parametrize("bits,group,batch,score,long", [
-    (128, 4, 16, 0, 40000), (256, 1, 16, 0, 40000), (256, 4, 17, 0, 32001), (128, 7, 16, 0, 40000), (64, 2, 16, 0, 60000),
+    (128, 4, 16, 0, 40000), (256, 1, 16, 0, 40000), (256, 4, 15, 0, 32001), (128, 7, 16, 0, 40000), (64, 2, 16, 0, 60000),
     (128, 4, 16, 1, 30000), (256, 2, 16, 1, 25000), (32, 4, 16, 0, 60000)])
 def test_two_blocks_per_sm(bits, group, batch, score, long):
     """Batches of unequal lengths (down to empty ones) on blocks of half the size, against one block per SM: the same selection, codes
