@@ -579,8 +579,8 @@ fit_gather_f32_kernel(const float* __restrict__ k_cache, const uint32_t* __restr
 // The bit-major words stay in registers where a warp has one group of keys, in tensor memory (a scratchpad here: the kernel
 // issues no tcgen05.mma) beside key-major words in shared memory, and over column 0 of T, which is dead after bit 0, where a block
 // has more keys than fit on chip.
-// Precision: T enters the sums as a 32-bit integer with a power-of-two scale, 2^-30 or finer of the largest |T| of the unit's block
-// of columns; everything after that is exact up to the fp64 scalars.  A key's own T stays the fp32 value.
+// Precision: T enters the sums as a 32-bit integer with a power-of-two scale, rounded by at most 2^-30 of the largest |T| of the
+// unit's block of columns; everything after that is exact up to the fp64 scalars.  A key's own T stays the fp32 value.
 
 constexpr int kOneGroup = 0, kWordsOnChip = 1, kWordsGlobal = 2;
 
