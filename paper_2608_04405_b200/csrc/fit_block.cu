@@ -1125,6 +1125,156 @@ fit_rows_kernel(const double* __restrict__ wpart, const int32_t* __restrict__ ap
   }
 }
 
+// The same in one launch, for a few units (see bpc_launch_fit_blocked): a cluster per unit adds the partial sums, forms the rows and then
+// the next block's scalars C = V D_next^T.  Block r of the cluster owns 16 channels of the rows, 1 / 8 of the inner products (sums sent to
+// every block) and 1 / 8 of the scalars.  Nothing here is limited by a rate of the chip but by a launch, a round of loads, two cluster
+// barriers and a chain of 32 FMAs, so every load is requested at the start, and both contractions take four rows per thread
+// and split their sums over the warps (with one output per thread they were bound by shared-memory reads, two per FMA).  Three kernels
+// take 21 to 27 us per 32 bits of 8 x 32K keys, this one 12 to 15.
+// The rows of the block enter each other's corrections in fp64, before they are rounded.
+constexpr int kFinishBlocks = 8;
+constexpr int kFinishThreads = 512;
+constexpr int kFinishChannels = BPC_D / kFinishBlocks;
+constexpr int kFinishRows = kBits / kFinishBlocks;         // rows of inner products, and per 32 bits so far of scalars, of a block
+constexpr int kFinishSlices = 4;                           // of the sum over the earlier rows
+constexpr int kDirStride = BPC_D + 1, kRowStride = kFinishChannels + 1;
+static_assert(kBits * kFinishChannels == kFinishThreads && kFinishChannels == kFinishThreads / 32, "a thread per row and channel; a warp per channel");
+static_assert(kFinishRows == 4 && kFinishThreads / 32 == 16, "four rows per thread, sums split over the warps");
+
+struct FinishSmem {                                        // (doubles)
+  int corr, v, w, d, p, part, total;                       // u_i . u_j over n; earlier rows, own channels; sums; next directions; rows of the own scalars; partial sums
+  __host__ __device__ explicit FinishSmem(int blk) {
+    corr = 0;                                              // [32][32 (blk + 1) + 2]
+    v = corr + kBits * (kBits * (blk + 1) + 2);            // [32 blk][16]
+    w = v + kBits * blk * kFinishChannels;                 // [4][32][17]
+    d = w + kFinishSlices * kBits * kRowStride;            // [32][129]
+    p = d + kBits * kDirStride;                            // [4 (blk + 1)][128]
+    part = p + kFinishRows * (blk + 1) * BPC_D;            // [16 warps][4][32]
+    total = part + 16 * kFinishRows * kBits;
+  }
+};
+
+__device__ __forceinline__ void store_peer(const double* dst, int r, double v) {
+  asm volatile("{\n\t.reg .b32 d;\n\tmapa.shared::cluster.u32 d, %0, %1;\n\tst.shared::cluster.f64 [d], %2;\n\t}\n" ::"r"(smem_u32(dst)), "r"(r), "d"(v) : "memory");
+}
+
+__global__ void __cluster_dims__(kFinishBlocks, 1, 1) __launch_bounds__(kFinishThreads, 1)
+fit_finish_kernel(const double* __restrict__ wpart, const int32_t* __restrict__ apart, const float* __restrict__ v_star, float* __restrict__ P,
+                  float* __restrict__ cross, const int32_t* __restrict__ unit_lens, int n_max, int b, int blk, int parts) {
+  extern __shared__ __align__(16) double finish_smem[];
+  const FinishSmem at(blk);
+  const int nj = kBits * (blk + 1), np = kBits * blk, cstride = nj + 2;
+  double *corr = finish_smem + at.corr, *v_s = finish_smem + at.v, *w_s = finish_smem + at.w, *d_s = finish_smem + at.d, *p_s = finish_smem + at.p,
+         *part_s = finish_smem + at.part;
+  const int rank = blockIdx.x % kFinishBlocks, unit = blockIdx.x / kFinishBlocks, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int i = tid / kFinishChannels, c = tid % kFinishChannels;        // this thread's row and channel
+  const int n = min(unit_lens[unit], n_max);
+  float* Pu = P + (size_t)unit * b * BPC_D;
+  if (n <= 0) {                                            // (the whole cluster)
+    Pu[(size_t)(np + i) * BPC_D + kFinishChannels * rank + c] = 0.f;
+    return;
+  }
+  const bool last = nj == b;                               // no further block
+  const int rows = block_rows(n, parts), used = (n + rows - 1) / rows;
+  const double inv_n = 1.0 / (double)n;
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  constexpr int kDirs = kBits * BPC_D / kFinishThreads;
+  float dir[kDirs];
+  if (!last) {
+#pragma unroll
+    for (int k = 0; k < kDirs; ++k) dir[k] = v_star[((size_t)unit * b + nj) * BPC_D + tid + k * kFinishThreads];
+  }
+  const double* w = wpart + (size_t)unit * parts * kBits * BPC_D + (size_t)i * BPC_D + kFinishChannels * rank + c;
+  double ws = w[0];
+#pragma unroll 16
+  for (int p = 1; p < used; ++p) ws += w[(size_t)p * kBits * BPC_D];
+  const int32_t* a = apart + ((size_t)unit * parts * kBits + kFinishRows * rank) * b;   // inner products of rows 4 rank .. 4 rank + 3
+  auto product = [&](int e) {
+    int s = 0;
+#pragma unroll 16
+    for (int p = 0; p < used; ++p) s += a[(size_t)p * kBits * b + (size_t)(e / nj) * b + e % nj];
+    return s;
+  };
+  const int first = tid < kFinishRows * nj ? product(tid) : 0;
+  for (int j = i; j < np; j += kBits) v_s[j * kFinishChannels + c] = (double)Pu[(size_t)j * BPC_D + kFinishChannels * rank + c];
+  if (!last) {
+#pragma unroll
+    for (int k = 0; k < kDirs; ++k) {
+      const int e = tid + k * kFinishThreads;
+      d_s[(e >> 7) * kDirStride + (e & 127)] = (double)dir[k];
+    }
+  }
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");    // (every block of the cluster runs: its shared memory may be written)
+  for (int e = tid; e < kFinishRows * nj; e += kFinishThreads) {
+    const double v = (double)(e == tid ? first : product(e)) * inv_n;
+#pragma unroll
+    for (int q = 0; q < kFinishBlocks; ++q) store_peer(corr + (size_t)(kFinishRows * rank + e / nj) * cstride + e % nj, q, v);
+  }
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  {                                                        // earlier rows: four rows and a quarter of the sum per thread
+    const int slice = tid >> 7, r0 = 4 * ((tid >> 4) & 7);
+    double x[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 2
+    for (int j = slice * (np / kFinishSlices); j < (slice + 1) * (np / kFinishSlices); j += 2) {
+      const double v0 = v_s[j * kFinishChannels + c], v1 = v_s[(j + 1) * kFinishChannels + c];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const double2 k = *reinterpret_cast<const double2*>(corr + (r0 + q) * cstride + j);
+        x[q] = fma(k.x, v0, x[q]);
+        x[q] = fma(k.y, v1, x[q]);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) w_s[(slice * kBits + r0 + q) * kRowStride + c] = x[q];
+    __syncthreads();
+    const double* y = w_s + i * kRowStride + c;
+    const double sum = (y[0] + y[kBits * kRowStride]) + (y[2 * kBits * kRowStride] + y[3 * kBits * kRowStride]);
+    w_s[i * kRowStride + c] = fma(ws, inv_n, -sum);        // (its own place; the other slices are not read again)
+  }
+  __syncthreads();
+  {                                                        // the block's own triangle: a warp per channel, a row per lane
+    double x = w_s[lane * kRowStride + warp];
+    const double* col = corr + (size_t)lane * cstride + np;
+#pragma unroll 4
+    for (int k = 0; k < kBits; ++k) {
+      const double v = __shfl_sync(0xffffffffu, x, k);
+      if (lane > k) x = fma(-col[k], v, x);
+    }
+    Pu[(size_t)(np + lane) * BPC_D + kFinishChannels * rank + warp] = (float)x;
+  }
+  if (last) return;                                        // (nobody writes to another block any more)
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");    // the unit's new rows are in memory
+  const int groups = blk + 1;                              // of four rows: this block's scalars
+  for (int e = tid; e < kFinishRows * groups * BPC_D; e += kFinishThreads) p_s[e] = (double)__ldcg(Pu + (size_t)kFinishRows * groups * rank * BPC_D + e);
+  __syncthreads();
+  const int slices = 16 / groups, slice = warp / groups, grp = warp % groups;   // (warps beyond groups x slices: none)
+  if (slice < slices) {
+    const int k0 = BPC_D * slice / slices & ~1, k1 = BPC_D * (slice + 1) / slices & ~1;
+    double x[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 2
+    for (int k = k0; k < k1; k += 2) {
+      const double d0 = d_s[lane * kDirStride + k], d1 = d_s[lane * kDirStride + k + 1];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const double2 v = *reinterpret_cast<const double2*>(p_s + (4 * grp + q) * BPC_D + k);
+        x[q] = fma(v.x, d0, x[q]);
+        x[q] = fma(v.y, d1, x[q]);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) part_s[(warp * 4 + q) * kBits + lane] = x[q];
+  }
+  __syncthreads();
+  for (int e = tid; e < kFinishRows * groups * kBits; e += kFinishThreads) {   // row e / 32 of the block's, column e % 32
+    const int q = e >> 5;
+    double s = 0.0;
+    for (int sl = 0; sl < slices; ++sl) s += part_s[((sl * groups + (q >> 2)) * 4 + (q & 3)) * kBits + (e & 31)];
+    cross[((size_t)unit * b + kFinishRows * groups * rank) * kBits + e] = (float)s;
+  }
+}
+
 // --------------------------------------------------------------------------- host side
 constexpr int kSms = 148;
 constexpr int kSweepMaxKeys = 1 << 24;                     // keys of a sweep block
@@ -1288,11 +1438,15 @@ cudaError_t bpc_launch_fit_blocked(bpc_ctx* ctx, const void* k_cache, const floa
   if (cs == 0) return cudaErrorNotSupported;
   const size_t sweep_smem = (size_t)sweep_share(c.n_max, cs) * 4;
   const bool tc = c.kv_dtype == BPC_BF16;
+  // One kernel after the gather while all its clusters are resident at once (15 of eight blocks, one to an SM; a guess that is wrong
+  // on some device costs time only).  Fits of 32K keys and 128 bits: 4 units 532 -> 506 us, 8 units 598 -> 569, 12 units 673 -> 657, but
+  // 16 units 854 -> 875.
+  const bool one_finish = ctx->units <= 15;
   const dim3 grid(parts, ctx->units);
   CUtensorMap kmap;
   if (tc) e = tma::make_key_map(&kmap, k_cache, (unsigned long long)ctx->units * c.n_max, ctx->row_stride);
   for (int blk = 0; blk < b / kBits && e == cudaSuccess; ++blk) {
-    if (blk > 0) {                                         // cross[j][l] = v_j . d_l for the bits so far and this block's columns
+    if (blk > 0 && !one_finish) {                          // cross[j][l] = v_j . d_l for the bits so far and this block's columns
       const size_t set = (size_t)b * BPC_D;
       e = bpc_launch_dots(ctx->P, set, v_star + (size_t)kBits * blk * BPC_D, set, cross, (size_t)b * kBits, kBits, blk, 1, ctx->units, stream);
       if (e != cudaSuccess) return e;
@@ -1324,6 +1478,15 @@ cudaError_t bpc_launch_fit_blocked(bpc_ctx* ctx, const void* k_cache, const floa
       fit_gather_f32_kernel<<<grid, 256, 0, stream>>>((const float*)k_cache, hfit, wpart, apart, ctx->unit_lens, c.n_max, ctx->row_stride, b, blk);
     }
     if (e != cudaSuccess) return e;
+    if (one_finish) {
+      e = allow_smem(fit_finish_kernel);
+      if (e != cudaSuccess) return e;
+      fit_finish_kernel<<<kFinishBlocks * ctx->units, kFinishThreads, FinishSmem(blk).total * sizeof(double), stream>>>(
+          wpart, apart, v_star, ctx->P, cross, ctx->unit_lens, c.n_max, b, blk, parts);
+      e = cudaGetLastError();
+      *launches += 4;
+      continue;
+    }
     fit_sum_parts_kernel<<<dim3(16 + 4 * (blk + 1), ctx->units), 256, 0, stream>>>(wpart, apart, ctx->unit_lens, c.n_max, b, blk, parts);
     const size_t rows_smem = (size_t)(kBits * kBits * (blk + 1) + kBits * blk * 32 + kBits * 32) * 8;
     e = allow_smem(fit_rows_kernel);
