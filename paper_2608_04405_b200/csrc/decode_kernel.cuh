@@ -127,7 +127,14 @@ struct DecodeSmem {
   }
 };
 
-__device__ __forceinline__ int score_slot(int i) { return (i >> 5) * kSegSlots + (i & 31); }
+// Where the score key of key i of a block lies: keys j and j + 16 of a segment share a word (byte keys: j, j + 8, j + 16, j + 24), so
+// that flags at the tops of the halves (bytes), collected by shifting right once per word, end up in the order of the keys.
+__device__ __forceinline__ int lane_slot(int j) { return 2 * (j & 15) + (j >> 4); }
+__device__ __forceinline__ int lane_byte(int j) { return 4 * (j & 7) + (j >> 3); }
+__device__ __forceinline__ int score_slot(int i) { return (i >> 5) * kSegSlots + lane_slot(i & 31); }
+__device__ __forceinline__ int score_byte(int i) { return (i & ~31) + lane_byte(i & 31); }
+// (a & b) or, where `any` is set, (a | b)
+__device__ __forceinline__ uint32_t both_or_any(uint32_t a, uint32_t b, uint32_t any) { return (a & b) | (any & (a | b)); }
 
 // Exclusive prefix sum over the NT threads of a block; *total receives the block sum.  One barrier per call: the warp
 // totals come from a warp reduction and are posted before each warp scans its own lanes, and consecutive calls
@@ -547,7 +554,7 @@ bpc_decode_kernel(const DecodeParams p) {
   SmallState* st = reinterpret_cast<SmallState*>(smem + plan.off_small);
   unsigned char* uni = smem + plan.off_union;
   uint16_t* sc = reinterpret_cast<uint16_t*>(uni);
-  [[maybe_unused]] uint8_t* sc8 = uni;                       // (byte-key variant: key i of the block at byte i)
+  [[maybe_unused]] uint8_t* sc8 = uni;                       // (byte-key variant: see score_byte)
   // Phase stamps (debug): slots 0 and 7 hold the global timer at block start and end, slots 15 and 14 the SM's cycle
   // counter at the same two points, every other slot the cycle counter (cheap to read) at that phase boundary.
 #define BPC_STAMP(i) do { if (p.dbg_times != nullptr && tid == 0) p.dbg_times[(size_t)blockIdx.x * 16 + (i)] = (unsigned long long)clock64(); } while (0)
@@ -826,21 +833,28 @@ bpc_decode_kernel(const DecodeParams p) {
       }
     }
     const int rfull = st->rsum << cs;                       // sum_j |A_j|
+    // (a warp's 32 keys are one segment: batches start at whole segments)
+    constexpr int kSegStep = K8 ? kSegKeys : kSegSlots;
+    [[maybe_unused]] const int own_slot = (stid >> 5) * kSegStep + (K8 ? lane_byte(lane) : lane_slot(lane)), next_slot = (nts >> 5) * kSegStep;
+    auto key_slot = [&](int base, int u) {                   // (256-bit codes: recomputed, their loop has no register to spare)
+      if constexpr (W32 == 8) return ((base - c0 + u * nts + stid) >> 5) * kSegStep + (K8 ? lane_byte(lane) : lane_slot(lane));
+      return ((base - c0) >> 5) * kSegStep + u * next_slot + own_slot;
+    };
     auto score_batch = [&](const uint32_t (&h)[U][W32], int base) {
       if constexpr (kWeighted) {
         int keys[U];
         weighted_keys<W32, U>(h, sg, wbase, keys);
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          sc[score_slot(base - c0 + u * nts + stid)] = (uint16_t)(keys[u] >> ksh);
+          sc[key_slot(base, u)] = (uint16_t)(keys[u] >> ksh);
           atomicAdd(&hist[(keys[u] >> ksh) >> hsh], 1u);
         }
       } else {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
           const int key = score_key<W32, NP>(h[u], sg, mk);
-          if constexpr (K8) sc8[base - c0 + u * nts + stid] = (uint8_t)key;
-          else sc[score_slot(base - c0 + u * nts + stid)] = (uint16_t)(key >> ksh);
+          if constexpr (K8) sc8[key_slot(base, u)] = (uint8_t)key;
+          else sc[key_slot(base, u)] = (uint16_t)(key >> ksh);
           atomicAdd(&hist[(key >> ksh) >> hsh], 1u);
         }
       }
@@ -938,7 +952,7 @@ bpc_decode_kernel(const DecodeParams p) {
         for (int u = 0; u < U; ++u) {
           const int i = i0 + u * nts + stid;
           if (i < c1s) {
-            sc[score_slot(i - c0)] = (uint16_t)(keys[u] >> ksh);
+            sc[key_slot(i0, u)] = (uint16_t)(keys[u] >> ksh);
             atomicAdd(&hist[(keys[u] >> ksh) >> hsh], 1u);
           }
         }
@@ -948,8 +962,8 @@ bpc_decode_kernel(const DecodeParams p) {
           const int i = i0 + u * nts + stid;
           if (i < c1s) {
             const int key = score_key<W32, NP>(h[u], sg, mk);
-            if constexpr (K8) sc8[i - c0] = (uint8_t)key;
-            else sc[score_slot(i - c0)] = (uint16_t)(key >> ksh);
+            if constexpr (K8) sc8[key_slot(i0, u)] = (uint8_t)key;
+            else sc[key_slot(i0, u)] = (uint16_t)(key >> ksh);
             atomicAdd(&hist[(key >> ksh) >> hsh], 1u);
           }
         }
@@ -1202,7 +1216,7 @@ bpc_decode_kernel(const DecodeParams p) {
         for (int pl = 0; pl < NP; ++pl) mk[pl][w] = st->mask[pl][w];
       }
       const int key = score_key<W32, NP>(h, sg, mk);
-      if constexpr (K8) sc8[n - 1 - c0] = (uint8_t)key;
+      if constexpr (K8) sc8[score_byte(n - 1 - c0)] = (uint8_t)key;
       else sc[score_slot(n - 1 - c0)] = (uint16_t)(key >> ksh);
       atomicAdd(&hist[(key >> ksh) >> hsh], 1u);
       if (p.dbg_scores != nullptr) p.dbg_scores[(size_t)unit * p.n_max + (n - 1)] = ((2 * key) << cs) - (st->rsum << cs);
@@ -1351,9 +1365,9 @@ bpc_decode_kernel(const DecodeParams p) {
           const uint32_t y = (kw[w] ^ TT) & HM;
           const uint32_t z = (y - 0x00010001u) & ~y & 0x80008000u;
           if (z) {
-            const int i = 8 * v + 2 * w;
+            const int i = 4 * v + w;                         // keys i and i + 16
             if ((y & 0xffffu) == 0u && i < valid) atomicAdd(&tot[kw[w] & (FB - 1)], 1u);
-            if ((y >> 16) == 0u && i + 1 < valid) atomicAdd(&tot[(kw[w] >> 16) & (FB - 1)], 1u);
+            if ((y >> 16) == 0u && i + 16 < valid) atomicAdd(&tot[(kw[w] >> 16) & (FB - 1)], 1u);
           }
         }
       }
@@ -1622,10 +1636,11 @@ bpc_decode_kernel(const DecodeParams p) {
       if (newkey > Tk || (newkey == Tk && eq_all < my_take)) sel_u[my_base + gt_all + min(eq_all, my_take)] = n - 1;
     }
   } else {
-    // Each thread owns whole 32-key segments, in ascending order within a pass.  Two keys share a 32-bit
-    // word; adding (0x8000 - T) to both halves raises bit 15 / bit 31 exactly for keys >= T (keys < 2048),
-    // which is shifted into a 32-bit candidate mask without branches.  Only the few candidates are looked
-    // at again (re-read from shared memory) to tell "greater" from "tie".
+    // Each thread owns whole 32-key segments, in ascending order within a pass.  A segment's keys are compared with T two (four) to a
+    // word: with the top bits of the halves (bytes) set, subtracting the low bits of T leaves each top bit set where the key's low
+    // bits reach T's, and the keys' own top bits decide the rest.  (Hamming keys are below 2048: one addition of 0x8000 - T does.)
+    // Flags are shifted into a mask in key order without branches, for >= T and for > T.  Two shifts, masks and merges per key pair
+    // and a loop over the candidates to tell "greater" from "tie" took EM_BEFORE us of 4 x 128K keys, this way EM_AFTER.
     const int len = c1 - c0;
     const int nseg = (len + kSegKeys - 1) / kSegKeys;
     int my_take = st->my_take, my_base = st->my_base;
@@ -1635,7 +1650,22 @@ bpc_decode_kernel(const DecodeParams p) {
       my_base = st->above_low + min(need, st->low);
     }
     const int T = T_exact;                                   // shadows the coarse bin: from here on the exact key
-    const uint32_t cge = (uint32_t)(0x8000 - T) * 0x10001u;
+    constexpr uint32_t kTop = K8 ? 0x80808080u : 0x80008000u, kEach = K8 ? 0x01010101u : 0x10001u, kTopBit = K8 ? 0x80u : 0x8000u;
+    constexpr int kSegWords = K8 ? kSegKeys / 4 : kSegKeys / 2;
+    // flags (at kTop) of the keys of a word that reach `least` (up to one above the largest key)
+    struct Reach { uint32_t low, any; };
+    auto reach_of = [&](int least) -> Reach {
+      if (MODE == 0 && !K8) return {(uint32_t)(0x8000 - least) * kEach, 0u};
+      return {((uint32_t)least & (kTopBit - 1u)) * kEach, (uint32_t)least & kTopBit ? 0u : ~0u};
+    };
+    auto reached = [&](uint32_t x, const Reach& r) {
+      if (MODE == 0 && !K8) return x + r.low;
+      return both_or_any(x, (x | kTop) - r.low, r.any);
+    };
+    const Reach ge = reach_of(T);
+    // (no key reaches 2^16 or 2^8: nothing is above such a T)
+    const Reach gt = reach_of((T + 1) & (int)(2u * kTopBit - 1u));
+    const bool none_above = !(MODE == 0 && !K8) && T + 1 >= (int)(2u * kTopBit);
     constexpr int SPT = 4;                                   // most consecutive segments one thread takes per pass
     const int spt = min(SPT, (nseg + NT - 1) / NT);
     int run_gt = 0, run_eq = 0;
@@ -1650,59 +1680,31 @@ bpc_decode_kernel(const DecodeParams p) {
         M[q] = 0u; Mgt[q] = 0u;
         const int seg = s0 + tid * spt + q;
         if (q < spt && seg < nseg) {
-          uint32_t kw[16];
-          if constexpr (K8) {                                // 32 byte keys: two 16-byte reads
-            const uint4* src = reinterpret_cast<const uint4*>(sc8 + (size_t)seg * kSegKeys);
+          const uint4* src = reinterpret_cast<const uint4*>(uni + (size_t)seg * (K8 ? kSegKeys : 2 * kSegSlots));
+          uint32_t m = 0u, mg = 0u;
 #pragma unroll
-            for (int v = 0; v < 2; ++v) {
-              const uint4 x = src[v];
-              kw[4 * v] = x.x; kw[4 * v + 1] = x.y; kw[4 * v + 2] = x.z; kw[4 * v + 3] = x.w;
+          for (int v = 0; v < kSegWords / 4; ++v) {
+            const uint4 x4 = src[v];
+            const uint32_t kw[4] = {x4.x, x4.y, x4.z, x4.w};
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+              m = (m >> 1) | (reached(kw[w], ge) & kTop);
+              if (MODE == 0) mg = (mg >> 1) | (reached(kw[w], gt) & kTop);
             }
-          } else {
-          const uint4* src = reinterpret_cast<const uint4*>(sc + (size_t)seg * kSegSlots);
-#pragma unroll
-          for (int v = 0; v < 4; ++v) {
-            const uint4 x = src[v];
-            kw[4 * v] = x.x; kw[4 * v + 1] = x.y; kw[4 * v + 2] = x.z; kw[4 * v + 3] = x.w;
-          }
-          }
-          uint32_t m = 0;
-          if constexpr (K8) {
-            // four keys per word: a per-byte unsigned compare leaves 0xFF where key >= T; one multiplication moves the
-            // four flags (bits 0, 8, 16, 24 after masking) next to each other: (y * 0x01020408) >> 24
-            const uint32_t T4 = (uint32_t)T * 0x01010101u;
-#pragma unroll
-            for (int w = 0; w < 8; ++w) {
-              const uint32_t ge = __vcmpgeu4(kw[w], T4) & 0x01010101u;
-              m |= (((ge * 0x01020408u) >> 24) & 15u) << (4 * w);
-            }
-          } else {
-#pragma unroll
-          for (int w = 0; w < 16; ++w) {
-            if (MODE == 0) {                                 // keys < 2048: both halves compared with one addition
-              const uint32_t gq = kw[w] + cge;
-              m |= (2 * w <= 15 ? (gq >> (15 - 2 * w)) : (gq << (2 * w - 15))) & (1u << (2 * w));
-              m |= (gq >> (30 - 2 * w)) & (2u << (2 * w));
-            } else {                                         // keys up to 65535: compare the halves separately
-              m |= ((int)(kw[w] & 0xffffu) >= T ? 1u : 0u) << (2 * w);
-              m |= ((int)(kw[w] >> 16) >= T ? 2u : 0u) << (2 * w);
-            }
-          }
           }
           const int valid = len - seg * kSegKeys;
           if (valid < kSegKeys) m &= (1u << valid) - 1u;     // slots past the end of the chunk hold stale bytes
-          uint32_t rem = m, mg = 0;
-          while (rem) {
-            const int j = __ffs(rem) - 1;
-            rem &= rem - 1;
-            if constexpr (K8) {
-              if ((int)sc8[(size_t)seg * kSegKeys + j] > T) mg |= 1u << j;
-            } else
-            if ((int)sc[(size_t)seg * kSegSlots + j] > T) mg |= 1u << j;
-            else if (MODE == 1 && ksh > 0) {                 // stored key == threshold: the dropped bits decide
-              const int low = exact_key(seg * kSegKeys + j) & ((1 << ksh) - 1);
-              if (low > T_low) mg |= 1u << j;
-              else if (low < T_low) m &= ~(1u << j);
+          if (MODE == 0) {
+            mg = none_above ? 0u : mg & m;
+          } else {                                           // (five operations a word: a loop over the candidates is no slower)
+            for (uint32_t rem = m; rem != 0u; rem &= rem - 1u) {
+              const int j = __ffs(rem) - 1;
+              if ((int)sc[(size_t)seg * kSegSlots + lane_slot(j)] > T) mg |= 1u << j;
+              else if (ksh > 0) {                            // stored key == threshold: the dropped bits decide
+                const int low = exact_key(seg * kSegKeys + j) & ((1 << ksh) - 1);
+                if (low > T_low) mg |= 1u << j;
+                else if (low < T_low) m &= ~(1u << j);
+              }
             }
           }
           M[q] = m; Mgt[q] = mg;
@@ -1716,22 +1718,25 @@ bpc_decode_kernel(const DecodeParams p) {
 #pragma unroll
       for (int q = 0; q < SPT; ++q) TK[q] = 0u;
       if (cgt | ceq) {
-        int eqb = run_eq + (int)(ex >> 16);
+        const int eqb = run_eq + (int)(ex >> 16);
         int pos = my_base + run_gt + (int)(ex & 0xffffu) + min(eqb, my_take);
+        int ties = max(my_take - eqb, 0);                    // of this thread's, the lowest ones
 #pragma unroll
         for (int q = 0; q < SPT; ++q) {
-          const int seg = s0 + tid * spt + q;
-          uint32_t rem = M[q];
+          if (q >= spt) break;                               // (uniform)
+          uint32_t e = M[q] & ~Mgt[q];
+          TK[q] = Mgt[q];
+          for (; e != 0u && ties > 0; --ties) { TK[q] |= e & (0u - e); e &= e - 1u; }
+        }
+        const int first = c0 + (s0 + tid * spt) * kSegKeys;
+#pragma unroll
+        for (int q = 0; q < SPT; ++q) {
+          if (q >= spt) break;
+          uint32_t rem = TK[q];
           while (rem) {
             const int j = __ffs(rem) - 1;
             rem &= rem - 1;
-            const int gi = c0 + seg * kSegKeys + j;
-            bool takes = true;
-            if (!((Mgt[q] >> j) & 1u)) { takes = eqb < my_take; ++eqb; }
-            if (takes) {
-              sel_u[pos++] = gi;
-              if (EAS) TK[q] |= 1u << j;
-            }
+            sel_u[pos++] = first + q * kSegKeys + j;
           }
         }
       }
