@@ -1274,7 +1274,7 @@ bpc_decode_kernel(const DecodeParams p) {
     {
       const int bq = max(bin, 0);
       if (pushed != nullptr) {
-#pragma unroll 1
+#pragma unroll 4
         for (int r = 0; r < CS; ++r) {
           const uint32_t v = bin >= 0 ? pushed[r * nbins + bq] : 0u;
           s_all += v;
@@ -1640,7 +1640,7 @@ bpc_decode_kernel(const DecodeParams p) {
     // word: with the top bits of the halves (bytes) set, subtracting the low bits of T leaves each top bit set where the key's low
     // bits reach T's, and the keys' own top bits decide the rest.  (Hamming keys are below 2048: one addition of 0x8000 - T does.)
     // Flags are shifted into a mask in key order without branches, for >= T and for > T.  Two shifts, masks and merges per key pair
-    // and a loop over the candidates to tell "greater" from "tie" took EM_BEFORE us of 4 x 128K keys, this way EM_AFTER.
+    // and a loop over the candidates to tell "greater" from "tie" took 1.48 us of 4 x 128K keys.
     const int len = c1 - c0;
     const int nseg = (len + kSegKeys - 1) / kSegKeys;
     int my_take = st->my_take, my_base = st->my_base;
@@ -1790,15 +1790,21 @@ bpc_decode_kernel(const DecodeParams p) {
     // Lane (g = lane/4, t = lane%4) holds the logits of head g for keys 2t, 2t+1 and, in every 8-dim output
     // tile, dims 2t, 2t+1 of head g (high part in d[0..1], low part in d[2..3]).
     const int g = lane >> 2, t = lane & 3;
+    // A dot product does not mind the order of its channels: lane t takes the 16-byte pieces t, 4 + t, 8 + t, 12 + t of a query and of a
+    // key row as its words of the eight MMAs, four vector reads each.  (Channels in order: 16 loads of q per lane, 0.5 us of the load
+    // pipe between the list and the first gather.)
     uint32_t qa0[8], qa2[8];
     {
-      const uint32_t* qw = reinterpret_cast<const uint32_t*>(qg + (size_t)g * BPC_D);
+      const uint4* qv = reinterpret_cast<const uint4*>(qg + (size_t)g * BPC_D);
 #pragma unroll
-      for (int s = 0; s < 8; ++s) {
-        qa0[s] = g < G ? qw[8 * s + t] : 0u;                 // dims 16s + 2t, +1
-        qa2[s] = g < G ? qw[8 * s + 4 + t] : 0u;             // dims 16s + 8 + 2t, +1
+      for (int i = 0; i < 4; ++i) {
+        const uint4 x = g < G ? qv[4 * i + t] : make_uint4(0u, 0u, 0u, 0u);
+        qa0[2 * i] = x.x; qa2[2 * i] = x.y; qa0[2 * i + 1] = x.z; qa2[2 * i + 1] = x.w;
       }
     }
+    // piece c of row r lies at place c ^ turn(r): the eight rows of a transposed read and the two rows of a quarter warp's key read
+    // are on different banks
+    auto turn = [](int r) { return ((r & 1) << 2) | (r >> 1); };
     float o[16][4];
 #pragma unroll
     for (int j = 0; j < 16; ++j) { o[j][0] = o[j][1] = o[j][2] = o[j][3] = 0.f; }
@@ -1841,7 +1847,7 @@ bpc_decode_kernel(const DecodeParams p) {
 #pragma unroll
         for (int it = 0; it < 8; ++it) {
           const int idx = __shfl_sync(0xffffffffu, myidx, it);
-          unsigned char* d = dst + it * ROWB + ((ch ^ it) << 4);
+          unsigned char* d = dst + it * ROWB + ((ch ^ turn(it)) << 4);
           if (idx >= 0) {
             cp_async16(d, srcbase + (size_t)idx * rstride);
           } else {
@@ -1862,14 +1868,18 @@ bpc_decode_kernel(const DecodeParams p) {
                                  : (rbase_c + 8 <= nrows ? 0xffu : ((1u << (nrows - rbase_c)) - 1u));
       const unsigned char* ks = wst + (size_t)(bi % NS) * WSTG;
       const unsigned char* vs = ks + 8 * ROWB;
+      // Two chains of four dependent MMAs instead of one of eight (8 x 1M keys of 64 bits 40.8 -> 40.2 us, weighted 256 bits 47.0 -> 46.4), but not
+      // for 128-bit codes, where the registers cost more than it saves (32K keys 17.1 -> 17.4).
+      constexpr bool kTwoChains = W32 != 4;
       float s[4] = {0.f, 0.f, 0.f, 0.f};
+      [[maybe_unused]] float z[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-      for (int jj = 0; jj < 4; ++jj) {                       // 32 dims per ldmatrix.x4: chunks 4jj .. 4jj+3
-        uint32_t b[4];
-        ldmatrix_x4(b, ks + (size_t)lrow * ROWB + (((4 * jj + lmat) ^ lrow) << 4));
-        mma_qk(s, qa0[2 * jj], qa2[2 * jj], b[0], b[1]);
-        mma_qk(s, qa0[2 * jj + 1], qa2[2 * jj + 1], b[2], b[3]);
+      for (int i = 0; i < 4; ++i) {
+        const uint4 x = *reinterpret_cast<const uint4*>(ks + (size_t)g * ROWB + (((4 * i + t) ^ turn(g)) << 4));   // key g
+        mma_qk(s, qa0[2 * i], qa2[2 * i], x.x, x.y);
+        mma_qk(kTwoChains ? z : s, qa0[2 * i + 1], qa2[2 * i + 1], x.z, x.w);
       }
+      if (kTwoChains) { s[0] += z[0]; s[1] += z[1]; }
       const bool v0 = (vmask >> (2 * t)) & 1u, v1 = (vmask >> (2 * t + 1)) & 1u;
       const float s0 = v0 ? s[0] * scale2 : -1e30f, s1 = v1 ? s[1] * scale2 : -1e30f;
       float tmax = fmaxf(s0, s1);
@@ -1879,8 +1889,10 @@ bpc_decode_kernel(const DecodeParams p) {
         if (tmax > m_run) {
           const float corr = exp2f(m_run - tmax);
           l_run *= corr;
+          if (bi > 0) {                                    // (nothing to scale before the first block)
 #pragma unroll
-          for (int j = 0; j < 16; ++j) { o[j][0] *= corr; o[j][1] *= corr; o[j][2] *= corr; o[j][3] *= corr; }
+            for (int j = 0; j < 16; ++j) { o[j][0] *= corr; o[j][1] *= corr; o[j][2] *= corr; o[j][3] *= corr; }
+          }
           m_run = tmax;
         }
       }
@@ -1893,7 +1905,7 @@ bpc_decode_kernel(const DecodeParams p) {
 #pragma unroll
       for (int jj = 0; jj < 4; ++jj) {
         uint32_t b[4];
-        ldmatrix_x4_trans(b, vs + (size_t)lrow * ROWB + (((4 * jj + lmat) ^ lrow) << 4));
+        ldmatrix_x4_trans(b, vs + (size_t)lrow * ROWB + (((4 * jj + lmat) ^ turn(lrow)) << 4));
         mma_pv(o[4 * jj], pa0, pa1, b[0]);
         mma_pv(o[4 * jj + 1], pa0, pa1, b[1]);
         mma_pv(o[4 * jj + 2], pa0, pa1, b[2]);
@@ -1910,10 +1922,7 @@ bpc_decode_kernel(const DecodeParams p) {
     if (g < GP) {
       acc_t* dst = part + ((size_t)warp * GP + g) * (BPC_D + 2);
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        dst[8 * j + 2 * t] = o[j][0] + o[j][2];
-        dst[8 * j + 2 * t + 1] = o[j][1] + o[j][3];
-      }
+      for (int j = 0; j < 16; ++j) *reinterpret_cast<float2*>(dst + 8 * j + 2 * t) = make_float2(o[j][0] + o[j][2], o[j][1] + o[j][3]);
       if (t == 0) { dst[BPC_D] = m_run; dst[BPC_D + 1] = l_run; }
     }
   } else {
@@ -2024,7 +2033,7 @@ bpc_decode_kernel(const DecodeParams p) {
       for (int gg = 0; gg < GP; ++gg) {
         acc_t* dst = part + ((size_t)warp * GP + gg) * (BPC_D + 2);
 #pragma unroll
-        for (int c = 0; c < 8; ++c) dst[8 * hl + c] = acc[gg][c];
+        for (int c = 0; c < 8; c += 2) *reinterpret_cast<double2*>(dst + 8 * hl + c) = make_double2(acc[gg][c], acc[gg][c + 1]);
         if (hl == 0) { dst[BPC_D] = m_run[gg]; dst[BPC_D + 1] = l_run[gg]; }
       }
     }
@@ -2080,11 +2089,13 @@ bpc_decode_kernel(const DecodeParams p) {
     for (int o = rank * per + tid; o < o_end; o += NT) {
       const int g = o >> 7, j = o - rank * per;
       acc_t mm = (acc_t)-1e30;
+#pragma unroll 4
       for (int r = 0; r < CS; ++r) {
         const acc_t v = inbox[r * istride + per + g];
         mm = v > mm ? v : mm;
       }
       acc_t num = 0, den = 0;
+#pragma unroll 4
       for (int r = 0; r < CS; ++r) {
         const acc_t wt = fast_exp2<acc_t>(inbox[r * istride + per + g] - mm);
         num = fma(inbox[r * istride + j], wt, num);
