@@ -134,7 +134,10 @@ def interleaved_kv(batch: int, n_kv_heads: int, n_max: int, head_dim: int, dtype
 
 
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    """The current stream of the current device, as torch.cuda.current_stream().cuda_stream without building the Stream object."""
+    if not torch.cuda.is_initialized():
+        torch.cuda.init()
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _check(status: int, what: str) -> None:
