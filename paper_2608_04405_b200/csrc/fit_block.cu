@@ -168,6 +168,7 @@ fit_project_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* 
     for (int p = 0; p < 3; ++p)
       *reinterpret_cast<__nv_bfloat16*>(b_s + sw128_offset(kProjN, p * kBits + l, ch >> 3) + (size_t)(ch & 7) * 2) = t3[p];
   }
+  asm volatile("griddepcontrol.wait;" ::: "memory");                   // (launched early by the kernel that forms the scalars)
   for (int c = tid; c < kBits * blk * kBits; c += kThreads) {
     const int j = c >> 5, l = c & 31;                                  // earlier bit, column
     __nv_bfloat16 t3[3];
@@ -365,6 +366,7 @@ fit_gather_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* _
   __shared__ uint32_t tmem_base_s;
   __shared__ int timed_out_g[GROUPS];
   const unsigned st_a = smem_u32(sign_table);
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int unit = blockIdx.y, words = b / 32;
   const int n = min(unit_lens[unit], n_max);
   const int rows = block_rows(n, gridDim.x);
@@ -1171,6 +1173,7 @@ fit_finish_kernel(const double* __restrict__ wpart, const int32_t* __restrict__ 
   const int n = min(unit_lens[unit], n_max);
   float* Pu = P + (size_t)unit * b * BPC_D;
   if (n <= 0) {                                            // (the whole cluster)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     Pu[(size_t)(np + i) * BPC_D + kFinishChannels * rank + c] = 0.f;
     return;
   }
@@ -1184,6 +1187,8 @@ fit_finish_kernel(const double* __restrict__ wpart, const int32_t* __restrict__ 
 #pragma unroll
     for (int k = 0; k < kDirs; ++k) dir[k] = v_star[((size_t)unit * b + nj) * BPC_D + tid + k * kFinishThreads];
   }
+  asm volatile("griddepcontrol.wait;" ::: "memory");         // (the lengths and directions are older than the kernel before)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const double* w = wpart + (size_t)unit * parts * kBits * BPC_D + (size_t)i * BPC_D + kFinishChannels * rank + c;
   double ws = w[0];
 #pragma unroll 16
@@ -1390,16 +1395,31 @@ int sweep_cluster(const bpc_config* c, const int* active) {
   return best;
 }
 
+// Ordinary launch, or one that may start while the kernel before it drains (both kernels then mark the point).
+template <typename... A, typename... B>
+cudaError_t launch_after(bool early, void (*kernel)(A...), dim3 grid, int threads, size_t smem, cudaStream_t stream, B... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = early ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<A>(args)...);
+}
+
 template <int GROUPS>
 cudaError_t launch_project_tc(const bpc_ctx* ctx, const CUtensorMap& kmap, const uint32_t* hfit, const float* v_star, const float* cross, float* T,
-                              uint32_t* t_max, int blk, int parts, int ts, cudaStream_t stream) {
+                              uint32_t* t_max, int blk, int parts, int ts, bool early, cudaStream_t stream) {
   const bpc_config& c = ctx->cfg;
   const size_t smem = (size_t)GROUPS * (kTileBytes + kTileKeys * kSignCols * 2) + (size_t)kProjN * 256 + (size_t)blk * kProjN * 64 + 1024;
   cudaError_t e = allow_smem(fit_project_tc_kernel<GROUPS>);
   if (e != cudaSuccess) return e;
-  fit_project_tc_kernel<GROUPS><<<dim3(parts, ctx->units), kGroupThreads * GROUPS, smem, stream>>>(
-      kmap, hfit, v_star, cross, T, t_max, ctx->unit_lens, ctx->dev_err, c.n_max, c.code_bits, blk, ts);
-  return cudaGetLastError();
+  return launch_after(early, fit_project_tc_kernel<GROUPS>, dim3(parts, ctx->units), kGroupThreads * GROUPS, smem, stream, kmap, hfit, v_star, cross, T, t_max,
+                      (const int32_t*)ctx->unit_lens, ctx->dev_err, (int)c.n_max, (int)c.code_bits, blk, ts);
 }
 
 template <int GROUPS>
@@ -1452,9 +1472,10 @@ cudaError_t bpc_launch_fit_blocked(bpc_ctx* ctx, const void* k_cache, const floa
       if (e != cudaSuccess) return e;
     }
     if (tc) {
+      const bool early = one_finish && blk > 0 && ctx->use_pdl;
       // three warpgroups while the scalars of the earlier bits leave room for them (up to five earlier words)
-      e = blk <= 5 ? launch_project_tc<3>(ctx, kmap, hfit, v_star, cross, T, t_max, blk, parts, ts, stream)
-                   : launch_project_tc<2>(ctx, kmap, hfit, v_star, cross, T, t_max, blk, parts, ts, stream);
+      e = blk <= 5 ? launch_project_tc<3>(ctx, kmap, hfit, v_star, cross, T, t_max, blk, parts, ts, early, stream)
+                   : launch_project_tc<2>(ctx, kmap, hfit, v_star, cross, T, t_max, blk, parts, ts, early, stream);
     } else {
       e = cudaMemset2DAsync(t_max, column_max_at(1, 0, parts) * 4, 0, kBits * 4, ctx->units, stream);
       if (e != cudaSuccess) return e;
@@ -1481,9 +1502,8 @@ cudaError_t bpc_launch_fit_blocked(bpc_ctx* ctx, const void* k_cache, const floa
     if (one_finish) {
       e = allow_smem(fit_finish_kernel);
       if (e != cudaSuccess) return e;
-      fit_finish_kernel<<<kFinishBlocks * ctx->units, kFinishThreads, FinishSmem(blk).total * sizeof(double), stream>>>(
-          wpart, apart, v_star, ctx->P, cross, ctx->unit_lens, c.n_max, b, blk, parts);
-      e = cudaGetLastError();
+      e = launch_after(tc && ctx->use_pdl, fit_finish_kernel, dim3(kFinishBlocks * ctx->units), kFinishThreads, FinishSmem(blk).total * sizeof(double), stream,
+                       (const double*)wpart, (const int32_t*)apart, v_star, ctx->P, cross, (const int32_t*)ctx->unit_lens, (int)c.n_max, b, blk, parts);
       *launches += 4;
       continue;
     }
