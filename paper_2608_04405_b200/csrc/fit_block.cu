@@ -169,6 +169,7 @@ fit_project_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* 
       *reinterpret_cast<__nv_bfloat16*>(b_s + sw128_offset(kProjN, p * kBits + l, ch >> 3) + (size_t)(ch & 7) * 2) = t3[p];
   }
   asm volatile("griddepcontrol.wait;" ::: "memory");                   // (launched early by the kernel that forms the scalars)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   for (int c = tid; c < kBits * blk * kBits; c += kThreads) {
     const int j = c >> 5, l = c & 31;                                  // earlier bit, column
     __nv_bfloat16 t3[3];
@@ -366,7 +367,6 @@ fit_gather_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* _
   __shared__ uint32_t tmem_base_s;
   __shared__ int timed_out_g[GROUPS];
   const unsigned st_a = smem_u32(sign_table);
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int unit = blockIdx.y, words = b / 32;
   const int n = min(unit_lens[unit], n_max);
   const int rows = block_rows(n, gridDim.x);
@@ -391,8 +391,10 @@ fit_gather_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* _
 #pragma unroll
     for (int w = 0; w < kMaxWords; ++w) nxt[w] = (w <= blk && r < row_end) ? h[w] : 0u;
   };
-  if (grp < ntile) load_words(grp);
   fill_sign_table(sign_table, tid);
+  asm volatile("griddepcontrol.wait;" ::: "memory");         // (launched early: the code words are there)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (grp < ntile) load_words(grp);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -901,10 +903,6 @@ fit_sweep_kernel(float* __restrict__ T, uint32_t* __restrict__ hfit, uint32_t* _
   uint32_t* ws = WORDS != kWordsGlobal ? reinterpret_cast<uint32_t*>(sweep_smem) : words_g + (size_t)unit * t_stride + row0;
   float* Tu = T + (size_t)unit * kBits * t_stride + row0;
   SweepWarp st;
-  if (warp * kSweepGroup < nk) {
-    load_entries(st.t, Tu + warp * kSweepGroup + 4 * lane);
-    load_entries(st.nx, Tu + t_stride + warp * kSweepGroup + 4 * lane);
-  }
 #pragma unroll
   for (int q = 0; q < kTabs; ++q) st.tab[q] = 0.f;
 #pragma unroll
@@ -915,6 +913,12 @@ fit_sweep_kernel(float* __restrict__ T, uint32_t* __restrict__ hfit, uint32_t* _
   for (int i = tid; i < 2 * 6 * kSumStride; i += kSweepThreads) (&sum_s[0][0])[i] = 0u;
   for (int i = tid; i < 32 * 33; i += kSweepThreads) (&inv_s[0][0])[i] = 0.0;
   if (tid < 4 * 32) { (&slot_s[0][0])[tid] = 0ull; (&slot_c[0][0])[tid] = 0; }
+  asm volatile("griddepcontrol.wait;" ::: "memory");         // (launched early: the columns are there)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (warp * kSweepGroup < nk) {
+    load_entries(st.t, Tu + warp * kSweepGroup + 4 * lane);
+    load_entries(st.nx, Tu + t_stride + warp * kSweepGroup + 4 * lane);
+  }
   {                                                        // largest |T| of the unit's columns (lane: column), by block of the projection
     const int used = t_parts > 1 ? (n + block_rows(n, parts) - 1) / block_rows(n, parts) : 1;
     uint32_t m = 0u;
@@ -1334,7 +1338,7 @@ struct SweepLimits {
 };
 SweepLimits g_sweep_limits[64];
 
-cudaLaunchConfig_t sweep_config(cudaLaunchAttribute* attr, int units, int cs, size_t smem, cudaStream_t stream) {
+cudaLaunchConfig_t sweep_config(cudaLaunchAttribute* attr, int units, int cs, size_t smem, cudaStream_t stream, bool early = false) {   // (two attributes)
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(units * cs));
   cfg.blockDim = dim3(kSweepThreads);
@@ -1345,6 +1349,11 @@ cudaLaunchConfig_t sweep_config(cudaLaunchAttribute* attr, int units, int cs, si
   attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  if (early) {
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 2;
+  }
   return cfg;
 }
 
@@ -1424,14 +1433,13 @@ cudaError_t launch_project_tc(const bpc_ctx* ctx, const CUtensorMap& kmap, const
 
 template <int GROUPS>
 cudaError_t launch_gather_tc(const bpc_ctx* ctx, const CUtensorMap& kmap, const uint32_t* hfit, double* wpart, int32_t* apart, int blk, int parts,
-                             cudaStream_t stream) {
+                             bool early, cudaStream_t stream) {
   const bpc_config& c = ctx->cfg;
   const size_t smem = gather_smem(GROUPS, blk);
   cudaError_t e = allow_smem(fit_gather_tc_kernel<GROUPS>);
   if (e != cudaSuccess) return e;
-  fit_gather_tc_kernel<GROUPS><<<dim3(parts, ctx->units), kGroupThreads * GROUPS, smem, stream>>>(
-      kmap, hfit, wpart, apart, ctx->unit_lens, ctx->dev_err, c.n_max, c.code_bits, blk);
-  return cudaGetLastError();
+  return launch_after(early, fit_gather_tc_kernel<GROUPS>, dim3(parts, ctx->units), kGroupThreads * GROUPS, smem, stream, kmap, hfit, wpart, apart,
+                      (const int32_t*)ctx->unit_lens, ctx->dev_err, (int)c.n_max, (int)c.code_bits, blk);
 }
 
 }  // namespace
@@ -1462,6 +1470,8 @@ cudaError_t bpc_launch_fit_blocked(bpc_ctx* ctx, const void* k_cache, const floa
   // on some device costs time only).  Fits of 32K keys and 128 bits: 4 units 532 -> 506 us, 8 units 598 -> 569, 12 units 673 -> 657, but
   // 16 units 854 -> 875.
   const bool one_finish = ctx->units <= 15;
+  // Then also each kernel is launched to start while the one before it drains.  (With more units every SM has work and it cost 1 to 3 %.)
+  const bool early = one_finish && tc && ctx->use_pdl;
   const dim3 grid(parts, ctx->units);
   CUtensorMap kmap;
   if (tc) e = tma::make_key_map(&kmap, k_cache, (unsigned long long)ctx->units * c.n_max, ctx->row_stride);
@@ -1472,10 +1482,9 @@ cudaError_t bpc_launch_fit_blocked(bpc_ctx* ctx, const void* k_cache, const floa
       if (e != cudaSuccess) return e;
     }
     if (tc) {
-      const bool early = one_finish && blk > 0 && ctx->use_pdl;
       // three warpgroups while the scalars of the earlier bits leave room for them (up to five earlier words)
-      e = blk <= 5 ? launch_project_tc<3>(ctx, kmap, hfit, v_star, cross, T, t_max, blk, parts, ts, early, stream)
-                   : launch_project_tc<2>(ctx, kmap, hfit, v_star, cross, T, t_max, blk, parts, ts, early, stream);
+      e = blk <= 5 ? launch_project_tc<3>(ctx, kmap, hfit, v_star, cross, T, t_max, blk, parts, ts, early && blk > 0, stream)
+                   : launch_project_tc<2>(ctx, kmap, hfit, v_star, cross, T, t_max, blk, parts, ts, early && blk > 0, stream);
     } else {
       e = cudaMemset2DAsync(t_max, column_max_at(1, 0, parts) * 4, 0, kBits * 4, ctx->units, stream);
       if (e != cudaSuccess) return e;
@@ -1483,18 +1492,18 @@ cudaError_t bpc_launch_fit_blocked(bpc_ctx* ctx, const void* k_cache, const floa
           (const float*)k_cache, hfit, v_star, cross, T, t_max, ctx->unit_lens, c.n_max, ctx->row_stride, b, blk, ts, parts);
     }
     if (e != cudaSuccess) return e;
-    cudaLaunchAttribute attr;
+    cudaLaunchAttribute attr[2];
     const bool words_fit = sweep_smem <= kSweepMaxSmem, one = sweep_share(c.n_max, cs) <= kSweepWarps * kSweepGroup;
-    cudaLaunchConfig_t cfg = sweep_config(&attr, ctx->units, cs, words_fit ? sweep_smem : 0, stream);
+    cudaLaunchConfig_t cfg = sweep_config(attr, ctx->units, cs, words_fit ? sweep_smem : 0, stream, early);
     auto sweep = !words_fit ? fit_sweep_kernel<kWordsGlobal> : one ? fit_sweep_kernel<kOneGroup> : fit_sweep_kernel<kWordsOnChip>;
     e = cudaLaunchKernelEx(&cfg, sweep, T, hfit, words_g, (const uint32_t*)t_max, (const int32_t*)ctx->unit_lens, ctx->dev_err, (int)c.n_max, b, blk,
                            ts, parts, tc ? parts : 1, cs, ctx->wait_tries);
     if (e != cudaSuccess) return e;
     if (tc) {
       // as many warpgroups as their tile and sign buffers leave room for (four up to the third word, two from the sixth)
-      if (gather_smem(4, blk) <= kMaxSmem) e = launch_gather_tc<4>(ctx, kmap, hfit, wpart, apart, blk, parts, stream);
-      else if (gather_smem(3, blk) <= kMaxSmem) e = launch_gather_tc<3>(ctx, kmap, hfit, wpart, apart, blk, parts, stream);
-      else e = launch_gather_tc<2>(ctx, kmap, hfit, wpart, apart, blk, parts, stream);
+      if (gather_smem(4, blk) <= kMaxSmem) e = launch_gather_tc<4>(ctx, kmap, hfit, wpart, apart, blk, parts, early, stream);
+      else if (gather_smem(3, blk) <= kMaxSmem) e = launch_gather_tc<3>(ctx, kmap, hfit, wpart, apart, blk, parts, early, stream);
+      else e = launch_gather_tc<2>(ctx, kmap, hfit, wpart, apart, blk, parts, early, stream);
     } else {
       fit_gather_f32_kernel<<<grid, 256, 0, stream>>>((const float*)k_cache, hfit, wpart, apart, ctx->unit_lens, c.n_max, ctx->row_stride, b, blk);
     }
@@ -1502,7 +1511,7 @@ cudaError_t bpc_launch_fit_blocked(bpc_ctx* ctx, const void* k_cache, const floa
     if (one_finish) {
       e = allow_smem(fit_finish_kernel);
       if (e != cudaSuccess) return e;
-      e = launch_after(tc && ctx->use_pdl, fit_finish_kernel, dim3(kFinishBlocks * ctx->units), kFinishThreads, FinishSmem(blk).total * sizeof(double), stream,
+      e = launch_after(early, fit_finish_kernel, dim3(kFinishBlocks * ctx->units), kFinishThreads, FinishSmem(blk).total * sizeof(double), stream,
                        (const double*)wpart, (const int32_t*)apart, v_star, ctx->P, cross, (const int32_t*)ctx->unit_lens, (int)c.n_max, b, blk, parts);
       *launches += 4;
       continue;
