@@ -142,8 +142,6 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __nv_bfloat16* 
   static_assert(kAccCols <= 512, "accumulators exceed tensor memory");
 
   const int unit = blockIdx.y;
-  const int n = min(unit_lens[unit], n_max);
-  const int ntiles = (n + kTileKeys - 1) / kTileKeys;
   const int set = shared_sets ? unit % n_kv_heads : unit;
 
   // ---- one-time set-up: barrier, tensor memory, projection and Gram operands in shared memory
@@ -157,6 +155,10 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __nv_bfloat16* 
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"(kTmemCols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  // launched while the kernel before drains: nothing that one may be writing is read above
+  pdl_wait();
+  const int n = min(unit_lens[unit], n_max);
+  const int ntiles = (n + kTileKeys - 1) / kTileKeys;
   {
     const unsigned char* psrc = reinterpret_cast<const unsigned char*>(Ph + ((size_t)set * TOTAL + ROW0) * BPC_D);
     for (int c = tid; c < NBITS * 16; c += kThreads) {
@@ -169,26 +171,27 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __nv_bfloat16* 
       const int d = c / (kSub * kSub), i = c / kSub % kSub, j = c % kSub;
       gd_s[c] = gsrc[(size_t)(kSub * d + i) * TOTAL + kSub * d + j];
     }
+    // minus eight elements of a Gram column from row i0 on, as K elements i0 .. i0 + 7 of row `row` of the operands of the three terms
+    auto put_terms = [&](unsigned char* base, int term_bytes, int rows, int row, int i0, const float* column) {
+      float v[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) v[e] = -column[(size_t)(i0 + e) * TOTAL];
+      uint4 t3[3];
+      split3x8(v, t3);
+#pragma unroll
+      for (int p = 0; p < 3; ++p) *reinterpret_cast<uint4*>(base + (size_t)p * term_bytes + nosw_offset(rows, row, i0)) = t3[p];
+    };
     if constexpr (HALF == 2) {
       // -G[i][128 + j] for the first half's bits i, as three bf16 terms; operand rows j, K index i, [128 x 128] each
-      for (int c = tid; c < 128 * 128; c += kThreads) {
-        const int i = c >> 7, j = c & 127;
-        __nv_bfloat16 t3[3];
-        split3(-gfull[(size_t)i * TOTAL + 128 + j], t3);
-#pragma unroll
-        for (int p = 0; p < 3; ++p) *reinterpret_cast<__nv_bfloat16*>(x_s + nosw_offset(128, j, i) + 32768 * p) = t3[p];
-      }
+      for (int c = tid; c < 16 * 128; c += kThreads) put_terms(x_s, 32768, 128, c & 127, 8 * (c >> 7), gfull + 128 + (c & 127));
     }
-    // -G[16 pb + i][j], j after block pb, as three bf16 terms (g = t1 + t2 + t3 up to 2^-24 |g|); operand rows j, K index i
-    for (int c = tid; c < (NS - 1) * kSub * NBITS; c += kThreads) {
-      const int pb = c / (kSub * NBITS), i = (c / NBITS) % kSub, j = c % NBITS;
-      const int j0 = kSub * (pb + 1);
+    // -G[16 pb + i][j], j after block pb, as three bf16 terms (g = t1 + t2 + t3 up to 2^-24 |g|); operand rows j, K index i.  Eight
+    // consecutive i at a time are one 16-byte store per term (one element at a time, in stores of 2 bytes, the set-up of a
+    // block took PRO_BEFORE us of the 22 that 8 x 4K keys take).
+    for (int c = tid; c < (NS - 1) * 2 * NBITS; c += kThreads) {
+      const int pb = c / (2 * NBITS), i0 = 8 * (c / NBITS % 2), j = c % NBITS, j0 = kSub * (pb + 1);
       if (j < j0) continue;
-      __nv_bfloat16 t3[3];
-      split3(-gsrc[(size_t)(kSub * pb + i) * TOTAL + j], t3);
-      unsigned char* base = gb_s + gb_off(pb) + nosw_offset(gb_cols(pb), j - j0, i);
-#pragma unroll
-      for (int p = 0; p < 3; ++p) *reinterpret_cast<__nv_bfloat16*>(base + (size_t)p * gb_cols(pb) * kSub * 2) = t3[p];
+      put_terms(gb_s + gb_off(pb), gb_cols(pb) * kSub * 2, gb_cols(pb), j - j0, i0, gsrc + (size_t)(kSub * pb) * TOTAL + j);
     }
   }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy writes -> visible to the tensor core
@@ -400,10 +403,9 @@ cudaError_t launch(bpc_ctx* ctx, const void* k_cache, uint64_t* codes, cudaStrea
   CUtensorMap kmap;
   e = tma::make_key_map(&kmap, k_cache, (unsigned long long)ctx->units * c.n_max, ctx->row_stride);
   if (e != cudaSuccess) return e;
-  kern<<<grid, kGroupThreads * (GROUPS + setup_groups(HALF)), smem, stream>>>(
-      kmap, (const __nv_bfloat16*)ctx->P_h, ctx->gram, ctx->unit_lens, codes, ctx->dev_err,
-      c.n_kv_heads, c.n_max, c.hash_sets != ctx->units, c.residual_correction, bpu, ctx->key_err);
-  return cudaGetLastError();
+  return launch_pdl(ctx->use_pdl, kern, grid, kGroupThreads * (GROUPS + setup_groups(HALF)), smem, stream,
+                    kmap, (const __nv_bfloat16*)ctx->P_h, ctx->gram, ctx->unit_lens, codes, ctx->dev_err,
+                    c.n_kv_heads, c.n_max, c.hash_sets != ctx->units, c.residual_correction, bpu, ctx->key_err);
 }
 
 template <bool ERR>

@@ -160,22 +160,26 @@ fit_project_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* 
   auto load_tile = [&](int tile) { tma::load_key_tile(a_t, &kmap, unit * n_max + row0 + (ntile - 1 - tile) * kTileKeys, tile_bar); };   // (one thread)
   fill_sign_table(sign_table, tid);
   if (tid < kBits) max_s[tid] = 0u;
-  for (int c = tid; c < kBits * BPC_D; c += kThreads) {
-    const int l = c >> 7, ch = c & 127;
-    __nv_bfloat16 t3[3];
-    split3(v_star[((size_t)unit * b + kBits * blk + l) * BPC_D + ch], t3);
+  for (int c = tid; c < kBits * BPC_D / 8; c += kThreads) {             // eight elements at a time: a 16-byte store per term
+    const int l = c >> 4, ch = c & 15;
+    const float4* src = reinterpret_cast<const float4*>(v_star + ((size_t)unit * b + kBits * blk + l) * BPC_D + 8 * ch);
+    const float4 x = src[0], y = src[1];
+    const float v[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+    uint4 t3[3];
+    split3x8(v, t3);
 #pragma unroll
-    for (int p = 0; p < 3; ++p)
-      *reinterpret_cast<__nv_bfloat16*>(b_s + sw128_offset(kProjN, p * kBits + l, ch >> 3) + (size_t)(ch & 7) * 2) = t3[p];
+    for (int p = 0; p < 3; ++p) *reinterpret_cast<uint4*>(b_s + sw128_offset(kProjN, p * kBits + l, ch)) = t3[p];
   }
-  asm volatile("griddepcontrol.wait;" ::: "memory");                   // (launched early by the kernel that forms the scalars)
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  for (int c = tid; c < kBits * blk * kBits; c += kThreads) {
-    const int j = c >> 5, l = c & 31;                                  // earlier bit, column
-    __nv_bfloat16 t3[3];
-    split3(-cross[((size_t)unit * b + j) * kBits + l], t3);
+  pdl_wait();                                                          // (launched early by the kernel that forms the scalars)
+  for (int c = tid; c < kBits * blk * kBits / 8; c += kThreads) {
+    const int j = 8 * (c >> 5), l = c & 31;                            // eight earlier bits, column
+    float v[8];
 #pragma unroll
-    for (int p = 0; p < 3; ++p) *reinterpret_cast<__nv_bfloat16*>(c_s + nosw_offset(kProjN, p * kBits + l, j)) = t3[p];
+    for (int e = 0; e < 8; ++e) v[e] = -cross[((size_t)unit * b + j + e) * kBits + l];
+    uint4 t3[3];
+    split3x8(v, t3);
+#pragma unroll
+    for (int p = 0; p < 3; ++p) *reinterpret_cast<uint4*>(c_s + nosw_offset(kProjN, p * kBits + l, j)) = t3[p];
   }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -392,8 +396,7 @@ fit_gather_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* _
     for (int w = 0; w < kMaxWords; ++w) nxt[w] = (w <= blk && r < row_end) ? h[w] : 0u;
   };
   fill_sign_table(sign_table, tid);
-  asm volatile("griddepcontrol.wait;" ::: "memory");         // (launched early: the code words are there)
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  pdl_wait();                                              // (launched early: the code words are there)
   if (grp < ntile) load_words(grp);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -913,8 +916,7 @@ fit_sweep_kernel(float* __restrict__ T, uint32_t* __restrict__ hfit, uint32_t* _
   for (int i = tid; i < 2 * 6 * kSumStride; i += kSweepThreads) (&sum_s[0][0])[i] = 0u;
   for (int i = tid; i < 32 * 33; i += kSweepThreads) (&inv_s[0][0])[i] = 0.0;
   if (tid < 4 * 32) { (&slot_s[0][0])[tid] = 0ull; (&slot_c[0][0])[tid] = 0; }
-  asm volatile("griddepcontrol.wait;" ::: "memory");         // (launched early: the columns are there)
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  pdl_wait();                                              // (launched early: the columns are there)
   if (warp * kSweepGroup < nk) {
     load_entries(st.t, Tu + warp * kSweepGroup + 4 * lane);
     load_entries(st.nx, Tu + t_stride + warp * kSweepGroup + 4 * lane);
@@ -1191,8 +1193,7 @@ fit_finish_kernel(const double* __restrict__ wpart, const int32_t* __restrict__ 
 #pragma unroll
     for (int k = 0; k < kDirs; ++k) dir[k] = v_star[((size_t)unit * b + nj) * BPC_D + tid + k * kFinishThreads];
   }
-  asm volatile("griddepcontrol.wait;" ::: "memory");         // (the lengths and directions are older than the kernel before)
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  pdl_wait();                                              // (the lengths and directions are older than the kernel before)
   const double* w = wpart + (size_t)unit * parts * kBits * BPC_D + (size_t)i * BPC_D + kFinishChannels * rank + c;
   double ws = w[0];
 #pragma unroll 16
@@ -1404,22 +1405,6 @@ int sweep_cluster(const bpc_config* c, const int* active) {
   return best;
 }
 
-// Ordinary launch, or one that may start while the kernel before it drains (both kernels then mark the point).
-template <typename... A, typename... B>
-cudaError_t launch_after(bool early, void (*kernel)(A...), dim3 grid, int threads, size_t smem, cudaStream_t stream, B... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = early ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kernel, static_cast<A>(args)...);
-}
-
 template <int GROUPS>
 cudaError_t launch_project_tc(const bpc_ctx* ctx, const CUtensorMap& kmap, const uint32_t* hfit, const float* v_star, const float* cross, float* T,
                               uint32_t* t_max, int blk, int parts, int ts, bool early, cudaStream_t stream) {
@@ -1427,7 +1412,7 @@ cudaError_t launch_project_tc(const bpc_ctx* ctx, const CUtensorMap& kmap, const
   const size_t smem = (size_t)GROUPS * (kTileBytes + kTileKeys * kSignCols * 2) + (size_t)kProjN * 256 + (size_t)blk * kProjN * 64 + 1024;
   cudaError_t e = allow_smem(fit_project_tc_kernel<GROUPS>);
   if (e != cudaSuccess) return e;
-  return launch_after(early, fit_project_tc_kernel<GROUPS>, dim3(parts, ctx->units), kGroupThreads * GROUPS, smem, stream, kmap, hfit, v_star, cross, T, t_max,
+  return launch_pdl(early, fit_project_tc_kernel<GROUPS>, dim3(parts, ctx->units), kGroupThreads * GROUPS, smem, stream, kmap, hfit, v_star, cross, T, t_max,
                       (const int32_t*)ctx->unit_lens, ctx->dev_err, (int)c.n_max, (int)c.code_bits, blk, ts);
 }
 
@@ -1438,7 +1423,7 @@ cudaError_t launch_gather_tc(const bpc_ctx* ctx, const CUtensorMap& kmap, const 
   const size_t smem = gather_smem(GROUPS, blk);
   cudaError_t e = allow_smem(fit_gather_tc_kernel<GROUPS>);
   if (e != cudaSuccess) return e;
-  return launch_after(early, fit_gather_tc_kernel<GROUPS>, dim3(parts, ctx->units), kGroupThreads * GROUPS, smem, stream, kmap, hfit, wpart, apart,
+  return launch_pdl(early, fit_gather_tc_kernel<GROUPS>, dim3(parts, ctx->units), kGroupThreads * GROUPS, smem, stream, kmap, hfit, wpart, apart,
                       (const int32_t*)ctx->unit_lens, ctx->dev_err, (int)c.n_max, (int)c.code_bits, blk);
 }
 
@@ -1511,7 +1496,7 @@ cudaError_t bpc_launch_fit_blocked(bpc_ctx* ctx, const void* k_cache, const floa
     if (one_finish) {
       e = allow_smem(fit_finish_kernel);
       if (e != cudaSuccess) return e;
-      e = launch_after(early, fit_finish_kernel, dim3(kFinishBlocks * ctx->units), kFinishThreads, FinishSmem(blk).total * sizeof(double), stream,
+      e = launch_pdl(early, fit_finish_kernel, dim3(kFinishBlocks * ctx->units), kFinishThreads, FinishSmem(blk).total * sizeof(double), stream,
                        (const double*)wpart, (const int32_t*)apart, v_star, ctx->P, cross, (const int32_t*)ctx->unit_lens, (int)c.n_max, b, blk, parts);
       *launches += 4;
       continue;

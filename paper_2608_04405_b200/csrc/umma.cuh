@@ -104,6 +104,24 @@ __device__ __forceinline__ void split3(float v, __nv_bfloat16 (&t)[3]) {
   t[2] = __float2bfloat16_rn(r1 - __bfloat162float(t[1]));
 }
 
+// the same for eight values: each term as 16 bytes, eight consecutive K elements of an operand row
+__device__ __forceinline__ void split3x8(const float (&v)[8], uint4 (&t)[3]) {
+  uint32_t w[3][4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    __nv_bfloat16 a[3], b[3];
+    split3(v[2 * e], a);
+    split3(v[2 * e + 1], b);
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+      const __nv_bfloat162 ab = __halves2bfloat162(a[p], b[p]);
+      w[p][e] = *reinterpret_cast<const uint32_t*>(&ab);
+    }
+  }
+#pragma unroll
+  for (int p = 0; p < 3; ++p) t[p] = make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]);
+}
+
 // the same MMA with operand A in tensor memory: one row per lane, two consecutive K elements per column
 __device__ __forceinline__ void umma_bf16_ta(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
