@@ -159,39 +159,69 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __nv_bfloat16* 
   pdl_wait();
   const int n = min(unit_lens[unit], n_max);
   const int ntiles = (n + kTileKeys - 1) / kTileKeys;
+  if (tid == 0) {                                            // the warpgroups' first key tiles come in under the set-up
+    for (int g = 0; g < kGroups; ++g)
+      if (kGroups * (int)blockIdx.x + g < ntiles)
+        tma::load_key_tile(smem + (size_t)g * A_BYTES, &kmap, unit * n_max + (kGroups * (int)blockIdx.x + g) * kTileKeys, &tile_bar_s[g]);
+  }
   {
-    const unsigned char* psrc = reinterpret_cast<const unsigned char*>(Ph + ((size_t)set * TOTAL + ROW0) * BPC_D);
-    for (int c = tid; c < NBITS * 16; c += kThreads) {
-      const int r = c >> 4, ch = c & 15;
-      *reinterpret_cast<uint4*>(b_s + sw128_offset(NBITS, r, ch)) = *reinterpret_cast<const uint4*>(psrc + (size_t)r * 256 + ch * 16);
-    }
+    // Projection rows, diagonal blocks (fp32, for the in-register sweep) and the Gram terms: everything is requested before anything is
+    // stored, one latency in all.
+    // -G[16 pb + i][j], j after block pb, as three bf16 terms (g = t1 + t2 + t3 up to 2^-24 |g|); operand rows j, K index i.  Eight
+    // consecutive i at a time are one 16-byte store per term.  (One element at a time, in stores of 2 bytes, and one loop after
+    // the other: 22.6 us for 8 x 4K keys, ENC4K now.)
+    const uint4* psrc = reinterpret_cast<const uint4*>(Ph + ((size_t)set * TOTAL + ROW0) * BPC_D);
     const float* gfull = gram + (size_t)set * TOTAL * TOTAL;
     const float* gsrc = gfull + (size_t)ROW0 * TOTAL + ROW0;  // this launch's diagonal block of the Gram matrix, row stride TOTAL
-    for (int c = tid; c < NS * kSub * kSub; c += kThreads) {  // diagonal blocks, kept in fp32 for the in-register sweep
-      const int d = c / (kSub * kSub), i = c / kSub % kSub, j = c % kSub;
-      gd_s[c] = gsrc[(size_t)(kSub * d + i) * TOTAL + kSub * d + j];
-    }
-    // minus eight elements of a Gram column from row i0 on, as K elements i0 .. i0 + 7 of row `row` of the operands of the three terms
-    auto put_terms = [&](unsigned char* base, int term_bytes, int rows, int row, int i0, const float* column) {
-      float v[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) v[e] = -column[(size_t)(i0 + e) * TOTAL];
+    constexpr int kRows = NBITS * 16, kDiag = NS * kSub * kSub, kTerms = (NS - 1) * 2 * NBITS;
+    constexpr int kRowsEach = (kRows + kThreads - 1) / kThreads, kDiagEach = (kDiag + kThreads - 1) / kThreads, kTermsEach = (kTerms + kThreads - 1) / kThreads;
+    uint4 row[kRowsEach];
+    float diag[kDiagEach], term[kTermsEach][8];
+    auto put_terms = [&](unsigned char* base, int term_bytes, int rows, int r, int i0, const float (&v)[8]) {   // K elements i0 .. i0 + 7 of operand row r
       uint4 t3[3];
       split3x8(v, t3);
 #pragma unroll
-      for (int p = 0; p < 3; ++p) *reinterpret_cast<uint4*>(base + (size_t)p * term_bytes + nosw_offset(rows, row, i0)) = t3[p];
+      for (int p = 0; p < 3; ++p) *reinterpret_cast<uint4*>(base + (size_t)p * term_bytes + nosw_offset(rows, r, i0)) = t3[p];
     };
+#pragma unroll
+    for (int k = 0; k < kRowsEach; ++k)
+      if (tid + k * kThreads < kRows) row[k] = psrc[tid + k * kThreads];
+#pragma unroll
+    for (int k = 0; k < kDiagEach; ++k) {
+      const int c = tid + k * kThreads, d = c / (kSub * kSub), i = c / kSub % kSub, j = c % kSub;
+      if (c < kDiag) diag[k] = gsrc[(size_t)(kSub * d + i) * TOTAL + kSub * d + j];
+    }
+#pragma unroll
+    for (int k = 0; k < kTermsEach; ++k) {
+      const int c = tid + k * kThreads, pb = c / (2 * NBITS), i0 = 8 * (c / NBITS % 2), j = c % NBITS;
+      if (c < kTerms && j >= kSub * (pb + 1)) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) term[k][e] = -gsrc[(size_t)(kSub * pb + i0 + e) * TOTAL + j];
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < kRowsEach; ++k) {
+      const int c = tid + k * kThreads;
+      if (c < kRows) *reinterpret_cast<uint4*>(b_s + sw128_offset(NBITS, c >> 4, c & 15)) = row[k];
+    }
+#pragma unroll
+    for (int k = 0; k < kDiagEach; ++k)
+      if (tid + k * kThreads < kDiag) gd_s[tid + k * kThreads] = diag[k];
+#pragma unroll
+    for (int k = 0; k < kTermsEach; ++k) {
+      const int c = tid + k * kThreads, pb = c / (2 * NBITS), i0 = 8 * (c / NBITS % 2), j = c % NBITS, j0 = kSub * (pb + 1);
+      if (c < kTerms && j >= j0) put_terms(gb_s + gb_off(pb), gb_cols(pb) * kSub * 2, gb_cols(pb), j - j0, i0, term[k]);
+    }
     if constexpr (HALF == 2) {
       // -G[i][128 + j] for the first half's bits i, as three bf16 terms; operand rows j, K index i, [128 x 128] each
-      for (int c = tid; c < 16 * 128; c += kThreads) put_terms(x_s, 32768, 128, c & 127, 8 * (c >> 7), gfull + 128 + (c & 127));
-    }
-    // -G[16 pb + i][j], j after block pb, as three bf16 terms (g = t1 + t2 + t3 up to 2^-24 |g|); operand rows j, K index i.  Eight
-    // consecutive i at a time are one 16-byte store per term (one element at a time, in stores of 2 bytes, the set-up of a
-    // block took PRO_BEFORE us of the 22 that 8 x 4K keys take).
-    for (int c = tid; c < (NS - 1) * 2 * NBITS; c += kThreads) {
-      const int pb = c / (2 * NBITS), i0 = 8 * (c / NBITS % 2), j = c % NBITS, j0 = kSub * (pb + 1);
-      if (j < j0) continue;
-      put_terms(gb_s + gb_off(pb), gb_cols(pb) * kSub * 2, gb_cols(pb), j - j0, i0, gsrc + (size_t)(kSub * pb) * TOTAL + j);
+#pragma unroll 2
+      for (int c = tid; c < 16 * 128; c += kThreads) {
+        const int i0 = 8 * (c >> 7), j = c & 127;
+        float v[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] = -gfull[(size_t)(i0 + e) * TOTAL + 128 + j];
+        put_terms(x_s, 32768, 128, j, i0, v);
+      }
     }
   }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy writes -> visible to the tensor core
@@ -257,10 +287,7 @@ encode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __nv_bfloat16* 
   const int tile_step = kGroups * blocks_per_unit;
   int tl = grp < kGroups ? kGroups * blockIdx.x + grp : ntiles;
   unsigned ph = 0;                                           // phase of the MMA barrier the next wait refers to
-  if (tl < ntiles && gtid == 0) {
-    load_tile(tl);
-    issue_gemm();
-  }
+  if (tl < ntiles && gtid == 0) issue_gemm();
   for (; tl < ntiles; tl += tile_step) {
     const int next = tl + tile_step;
     // decision values of this tile: wait for the MMAs, then one TMEM lane (one key) per thread

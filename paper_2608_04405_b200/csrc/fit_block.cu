@@ -151,6 +151,9 @@ fit_project_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* 
   if (tid == 0) {
     for (int g = 0; g < GROUPS; ++g) { mbar_init(&bar_s[g], 1); mbar_init(&tile_bar_s[g], 1); timed_out_g[g] = 0; }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    // (the warpgroups' first tiles: no kernel of the fit writes keys)
+    for (int g = 0; g < min(GROUPS, ntile); ++g)
+      tma::load_key_tile(smem + (size_t)g * kTileBytes, &kmap, unit * n_max + row0 + (ntile - 1 - g) * kTileKeys, &tile_bar_s[g]);
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"(512) : "memory");
@@ -191,7 +194,6 @@ fit_project_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* 
   unsigned long long* bar = &bar_s[grp];
   const uint32_t idesc = umma_idesc_bf16(kTileKeys, kProjN);
 
-  if (grp < ntile && gtid == 0) load_tile(grp);
   unsigned ph = 0, tph = 0;
   uint32_t first[kSignCols / 32];                                      // the next tile's first code words of this thread's key
   auto load_words = [&](int tile) {
@@ -381,6 +383,8 @@ fit_gather_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* _
   if (tid == 0) {
     for (int g = 0; g < GROUPS; ++g) { mbar_init(&bar_s[g], 1); mbar_init(&tile_bar_s[g], 1); timed_out_g[g] = 0; }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    for (int g = 0; g < min(GROUPS, ntile); ++g)           // (the warpgroups' first tiles: no kernel of the fit writes keys)
+      tma::load_key_tile(smem + (size_t)g * kTileBytes, &kmap, unit * n_max + row0 + g * kTileKeys, &tile_bar_s[g]);
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"(512) : "memory");
@@ -409,7 +413,6 @@ fit_gather_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* _
   double acc[kBits];                                       // channel gtid
 #pragma unroll
   for (int i = 0; i < kBits; ++i) acc[i] = 0.0;
-  if (grp < ntile && gtid == 0) load_tile(grp);
   unsigned ph = 0, tph = 0;
   int since_flush = 0;
   bool first = true;
