@@ -188,7 +188,7 @@ inline cudaError_t launch_pdl(bool early, void (*kernel)(P...), dim3 grid, unsig
 // ---- prefill-side launchers (prefill.cu)
 // C[set][i][j] = A[set][i] . B[set][j] over BPC_D channels in fp64, for 32 x 32 tiles of rows (strides in elements)
 cudaError_t bpc_launch_dots(const float* A, size_t a_set, const float* B, size_t b_set, float* C, size_t c_set, int ldc, int tiles_a, int tiles_b,
-                            int sets, cudaStream_t stream);
+                            int sets, bool early, cudaStream_t stream);
 cudaError_t bpc_launch_finalize_projection(bpc_ctx* ctx, cudaStream_t stream);
 cudaError_t bpc_launch_encode_simple(bpc_ctx* ctx, const void* k_cache, uint64_t* codes, cudaStream_t stream);
 cudaError_t bpc_launch_append(bpc_ctx* ctx, const void* k_new, const void* v_new, void* k_cache, void* v_cache,

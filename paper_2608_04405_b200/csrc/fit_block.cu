@@ -1067,6 +1067,7 @@ fit_sweep_kernel(float* __restrict__ T, uint32_t* __restrict__ hfit, uint32_t* _
 __global__ void __launch_bounds__(256)
 fit_sum_parts_kernel(double* __restrict__ wpart, int32_t* __restrict__ apart, const int32_t* __restrict__ unit_lens, int n_max, int b,
                      int blk, int parts) {
+  pdl_wait();
   const int unit = blockIdx.y;
   const int n = min(unit_lens[unit], n_max);
   if (n <= 0) return;
@@ -1092,6 +1093,7 @@ fit_sum_parts_kernel(double* __restrict__ wpart, int32_t* __restrict__ apart, co
 __global__ void __launch_bounds__(512)
 fit_rows_kernel(const double* __restrict__ wpart, const int32_t* __restrict__ apart, float* __restrict__ P,
                 const int32_t* __restrict__ unit_lens, int n_max, int b, int blk, int parts) {
+  pdl_wait();
   extern __shared__ __align__(16) double rows_smem[];
   const int nj = kBits * (blk + 1), np = kBits * blk;
   double* corr = rows_smem;                                // [32][nj] u_i . u_j
@@ -1458,15 +1460,17 @@ cudaError_t bpc_launch_fit_blocked(bpc_ctx* ctx, const void* k_cache, const floa
   // on some device costs time only).  Fits of 32K keys and 128 bits: 4 units 532 -> 506 us, 8 units 598 -> 569, 12 units 673 -> 657, but
   // 16 units 854 -> 875.
   const bool one_finish = ctx->units <= 15;
-  // Then also each kernel is launched to start while the one before it drains.  (With more units every SM has work and it cost 1 to 3 %.)
-  const bool early = one_finish && tc && ctx->use_pdl;
+  // Each kernel is launched to start while the one before it drains: what it can set up, and request, lies before its wait.  (fp32 caches: their
+  // project and gather do not wait.)  Fits of 32K keys and 128 bits: 4 units 502 -> 461 us, 8 units 575 -> 535, 16 units 849 -> 809,
+  // 32 units 1183 -> 1171.
+  const bool early = tc && ctx->use_pdl;
   const dim3 grid(parts, ctx->units);
   CUtensorMap kmap;
   if (tc) e = tma::make_key_map(&kmap, k_cache, (unsigned long long)ctx->units * c.n_max, ctx->row_stride);
   for (int blk = 0; blk < b / kBits && e == cudaSuccess; ++blk) {
     if (blk > 0 && !one_finish) {                          // cross[j][l] = v_j . d_l for the bits so far and this block's columns
       const size_t set = (size_t)b * BPC_D;
-      e = bpc_launch_dots(ctx->P, set, v_star + (size_t)kBits * blk * BPC_D, set, cross, (size_t)b * kBits, kBits, blk, 1, ctx->units, stream);
+      e = bpc_launch_dots(ctx->P, set, v_star + (size_t)kBits * blk * BPC_D, set, cross, (size_t)b * kBits, kBits, blk, 1, ctx->units, early, stream);
       if (e != cudaSuccess) return e;
     }
     if (tc) {
@@ -1504,12 +1508,12 @@ cudaError_t bpc_launch_fit_blocked(bpc_ctx* ctx, const void* k_cache, const floa
       *launches += 4;
       continue;
     }
-    fit_sum_parts_kernel<<<dim3(16 + 4 * (blk + 1), ctx->units), 256, 0, stream>>>(wpart, apart, ctx->unit_lens, c.n_max, b, blk, parts);
+    e = launch_pdl(early, fit_sum_parts_kernel, dim3(16 + 4 * (blk + 1), ctx->units), 256, 0, stream, wpart, apart, ctx->unit_lens, c.n_max, b, blk, parts);
+    if (e != cudaSuccess) return e;
     const size_t rows_smem = (size_t)(kBits * kBits * (blk + 1) + kBits * blk * 32 + kBits * 32) * 8;
     e = allow_smem(fit_rows_kernel);
     if (e != cudaSuccess) return e;
-    fit_rows_kernel<<<dim3(4, ctx->units), 512, rows_smem, stream>>>(wpart, apart, ctx->P, ctx->unit_lens, c.n_max, b, blk, parts);
-    e = cudaGetLastError();
+    e = launch_pdl(early, fit_rows_kernel, dim3(4, ctx->units), 512, rows_smem, stream, wpart, apart, ctx->P, ctx->unit_lens, c.n_max, b, blk, parts);
     *launches += blk > 0 ? 6 : 5;
   }
   return e;

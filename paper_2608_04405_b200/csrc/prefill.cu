@@ -37,6 +37,7 @@ constexpr int kDotChannels = 64;
 __global__ void __launch_bounds__(kDotThreads)
 dots_kernel(const float* __restrict__ A, size_t a_set, const float* __restrict__ B, size_t b_set, float* __restrict__ C, size_t c_set, int ldc,
             int symmetric) {
+  pdl_wait();
   __shared__ double as[16][kDotChannels + 1], bs[32][kDotChannels + 1];
   const int i0 = 16 * blockIdx.x, j0 = 32 * blockIdx.y;
   if (symmetric && j0 + 31 < i0) return;
@@ -763,9 +764,8 @@ build_eas_kernel(const float* __restrict__ key_err, const int32_t* __restrict__ 
 
 // =========================================================================== host launchers
 cudaError_t bpc_launch_dots(const float* A, size_t a_set, const float* B, size_t b_set, float* C, size_t c_set, int ldc, int tiles_a, int tiles_b,
-                            int sets, cudaStream_t stream) {
-  dots_kernel<<<dim3(2 * tiles_a, tiles_b, sets), kDotThreads, 0, stream>>>(A, a_set, B, b_set, C, c_set, ldc, A == B);
-  return cudaGetLastError();
+                            int sets, bool early, cudaStream_t stream) {
+  return launch_pdl(early, dots_kernel, dim3(2 * tiles_a, tiles_b, sets), kDotThreads, 0, stream, A, a_set, B, b_set, C, c_set, ldc, A == B);
 }
 
 cudaError_t bpc_launch_finalize_projection(bpc_ctx* ctx, cudaStream_t stream) {
@@ -780,7 +780,7 @@ cudaError_t bpc_launch_finalize_projection(bpc_ctx* ctx, cudaStream_t stream) {
   ctx->launches += 2;
   const size_t set = (size_t)c.code_bits * BPC_D;
   return bpc_launch_dots(ctx->P_hf, set, ctx->P_hf, set, ctx->gram, (size_t)c.code_bits * c.code_bits, c.code_bits, c.code_bits / 32,
-                         c.code_bits / 32, c.hash_sets, stream);
+                         c.code_bits / 32, c.hash_sets, ctx->use_pdl, stream);
 }
 
 template <typename KV, int NB>
