@@ -169,7 +169,8 @@ __host__ __device__ inline int bpc_duo_unit(unsigned long long order, int first,
   return (int)((order >> (4 * (r / heads))) & 15u) * heads + r % heads;
 }
 
-// ---- a kernel that may be scheduled while its predecessor in the stream drains; it starts with pdl_wait()
+// ---- a kernel that may be scheduled while its predecessor in the stream drains; ahead of pdl_wait() it reads nothing that a kernel
+// before it may still be writing
 template <typename... P, typename... A>
 inline cudaError_t launch_pdl(bool early, void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t stream, A... args) {
   cudaLaunchConfig_t cfg = {};
@@ -214,7 +215,7 @@ cudaError_t bpc_launch_encode_tc(bpc_ctx* ctx, const void* k_cache, uint64_t* co
 
 // --------------------------------------------------------------------------- device helpers
 #ifdef __CUDACC__
-// First statement of a kernel launched with launch_pdl: waits for the kernels before it in the stream (their results are
+// In a kernel launched with launch_pdl, ahead of the first read of earlier results: waits for the kernels before it in the stream (their results are
 // visible afterwards), then lets the next one be scheduled.  No effect in an ordinary launch.
 __device__ __forceinline__ void pdl_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
