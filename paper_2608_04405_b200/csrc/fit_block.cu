@@ -1480,8 +1480,8 @@ cudaError_t bpc_launch_fit_blocked(bpc_ctx* ctx, const void* k_cache, const floa
     } else {
       e = cudaMemset2DAsync(t_max, column_max_at(1, 0, parts) * 4, 0, kBits * 4, ctx->units, stream);
       if (e != cudaSuccess) return e;
-      fit_project_f32_kernel<<<dim3(ts / kTileKeys, ctx->units), kTileKeys, 0, stream>>>(
-          (const float*)k_cache, hfit, v_star, cross, T, t_max, ctx->unit_lens, c.n_max, ctx->row_stride, b, blk, ts, parts);
+      e = launch_pdl(false, fit_project_f32_kernel, dim3(ts / kTileKeys, ctx->units), kTileKeys, 0, stream, (const float*)k_cache, hfit, v_star, cross, T,
+                     t_max, ctx->unit_lens, c.n_max, ctx->row_stride, b, blk, ts, parts);
     }
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr[2];
@@ -1497,7 +1497,8 @@ cudaError_t bpc_launch_fit_blocked(bpc_ctx* ctx, const void* k_cache, const floa
       else if (gather_smem(3, blk) <= kMaxSmem) e = launch_gather_tc<3>(ctx, kmap, hfit, wpart, apart, blk, parts, early, stream);
       else e = launch_gather_tc<2>(ctx, kmap, hfit, wpart, apart, blk, parts, early, stream);
     } else {
-      fit_gather_f32_kernel<<<grid, 256, 0, stream>>>((const float*)k_cache, hfit, wpart, apart, ctx->unit_lens, c.n_max, ctx->row_stride, b, blk);
+      e = launch_pdl(false, fit_gather_f32_kernel, grid, 256, 0, stream, (const float*)k_cache, hfit, wpart, apart, ctx->unit_lens, c.n_max, ctx->row_stride,
+                     b, blk);
     }
     if (e != cudaSuccess) return e;
     if (one_finish) {

@@ -773,10 +773,10 @@ cudaError_t bpc_launch_finalize_projection(bpc_ctx* ctx, cudaStream_t stream) {
   const size_t n = (size_t)c.hash_sets * c.code_bits * BPC_D;
   const int th = 256;
   const unsigned blocks = (unsigned)((n + th - 1) / th);
-  if (c.kv_dtype == BPC_BF16)
-    round_projection_kernel<__nv_bfloat16><<<blocks, th, 0, stream>>>(ctx->P, (__nv_bfloat16*)ctx->P_h, ctx->P_hf, n);
-  else
-    round_projection_kernel<float><<<blocks, th, 0, stream>>>(ctx->P, (float*)ctx->P_h, ctx->P_hf, n);
+  const cudaError_t e = c.kv_dtype == BPC_BF16
+      ? launch_pdl(false, round_projection_kernel<__nv_bfloat16>, blocks, th, 0, stream, ctx->P, (__nv_bfloat16*)ctx->P_h, ctx->P_hf, n)
+      : launch_pdl(false, round_projection_kernel<float>, blocks, th, 0, stream, ctx->P, (float*)ctx->P_h, ctx->P_hf, n);
+  if (e != cudaSuccess) return e;
   ctx->launches += 2;
   const size_t set = (size_t)c.code_bits * BPC_D;
   return bpc_launch_dots(ctx->P_hf, set, ctx->P_hf, set, ctx->gram, (size_t)c.code_bits * c.code_bits, c.code_bits, c.code_bits / 32,
