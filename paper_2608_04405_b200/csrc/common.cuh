@@ -215,12 +215,12 @@ cudaError_t bpc_launch_encode_tc(bpc_ctx* ctx, const void* k_cache, uint64_t* co
 
 // --------------------------------------------------------------------------- device helpers
 #ifdef __CUDACC__
-// In a kernel launched with launch_pdl, ahead of the first read of earlier results: waits for the kernels before it in the stream (their results are
-// visible afterwards), then lets the next one be scheduled.  No effect in an ordinary launch.
-__device__ __forceinline__ void pdl_wait() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
+// In a kernel launched with launch_pdl, ahead of the first read of earlier results: waits for the kernels before it in the stream (their
+// results are visible afterwards).  No effect in an ordinary launch.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// After it: lets the next kernel be scheduled once every block is here (one thread speaks for its block).  The next kernel may allocate tensor
+// memory ahead of its own wait, so a kernel that allocates some does this behind a barrier that follows the allocation.
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 __device__ __forceinline__ float bf16_lo(uint32_t x) { return __uint_as_float(x << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t x) { return __uint_as_float(x & 0xffff0000u); }

@@ -187,6 +187,7 @@ fit_project_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* 
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
+  pdl_release();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_all = tmem_base_s;
   const uint32_t tm_d = tmem_all + (uint32_t)(grp * kProjN);
@@ -404,6 +405,7 @@ fit_gather_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* _
   if (grp < ntile) load_words(grp);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
+  pdl_release();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_all = tmem_base_s;
   const uint32_t tm_w = tmem_all + (uint32_t)(grp * 96), tm_a = tm_w + 32;   // channel sums; inner products, 128 bits per 32 columns
@@ -945,6 +947,7 @@ fit_sweep_kernel(float* __restrict__ T, uint32_t* __restrict__ hfit, uint32_t* _
   if (WORDS == kWordsOnChip) asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");      // every rank's barriers are armed
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  pdl_release();
   if (WORDS == kWordsOnChip) asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   double new_row = 0.0;
   const uint32_t aw_tmem = WORDS == kWordsOnChip ? tmem_base_s + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(warp >> 2) * 128u : 0u;
@@ -1068,6 +1071,7 @@ __global__ void __launch_bounds__(256)
 fit_sum_parts_kernel(double* __restrict__ wpart, int32_t* __restrict__ apart, const int32_t* __restrict__ unit_lens, int n_max, int b,
                      int blk, int parts) {
   pdl_wait();
+  pdl_release();
   const int unit = blockIdx.y;
   const int n = min(unit_lens[unit], n_max);
   if (n <= 0) return;
@@ -1094,6 +1098,7 @@ __global__ void __launch_bounds__(512)
 fit_rows_kernel(const double* __restrict__ wpart, const int32_t* __restrict__ apart, float* __restrict__ P,
                 const int32_t* __restrict__ unit_lens, int n_max, int b, int blk, int parts) {
   pdl_wait();
+  pdl_release();
   extern __shared__ __align__(16) double rows_smem[];
   const int nj = kBits * (blk + 1), np = kBits * blk;
   double* corr = rows_smem;                                // [32][nj] u_i . u_j
@@ -1184,7 +1189,7 @@ fit_finish_kernel(const double* __restrict__ wpart, const int32_t* __restrict__ 
   const int n = min(unit_lens[unit], n_max);
   float* Pu = P + (size_t)unit * b * BPC_D;
   if (n <= 0) {                                            // (the whole cluster)
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    pdl_wait();
     Pu[(size_t)(np + i) * BPC_D + kFinishChannels * rank + c] = 0.f;
     return;
   }
@@ -1199,6 +1204,7 @@ fit_finish_kernel(const double* __restrict__ wpart, const int32_t* __restrict__ 
     for (int k = 0; k < kDirs; ++k) dir[k] = v_star[((size_t)unit * b + nj) * BPC_D + tid + k * kFinishThreads];
   }
   pdl_wait();                                              // (the lengths and directions are older than the kernel before)
+  pdl_release();
   const double* w = wpart + (size_t)unit * parts * kBits * BPC_D + (size_t)i * BPC_D + kFinishChannels * rank + c;
   double ws = w[0];
 #pragma unroll 16

@@ -38,6 +38,7 @@ __global__ void __launch_bounds__(kDotThreads)
 dots_kernel(const float* __restrict__ A, size_t a_set, const float* __restrict__ B, size_t b_set, float* __restrict__ C, size_t c_set, int ldc,
             int symmetric) {
   pdl_wait();
+  pdl_release();
   __shared__ double as[16][kDotChannels + 1], bs[32][kDotChannels + 1];
   const int i0 = 16 * blockIdx.x, j0 = 32 * blockIdx.y;
   if (symmetric && j0 + 31 < i0) return;
@@ -109,6 +110,7 @@ encode_simple_kernel(const KV* __restrict__ k_cache, const float* __restrict__ P
   float* g_s = reinterpret_cast<float*>(smem + sizeof(EncSmem<NB>));     // [b][b] where it fits
   const int unit = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   pdl_wait();
+  pdl_release();
   const int n = min(unit_lens[unit], n_max);
   if (blockIdx.x * kEncKeys >= n) return;                            // uniform over the block
   const int set = shared_sets ? unit % n_kv_heads : unit;
@@ -247,6 +249,7 @@ append_kernel(const KV* __restrict__ k_new, const KV* __restrict__ v_new, KV* __
               int32_t* __restrict__ unit_lens, int32_t* __restrict__ err, int n_kv_heads, int n_max, int row_stride,
               int b, int shared_sets, int residual_correction) {
   pdl_wait();
+  pdl_release();
   extern __shared__ __align__(16) unsigned char smem[];
   // the 32 x 32 blocks of the Gram matrix on and to the right of the diagonal (the only ones the sweep reads), block
   // (r, c) at slot r * nb - r (r - 1) / 2 + (c - r): 144 KB at 256 bits
