@@ -915,6 +915,7 @@ fit_sweep_kernel(float* __restrict__ T, uint32_t* __restrict__ hfit, uint32_t* _
   for (int q = 0; q < kTabs; ++q) st.tab[q] = 0.f;
 #pragma unroll
   for (int q = 0; q < 4; ++q) st.aw[q][0] = st.aw[q][1] = st.w[2 * q] = st.w[2 * q + 1] = 0u;
+  if (WORDS == kWordsGlobal) pdl_wait();                   // (the words below are not this block's own memory)
   for (int i = tid; i < nk / 4; i += kSweepThreads) reinterpret_cast<uint4*>(ws)[i] = make_uint4(0u, 0u, 0u, 0u);
   if (tid < kTabs * kTabBits) c_s[tid] = 0.0;
   if (tid < kStageRow / 4) ones_s[tid] = 0x01010101u;

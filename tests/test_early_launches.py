@@ -6,6 +6,7 @@ import re
 import pytest
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2608_04405_b200", "csrc")
+WAIT = r"pdl_wait\(\)|griddepcontrol\.wait"
 RELEASE, ALLOC = r"pdl_release\(\)|griddepcontrol\.launch_dependents", r"tcgen05\.alloc"
 BLOCK_BARRIER = r"__syncthreads\(\)|barrier\.cluster\.wait"
 
@@ -50,3 +51,17 @@ def test_tensor_memory_is_held_before_the_next_kernel_may_start(kernel):
     alloc = re.search(ALLOC, body).end()
     barrier = alloc + re.search(BLOCK_BARRIER, body[alloc:]).end()
     assert not re.search(RELEASE, body[:barrier])
+
+
+@pytest.mark.parametrize("kernel", EARLY)
+def test_nothing_is_written_to_global_memory_ahead_of_the_wait(kernel):
+    """What lies there may be in use by the kernel before, or by the one before that."""
+    params, body = KERNELS[kernel]
+    ahead = body[:re.search(WAIT, body).start()]
+    for f in re.findall(r"\*\s*(?:__restrict__\s+)?(\w+)", ",".join(p for p in params.split(",") if "const" not in p)):
+        names = {f}
+        for m in re.finditer(r"\*\s*(\w+)\s*=([^;]*);", ahead):
+            if names & set(re.findall(r"\w+", m.group(2))):
+                names.add(m.group(1))
+        for name in names:
+            assert not re.search(r"(?:\b%s|\(%s\))\s*\[[^;=]*\]\s*[-+|&]?=(?!=)" % (name, name), ahead), name
