@@ -170,8 +170,9 @@ __host__ __device__ inline int bpc_duo_unit(unsigned long long order, int first,
 }
 
 // ---- a kernel that may be scheduled while its predecessor in the stream drains; ahead of pdl_wait() it reads nothing that a kernel
-// before it may still be writing, and writes nothing to global memory.  Returns the launch's own status: that of a <<< >>> launch
-// before it would stay behind unseen.
+// before it may still be writing, and writes nothing to global memory.  What such a kernel writes is read through pointers that
+// are not `const __restrict__` (see tests/test_early_launches.py).  Returns the launch's own status: that of a <<< >>> launch before it would stay
+// behind unseen.
 template <typename... P, typename... A>
 inline cudaError_t launch_pdl(bool early, void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t stream, A... args) {
   cudaLaunchConfig_t cfg = {};

@@ -100,8 +100,8 @@ __device__ __forceinline__ void diag_sweep(float (&t)[kSub], uint32_t& word, flo
 
 template <int NBITS, int GROUPS, int HALF, bool ERR>
 __global__ void __launch_bounds__(kGroupThreads * (GROUPS + setup_groups(HALF)), 1)
-encode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __nv_bfloat16* __restrict__ Ph, const float* __restrict__ gram,
-                 const int32_t* __restrict__ unit_lens, uint64_t* __restrict__ codes, int32_t* __restrict__ err,
+encode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __nv_bfloat16* Ph, const float* gram,
+                 const int32_t* unit_lens, uint64_t* __restrict__ codes, int32_t* __restrict__ err,
                  int n_kv_heads, int n_max, int shared_sets, int residual_correction, int blocks_per_unit,
                  float* __restrict__ key_err) {
   extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -119,8 +119,8 @@ constexpr int kProjN = 3 * kBits;
 
 template <int GROUPS>
 __global__ void __launch_bounds__(kGroupThreads * GROUPS, 1)
-fit_project_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* __restrict__ hfit, const float* __restrict__ v_star,
-                      const float* __restrict__ cross, float* __restrict__ T, uint32_t* __restrict__ t_max,
+fit_project_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* hfit, const float* __restrict__ v_star,
+                      const float* cross, float* __restrict__ T, uint32_t* __restrict__ t_max,
                       const int32_t* __restrict__ unit_lens, int32_t* __restrict__ err, int n_max, int b, int blk, int t_stride) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -356,7 +356,7 @@ constexpr int kFlushTiles = 3;
 
 template <int GROUPS>
 __global__ void __launch_bounds__(kGroupThreads * GROUPS, 1)
-fit_gather_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* __restrict__ hfit, double* __restrict__ wpart,
+fit_gather_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* hfit, double* __restrict__ wpart,
                      int32_t* __restrict__ apart, const int32_t* __restrict__ unit_lens, int32_t* __restrict__ err, int n_max,
                      int b, int blk) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -881,7 +881,7 @@ __device__ __forceinline__ void add_b32(const void* dst, const void* bar, int r,
 
 template <int WORDS>
 __global__ void __launch_bounds__(kSweepThreads, 1)
-fit_sweep_kernel(float* __restrict__ T, uint32_t* __restrict__ hfit, uint32_t* __restrict__ words_g, const uint32_t* __restrict__ t_max,
+fit_sweep_kernel(float* __restrict__ T, uint32_t* __restrict__ hfit, uint32_t* __restrict__ words_g, const uint32_t* t_max,
                  const int32_t* __restrict__ unit_lens, int32_t* __restrict__ err, int n_max, int b, int blk, int t_stride, int parts,
                  int t_parts, int cluster_size, int wait_tries) {
   extern __shared__ __align__(16) unsigned char sweep_smem[];   // this block's code words (unless global)
@@ -1096,7 +1096,7 @@ fit_sum_parts_kernel(double* __restrict__ wpart, int32_t* __restrict__ apart, co
 // v_i = (W_i - sum_{j<i} (u_i . u_j) v_j) / n for the block's 32 bits; grid (4, units), a block has 32 channels.  Thread
 // (row pair, channel) takes off the earlier blocks' rows, then one warp runs the block's own triangle in registers.
 __global__ void __launch_bounds__(512)
-fit_rows_kernel(const double* __restrict__ wpart, const int32_t* __restrict__ apart, float* __restrict__ P,
+fit_rows_kernel(const double* wpart, const int32_t* apart, float* __restrict__ P,
                 const int32_t* __restrict__ unit_lens, int n_max, int b, int blk, int parts) {
   pdl_wait();
   pdl_release();
@@ -1178,7 +1178,7 @@ __device__ __forceinline__ void store_peer(const double* dst, int r, double v) {
 }
 
 __global__ void __cluster_dims__(kFinishBlocks, 1, 1) __launch_bounds__(kFinishThreads, 1)
-fit_finish_kernel(const double* __restrict__ wpart, const int32_t* __restrict__ apart, const float* __restrict__ v_star, float* __restrict__ P,
+fit_finish_kernel(const double* wpart, const int32_t* apart, const float* __restrict__ v_star, float* __restrict__ P,
                   float* __restrict__ cross, const int32_t* __restrict__ unit_lens, int n_max, int b, int blk, int parts) {
   extern __shared__ __align__(16) double finish_smem[];
   const FinishSmem at(blk);

@@ -35,7 +35,7 @@ template <> __global__ void round_projection_kernel<__nv_bfloat16>(const float* 
 constexpr int kDotThreads = 128;
 constexpr int kDotChannels = 64;
 __global__ void __launch_bounds__(kDotThreads)
-dots_kernel(const float* __restrict__ A, size_t a_set, const float* __restrict__ B, size_t b_set, float* __restrict__ C, size_t c_set, int ldc,
+dots_kernel(const float* A, size_t a_set, const float* B, size_t b_set, float* __restrict__ C, size_t c_set, int ldc,
             int symmetric) {
   pdl_wait();
   pdl_release();
@@ -84,8 +84,8 @@ dots_kernel(const float* __restrict__ A, size_t a_set, const float* __restrict__
 // one FMA per 32 columns, and a block's word is one ballot at its end, because a decided column keeps its decision value.  The
 // chunks of the projection are requested one ahead and the Gram matrix arrives by asynchronous copies, so that no global latency but
 // the first is waited for.  Bound by the product's fp64 issue and shared-memory reads (two channels a read) and by the chain of
-// decisions, with eight warps per SM to hide it.  4096 keys x 64 bits: 18.4 -> 12.3 us with those (160 with one thread per key, its
-// own conversions and a column-by-column sweep, which filled 32 SMs).
+// decisions, with eight warps per SM to hide it.  4096 keys x 64 bits: 18.4 -> 12.3 us with those, 12.1 with the keys requested
+// before anything is waited for (160 with one thread per key, its own conversions and a column-by-column sweep, which filled 32 SMs).
 constexpr int kEncThreads = 256;
 constexpr int kEncKeys = 32;
 constexpr int kEncBits = 64;                                         // bits of a projection pass
@@ -101,8 +101,8 @@ struct EncSmem {
 
 template <typename KV, int NB>                                       // NB = code words per key
 __global__ void __launch_bounds__(kEncThreads)
-encode_simple_kernel(const KV* __restrict__ k_cache, const float* __restrict__ Phf, const float* __restrict__ gram,
-                     const int32_t* __restrict__ unit_lens, uint64_t* __restrict__ codes, int n_kv_heads, int n_max,
+encode_simple_kernel(const KV* k_cache, const float* Phf, const float* gram,
+                     const int32_t* unit_lens, uint64_t* __restrict__ codes, int n_kv_heads, int n_max,
                      int row_stride, int shared_sets, int residual_correction, float* __restrict__ key_err) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int b = 32 * NB;
@@ -116,9 +116,6 @@ encode_simple_kernel(const KV* __restrict__ k_cache, const float* __restrict__ P
   const int set = shared_sets ? unit % n_kv_heads : unit;
   const float* Pset = Phf + (size_t)set * b * BPC_D;
   const float* Gset = gram + (size_t)set * b * b;
-  if (b <= kEncGramBits && residual_correction)
-    for (int i = tid; i < b * b / 4; i += kEncThreads)               // (lands during the product)
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(g_s + 4 * i)), "l"(Gset + 4 * i) : "memory");
   // the rows of the projection one chunk ahead, in registers: chunk s holds channels 32 (s % 4) .. of bits 64 (s / 4) ..
   constexpr int JN = (b < kEncBits ? b : kEncBits) / 16;             // bits of a thread: tx, tx + 16, ...
   constexpr int kChunks = BPC_D / kEncChannels, kSteps = (b + kEncBits - 1) / kEncBits * kChunks;
@@ -132,11 +129,39 @@ encode_simple_kernel(const KV* __restrict__ k_cache, const float* __restrict__ P
     }
   };
   fetch(0);
+  // the keys as well, in 16-byte pieces (cache rows start on 16 bytes), but with 32 bits, where the registers cost more than the latency
+  // (8 x 4K keys 35.2 us against 37.2; 4K keys of 64 bits 12.4 with, 12.7 without, 4K of 256 55.2 and 56.6)
+  constexpr bool kKeysAhead = NB > 1;
+  constexpr int kVec = 16 / (int)sizeof(KV), kKeysEach = kEncKeys * BPC_D / kVec / kEncThreads;
+  uint4 keys[kKeysEach];
+  auto fetch_keys = [&](int key0) {
+#pragma unroll
+    for (int m = 0; m < kKeysEach; ++m) {
+      const int e = (tid + m * kEncThreads) * kVec, r = e / BPC_D, c = e % BPC_D;
+      keys[m] = key0 + r < n ? *reinterpret_cast<const uint4*>(k_cache + ((size_t)unit * n_max + key0 + r) * row_stride + c) : make_uint4(0u, 0u, 0u, 0u);
+    }
+  };
+  if constexpr (kKeysAhead) fetch_keys(blockIdx.x * kEncKeys);
+  if (b <= kEncGramBits && residual_correction)
+    for (int i = tid; i < b * b / 4; i += kEncThreads)               // (lands during the product)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(g_s + 4 * i)), "l"(Gset + 4 * i) : "memory");
   for (int key0 = blockIdx.x * kEncKeys; key0 < n; key0 += gridDim.x * kEncKeys) {
+    if (kKeysAhead && key0 != blockIdx.x * kEncKeys) fetch_keys(key0);
     __syncthreads();
-    for (int e = tid; e < kEncKeys * BPC_D; e += kEncThreads) {
-      const int r = e / BPC_D, c = e % BPC_D;
-      sm.k[r][c] = key0 + r < n ? (double)to_float(k_cache[((size_t)unit * n_max + key0 + r) * row_stride + c]) : 0.0;
+    if constexpr (kKeysAhead) {
+#pragma unroll
+      for (int m = 0; m < kKeysEach; ++m) {
+        const int e = (tid + m * kEncThreads) * kVec;
+        const KV* x = reinterpret_cast<const KV*>(&keys[m]);
+        double* row = &sm.k[e / BPC_D][e % BPC_D];
+#pragma unroll
+        for (int i = 0; i < kVec; i += 2) *reinterpret_cast<double2*>(row + i) = make_double2((double)to_float(x[i]), (double)to_float(x[i + 1]));
+      }
+    } else {
+      for (int e = tid; e < kEncKeys * BPC_D; e += kEncThreads) {
+        const int r = e / BPC_D, c = e % BPC_D;
+        sm.k[r][c] = key0 + r < n ? (double)to_float(k_cache[((size_t)unit * n_max + key0 + r) * row_stride + c]) : 0.0;
+      }
     }
     const int tx = tid & 15, ty = tid >> 4;
     for (int j0 = 0; j0 < b; j0 += kEncBits) {
@@ -197,7 +222,7 @@ encode_simple_kernel(const KV* __restrict__ k_cache, const float* __restrict__ P
 #pragma unroll
           for (int w = cb; w < NB; ++w) {
             const size_t at = (size_t)(32 * cb + i) * b + 32 * w + lane;
-            g[w] = b <= kEncGramBits ? g_s[at] : __ldg(Gset + at);
+            g[w] = b <= kEncGramBits ? g_s[at] : Gset[at];
           }
 #pragma unroll
           for (int r = 0; r < 4; ++r) {
@@ -222,7 +247,7 @@ encode_simple_kernel(const KV* __restrict__ k_cache, const float* __restrict__ P
     if (key_err != nullptr) {
       // squared reconstruction error (Eq. 8) from the sweep: ||k - hP||^2 = ||k||^2 - 2 sum|t_i| + trace(G)
       double trg = 0.0;
-      for (int i = lane; i < b; i += 32) trg += (double)__ldg(Gset + (size_t)i * b + i);
+      for (int i = lane; i < b; i += 32) trg += (double)Gset[(size_t)i * b + i];
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
         double v = trg - 2.0 * abs_sum[r];
@@ -244,8 +269,8 @@ constexpr int kAppThreads = 256;
 
 template <typename KV>
 __global__ void __launch_bounds__(kAppThreads)
-append_kernel(const KV* __restrict__ k_new, const KV* __restrict__ v_new, KV* __restrict__ k_cache, KV* __restrict__ v_cache,
-              uint64_t* __restrict__ codes, const KV* __restrict__ Ph, const float* __restrict__ gram,
+append_kernel(const KV* k_new, const KV* v_new, KV* __restrict__ k_cache, KV* __restrict__ v_cache,
+              uint64_t* __restrict__ codes, const KV* Ph, const float* gram,
               int32_t* __restrict__ unit_lens, int32_t* __restrict__ err, int n_kv_heads, int n_max, int row_stride,
               int b, int shared_sets, int residual_correction) {
   pdl_wait();

@@ -65,3 +65,13 @@ def test_nothing_is_written_to_global_memory_ahead_of_the_wait(kernel):
                 names.add(m.group(1))
         for name in names:
             assert not re.search(r"(?:\b%s|\(%s\))\s*\[[^;=]*\]\s*[-+|&]?=(?!=)" % (name, name), ahead), name
+
+
+@pytest.mark.parametrize("kernel", EARLY)
+def test_what_the_kernel_before_writes_is_read_coherently(kernel):
+    """`const` with `__restrict__` allows loads through the read-only path and ahead of the wait: both need memory that nobody writes while the
+    kernel is resident, and it is resident while the one before still writes.  The directions and lengths of a fit are older."""
+    params, body = KERNELS[kernel]
+    older = {"v_star", "unit_lens"} if kernel.startswith("fit_block.cu") else set()
+    assert set(re.findall(r"const\s+\w+\s*\*\s*__restrict__\s+(\w+)", params)) <= older
+    assert "__ldg" not in body
