@@ -75,3 +75,9 @@ def test_what_the_kernel_before_writes_is_read_coherently(kernel):
     older = {"v_star", "unit_lens"} if kernel.startswith("fit_block.cu") else set()
     assert set(re.findall(r"const\s+\w+\s*\*\s*__restrict__\s+(\w+)", params)) <= older
     assert "__ldg" not in body
+
+
+def test_no_load_through_the_read_only_path():
+    """(the same for loads written out: the codes of a step may be those of the kernel before)"""
+    for f in os.listdir(CSRC):
+        assert "ld.global.nc" not in open(os.path.join(CSRC, f)).read(), f
