@@ -218,7 +218,8 @@ cudaError_t bpc_launch_encode_tc(bpc_ctx* ctx, const void* k_cache, uint64_t* co
 // --------------------------------------------------------------------------- device helpers
 #ifdef __CUDACC__
 // In a kernel launched with launch_pdl, ahead of the first read of earlier results: waits for the kernels before it in the stream (their
-// results are visible afterwards).  No effect in an ordinary launch.
+// results are visible afterwards).  Also where a block leaves early: a kernel that nobody in waits is no link of the chain.  No effect in an
+// ordinary launch.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // After it: lets the next kernel be scheduled once every block is here (one thread speaks for its block).  The next kernel may allocate tensor
 // memory ahead of its own wait, so a kernel that allocates some does this behind a barrier that follows the allocation.

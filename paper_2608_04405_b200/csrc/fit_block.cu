@@ -143,7 +143,7 @@ fit_project_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* 
   const int n = min(unit_lens[unit], n_max);
   const int rows = block_rows(n, gridDim.x);
   const int row0 = part * rows;
-  if (row0 >= n) return;                                               // uniform over the block, nothing set up yet
+  if (row0 >= n) { pdl_wait(); return; }                               // uniform over the block, nothing set up yet
   const int row_end = min(n, row0 + rows);
   const int ntile = (row_end - row0 + kTileKeys - 1) / kTileKeys;
   const int words = b / 32;
@@ -378,7 +378,7 @@ fit_gather_tc_kernel(const __grid_constant__ CUtensorMap kmap, const uint32_t* h
   const int n = min(unit_lens[unit], n_max);
   const int rows = block_rows(n, gridDim.x);
   const int row0 = blockIdx.x * rows;
-  if (row0 >= n) return;                                   // (the reduction skips blocks without rows)
+  if (row0 >= n) { pdl_wait(); return; }                   // (the reduction skips blocks without rows)
   const int row_end = min(n, row0 + rows);
   const int ntile = (row_end - row0 + kTileKeys - 1) / kTileKeys;
   if (tid == 0) {
@@ -903,7 +903,7 @@ fit_sweep_kernel(float* __restrict__ T, uint32_t* __restrict__ hfit, uint32_t* _
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int rank = blockIdx.x % cluster_size, unit = blockIdx.x / cluster_size;
   const int n = min(unit_lens[unit], n_max);
-  if (n <= 0) return;                                      // (the whole cluster)
+  if (n <= 0) { pdl_wait(); return; }                      // (the whole cluster)
   const int share = sweep_share(n, cluster_size);
   const int row0 = rank * share;
   const int nkeys = max(0, min(n - row0, share));          // keys of this block; nk = the same in whole groups

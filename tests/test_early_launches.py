@@ -81,3 +81,14 @@ def test_no_load_through_the_read_only_path():
     """(the same for loads written out: the codes of a step may be those of the kernel before)"""
     for f in os.listdir(CSRC):
         assert "ld.global.nc" not in open(os.path.join(CSRC, f)).read(), f
+
+
+@pytest.mark.parametrize("kernel", EARLY)
+def test_no_block_leaves_ahead_of_the_wait(kernel):
+    """A kernel whose blocks all leave ahead of their wait (lengths of zero) is over before the one before it, and what follows would start
+    beside that one."""
+    body = KERNELS[kernel][1]
+    ahead = body[:re.search(r"\n  (?:%s|asm volatile\(\"griddepcontrol\.wait)" % WAIT.split("|")[0], body).start()]
+    for m in re.finditer(r"\breturn;", ahead):
+        statement = ahead[max(ahead.rfind("if (", 0, m.start()), 0):m.start()]
+        assert re.search(WAIT, statement), statement
