@@ -1343,7 +1343,7 @@ struct Layout {
 };
 
 // Resident sweep clusters by size on a device (the kernel takes a whole SM per block, so this depends on nothing else);
-// asked for until it succeeds, then kept.
+// asked for until it succeeds, then kept.  The kernel after the gather is such a kernel too.
 struct SweepLimits {
   std::mutex lock;
   bool known;
@@ -1463,10 +1463,11 @@ cudaError_t bpc_launch_fit_blocked(bpc_ctx* ctx, const void* k_cache, const floa
   if (cs == 0) return cudaErrorNotSupported;
   const size_t sweep_smem = (size_t)sweep_share(c.n_max, cs) * 4;
   const bool tc = c.kv_dtype == BPC_BF16;
-  // One kernel after the gather while all its clusters are resident at once (15 of eight blocks, one to an SM; a guess that is wrong
-  // on some device costs time only).  Fits of 32K keys and 128 bits: 4 units 532 -> 506 us, 8 units 598 -> 569, 12 units 673 -> 657, but
-  // 16 units 854 -> 875.
-  const bool one_finish = ctx->units <= 15;
+  // One kernel after the gather while all its clusters are resident at once: like the sweep it takes an SM per block, so the sweep's limit is
+  // its own (15 clusters of eight on a B200).  Three kernels -> one, 128 bits, early launches: 32K keys 8 units 537 -> 511 us, 12 605 -> 595,
+  // 15 658 -> 644, but 16 785 -> 812 and 20 847 -> 871; 2K keys 8 units 329 -> 312, 15 329 -> 317, but 16 331 -> 355.  32 and 256 bits: the
+  // same line (15 units of 32K keys 158 -> 157 and 1546 -> 1518, 16 189 -> 195 and 1806 -> 1880).
+  const bool one_finish = ctx->units <= lim->active[kFinishBlocks];
   // Each kernel is launched to start while the one before it drains: what it can set up, and request, lies before its wait.  (fp32 caches: their
   // project and gather do not wait.)  Fits of 32K keys and 128 bits: 4 units 502 -> 461 us, 8 units 575 -> 535, 16 units 849 -> 809,
   // 32 units 1183 -> 1171.

@@ -66,7 +66,7 @@ cudaError_t cudaFuncGetAttributes(cudaFuncAttributes* a, const void*) { memset(a
 cudaError_t cudaGetSymbolAddress(void** p, const void*) { static char word[64]; *p = word; return cudaSuccess; }
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void*, int, size_t, unsigned) { *n = 1; return cudaSuccess; }
 cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void*, const cudaLaunchConfig_t* c) {
-  *n = 148 / (int)c->attrs[0].val.clusterDim.x;
+  *n = 120 / (int)c->attrs[0].val.clusterDim.x;          // (15 of eight, as on a B200)
   return cudaSuccess;
 }
 cudaError_t cudaGetDriverEntryPointByVersion(const char*, void** fn, unsigned, unsigned long long, cudaDriverEntryPointQueryResult* found) {
