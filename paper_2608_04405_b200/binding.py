@@ -133,11 +133,18 @@ def interleaved_kv(batch: int, n_kv_heads: int, n_max: int, head_dim: int, dtype
     return buf, buf[:, :, :, 0, :], buf[:, :, :, 1, :]
 
 
+# private to torch: 3.3 us less per call than the Stream object of the public function, which serves where a release has them no more
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream() -> int:
-    """The current stream of the current device, as torch.cuda.current_stream().cuda_stream without building the Stream object."""
+    """The current stream of the current device."""
+    if _raw_stream is None or _current_device is None:
+        return torch.cuda.current_stream().cuda_stream
     if not torch.cuda.is_initialized():
         torch.cuda.init()
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return _raw_stream(_current_device())
 
 
 def _check(status: int, what: str) -> None:

@@ -187,3 +187,25 @@ def test_fit_cluster_size_bounds_the_keys_of_a_block():
     assert B.plan_fit_cluster_size(B.make_config(1, 1, 1, (1 << 24) + 256, 128, torch.bfloat16), WHOLE[:2] + [0] * 15) == 0
     assert B.plan_fit_cluster_size(B.make_config(1, 32, 8, 32768, 128, torch.bfloat16), WHOLE) > 4
     assert B.plan_fit_cluster_size(longest, [0] * 17) == 0
+
+
+def test_stream_where_torch_has_no_raw_one(monkeypatch):
+    """The current stream comes from the public function where torch lacks the private ones."""
+    B = _binding()
+
+    class Stream:
+        cuda_stream = 4711
+
+    monkeypatch.setattr(torch.cuda, "current_stream", Stream)
+    for name in ("_raw_stream", "_current_device"):
+        with monkeypatch.context() as m:
+            m.setattr(B, name, None)
+            assert B._stream() == 4711
+
+
+@pytest.mark.gpu
+def test_stream_is_the_current_one():
+    B = _binding()
+    for s in (torch.cuda.current_stream(), torch.cuda.Stream(), torch.cuda.default_stream()):
+        with torch.cuda.stream(s):
+            assert B._stream() == s.cuda_stream
