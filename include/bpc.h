@@ -293,7 +293,7 @@ bpc_status bpc_debug_set_work_item_trace(bpc_ctx* ctx, uint64_t* trace);
  * otherwise.  bpc_status_of_device_error is that mapping as a pure function.  Then: last CUDA error code seen by the
  * context, number of kernels this context has launched so far.
  * Diagnostic switches (explicit calls; the library reads no environment variable): bpc_debug_set_pdl(ctx, 0) launches
- * the decode kernel without programmatic dependent launch; bpc_debug_set_tensor_core_encode(ctx, 0) makes
+ * every kernel (fit, projection, encode, append, decode) behind the end of the one before it; bpc_debug_set_tensor_core_encode(ctx, 0) makes
  * bpc_encode_keys and bpc_fit take the CUDA-core kernels instead of the tensor-core ones (bpc_fit then makes one pass
  * over the keys per bit); bpc_debug_force_streaming(ctx, 1) selects the streaming selection at any context length
  * (Hamming scores without the safeguard only) and re-plans the launch geometry;

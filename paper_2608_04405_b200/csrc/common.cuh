@@ -47,7 +47,7 @@ struct bpc_ctx {
   bool step_duo;            // the last decode step ran two blocks per SM
   bool cluster_forced;      // the caller has set a cluster size
   int wait_tries;           // tries after which waits for other blocks of a cluster give up
-  bool use_pdl;             // launch the decode kernel with programmatic stream serialization
+  bool use_pdl;             // launch kernels of fit, projection, encode, append and decode while the one before drains
   int duo_active[BPC_MAX_CLUSTER + 1];   // [cs]: resident clusters with two blocks per SM (0 = variant not used)
   int duo_cap;              // keys such a block can hold
   bool streaming;           // the scores of a full unit do not fit the largest cluster: two-pass (streaming) selection
