@@ -579,7 +579,7 @@ def run_ours(args):
         "roofline": _roofline(spec, lens_now, ms_step, peaks,
                               # dram__bytes_read.sum + dram__bytes_write.sum of one launch: not measured by this run, quoted
                               # from the committed profiler capture of this workload
-                              traffic=116.5e6 if (args.workload == 2 and not args.separate_kv) else None,
+                              traffic=116.8e6 if (args.workload == 2 and not args.separate_kv) else None,
                               traffic_source="ncu capture of one launch, profiles/decode_fused_cfg2_ncu.md (not measured in this run)"
                               if (args.workload == 2 and not args.separate_kv) else None),
         "timing": {"reps": args.reps, "us_per_step_median": ms_step * 1e3, "us_per_step_min": min(rep_ms) / K * 1e3,
