@@ -57,6 +57,7 @@ def test_tensor_memory_is_held_before_the_next_kernel_may_start(kernel):
 def test_nothing_is_written_to_global_memory_ahead_of_the_wait(kernel):
     """What lies there may be in use by the kernel before, or by the one before that."""
     params, body = KERNELS[kernel]
+    body = re.sub(r"\{\s*pdl_wait\(\);[^{}]*\breturn;\s*\}", "return;", body)   # (a block that leaves behind a wait of its own)
     ahead = body[:re.search(WAIT, body).start()]
     for f in re.findall(r"\*\s*(?:__restrict__\s+)?(\w+)", ",".join(p for p in params.split(",") if "const" not in p)):
         names = {f}
